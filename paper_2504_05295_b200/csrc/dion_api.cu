@@ -15,7 +15,7 @@
 #include "dion_internal.h"
 #include "orth_kernels.cuh"
 #include "simt_gemm.cuh"
-#include "umma_gemm.cuh"
+#include "umma_api.cuh"
 
 using namespace dion;
 
@@ -44,6 +44,13 @@ constexpr double GRAM_PAIR_MIN_FLOPS = 2e9;     // smallest rows r^2 whose Gram 
 constexpr double P_PAIR_MIN_MNR = 1.5e10;       // smallest m n r whose P = (M + G) Q runs on bf16 operand pairs first
 
 constexpr i64 NBO_COLS = 512;  // = NBO, the outer block of the two-level Cholesky (defined below)
+
+// One launch of k_chol_flow factors Gram matrices up to this order; beyond it blocks of 512 columns.
+constexpr i64 FLOW_MAX_R = 2048;
+constexpr double FLOW_SOLVE_MAX = 6e9;          // largest rows r^2 whose panel that launch solves too
+constexpr int FLOW_EXCLUSIVE_MAX = 8;           // matrices of a chain up to which its runners get an SM each
+constexpr int FLOW_AHEAD_MAX = 16;              // steps by which its preparations are handed out early
+constexpr i64 FLOW_MAX_PANEL_TILES = 800;       // ... and most 64-row blocks of it (the control block holds 64 such matrices)
 
 inline i64 align64(i64 floats) { return (floats + 63) / 64 * 64; }  // 256-byte granules
 
@@ -77,6 +84,8 @@ struct dion_ctx {
   size_t ws_bytes;
   int* dev_ints;  // [0] status, [1] skipped, [2..] per-step flags
   int flag_cursor;
+  int* flow_ctl = nullptr;   // progress counters of k_chol_flow (zero between launches)
+  i64 flow_ctl_cap = 0;
   int64_t launches;
   // per-phase profiling (off by default)
   bool prof_on;
@@ -296,6 +305,7 @@ int launch_gemm_simt(dion_ctx* c, GemmArgs g, cudaStream_t st, float* part, i64 
   if (use128) launch_pdl(k_gemm_simt<128, 128, 8, 8, 8>, grid, dim3(256), 0, st, g);
   else launch_pdl(k_gemm_simt<64, 64, 16, 4, 4>, grid, dim3(256), 0, st, g);
   DION_CHECK_LAUNCH(c);
+  if (g.splits_out != nullptr) { *g.splits_out = splits; return DION_OK; }      // (the caller sums the partial products itself)
   if (splits > 1) {
     const i64 total = g.M * g.N;
     int blocks = (int)((total + 255) / 256);
@@ -469,12 +479,29 @@ int launch_gemm_group(StepCtx& s, const std::vector<GemmArgs>& v) {
 int configure_kernels() {
   if (umma_configure() != DION_OK) return DION_ERR_CUDA;
   if (cudaFuncSetAttribute(k_probe_y4, cudaFuncAttributeMaxDynamicSharedMemorySize, PY_SMEM) != cudaSuccess ||
-      cudaFuncSetAttribute(k_chol_step, cudaFuncAttributeMaxDynamicSharedMemorySize, CHOL_STEP_SMEM) != cudaSuccess ||
+      cudaFuncSetAttribute(k_chol_flow<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, FLOW_SMEM) != cudaSuccess ||
+      cudaFuncSetAttribute(k_chol_flow<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, FLOW_SMEM) != cudaSuccess ||
       cudaFuncSetAttribute(k_tiny_cholqr2, cudaFuncAttributeMaxDynamicSharedMemorySize, tiny_cholqr2_smem(TINY_MAX_ROWS)) != cudaSuccess) {
     cudaGetLastError();
     return DION_ERR_CUDA;
   }
   return DION_OK;
+}
+
+// CTAs of k_chol_flow that fit an SM (the cooperative launch must not ask for more).
+int flow_ctas_per_sm() {
+  static std::atomic<int> cached{0};
+  int n = cached.load(std::memory_order_relaxed);
+  if (n > 0) return n;
+  int a = 0, b = 0;
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&a, k_chol_flow<true>, FLOW_THREADS, FLOW_SMEM) != cudaSuccess ||
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_chol_flow<false>, FLOW_THREADS, FLOW_SMEM) != cudaSuccess) {
+    cudaGetLastError();
+    return 1;
+  }
+  n = a < b ? a : b;
+  if (n > 0) cached.store(n, std::memory_order_relaxed);
+  return n;
 }
 
 constexpr i64 NBO = NBO_COLS;  // outer block of the two-level Cholesky
@@ -493,56 +520,6 @@ void over_batch(const StepCtx& s, GemmArgs& g) {
   g.skip_stride = OS_SLOT_INTS;
 }
 
-// Inverse of a lower-triangular matrix by doubling, on the diagonal square [o, o+sz):
-// [[L11,0],[L21,L22]]^-1 = [[X11,0],[-X22 L21 X11, X22]], for block sizes b_from, 2 b_from, ...
-// while b < sz.  The diagonal blocks of size b_from of Linv must already hold their inverses.
-// Offsets are relative to each matrix's scratch slice.
-int trtri_levels(StepCtx& s, i64 r, i64 o, i64 sz, i64 b_from, const int* skip, int precise) {
-  const float* Gm = s.ws + s.L.Gram;
-  float* Linv = s.ws + s.L.Linv;
-  float* Tbuf = s.ws + s.L.Tbuf;
-  for (i64 b = b_from; b < sz; b *= 2) {
-    const i64 nfull = sz / (2 * b);
-    const i64 tail0 = nfull * 2 * b;
-    const i64 b2_tail = (sz - tail0 > b) ? (sz - tail0 - b) : 0;
-    for (int pass = 0; pass < 2; ++pass) {
-      const i64 base = o + ((pass == 0) ? 0 : tail0);
-      const i64 rows = (pass == 0) ? b : b2_tail;
-      const int batch = (pass == 0) ? (int)nfull : 1;
-      if (rows <= 0 || batch <= 0) continue;
-      const i64 off21 = (base + b) * r + base, off11 = base * r + base, off22 = (base + b) * r + (base + b);
-      const i64 bs = 2 * b * (r + 1);
-      const bool big = b >= NBO;   // large blocks: one launch per pair and matrix, tensor cores where they qualify
-      const int launches = big ? batch : 1;
-      for (int q = 0; q < launches; ++q) {
-        const i64 sh = big ? (i64)q * bs : 0;
-        GemmArgs g1 = gemm_args();  // T = L21 * X11
-        g1.M = rows; g1.N = b; g1.K = b;
-        g1.A = Gm + off21 + sh; g1.a_si = r; g1.a_sk = 1;
-        g1.B = Linv + off11 + sh; g1.b_sk = r; g1.b_sn = 1;
-        g1.C = Tbuf + off21 + sh; g1.ldc = r; g1.epi = EPI_STORE; g1.skip_flag = skip; g1.precise = precise;
-        GemmArgs g2 = gemm_args();  // X21 = -X22 * T
-        g2.M = rows; g2.N = b; g2.K = rows;
-        g2.A = Linv + off22 + sh; g2.a_si = r; g2.a_sk = 1;
-        g2.B = Tbuf + off21 + sh; g2.b_sk = r; g2.b_sn = 1;
-        g2.C = Linv + off21 + sh; g2.ldc = r; g2.epi = EPI_STORE; g2.alpha = -1.f; g2.skip_flag = skip; g2.precise = precise;
-        if (big) {
-          DION_TRY(launch_gemm_chain(s, g1));
-          DION_TRY(launch_gemm_chain(s, g2));
-        } else {
-          g1.batch = batch; g1.bsA = bs; g1.bsB = bs; g1.bsC = bs; over_batch(s, g1);
-          g2.batch = batch; g2.bsA = bs; g2.bsB = bs; g2.bsC = bs; over_batch(s, g2);
-          DION_TRY(launch_gemm_simt(s.c, g1, s.st, nullptr, 0, false));
-          DION_TRY(launch_gemm_simt(s.c, g2, s.st, nullptr, 0, false));
-        }
-      }
-    }
-  }
-  return DION_OK;
-}
-
-// Cholesky of the diagonal square [o, o+sz) of each Gram matrix (sz <= NBO), right-looking with
-// 64-wide blocks on the FMA engine, followed by the inverse of that square's factor into Linv.
 // How a Cholesky-QR round runs.
 enum : int {
   RM_PLAIN = 0,     // no device-side control
@@ -556,67 +533,90 @@ enum : int {
 inline bool rm_skips(int mode) { return mode == RM_ADAPTIVE || mode == RM_CHECKED || mode == RM_REDO; }
 inline bool rm_precise(int mode) { return mode == RM_ADAPTIVE || mode == RM_FIRST || mode == RM_REDO; }
 
-int potrf_inner(StepCtx& s, i64 r, i64 o, i64 sz, int mode) {
-  const bool adaptive = rm_skips(mode);
+// ints of the control block per matrix: progress of the rows of L and of the preparations, of D, of the panel's rows
+int flow_ctl_ints(i64 sz, i64 rows) {
+  const i64 T = (sz + CB - 1) / CB, NR = (rows + CB - 1) / CB;
+  return (int)((2 * T + 1 + (NR > T ? NR : T) + 31) / 32 * 32);
+}
+// Panels that the factorization's launch solves too (beside the factorization, on the FMA pipes: rows r^2 multiply-adds);
+// larger ones take tensor-core products behind it.  The rule looks at the shape alone (grouped calls compute what
+// single ones do).
+bool flow_solves(const StepCtx& s, i64 rows, i64 r) {
+  return (double)rows * (double)r * (double)r <= FLOW_SOLVE_MAX &&
+         (rows + CB - 1) / CB <= FLOW_MAX_PANEL_TILES;
+}
+
+// One launch of the factorization (k_chol_flow) on the diagonal square [o, o + sz) of the Gram matrices, with either
+// the solve of the panel at pin_off into pout_off (rows > 0; the whole Gram matrix, o = 0 and sz = r) or the inverses of its
+// diagonal squares of 512 (transposed: L^-T, upper triangular) into L.Linv.  nsplit > 1: the Gram matrix is still the
+// product's partial sums (alpha_dev: their scale).
+int chol_flow(StepCtx& s, i64 r, i64 o, i64 sz, int mode, i64 pin_off, i64 pout_off, i64 rows, int nsplit, const float* alpha_dev,
+              bool round_end) {
   dion_ctx* c = s.c;
-  float* Gm = s.ws + s.L.Gram;
-  float* Dinv = s.ws + s.L.Dinv;
-  float* DinvP = s.ws + s.L.DinvP;
-  float* Linv = s.ws + s.L.Linv;
-  float* Tbuf = s.ws + s.L.Tbuf;
-  const float* gdiag = s.ws + s.L.gdiag;
-  int* status = s.quiet_fail ? nullptr : c->dev_ints;
-  const int* skip = adaptive ? (s.os + OS_DONE) : nullptr;
-  const float floor_rel = (mode == RM_ADAPTIVE) ? FLOOR_REL : 0.f;
-  const int nblk = (int)((sz + NB - 1) / NB);
-  {
-    const int jb = (int)((sz < NB) ? sz : NB);
-    launch_pdl(k_potrf_diag, dim3((unsigned)s.nb), dim3(256), 0, s.st, Gm + o * r + o, r, jb, Dinv + (o / NB) * (NB * NB),
-               DinvP + (o / NB) * (NB * NB), gdiag + o, floor_rel, s.os, adaptive ? 1 : 0, status, s.wstride);
-    DION_CHECK_LAUNCH(c);
+  const bool adaptive = (mode == RM_ADAPTIVE);
+  FlowArgs f;
+  memset(&f, 0, sizeof(f));
+  f.A = s.ws + s.L.Gram;
+  f.L = s.ws + s.L.Tbuf;
+  if (nsplit > 1) { f.part = s.ws + s.L.part; f.nsplit = nsplit; f.alpha_dev = alpha_dev; f.alpha_stride = s.wstride; }
+  f.Dinv = s.ws + s.L.Dinv;
+  f.DinvP = adaptive ? s.ws + s.L.DinvP : f.Dinv;
+  f.gdiag = s.ws + s.L.gdiag;
+  f.gdiag_given = (sz < r) ? 1 : 0;
+  const bool solve = rows > 0;
+  f.Pin = solve ? s.ws + pin_off : nullptr;
+  f.Pout = s.ws + (solve ? pout_off : s.L.Linv);
+  f.rows = rows;
+  f.r = r; f.o = o; f.sz = sz;
+  f.floor_rel = adaptive ? FLOOR_REL : 0.f;
+  f.os = s.os; f.skips = rm_skips(mode) ? 1 : 0;
+  f.status = s.quiet_fail ? nullptr : c->dev_ints;
+  f.status_always = c->dev_ints;
+  const i64 T = (sz + CB - 1) / CB, NR = (rows + CB - 1) / CB;
+  f.ctl = c->flow_ctl;
+  f.ctl_stride = flow_ctl_ints(sz, rows);
+  f.wstride = s.wstride; f.nb = s.nb;
+  f.round_end = (round_end && adaptive) ? 1 : 0;
+  f.good_rel = GOOD_REL; f.done_rel = DONE_REL; f.rounds_total = c->dev_ints + 2;
+  f.limit = umma::SPIN_LIMIT_CYCLES;
+  if (FLOW_HEAD_INTS + (i64)s.nb * f.ctl_stride > c->flow_ctl_cap) return DION_ERR_UNSUPPORTED;
+  // one runner per matrix; as many helpers as can be resident beside them, at most one per task
+  i64 tasks = (T > 2) ? (T - 2) * (T - 3) / 2 + 2 * (T - 2) : 0;
+  if (solve) tasks += NR * T;
+  else for (i64 k = 0; k < T; ++k) tasks += (T - k / FLOW_ISQ * FLOW_ISQ < FLOW_ISQ) ? T - k / FLOW_ISQ * FLOW_ISQ : FLOW_ISQ;
+  const i64 cap = (i64)flow_ctas_per_sm() * c->sm_count;
+  i64 grid = s.nb + tasks * s.nb;
+  if (grid > cap) grid = cap;
+  if (grid < s.nb + 1) return DION_ERR_UNSUPPORTED;
+  // With few matrices the helper that shares a runner's SM would slow the chain down more than it helps; it leaves if
+  // others are sure to stay.
+  const i64 ahead = (grid - s.nb) / (4 * s.nb) - 1;      // (2 nb (ahead + 1) preparations at most wait for tasks handed out later)
+  f.ahead = (int)(ahead < 0 ? 0 : ahead > FLOW_AHEAD_MAX ? FLOW_AHEAD_MAX : ahead);
+  f.exclusive = (s.nb <= FLOW_EXCLUSIVE_MAX && grid - s.nb > (i64)s.nb * (flow_ctas_per_sm() - 1)) ? 1 : 0;
+  void* args[] = {&f};
+  const void* fn = (r % 4 == 0) ? (const void*)k_chol_flow<true> : (const void*)k_chol_flow<false>;
+  if (cudaLaunchCooperativeKernel(fn, dim3((unsigned)grid), dim3(FLOW_THREADS), args, FLOW_SMEM, s.st) != cudaSuccess) {
+    cudaGetLastError();
+    return DION_ERR_CUDA;
   }
-  // one launch per block column: panel, trailing update and the next diagonal block; behind them the CTAs
-  // that add one term to every unfinished block row of the inverse of the square's factor (j blocks in each
-  // of the rows j .. nblk-1), off the critical path
-  for (int j = 0; j + 1 < nblk; ++j) {
-    const int nt = nblk - 1 - j;
-    const int extra = (nblk - j) * j;
-    dim3 grid((unsigned)(nt * (nt + 1) / 2 + extra), (unsigned)s.nb);
-    launch_pdl(k_chol_step, grid, dim3(256), CHOL_STEP_SMEM, s.st, Gm, r, o, sz, j, Dinv, DinvP, Tbuf, Linv, gdiag, floor_rel,
-               s.os, adaptive ? 1 : 0, status, s.wstride);
-    DION_CHECK_LAUNCH(c);
-  }
-  {
-    // last block row of the inverse, the factor's blocks into the Gram buffer, diagonal inverses into Linv
-    dim3 grid((unsigned)(nblk - 1 + grid_for(c, sz * sz)), (unsigned)s.nb);
-    launch_pdl(k_inv_finish, grid, dim3(256), INV_FINISH_SMEM, s.st, (const float*)Tbuf, Gm, Linv, r, o, sz, (const float*)Dinv, skip,
-               s.wstride);
-    DION_CHECK_LAUNCH(c);
-  }
+  c->launches++;
   return DION_OK;
 }
 
-// Two-level blocked Cholesky of each r x r Gram matrix (lower) and the full inverse of its
-// factor into Linv.  Outer blocks of 512 columns: the diagonal square is factored and
-// inverted by potrf_inner, the panel below it is multiplied by that inverse and the
-// trailing matrix is updated with one rank-512 product (tensor cores where it qualifies).
-int potrf_trtri(StepCtx& s, i64 r, int mode, bool full_inverse,
-                const std::function<int(i64, i64)>* after_block = nullptr) {
-  const bool adaptive = rm_skips(mode);
+// Cholesky of an r x r Gram matrix (lower) that is too large for one data-flow launch, with the inverses of its diagonal
+// squares (L.Linv): outer blocks of 512 columns.  The diagonal square is factored and inverted by k_chol_flow, the panel
+// below it is multiplied by that inverse and the trailing matrix is updated with one rank-512 product (tensor cores
+// where it qualifies).
+int potrf_blocked(StepCtx& s, i64 r, int mode, const std::function<int(i64, i64)>* after_block) {
   dion_ctx* c = s.c;
   float* Gm = s.ws + s.L.Gram;
   float* Linv = s.ws + s.L.Linv;
   float* Tbuf = s.ws + s.L.Tbuf;
-  const int* skip = adaptive ? (s.os + OS_DONE) : nullptr;
+  const int* skip = rm_skips(mode) ? (s.os + OS_DONE) : nullptr;
   const int precise = rm_precise(mode) ? 1 : 0;
-  if (r > NBO && full_inverse) {
-    // everything outside the diagonal squares starts at zero (the product U = P Linv^T reads whole tiles)
-    for (int m = 0; m < s.nb; ++m)
-      if (cudaMemsetAsync(s.W(m, s.L.Linv), 0, sizeof(float) * (size_t)r * (size_t)r, s.st) != cudaSuccess) return DION_ERR_CUDA;
-  }
   for (i64 J0 = 0; J0 < r; J0 += NBO) {
     const i64 sz = (r - J0 < NBO) ? (r - J0) : NBO;
-    DION_TRY(potrf_inner(s, r, J0, sz, mode));
+    DION_TRY(chol_flow(s, r, J0, sz, mode, 0, 0, 0, 1, nullptr, false));
     if (after_block != nullptr) DION_TRY((*after_block)(J0, sz));   // block column J of the factor and its inverse are final
     const i64 rem = r - J0 - sz;
     if (rem > 0) {
@@ -625,7 +625,7 @@ int potrf_trtri(StepCtx& s, i64 r, int mode, bool full_inverse,
       GemmArgs g = gemm_args();  // Lpanel = panel * Linv_JJ^T (out of place, then copied back)
       g.M = rem; g.N = sz; g.K = sz;
       g.A = panel; g.a_si = r; g.a_sk = 1;
-      g.B = Linv + J0 * r + J0; g.b_sk = 1; g.b_sn = r; g.klimit = 1;
+      g.B = Linv + J0 * r + J0; g.b_sk = r; g.b_sn = 1; g.klimit = 1;
       g.C = ptmp; g.ldc = r; g.epi = EPI_STORE; g.skip_flag = skip; g.precise = precise;
       DION_TRY(launch_gemm_chain(s, g));
       // With the solves on the second stream, the copy of Lpanel into the Gram buffer goes there too: its
@@ -654,7 +654,6 @@ int potrf_trtri(StepCtx& s, i64 r, int mode, bool full_inverse,
       DION_TRY(launch_gemm_chain(s, t));
     }
   }
-  if (r > NBO && full_inverse) DION_TRY(trtri_levels(s, r, 0, r, NBO, skip, precise));
   return DION_OK;
 }
 
@@ -707,11 +706,11 @@ bool gram_on_pairs(const StepCtx& s, i64 rows, i64 r) {
 
 // One Cholesky-QR round on every matrix of the chain: Pout = Pin * chol(Pin^T Pin)^-T.
 // rows x r panels, ld = r; pin_off / pout_off are offsets in the scratch slice.
-// adaptive: columns with negligible pivots are deflated, the round is skipped (Pout = Pin)
+// adaptive: columns with negligible pivots are deflated, the round is skipped
 // once the panel is orthonormal, and the round statistics are evaluated at the end.
 int cholqr_round(StepCtx& s, i64 pin_off, i64 pout_off, i64 rows, i64 r, int mode, i64 gram_rows = 0,
-                 bool passthrough = true, int probe_phase = PROBE_CHECK) {
-  // passthrough = false: a skipped round leaves Pout untouched (the caller keeps using Pin)
+                 int probe_phase = PROBE_CHECK) {
+  // A skipped round leaves Pout untouched (the caller keeps using Pin).
   // gram_rows > 0: the Gram matrix is formed from the first gram_rows rows only (a sketch stacked on
   // top of the panel); the factor is applied to all rows
   dion_ctx* c = s.c;
@@ -749,28 +748,26 @@ int cholqr_round(StepCtx& s, i64 pin_off, i64 pout_off, i64 rows, i64 r, int mod
     g.alpha_dev = s.ws + s.L.gmax + AMAX_PARTS; g.alpha_dev_stride = s.wstride;
   }
   g.C = s.ws + s.L.Gram; g.ldc = r; g.epi = EPI_STORE; g.tri = TRI_LOWER; g.skip_flag = skips ? skip : nullptr; g.precise = rm_precise(mode) ? 1 : 0;
+  const bool flow_all = r <= FLOW_MAX_R;      // the whole factorization in one launch
+  int nsplit = 1;
+  if (flow_all) g.splits_out = &nsplit;       // (which also adds up the partial products)
   DION_TRY(launch_gemm_chain(s, g));
-  launch_pdl(k_round_begin, dim3((unsigned)(s.nb)), dim3(256), 0, s.st, s.ws + s.L.Gram, r, r, 0.f, s.ws + s.L.gdiag, s.ws + s.L.scal, s.os,
-                                        skips ? 1 : 0, s.wstride, c->dev_ints);
-  DION_CHECK_LAUNCH(c);
-  // Tall panels with r > 512: blocked triangular solve with the 512-column diagonal inverses
-  // only (the levels of the triangular inverse above 512 are never formed).
-  // alone, 512-column products need >= 128 row tiles to fill the GPU; beside the factorization
-  // (second stream) they are background work at any height
-  const bool trsm = (r > NBO) && (rows >= 8192 || c->side != nullptr);
-  if (skips && passthrough) {   // a finished panel is passed through (before anything writes Pout)
-    dim3 grid((unsigned)grid_for(c, rows * r), (unsigned)s.nb);
-    launch_pdl(k_copy_panel, grid, dim3(256), 0, s.st, s.ws + pin_off, r, s.ws + pout_off, r, rows, r, nullptr, s.os + OS_DONE, s.wstride);
+  const float* part_scale = g.alpha_dev;
+  if (flow_all && flow_solves(s, rows, r))
+    return chol_flow(s, r, 0, r, mode, pin_off, pout_off, rows, nsplit, part_scale, true);
+  if (!flow_all) {
+    launch_pdl(k_round_begin, dim3((unsigned)(s.nb)), dim3(256), 0, s.st, s.ws + s.L.Gram, r, r, 0.f, s.ws + s.L.gdiag, s.ws + s.L.scal, s.os,
+                                          skips ? 1 : 0, s.wstride, c->dev_ints);
     DION_CHECK_LAUNCH(c);
   }
-  if (trsm) {
+  if (r > NBO) {
     // Pout_J = (Pin_J - sum_{K<J} Pout_K L_{J,K}^T) Linv_JJ^T, block columns J of 512.
     // The solves run with the plain 3xTF32 product: their rounding error enters U once (~1e-6),
     // whereas an error in the Gram matrix or its factor is amplified by the panel's conditioning.
     // Block column J needs row block J of the factor and the inverse of its diagonal square, both
     // final once the factorization has passed J: the solves run on a second stream beside the rest
     // of the factorization, whose serial 64-column chain leaves most SMs idle.
-    const float* Lm = s.ws + s.L.Gram;     // the factor, lower
+    const float* Lm = s.ws + (flow_all ? s.L.Tbuf : s.L.Gram);     // the factor, lower
     float* Wt = s.ws + (s.wt_off >= 0 ? s.wt_off : s.L.R);   // rows x 512 temporary (R is free during the orthonormalization)
     // On tall panels the two products of a block column run on scaled half pairs (22 significant bits in three
     // kind::f16 MMAs; 1024-k chains) like the Gram matrix: the right-hand side, the factor's row block and the
@@ -816,7 +813,7 @@ int cholqr_round(StepCtx& s, i64 pin_off, i64 pout_off, i64 rows, i64 r, int mod
       }
       // V = rhs Linv_JJ^T
       DION_TRY(absmax_split(rhs, rhs_ld, rows, sz, s.L.SolveP, 1, 1.f, nullptr));
-      const i64 li_off = s.L.LfP + NBO * r;
+      const i64 li_off = s.L.LfP + NBO * r;      // (L^-T: row k, column j of the product's right operand)
       DION_TRY(absmax_split(s.ws + s.L.Linv + J0 * r + J0, r, sz, sz, li_off, 2, 1.f, sc + (AMAX_PARTS + 64) + AMAX_PARTS));
       __half* rh = reinterpret_cast<__half*>(s.ws + s.L.SolveP);
       __half* ih = reinterpret_cast<__half*>(s.ws + li_off);
@@ -824,7 +821,7 @@ int cholqr_round(StepCtx& s, i64 pin_off, i64 pout_off, i64 rows, i64 r, int mod
       v.M = rows; v.N = sz; v.K = sz;
       v.ab16 = 1; v.f16 = 1;
       v.A = (const float*)rh; v.A16lo = rh + rows * sz; v.a_si = sz; v.a_sk = 1;
-      v.B = (const float*)ih; v.B16lo = ih + sz * sz; v.b_sk = 1; v.b_sn = sz; v.klimit = 1;
+      v.B = (const float*)ih; v.B16lo = ih + sz * sz; v.b_sk = sz; v.b_sn = 1; v.klimit = 1;
       v.C = s.ws + pout_off + J0; v.ldc = r; v.epi = EPI_STORE; v.skip_flag = skip;
       v.alpha_dev = sc + 2 * (AMAX_PARTS + 64) + AMAX_PARTS; v.alpha_dev_stride = s.wstride;
       DION_TRY(launch_gemm_chain(s, v));
@@ -854,12 +851,12 @@ int cholqr_round(StepCtx& s, i64 pin_off, i64 pout_off, i64 rows, i64 r, int mod
       GemmArgs v = gemm_args();
       v.M = rows; v.N = sz; v.K = sz;
       v.A = rhs; v.a_si = rhs_ld; v.a_sk = 1;
-      v.B = s.ws + s.L.Linv + J0 * r + J0; v.b_sk = 1; v.b_sn = r; v.klimit = 1;
+      v.B = s.ws + s.L.Linv + J0 * r + J0; v.b_sk = r; v.b_sn = 1; v.klimit = 1;
       v.C = s.ws + pout_off + J0; v.ldc = r; v.epi = EPI_STORE; v.skip_flag = skip;
       DION_TRY(launch_gemm_chain(s, v));
       return DION_OK;
     };
-    if (c->side != nullptr) {
+    if (!flow_all && c->side != nullptr) {
       cudaStream_t main_st = s.st;
       auto next_event = [&]() { cudaEvent_t e = c->side_ev[c->side_cursor]; c->side_cursor = (c->side_cursor + 1) % 32; return e; };
       const std::function<int(i64, i64)> after_block = [&](i64 J0, i64 sz) -> int {
@@ -870,11 +867,12 @@ int cholqr_round(StepCtx& s, i64 pin_off, i64 pout_off, i64 rows, i64 r, int mod
         s.st = main_st; s.no_split = false;
         return rc;
       };
-      DION_TRY(potrf_trtri(s, r, mode, false, &after_block));
+      DION_TRY(potrf_blocked(s, r, mode, &after_block));
       cudaEvent_t e = next_event();   // join: the round ends when the last solve has finished
       if (cudaEventRecord(e, c->side) != cudaSuccess || cudaStreamWaitEvent(main_st, e, 0) != cudaSuccess) return DION_ERR_CUDA;
     } else {
-      DION_TRY(potrf_trtri(s, r, mode, false));
+      if (flow_all) DION_TRY(chol_flow(s, r, 0, r, mode, 0, 0, 0, nsplit, part_scale, false));
+      else DION_TRY(potrf_blocked(s, r, mode, nullptr));
       for (i64 J0 = 0; J0 < r; J0 += NBO) DION_TRY(solve_block(J0, (r - J0 < NBO) ? (r - J0) : NBO));
     }
     if (adaptive) {
@@ -883,11 +881,11 @@ int cholqr_round(StepCtx& s, i64 pin_off, i64 pout_off, i64 rows, i64 r, int mod
     }
     return DION_OK;
   }
-  DION_TRY(potrf_trtri(s, r, mode, true));
+  DION_TRY(chol_flow(s, r, 0, r, mode, 0, 0, 0, nsplit, part_scale, false));
   GemmArgs u = gemm_args();
   u.M = rows; u.N = r; u.K = r;
   u.A = s.ws + pin_off; u.a_si = r; u.a_sk = 1;
-  u.B = s.ws + s.L.Linv; u.b_sk = 1; u.b_sn = r; u.klimit = 1;
+  u.B = s.ws + s.L.Linv; u.b_sk = r; u.b_sn = 1; u.klimit = 1;
   u.C = s.ws + pout_off; u.ldc = r; u.epi = EPI_STORE; u.skip_flag = skip;
   DION_TRY(launch_gemm_chain(s, u));
   if (adaptive) {
@@ -944,9 +942,24 @@ int adaptive_rounds(StepCtx& s, i64 off_a, i64 off_b, i64 rows, i64 r, i64 gram_
     DION_TRY(cholqr_round(s, off_a, off_b, rows, r, RM_ADAPTIVE, gram_rows));
     DION_TRY(cholqr_round(s, off_b, off_a, rows, r, RM_ADAPTIVE, gram_rows));
   }
+  {   // an odd number of rounds left the result in the second buffer
+    dim3 grid((unsigned)grid_for(s.c, rows * r), (unsigned)s.nb);
+    launch_pdl(k_copy_panel, grid, dim3(256), 0, s.st, (const float*)(s.ws + off_b), r, s.ws + off_a, r, rows, r, (const int*)nullptr,
+               (const int*)(s.os + OS_ROUNDS), s.wstride, 1);
+    s.c->launches++;
+  }
   launch_pdl(k_orth_finish, dim3((unsigned)(s.nb)), dim3(1), 0, s.st, s.os, s.c->dev_ints);
   s.c->launches++;
   if (cudaGetLastError() != cudaSuccess) return DION_ERR_CUDA;
+  return DION_OK;
+}
+
+// The second round of CholeskyQR2, when it ran, went P0 -> P1: its result back to P0.
+int second_round_back(StepCtx& s, i64 rows, i64 r) {
+  dim3 grid((unsigned)grid_for(s.c, rows * r), (unsigned)s.nb);
+  launch_pdl(k_copy_panel, grid, dim3(256), 0, s.st, (const float*)(s.ws + s.L.P1), r, s.ws + s.L.P0, r, rows, r,
+             (const int*)(s.os + OS_DONE), (const int*)nullptr, s.wstride, -1);
+  DION_CHECK_LAUNCH(s.c);
   return DION_OK;
 }
 
@@ -983,8 +996,9 @@ int rcqr(StepCtx& s, i64 rows, i64 r) {
   // B = the panel rows of the stack; the step's state slot starts afresh for its Cholesky QR
   launch_pdl(k_reset_rounds, dim3((unsigned)s.nb), dim3(1), 0, s.st, s.os);
   DION_CHECK_LAUNCH(c);
-  DION_TRY(cholqr_round(s, s.L.Sk + k * r, s.L.P1, rows, r, RM_FIRST));
-  return cholqr_round(s, s.L.P1, s.L.P0, rows, r, RM_CHECKED);
+  DION_TRY(cholqr_round(s, s.L.Sk + k * r, s.L.P0, rows, r, RM_FIRST));
+  DION_TRY(cholqr_round(s, s.L.P0, s.L.P1, rows, r, RM_CHECKED));
+  return second_round_back(s, rows, r);
 }
 
 // The orthonormalization a step on (m, n, r) will use.
@@ -1069,17 +1083,12 @@ int orthonormalize(StepCtx& s, i64 rows, i64 r, i64 short_dim, i64 pin_off, i64*
       // with the accurate product and repeats the round; all of that is launched and skipped in the common case.
       if (rc == DION_OK) rc = probe(s, s.L.P0, rows, r, PROBE_FAST);
       if (rc == DION_OK) rc = (*s.redo_p)();
-      if (rc == DION_OK) rc = cholqr_round(s, pin_off, s.L.P0, rows, r, RM_REDO, 0, false);
+      if (rc == DION_OK) rc = cholqr_round(s, pin_off, s.L.P0, rows, r, RM_REDO);
     }
-    if (rc == DION_OK) rc = cholqr_round(s, s.L.P0, s.L.P1, rows, r, RM_CHECKED, 0, false, redo ? PROBE_AFTER_REDO : PROBE_CHECK);
+    if (rc == DION_OK) rc = cholqr_round(s, s.L.P0, s.L.P1, rows, r, RM_CHECKED, 0, redo ? PROBE_AFTER_REDO : PROBE_CHECK);
     s.quiet_fail = false;
     DION_TRY(rc);
-    {
-      dim3 grid((unsigned)grid_for(s.c, rows * r), (unsigned)s.nb);
-      launch_pdl(k_copy_panel, grid, dim3(256), 0, s.st, (const float*)(s.ws + s.L.P1), r, s.ws + s.L.P0, r, rows, r,
-                 (const int*)(s.os + OS_DONE), (const int*)nullptr, s.wstride);
-      DION_CHECK_LAUNCH(s.c);
-    }
+    DION_TRY(second_round_back(s, rows, r));
     if (fb) DION_TRY(cgs_fallback(s, pin_off, s.L.P0, rows, r));   // else: the failed pivot was reported as a breakdown
     *U_off = s.L.P0;
   } else if (mode == DION_ORTH_SHIFTED3) {
@@ -1937,7 +1946,7 @@ int lazy_one(dion_ctx* c, const dion_matrix* a, float lr, int refresh, cudaStrea
     const i64 total = n * r;
     int blocks = (int)((total + 255) / 256);
     if (blocks > 8 * c->sm_count) blocks = 8 * c->sm_count;
-    launch_pdl(k_copy_panel, dim3((unsigned)(blocks)), dim3(256), 0, st, V, r, (float*)a->Q, a->ldq, n, r, s.flag, nullptr, 0);
+    launch_pdl(k_copy_panel, dim3((unsigned)(blocks)), dim3(256), 0, st, V, r, (float*)a->Q, a->ldq, n, r, (const int*)s.flag, (const int*)nullptr, (i64)0, -1);
     DION_CHECK_LAUNCH(c);
   }
   // W = (M + G) Q
@@ -2031,9 +2040,12 @@ int dion_init(dion_ctx** out, const dion_config* cfg) {
   c->cfg = *cfg;
   c->sm_count = prop.multiProcessorCount;
   void* p = nullptr;
-  if (cudaMalloc(&p, sizeof(int) * (8 + MAX_FLAG_SLOTS * OS_SLOT_INTS)) != cudaSuccess) { delete c; return DION_ERR_NOMEM; }
+  constexpr size_t int_bytes = sizeof(int) * (8 + MAX_FLAG_SLOTS * OS_SLOT_INTS + 24 + FLOW_CTL_INTS);
+  if (cudaMalloc(&p, int_bytes) != cudaSuccess) { delete c; return DION_ERR_NOMEM; }
   c->dev_ints = (int*)p;
-  if (cudaMemset(p, 0, sizeof(int) * (8 + MAX_FLAG_SLOTS * OS_SLOT_INTS)) != cudaSuccess) { cudaFree(p); delete c; return DION_ERR_CUDA; }
+  c->flow_ctl = c->dev_ints + 8 + MAX_FLAG_SLOTS * OS_SLOT_INTS + 24;      // (128-byte aligned)
+  c->flow_ctl_cap = FLOW_CTL_INTS;
+  if (cudaMemset(p, 0, int_bytes) != cudaSuccess) { cudaFree(p); delete c; return DION_ERR_CUDA; }
   if (configure_kernels() != DION_OK) { cudaFree(p); delete c; return DION_ERR_CUDA; }
   if (cudaStreamCreateWithFlags(&c->side, cudaStreamNonBlocking) != cudaSuccess) { cudaGetLastError(); c->side = nullptr; }
   // graph replay of small steps: a capture stream and the scalars the graphs read; off if either cannot be had
@@ -2432,6 +2444,7 @@ namespace {
 
 constexpr size_t NOALLOC_SCRATCH_BYTES = (size_t)24 << 20;  // 24 MiB, resident on every device that loads the library
 constexpr size_t NOALLOC_INT_BYTES = 256;                   // status word, counters and one step slot
+constexpr size_t NOALLOC_CTL_BYTES = 16 * 1024;             // progress counters of the factorization
 constexpr int NOALLOC_MAX_DEVICES = 64;
 
 // Scratch of dion_step_noalloc.  In host code this name is only a handle for
@@ -2459,8 +2472,8 @@ bool touch_kernel(K kernel) {
 bool preload_kernels() {
   bool ok = true;
   ok = ok && touch_kernel(k_gemm_simt<128, 128, 8, 8, 8>) && touch_kernel(k_gemm_simt<64, 64, 16, 4, 4>);
-  ok = ok && touch_kernel(k_splitk_reduce) && touch_kernel(k_round_begin) && touch_kernel(k_potrf_diag);
-  ok = ok && touch_kernel(k_chol_step) && touch_kernel(k_inv_finish) && touch_kernel(k_round_end) && touch_kernel(k_tiny_cholqr2);
+  ok = ok && touch_kernel(k_splitk_reduce) && touch_kernel(k_round_begin) && touch_kernel(k_chol_flow<true>);
+  ok = ok && touch_kernel(k_chol_flow<false>) && touch_kernel(k_round_end) && touch_kernel(k_tiny_cholqr2);
   ok = ok && touch_kernel(k_probe_y) && touch_kernel(k_probe_y4) && touch_kernel(k_probe_w) && touch_kernel(k_probe_decide) && touch_kernel(k_reset_rounds);
   ok = ok && touch_kernel(k_orth_finish) && touch_kernel(k_cgs_fallback) && touch_kernel(k_copy_block);
   ok = ok && touch_kernel(k_colsumsq_partial) && touch_kernel(k_colnorm_apply) && touch_kernel(k_copy_panel);
@@ -2520,8 +2533,10 @@ extern "C" int dion_step_noalloc(const dion_matrix* a, float lr, float mu, float
   c.cfg.device = device;
   c.sm_count = nd->sm_count;
   c.dev_ints = (int*)nd->base;
-  c.ws = (float*)(nd->base + NOALLOC_INT_BYTES);
-  c.ws_bytes = NOALLOC_SCRATCH_BYTES - NOALLOC_INT_BYTES;
+  c.flow_ctl = (int*)(nd->base + NOALLOC_INT_BYTES);
+  c.flow_ctl_cap = NOALLOC_CTL_BYTES / sizeof(int);
+  c.ws = (float*)(nd->base + NOALLOC_INT_BYTES + NOALLOC_CTL_BYTES);
+  c.ws_bytes = NOALLOC_SCRATCH_BYTES - NOALLOC_INT_BYTES - NOALLOC_CTL_BYTES;
   c.flag_cursor = 0;
   c.launches = 0;
   c.prof_on = false;
@@ -2535,7 +2550,7 @@ extern "C" int dion_step_noalloc(const dion_matrix* a, float lr, float mu, float
   return step_one(&c, a, lr, (cudaStream_t)cuda_stream);
 }
 
-extern "C" size_t dion_noalloc_scratch_limit(void) { return NOALLOC_SCRATCH_BYTES - NOALLOC_INT_BYTES; }
+extern "C" size_t dion_noalloc_scratch_limit(void) { return NOALLOC_SCRATCH_BYTES - NOALLOC_INT_BYTES - NOALLOC_CTL_BYTES; }
 
 // ---------------------------------------------------------------------------
 // Internal test hook (dion_internal.h)

@@ -58,8 +58,22 @@ struct GemmArgs {
   const void* A16lo;             // with ab16: A and B are PAIRS of bf16 arrays, x ~ hi + lo (A, B point to the "hi" arrays, these
   const void* B16lo;             // to the "lo" arrays of the same shape and strides): three bf16 MMAs per K step, ~1e-5 relative
   int f16;                       // with ab16 (no pairs): the arrays hold IEEE half values instead of bf16 (11 significant bits)
+  int* splits_out;               // HOST, optional: a product that splits K leaves its partial sums unreduced and reports their number here
   int tf32x1;                    // tensor engine, fp32 mode: the operands' values fit TF32 already (k_round_tf32): one MMA
                                  // per K step instead of the three-term split.  Ignored by the FMA engine.
+};
+
+// Per-step device state of the orthonormalization (ints, one slot per step).
+enum : int {
+  OS_FAIL = 0,      // the step must not write X, M, Q (breakdown)
+  OS_DONE = 1,      // adaptive rounds: the panel is orthonormal, later rounds are skipped
+  OS_GOOD = 2,      // adaptive rounds: the last round saw a well-conditioned panel
+  OS_FLOORED = 3,   // pivots raised to the floor in the current round
+  OS_MINREL = 4,    // float bits: min over columns of pivot / original diagonal, current round
+  OS_ROUNDS = 5,    // rounds that did work
+  OS_MAXDEV = 6,    // float bits: the estimate of |U1^T U1 - I|_F^2 of the CholeskyQR2 check
+  OS_BARRIER = 7,   // arrival counter of the fallback kernel's grid-wide barriers (zero at the start of a step)
+  OS_SLOT_INTS = 8
 };
 
 // Programmatic dependent launch (the small kernels of the serial Cholesky chain): lets the next

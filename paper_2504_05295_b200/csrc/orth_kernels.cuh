@@ -1,24 +1,12 @@
 // Small kernels of the orthonormalization (r x r factor work) and of ColNorm.
 #pragma once
 
+#include "chol_flow.cuh"
 #include "dion_common.cuh"
 
 namespace dion {
 
-constexpr int NB = 64;  // diagonal block of the blocked Cholesky / triangular inverse
-
-// Per-step device state of the orthonormalization (ints, one slot per step).
-enum : int {
-  OS_FAIL = 0,      // the step must not write X, M, Q (breakdown)
-  OS_DONE = 1,      // adaptive rounds: the panel is orthonormal, later rounds are skipped
-  OS_GOOD = 2,      // adaptive rounds: the last round saw a well-conditioned panel
-  OS_FLOORED = 3,   // pivots raised to the floor in the current round
-  OS_MINREL = 4,    // float bits: min over columns of pivot / original diagonal, current round
-  OS_ROUNDS = 5,    // rounds that did work
-  OS_MAXDEV = 6,    // float bits: the estimate of |U1^T U1 - I|_F^2 of the CholeskyQR2 check
-  OS_BARRIER = 7,   // arrival counter of the fallback kernel's grid-wide barriers (zero at the start of a step)
-  OS_SLOT_INTS = 8
-};
+constexpr int NB = CB;  // tile of the factorization
 
 // Round set-up on the r x r Gram matrix G (one block): saves diag(G) to gdiag, writes
 // shift = scale * trace(G) (fixed summation order) and resets the round statistics.
@@ -57,262 +45,9 @@ __global__ void k_round_begin(const float* __restrict__ G, i64 ld, i64 r, float 
   }
 }
 
-typedef float (*blk_t)[NB + 1];
-typedef float (*half_blk_t)[NB / 2 + 1];
-
-// One doubling level of the triangular inverse inside a 64 x 64 block: for every pair of
-// adjacent B x B diagonal blocks, X21 = -X22 (L21 X11).  256 threads, two block-wide barriers.
-// SUB: the 256 calling threads are the first eight warps of a larger CTA; they meet at a named barrier of their own.
-template <bool SUB>
-__device__ __forceinline__ void block_sync() {
-  if constexpr (SUB) asm volatile("bar.sync 1, 256;" ::: "memory");
-  else __syncthreads();
-}
-
-template <int B, bool SUB = false>
-__device__ __forceinline__ void trtri_level(blk_t L, blk_t X, half_blk_t T, int tid) {
-  constexpr int NPAIRS = NB / (2 * B);
-  for (int e = tid; e < NPAIRS * B * B; e += 256) {
-    const int pr = e / (B * B), rr = (e / B) % B, cc = e % B, base = pr * 2 * B;
-    float s0 = 0.f, s1 = 0.f, s2 = 0.f, s3 = 0.f;   // X11 is lower triangular: k >= cc; zeros above are stored
-    for (int k = cc & ~3; k < B; k += 4) {
-      s0 = fmaf(L[base + B + rr][base + k], X[base + k][base + cc], s0);
-      s1 = fmaf(L[base + B + rr][base + k + 1], X[base + k + 1][base + cc], s1);
-      s2 = fmaf(L[base + B + rr][base + k + 2], X[base + k + 2][base + cc], s2);
-      s3 = fmaf(L[base + B + rr][base + k + 3], X[base + k + 3][base + cc], s3);
-    }
-    T[pr * B + rr][cc] = (s0 + s1) + (s2 + s3);
-  }
-  block_sync<SUB>();
-  for (int e = tid; e < NPAIRS * B * B; e += 256) {
-    const int pr = e / (B * B), rr = (e / B) % B, cc = e % B, base = pr * 2 * B;
-    float s0 = 0.f, s1 = 0.f, s2 = 0.f, s3 = 0.f;   // X22 is lower triangular: k <= rr; zeros above are stored
-    for (int k = 0; k <= rr; k += 4) {
-      s0 = fmaf(X[base + B + rr][base + B + k], T[pr * B + k][cc], s0);
-      s1 = fmaf(X[base + B + rr][base + B + k + 1], T[pr * B + k + 1][cc], s1);
-      s2 = fmaf(X[base + B + rr][base + B + k + 2], T[pr * B + k + 2][cc], s2);
-      s3 = fmaf(X[base + B + rr][base + B + k + 3], T[pr * B + k + 3][cc], s3);
-    }
-    X[base + B + rr][base + cc] = -((s0 + s1) + (s2 + s3));
-  }
-  block_sync<SUB>();
-}
-
-// Inverse X of the lower-triangular 64 x 64 block L (shared memory; rdiag[i] = 1 / L[i][i];
-// X zero on entry): 16 x 16 diagonal inverses by forward substitution, then doubling.
-// Called by all 256 threads after a block-wide barrier; ends with one.
-template <bool SUB = false>
-__device__ __forceinline__ void invert_block(blk_t L, blk_t X, half_blk_t T, const float* rdiag, int tid) {
-  constexpr int W = 16;
-  if (tid < NB) {
-    const int b0 = (tid / W) * W, q = tid % W;
-    float x[W];
-#pragma unroll
-    for (int i = 0; i < W; ++i) {
-      float sacc = (i == q) ? 1.f : 0.f;
-#pragma unroll
-      for (int k = 0; k < i; ++k)
-        if (k >= q) sacc = fmaf(-L[b0 + i][b0 + k], x[k], sacc);
-      x[i] = (i >= q) ? sacc * rdiag[b0 + i] : 0.f;
-    }
-#pragma unroll
-    for (int i = 0; i < W; ++i) X[b0 + i][b0 + q] = x[i];
-  }
-  block_sync<SUB>();
-  // ... then [[X11, 0], [-X22 L21 X11, X22]] for block sizes 16 and 32
-  trtri_level<16, SUB>(L, X, T, tid);
-  trtri_level<32, SUB>(L, X, T, tid);
-}
-
-// Cholesky factor and its inverse of the 64 x 64 block held in L (shared memory; lower
-// triangle, identity padding beyond a ragged block of jb columns), by the 256 threads of
-// a CTA.  On return L holds the factor, X its inverse, deflated[] the deflated columns.
-// X must be zero on entry, gd[] hold the floors' reference values, deflated[] zeros,
-// and a block-wide barrier must separate those writes from the call.
-// The block is factored in four 16-column sub-panels: the 16 x 16 diagonal piece by
-// one warp (rows in registers, shuffles, no barrier), the rows below it by one thread per
-// row, the trailing update by all threads -- three block-wide barriers per sub-panel
-// instead of three per column.  The inverse is built from 16 x 16 inverses by doubling.
-template <bool SUB = false>
-__device__ __forceinline__ void potrf_block(blk_t L, blk_t X, half_blk_t T, const float* gd, float* rdiag,
-                                            int* deflated, int jb, float floor_rel, int* __restrict__ os,
-                                            int* __restrict__ status) {
-  constexpr int W = 16;    // base blocks of the inverse
-  constexpr int WF = 8;    // sub-panel width of the factorization
-  const int tid = threadIdx.x;
-  int floored = 0, failed = 0;
-  float minrel = __int_as_float(0x7f800000);
-  const float inf = __int_as_float(0x7f800000);
-#pragma unroll 1
-  for (int c0 = 0; c0 < NB; c0 += WF) {
-    if (tid == 0) {
-      // WF x WF diagonal piece: one thread, the lower triangle in registers.  The chain
-      // pivot -> rsqrt -> scale -> update of the next pivot is serial whatever the thread
-      // count; one thread runs it without any barrier or shuffle.  Padding columns of a
-      // ragged block (unit diagonal, gd = 0) pass every test.
-      float a[WF][WF], g[WF];
-#pragma unroll
-      for (int i = 0; i < WF; ++i) {
-        g[i] = gd[c0 + i];
-#pragma unroll
-        for (int c = 0; c <= i; ++c) a[i][c] = L[c0 + i][c0 + c];
-      }
-#pragma unroll
-      for (int j = 0; j < WF; ++j) {
-        float p = a[j][j];
-        const float fl = floor_rel * g[j];           // 0 in the plain mode
-        bool defl = false;
-        if (!(p > fl) || !(p < inf)) {
-          if (floor_rel > 0.f) {
-            p = (fl > 0.f && fl < inf) ? fl : 1.f;   // zero or non-finite column: unit pivot
-            defl = true;
-            ++floored;
-          } else {
-            failed = 1;
-            p = 1.f;
-          }
-        } else {
-          minrel = fminf(minrel, __fdividef(p, g[j]));
-        }
-        const float inv = rsqrtf(p);
-        const float sc = defl ? 0.f : inv;
-        a[j][j] = p * inv;
-        rdiag[c0 + j] = inv;
-        if (defl) deflated[c0 + j] = 1;
-#pragma unroll
-        for (int i = j + 1; i < WF; ++i) a[i][j] *= sc;
-#pragma unroll
-        for (int c = j + 1; c < WF; ++c)
-#pragma unroll
-          for (int i = c; i < WF; ++i) a[i][c] = fmaf(-a[i][j], a[c][j], a[i][c]);
-      }
-#pragma unroll
-      for (int i = 0; i < WF; ++i)
-#pragma unroll
-        for (int c = 0; c <= i; ++c) L[c0 + i][c0 + c] = a[i][c];
-    }
-    else if (tid >= 32 && c0 > 0) {
-      // meanwhile warps 1-7 finish the trailing update of the previous sub-panel: its columns from
-      // c0 + WF on (the WF columns the piece and the next panel need were updated right away)
-      const int p0 = c0 - WF;                       // the previous sub-panel's first column
-      const int t2 = tid - 32, ty = t2 >> 4, tx = t2 & 15;
-      for (int i = c0 + WF + ty; i < NB; i += 14)
-        for (int c = c0 + WF + tx; c <= i; c += 16) {
-          float sacc = 0.f;
-#pragma unroll
-          for (int k = 0; k < WF; ++k) sacc = fmaf(L[i][p0 + k], L[c][p0 + k], sacc);
-          L[i][c] -= sacc;
-        }
-    }
-    block_sync<SUB>();
-    const int below = NB - c0 - WF;   // rows under the diagonal piece
-    if (tid < below) {
-      const int i = c0 + WF + tid;
-      float x[WF];
-#pragma unroll
-      for (int j = 0; j < WF; ++j) {
-        float sacc = L[i][c0 + j];
-#pragma unroll
-        for (int k = 0; k < j; ++k) sacc = fmaf(-x[k], L[c0 + j][c0 + k], sacc);
-        x[j] = deflated[c0 + j] ? 0.f : sacc * rdiag[c0 + j];
-      }
-#pragma unroll
-      for (int j = 0; j < WF; ++j) L[i][c0 + j] = x[j];
-    }
-    block_sync<SUB>();
-    // trailing update, first part: the WF columns that the next diagonal piece and the panel below
-    // it need (thread -> (row, column)); the rest is deferred to run beside the next diagonal piece
-    for (int e = tid; e < below * WF; e += 256) {
-      const int i = c0 + WF + e / WF, c = c0 + WF + e % WF;
-      if (c <= i) {
-        float sacc = 0.f;
-#pragma unroll
-        for (int k = 0; k < WF; ++k) sacc = fmaf(L[i][c0 + k], L[c][c0 + k], sacc);
-        L[i][c] -= sacc;
-      }
-    }
-    block_sync<SUB>();
-  }
-  if (tid == 0) {
-    if (floor_rel > 0.f) {
-      if (floored) atomicAdd(&os[OS_FLOORED], floored);
-      atomicMin(&os[OS_MINREL], __float_as_int(minrel));
-    } else if (failed) {
-      os[OS_FAIL] = 1;
-      if (status != nullptr) atomicOr(status, DION_STATUS_BREAKDOWN);   // nullptr: a fallback follows in the same step
-    }
-  }
-
-  invert_block<SUB>(L, X, T, rdiag, tid);
-}
-
-// Cholesky of one jb x jb (jb <= 64) diagonal block, in place (lower factor, the
-// strict upper part of the block is zeroed), plus the inverse of that factor into
-// Dinv (64 x 64, row-major, zero padded).
-// floor_rel == 0 (plain Cholesky QR): a pivot that is <= 0 or not finite sets
-//   os[OS_FAIL] and the BREAKDOWN status bit and is replaced by 1 so that everything
-//   downstream stays finite.
-// floor_rel > 0 (adaptive rounds): a pivot below floor_rel * gdiag[j] (gdiag = the
-//   diagonal of the Gram matrix before elimination) is below the rounding noise of
-//   the Gram matrix.  Column j is then deflated: its diagonal entry becomes
-//   sqrt(floor), the entries below it zero, so the noisy column never reaches the
-//   trailing matrix.  The factor stays triangular and nonsingular for any panel;
-//   the round only improves the conditioning and a later round finishes the job.
-//   DinvP is Dinv with the rows of deflated columns zeroed: the panel below this
-//   block is multiplied by DinvP^T, which yields the zero columns of the factor.
-__global__ void __launch_bounds__(256) k_potrf_diag(float* __restrict__ A, i64 ld, int jb,
-                                                    float* __restrict__ Dinv, float* __restrict__ DinvP,
-                                                    const float* __restrict__ gdiag, float floor_rel,
-                                                    int* __restrict__ os, int adaptive,
-                                                    int* __restrict__ status, i64 wstride) {
-  {  // batched: block b -> matrix b
-    const i64 wo = (i64)blockIdx.x * wstride;
-    A += wo; Dinv += wo; DinvP += wo; gdiag += wo;
-    os += (i64)blockIdx.x * OS_SLOT_INTS;
-  }
-  pdl_enter();
-  if (adaptive && os[OS_DONE] != 0) return;
-  __shared__ float L[NB][NB + 1];
-  __shared__ float X[NB][NB + 1];
-  __shared__ float T[NB / 2][NB / 2 + 1];
-  __shared__ float gd[NB];
-  __shared__ float rdiag[NB];     // 1 / L[j][j]
-  __shared__ int deflated[NB];
-  const int tid = threadIdx.x;
-  if (tid < NB) {
-    deflated[tid] = 0;
-    gd[tid] = (floor_rel > 0.f && tid < jb) ? gdiag[tid] : 0.f;
-  }
-  {
-    float v[NB * NB / 256];
-#pragma unroll
-    for (int l = 0; l < NB * NB / 256; ++l) {
-      const int e = tid + l * 256, i = e / NB, c = e % NB;
-      v[l] = (i < jb && c <= i) ? A[(i64)i * ld + c] : 0.f;
-    }
-#pragma unroll
-    for (int l = 0; l < NB * NB / 256; ++l) {
-      const int e = tid + l * 256, i = e / NB, c = e % NB;
-      float x = v[l];
-      if (i == c && i >= jb) x = 1.f;   // identity padding of a ragged last block
-      L[i][c] = x;
-      X[i][c] = 0.f;
-    }
-  }
-  __syncthreads();
-
-  potrf_block(L, X, T, gd, rdiag, deflated, jb, floor_rel, os, status);
-  for (int e = tid; e < NB * NB; e += 256) {
-    const int i = e / NB, c = e % NB;
-    if (i < jb && c < jb) A[(i64)i * ld + c] = (c <= i) ? L[i][c] : 0.f;
-    Dinv[e] = X[i][c];
-    DinvP[e] = deflated[i] ? 0.f : X[i][c];
-  }
-}
-
 // CholeskyQR2 of a small panel (rows x r, r <= 64, rows <= TINY_MAX_ROWS, leading dimension r) in ONE launch, one
-// CTA of 1024 threads per matrix, the panel resident in shared memory: Gram matrix (3xTF32 on the warp-level tensor
-// path), Cholesky factor and its inverse (potrf_block, on the first eight warps), U1 = P L^-T (3xTF32), then the second round's Gram matrix G2 = U1^T U1, which
+// CTA of 512 threads per matrix, the panel resident in shared memory: Gram matrix (3xTF32 on the warp-level tensor
+// path), Cholesky factor and its inverse (potrf64, on the first eight warps), U1 = P L^-T (3xTF32), then the second round's Gram matrix G2 = U1^T U1, which
 // also says exactly how far U1 is from orthonormal: |G2 - I|_F^2 <= tau_f^2 r -> done after one round (the same
 // test the probe of the large panels estimates), else the second round runs on G2.  Replaces some seventeen
 // launches of a step on such a panel.  Every sum has a fixed order: same bits on every run.
@@ -321,17 +56,15 @@ __global__ void __launch_bounds__(256) k_potrf_diag(float* __restrict__ A, i64 l
 // fallback follows), the panel is then left to the fallback; a Gram trace that is not finite raises OS_FAIL and
 // DION_STATUS_NONFINITE.  Pin may equal Pout.
 constexpr int TINY_MAX_ROWS = 512;
-constexpr int TINY_THREADS = 1024;
+constexpr int TINY_THREADS = 512;      // (128 registers a thread: potrf64 keeps an 8 x 8 piece in them)
 // Row strides (floats) that keep the fragment loads of the two products off each other's banks: a lane reads
 // (row ft, column fg) of the panel for the Gram matrix (stride = 8 mod 32: no conflict) and (row fg, column ft)
 // of it (two-way) and of the inverse (copied to stride = 4 mod 32: none) for U.
 constexpr int TINY_LD = NB + 8;
-constexpr int TINY_XLD = NB + 4;
-constexpr int TINY_BLK = NB * (NB + 1);     // floats of a 64 x 65 block
+constexpr int TINY_BLK = CB * CLD;          // floats of a 64 x 64 tile (row stride = 4 mod 32: none for the inverse)
 inline int tiny_rows_pad(i64 rows) { return (int)((rows + 15) / 16 * 16); }
-inline int tiny_cholqr2_smem(i64 rows) {    // panel (rows padded to 16), L, X, the copy of X, T, gd, rdiag, red, deflated
-  return (int)sizeof(float) * (tiny_rows_pad(rows) * TINY_LD + 2 * TINY_BLK + NB * TINY_XLD + (NB / 2) * (NB / 2 + 1) + 2 * NB + TINY_THREADS) +
-         (int)sizeof(int) * NB;
+inline int tiny_cholqr2_smem(i64 rows) {    // panel (rows padded to 16), L, X, red, what potrf64 needs beside them
+  return (int)sizeof(float) * (tiny_rows_pad(rows) * TINY_LD + 2 * TINY_BLK + TINY_THREADS) + (int)(sizeof(Potrf64Set) + sizeof(Potrf64Aux));
 }
 
 // The two small products of the kernel run on the warp-level tensor-core path (m16n8k8, TF32 operands, fp32
@@ -369,14 +102,11 @@ __global__ void __launch_bounds__(TINY_THREADS) k_tiny_cholqr2(const float* __re
   const int rows_pad = (rows + 15) / 16 * 16;
   float* Ps = tiny_smem;                                              // rows_pad x TINY_LD; rows beyond `rows` and columns beyond r are zero
   float* blocks = Ps + rows_pad * TINY_LD;
-  blk_t L = reinterpret_cast<blk_t>(blocks);
-  blk_t X = reinterpret_cast<blk_t>(blocks + TINY_BLK);
-  float* XS = blocks + 2 * TINY_BLK;                                  // the inverse, row stride TINY_XLD
-  half_blk_t T = reinterpret_cast<half_blk_t>(XS + NB * TINY_XLD);
-  float* gd = XS + NB * TINY_XLD + (NB / 2) * (NB / 2 + 1);
-  float* rdiag = gd + NB;
-  float* red = rdiag + NB;                                            // TINY_THREADS
-  int* deflated = reinterpret_cast<int*>(red + TINY_THREADS);
+  ctile_t L = reinterpret_cast<ctile_t>(blocks);
+  ctile_t X = reinterpret_cast<ctile_t>(blocks + TINY_BLK);
+  float* red = blocks + 2 * TINY_BLK;                                 // TINY_THREADS
+  Potrf64Set& set = *reinterpret_cast<Potrf64Set*>(red + TINY_THREADS);
+  Potrf64Aux& aux = *reinterpret_cast<Potrf64Aux*>(&set + 1);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int fg = lane >> 2, ft = lane & 3;                            // fragment coordinates of the lane
 
@@ -412,40 +142,49 @@ __global__ void __launch_bounds__(TINY_THREADS) k_tiny_cholqr2(const float* __re
   for (int e = rows * NB + tid; e < rows_pad * NB; e += TINY_THREADS) Ps[(e / NB) * TINY_LD + e % NB] = 0.f;
   __syncthreads();
 
-  // G = P^T P (64 x 64, K = rows_pad): warp w owns the 16 x 8 tile (w / 8, w % 8); lane (fg, ft) then holds
-  // G[m0 + fg][n0 + 2 ft], [..][n0 + 2 ft + 1], G[m0 + fg + 8][n0 + 2 ft], [..][n0 + 2 ft + 1].
-  const int m0 = (warp >> 3) * 16, n0 = (warp & 7) * 8;
-  float acc[4];
+  // G = P^T P (64 x 64, K = rows_pad): warp w owns the 16 x 8 tiles (w / 4, 2 (w % 4)) and (w / 4, 2 (w % 4) + 1); lane
+  // (fg, ft) then holds G[m0 + fg][n0 + 2 ft], [..][n0 + 2 ft + 1], G[m0 + fg + 8][n0 + 2 ft], [..][n0 + 2 ft + 1] of each
+  // (n0 = nb0, nb0 + 8).
+  const int m0 = (warp >> 2) * 16, nb0 = (warp & 3) * 16;
+  float acc[2][4];
   auto gram = [&]() {
-    acc[0] = acc[1] = acc[2] = acc[3] = 0.f;
+#pragma unroll
+    for (int t = 0; t < 2; ++t) acc[t][0] = acc[t][1] = acc[t][2] = acc[t][3] = 0.f;
 #pragma unroll 4
     for (int k0 = 0; k0 < rows_pad; k0 += 8) {
       const float* r0 = Ps + (k0 + ft) * TINY_LD;
       const float* r1 = Ps + (k0 + ft + 4) * TINY_LD;
       const float a[4] = {r0[m0 + fg], r0[m0 + fg + 8], r1[m0 + fg], r1[m0 + fg + 8]};    // A(m, k) = P[k][m]
-      const float b[2] = {r0[n0 + fg], r1[n0 + fg]};                                      // B(k, n) = P[k][n]
-      mma_3xtf32(acc, a, b);
+#pragma unroll
+      for (int t = 0; t < 2; ++t) {
+        const float b[2] = {r0[nb0 + 8 * t + fg], r1[nb0 + 8 * t + fg]};                  // B(k, n) = P[k][n]
+        mma_3xtf32(acc[t], a, b);
+      }
     }
   };
-  // the Gram matrix from the registers into L: lower triangle, zero above, identity beyond column r; X, gd,
-  // deflated reset
+  // the Gram matrix from the registers into L: lower triangle, zero above, identity beyond column r; what
+  // potrf64 needs beside it
   auto stage_factor_input = [&]() {
 #pragma unroll
-    for (int x = 0; x < 4; ++x) {
-      const int i = m0 + fg + ((x & 2) ? 8 : 0), c = n0 + 2 * ft + (x & 1);
-      float v = (i < r && c <= i) ? acc[x] : 0.f;
+    for (int x = 0; x < 8; ++x) {
+      const int i = m0 + fg + ((x & 2) ? 8 : 0), c = nb0 + 8 * (x >> 2) + 2 * ft + (x & 1);
+      if (i == c) red[i] = (i < r) ? acc[x >> 2][x & 3] : 0.f;      // the diagonal (also for the trace)
+    }
+    __syncthreads();
+    if (warp == 0) potrf64_setup(set, red[lane], red[lane + 32], 0.f, lane);
+    __syncthreads();
+    const float s2 = set.s2;
+#pragma unroll
+    for (int x = 0; x < 8; ++x) {
+      const int i = m0 + fg + ((x & 2) ? 8 : 0), c = nb0 + 8 * (x >> 2) + 2 * ft + (x & 1);
+      float v = (i < r && c <= i) ? acc[x >> 2][x & 3] * s2 : 0.f;
       if (i == c && i >= r) v = 1.f;
       L[i][c] = v;
-      X[i][c] = 0.f;
-      if (i == c) red[i] = (i < r) ? acc[x] : 0.f;      // the diagonal, for the trace
     }
-    if (tid < NB) { deflated[tid] = 0; gd[tid] = 0.f; }
   };
   // U = P X^T in place (X lower triangular, its zeros above the diagonal stored): work item = 16 rows x 32
   // columns, K = 64; the items of a sweep are all computed before any entry of the panel is overwritten.
   auto apply_inverse = [&]() {
-    for (int e = tid; e < NB * NB; e += TINY_THREADS) XS[(e / NB) * TINY_XLD + e % NB] = X[e / NB][e % NB];
-    __syncthreads();
     const int items = (rows_pad / 16) * 2;
     for (int it0 = 0; it0 < items; it0 += TINY_THREADS / 32) {
       const int it = it0 + warp;
@@ -461,7 +200,7 @@ __global__ void __launch_bounds__(TINY_THREADS) k_tiny_cholqr2(const float* __re
           const float a[4] = {r0[ft], r1[ft], r0[ft + 4], r1[ft + 4]};                    // A(m, k) = P[i0 + m][k]
 #pragma unroll
           for (int nt = 0; nt < 4; ++nt) {
-            const float* xr = XS + (c0 + 8 * nt + fg) * TINY_XLD + k0;
+            const float* xr = &X[c0 + 8 * nt + fg][k0];
             const float b[2] = {xr[ft], xr[ft + 4]};                                      // B(k, n) = X[n][k]
             mma_3xtf32(y[nt], a, b);
           }
@@ -493,7 +232,7 @@ __global__ void __launch_bounds__(TINY_THREADS) k_tiny_cholqr2(const float* __re
       atomicOr(status_always, DION_STATUS_NONFINITE);
     }
   }
-  if (tid < 256) potrf_block<true>(L, X, T, gd, rdiag, deflated, r, 0.f, os, status_fail);   // (ends with its own barrier)
+  if (tid < 256) potrf64(L, X, set, aux, 0.f, os, status_fail, tid);   // (ends with its own barrier)
   __syncthreads();
   const bool failed1 = reinterpret_cast<volatile int*>(os)[OS_FAIL] != 0;   // (written by this CTA's thread 0 before that barrier, or before this launch)
   apply_inverse();
@@ -502,9 +241,9 @@ __global__ void __launch_bounds__(TINY_THREADS) k_tiny_cholqr2(const float* __re
   gram();
   float e = 0.f;
 #pragma unroll
-  for (int x = 0; x < 4; ++x) {
-    const int i = m0 + fg + ((x & 2) ? 8 : 0), c = n0 + 2 * ft + (x & 1);
-    if (i < r && c < r) { const float d = acc[x] - ((i == c) ? 1.f : 0.f); e = fmaf(d, d, e); }
+  for (int x = 0; x < 8; ++x) {
+    const int i = m0 + fg + ((x & 2) ? 8 : 0), c = nb0 + 8 * (x >> 2) + 2 * ft + (x & 1);
+    if (i < r && c < r) { const float d = acc[x >> 2][x & 3] - ((i == c) ? 1.f : 0.f); e = fmaf(d, d, e); }
   }
   red[tid] = e;
   __syncthreads();
@@ -518,7 +257,7 @@ __global__ void __launch_bounds__(TINY_THREADS) k_tiny_cholqr2(const float* __re
     __syncthreads();                 // everyone has read red[0]
     stage_factor_input();
     __syncthreads();
-    if (tid < 256) potrf_block<true>(L, X, T, gd, rdiag, deflated, r, 0.f, os, status_fail);
+    if (tid < 256) potrf64(L, X, set, aux, 0.f, os, status_fail, tid);
     __syncthreads();
     apply_inverse();
   }
@@ -535,286 +274,12 @@ __global__ void __launch_bounds__(TINY_THREADS) k_tiny_cholqr2(const float* __re
   }
 }
 
-// Operand tiles of the 64 x 64 x 64 products: rows of 68 floats (16-byte aligned rows for
-// 128-bit loads along k; the row patterns below stay free of bank conflicts).
-constexpr int MMS = NB + 4;
-typedef float (*mm_t)[MMS];
-
-// acc[a][b] += sum_k A[4 ty + a][k] * B[tx + 16 b][k]  (64 x 64 x 64, operands in shared memory)
-__device__ __forceinline__ void mm_nt_64(mm_t A, mm_t B, int ty, int tx, float (&acc)[4][4]) {
-#pragma unroll 4
-  for (int k = 0; k < NB; k += 4) {
-    float4 av[4], bv[4];
-#pragma unroll
-    for (int a = 0; a < 4; ++a) av[a] = *reinterpret_cast<const float4*>(&A[ty * 4 + a][k]);
-#pragma unroll
-    for (int b = 0; b < 4; ++b) bv[b] = *reinterpret_cast<const float4*>(&B[tx + 16 * b][k]);
-#pragma unroll
-    for (int a = 0; a < 4; ++a)
-#pragma unroll
-      for (int b = 0; b < 4; ++b) {
-        float t = acc[a][b];
-        t = fmaf(av[a].x, bv[b].x, t);
-        t = fmaf(av[a].y, bv[b].y, t);
-        t = fmaf(av[a].z, bv[b].z, t);
-        t = fmaf(av[a].w, bv[b].w, t);
-        acc[a][b] = t;
-      }
-  }
-}
-
-constexpr int CHOL_STEP_SMEM = 3 * NB * MMS * (int)sizeof(float);
-
-// The inverse X of the factor of the diagonal square [o, o+sz), 64 x 64 blocks:
-//   X_im = -Dinv_i * S_im,   S_im = sum_{k=m}^{i-1} L_ik X_km,   X_mm = Dinv_m   (m < i).
-// The sums are accumulated right-looking, one term per launch: as soon as block column kk of the factor
-// and block row kk of X are final, every later row adds its term k = kk,
-//   S_im (+)= L_{i,kk} X_{kk,m}   (the first term, m = kk, takes X_kk,kk = Dinv_kk),
-// and the row that is complete with it (i = kk + 1, `finish`) is multiplied by -Dinv_i.  S_im lives in
-// X_im's place in Linv until then.  L is read from Lsrc (the panels the steps have written).  One CTA of
-// 256 threads per block and launch: one 64^3 product, two for the finishing row; smem holds two tiles.
-__device__ __forceinline__ void inv_term(const float* __restrict__ Lsrc, float* __restrict__ Linv, i64 ld,
-                                         const float* __restrict__ Dinv, i64 o, i64 sz, int i, int m, int kk,
-                                         bool finish, float* smem) {
-  mm_t S0 = reinterpret_cast<mm_t>(smem);
-  mm_t S1 = reinterpret_cast<mm_t>(smem + NB * MMS);
-  const int tid = threadIdx.x, ty = tid >> 4, tx = tid & 15;
-  const i64 ri = o + (i64)i * NB, cm = o + (i64)m * NB, rk = o + (i64)kk * NB;
-  const int rows_i = (int)((o + sz - ri < NB) ? (o + sz - ri) : NB);
-  const bool first = (m == kk);
-  const float* Dk = Dinv + (rk / NB) * (NB * NB);
-  float acc[4][4];
-#pragma unroll
-  for (int a = 0; a < 4; ++a)
-#pragma unroll
-    for (int b = 0; b < 4; ++b)
-      acc[a][b] = (!first && ty * 4 + a < rows_i) ? Linv[(ri + ty * 4 + a) * ld + cm + tx + 16 * b] : 0.f;
-#pragma unroll 4
-  for (int l = 0; l < NB * NB / 256; ++l) {
-    const int e = tid + l * 256, rr = e / NB, cc = e % NB;
-    S0[rr][cc] = (rr < rows_i) ? Lsrc[(ri + rr) * ld + rk + cc] : 0.f;
-    S1[cc][rr] = first ? Dk[e] : Linv[(rk + rr) * ld + cm + cc];   // transposed: the product below is A * B^T
-  }
-  __syncthreads();
-  mm_nt_64(S0, S1, ty, tx, acc);
-  if (!finish) {
-#pragma unroll
-    for (int a = 0; a < 4; ++a)
-#pragma unroll
-      for (int b = 0; b < 4; ++b)
-        if (ty * 4 + a < rows_i) Linv[(ri + ty * 4 + a) * ld + cm + tx + 16 * b] = acc[a][b];
-    return;
-  }
-  __syncthreads();
-  const float* Di = Dinv + (ri / NB) * (NB * NB);
-#pragma unroll
-  for (int a = 0; a < 4; ++a)
-#pragma unroll
-    for (int b = 0; b < 4; ++b) S1[tx + 16 * b][ty * 4 + a] = acc[a][b];
-#pragma unroll 4
-  for (int l = 0; l < NB * NB / 256; ++l) {
-    const int e = tid + l * 256;
-    S0[e / NB][e % NB] = Di[e];
-  }
-  __syncthreads();
-  float x[4][4] = {};
-  mm_nt_64(S0, S1, ty, tx, x);
-#pragma unroll
-  for (int a = 0; a < 4; ++a)
-#pragma unroll
-    for (int b = 0; b < 4; ++b)
-      if (ty * 4 + a < rows_i) Linv[(ri + ty * 4 + a) * ld + cm + tx + 16 * b] = -x[a][b];
-}
-
-// One step of the right-looking 64-column Cholesky inside the diagonal square [o, o+sz)
-// of the Gram matrix, in ONE launch: with the diagonal block of block column j already
-// factored (its inverse in DinvP), CTA (bi, bk), bk <= bi, forms the two 64-row pieces
-// L_i = A[i][j] DinvP^T and L_k of block column j of the factor, and subtracts
-// L_i L_k^T from the trailing block (i, k).  The CTA of the next diagonal block
-// (bi = bk = 0) then factors and inverts that block right away, so that the next step
-// can start at the next launch; the other CTAs run beside it.  The L pieces go to Lout
-// (same offsets as in A): block column j of A is still read by the other CTAs of this
-// launch, so it cannot be overwritten here; the caller copies Lout back after the last step.
-__global__ void __launch_bounds__(256) k_chol_step(float* __restrict__ A, i64 ld, i64 o, i64 sz, int j,
-                                                   float* __restrict__ Dinv, float* __restrict__ DinvP,
-                                                   float* __restrict__ Lout, float* __restrict__ Linv,
-                                                   const float* __restrict__ gdiag, float floor_rel,
-                                                   int* __restrict__ os, int adaptive,
-                                                   int* __restrict__ status, i64 wstride) {
-  {
-    const i64 wo = (i64)blockIdx.y * wstride;
-    A += wo; Dinv += wo; DinvP += wo; Lout += wo; Linv += wo; gdiag += wo;
-    os += (i64)blockIdx.y * OS_SLOT_INTS;
-  }
-  // Launched with programmatic stream serialization: the next step's CTAs may be scheduled while
-  // this grid still runs (they wait here), which takes the launch latency off the serial chain.
-  pdl_enter();
-  if (adaptive && os[OS_DONE] != 0) return;
-  extern __shared__ __align__(16) float chol_smem[];
-  {
-    // the CTAs behind the trailing blocks: block column j - 1 of the factor and block row j - 1 of the
-    // square's inverse are final since the last launch; every row i >= j of the inverse adds that term
-    // (j blocks per row), and row j is complete with it
-    const int nblk = (int)((sz + NB - 1) / NB);
-    const int nt = nblk - 1 - j;
-    const int ntri = nt * (nt + 1) / 2;
-    if ((int)blockIdx.x >= ntri) {
-      const int x = (int)blockIdx.x - ntri;
-      const int i = j + x / j, m = x % j;
-      inv_term(Lout, Linv, ld, Dinv, o, sz, i, m, j - 1, i == j, chol_smem);
-      return;
-    }
-  }
-  mm_t S0 = reinterpret_cast<mm_t>(chol_smem);
-  mm_t S1 = reinterpret_cast<mm_t>(chol_smem + NB * MMS);
-  mm_t S2 = reinterpret_cast<mm_t>(chol_smem + 2 * NB * MMS);
-  __shared__ float gd[NB];
-  __shared__ float rdiag[NB];
-  __shared__ int deflated[NB];
-  const int tid = threadIdx.x, ty = tid >> 4, tx = tid & 15;
-  int bi = 0;
-  while ((bi + 1) * (bi + 2) / 2 <= (int)blockIdx.x) ++bi;
-  const int bk = (int)blockIdx.x - bi * (bi + 1) / 2;
-  const i64 cj = o + (i64)j * NB;                    // first column of block column j
-  const i64 ri = cj + (i64)NB * (1 + bi), rk = cj + (i64)NB * (1 + bk);
-  const int rows_i = (int)((o + sz - ri < NB) ? (o + sz - ri) : NB);
-  const int rows_k = (int)((o + sz - rk < NB) ? (o + sz - rk) : NB);
-  const bool diag = (bi == bk);
-  const bool next_diag = (bi == 0 && bk == 0);
-  const float* DPj = DinvP + (cj / NB) * (NB * NB);
-  float cblk[4][4];      // this thread's entries of trailing block (i, k), fetched ahead of the products
-  {
-    float vi[NB * NB / 256], vk[NB * NB / 256], vd[NB * NB / 256];
-#pragma unroll
-    for (int l = 0; l < NB * NB / 256; ++l) {
-      const int e = tid + l * 256, i = e / NB, c = e % NB;
-      vi[l] = (i < rows_i) ? A[(ri + i) * ld + cj + c] : 0.f;
-      vk[l] = (!diag && i < rows_k) ? A[(rk + i) * ld + cj + c] : 0.f;
-      vd[l] = DPj[e];
-    }
-#pragma unroll
-    for (int a = 0; a < 4; ++a)
-#pragma unroll
-      for (int b = 0; b < 4; ++b) {
-        const int i = ty * 4 + a, c = tx + 16 * b;
-        cblk[a][b] = (i < rows_i && c < rows_k) ? A[(ri + i) * ld + rk + c] : 0.f;
-      }
-#pragma unroll
-    for (int l = 0; l < NB * NB / 256; ++l) {
-      const int e = tid + l * 256, i = e / NB, c = e % NB;
-      S0[i][c] = vi[l];
-      S1[i][c] = vk[l];
-      S2[i][c] = vd[l];
-    }
-  }
-  __syncthreads();
-  float li[4][4] = {}, lk[4][4] = {};
-  mm_nt_64(S0, S2, ty, tx, li);
-  if (!diag) mm_nt_64(S1, S2, ty, tx, lk);
-  __syncthreads();
-#pragma unroll
-  for (int a = 0; a < 4; ++a)
-#pragma unroll
-    for (int b = 0; b < 4; ++b) {
-      S0[ty * 4 + a][tx + 16 * b] = li[a][b];
-      if (!diag) S1[ty * 4 + a][tx + 16 * b] = lk[a][b];
-      if (bk == 0 && ty * 4 + a < rows_i) Lout[(ri + ty * 4 + a) * ld + cj + tx + 16 * b] = li[a][b];
-    }
-  __syncthreads();
-  float acc[4][4] = {};
-  mm_nt_64(S0, diag ? S0 : S1, ty, tx, acc);
-  if (!next_diag) {
-#pragma unroll
-    for (int a = 0; a < 4; ++a)
-#pragma unroll
-      for (int b = 0; b < 4; ++b) {
-        const int i = ty * 4 + a, c = tx + 16 * b;
-        if (i < rows_i && c < rows_k) A[(ri + i) * ld + rk + c] = cblk[a][b] - acc[a][b];
-      }
-    return;
-  }
-  // the next diagonal block: factor and invert it here.  The three buffers are reused as the
-  // factor L (65-float rows, S2: the inverse of the previous block is no longer needed), its
-  // inverse X (S1) and the scratch T of the inverse levels (S0).
-  blk_t Lb = reinterpret_cast<blk_t>(chol_smem + 2 * NB * MMS);
-  blk_t Xb = reinterpret_cast<blk_t>(chol_smem + NB * MMS);
-  if (tid < NB) {
-    deflated[tid] = 0;
-    gd[tid] = (floor_rel > 0.f && tid < rows_i) ? gdiag[ri + tid] : 0.f;
-  }
-  __syncthreads();                // every thread is done reading S0 / S1 / S2
-#pragma unroll
-  for (int a = 0; a < 4; ++a)
-#pragma unroll
-    for (int b = 0; b < 4; ++b) {
-      const int i = ty * 4 + a, c = tx + 16 * b;
-      const float v = cblk[a][b] - acc[a][b];
-      Lb[i][c] = (c < i) ? v : ((c == i) ? ((i < rows_i) ? v : 1.f) : 0.f);
-    }
-  for (int e = tid; e < NB * NB; e += 256) Xb[e / NB][e % NB] = 0.f;
-  __syncthreads();
-  potrf_block(Lb, Xb, reinterpret_cast<half_blk_t>(chol_smem), gd, rdiag, deflated, rows_i, floor_rel, os, status);
-  float* Dn = Dinv + (ri / NB) * (NB * NB);
-  float* DPn = DinvP + (ri / NB) * (NB * NB);
-  for (int e = tid; e < NB * NB; e += 256) {
-    const int i = e / NB, c = e % NB;
-    if (i < rows_i && c < rows_i) A[(ri + i) * ld + ri + c] = (c <= i) ? Lb[i][c] : 0.f;
-    Dn[e] = Xb[i][c];
-    DPn[e] = deflated[i] ? 0.f : Xb[i][c];
-  }
-}
-
-// After the last k_chol_step of a square [o, o+sz): the first CTAs complete the last block row of the
-// inverse of the factor (inv_term); the others move the factor's blocks below the block diagonal from
-// Lout into A, put the diagonal inverses into Linv and clear Linv above the block diagonal.
-constexpr int INV_FINISH_SMEM = 2 * NB * MMS * (int)sizeof(float);
-__global__ void __launch_bounds__(256) k_inv_finish(const float* __restrict__ Lout, float* __restrict__ A,
-                                                    float* __restrict__ Linv, i64 ld, i64 o, i64 sz,
-                                                    const float* __restrict__ Dinv,
-                                                    const int* __restrict__ skip_flag, i64 wstride) {
-  Lout += (i64)blockIdx.y * wstride; A += (i64)blockIdx.y * wstride;
-  Linv += (i64)blockIdx.y * wstride; Dinv += (i64)blockIdx.y * wstride;
-  pdl_enter();
-  if (skip_flag != nullptr && skip_flag[(i64)blockIdx.y * OS_SLOT_INTS] != 0) return;
-  extern __shared__ __align__(16) float fin_smem[];
-  const int nblk = (int)((sz + NB - 1) / NB);
-  if ((int)blockIdx.x < nblk - 1) {   // the last row's last term (block column nblk - 2), and its finish
-    inv_term(Lout, Linv, ld, Dinv, o, sz, nblk - 1, (int)blockIdx.x, nblk - 2, true, fin_smem);
-    return;
-  }
-  const i64 total = sz * sz;
-  const i64 first = (i64)((int)blockIdx.x - (nblk - 1)) * blockDim.x + threadIdx.x;
-  const i64 step = (i64)((int)gridDim.x - (nblk - 1)) * blockDim.x;
-  for (i64 e = first; e < total; e += step) {
-    const i64 i = e / sz, c = e % sz;
-    const i64 bi = i / NB, bc = c / NB;
-    if (bi > bc) {
-      A[(o + i) * ld + o + c] = Lout[(o + i) * ld + o + c];
-    } else {
-      Linv[(o + i) * ld + o + c] = (bi == bc) ? Dinv[((o + i) / NB) * (NB * NB) + (i % NB) * NB + (c % NB)] : 0.f;
-    }
-  }
-}
-
-// End of an adaptive round (one thread).  `minrel`, the smallest pivot relative to its
-// column's squared norm, estimates 1 / cond^2 of the round's input panel.
-//   - no pivot raised and minrel >= done_rel: the input was already orthonormal to
-//     ~(1 - done_rel), so this round's output is orthonormal to rounding level: done;
-//   - no pivot raised and minrel >= good_rel: cond <~ 1 / sqrt(good_rel); one more
-//     round brings orthonormality to rounding level (the CholeskyQR2 argument), after
-//     which the remaining rounds are skipped.
+// End of an adaptive round whose panel was solved by products behind the factorization (one thread per matrix).
 __global__ void k_round_end(int* __restrict__ os, float good_rel, float done_rel, int* __restrict__ rounds_total) {
   pdl_enter();
   os += (i64)blockIdx.x * OS_SLOT_INTS;
   if (os[OS_DONE] != 0) return;
-  os[OS_ROUNDS] += 1;
-  atomicAdd(rounds_total, 1);
-  if (os[OS_GOOD] != 0) { os[OS_DONE] = 1; return; }
-  const float minrel = __int_as_float(os[OS_MINREL]);
-  if (os[OS_FLOORED] == 0) {
-    if (minrel >= done_rel) os[OS_DONE] = 1;
-    else if (minrel >= good_rel) os[OS_GOOD] = 1;
-  }
+  round_evaluate(os, good_rel, done_rel, rounds_total);
 }
 
 // ---------------------------------------------------------------------------
@@ -1338,15 +803,15 @@ __global__ void __launch_bounds__(128) k_colnorm_apply(const float* __restrict__
 }
 
 // Copies a rows x r panel (ld = ldv) into Q (ld = ldq) unless the step was flagged.
-// `only_if` (optional): the copy happens only when *only_if != 0.
+// `only_if` (optional): the copy happens only when (*only_if & only_mask) != 0.
 __global__ void k_copy_panel(const float* __restrict__ V, i64 ldv, float* __restrict__ Q, i64 ldq,
                              i64 rows, i64 r, const int* __restrict__ skip_flag,
-                             const int* __restrict__ only_if, i64 wstride) {
+                             const int* __restrict__ only_if, i64 wstride, int only_mask) {
   pdl_enter();
   V += (i64)blockIdx.y * wstride;                                         // batched over blockIdx.y
   if (wstride != 0) Q += (i64)blockIdx.y * wstride;
   if (skip_flag != nullptr && skip_flag[(i64)blockIdx.y * OS_SLOT_INTS] != 0) return;
-  if (only_if != nullptr && only_if[(i64)blockIdx.y * OS_SLOT_INTS] == 0) return;
+  if (only_if != nullptr && (only_if[(i64)blockIdx.y * OS_SLOT_INTS] & only_mask) == 0) return;
   const i64 total = rows * r;
   for (i64 e = (i64)blockIdx.x * blockDim.x + threadIdx.x; e < total; e += (i64)gridDim.x * blockDim.x) {
     const i64 i = e / r, c = e % r;

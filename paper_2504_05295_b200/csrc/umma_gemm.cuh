@@ -34,6 +34,7 @@
 
 #include "dion_common.cuh"
 #include "simt_gemm.cuh"
+#include "umma_api.cuh"
 
 namespace dion {
 namespace umma {
@@ -44,7 +45,6 @@ constexpr int NUM_PROD_WARPS = 8;
 constexpr int NUM_PROD_THREADS = NUM_PROD_WARPS * 32;
 constexpr int NUM_THREADS = (NUM_EPI_WARPS + NUM_PROD_WARPS + 1) * 32;
 constexpr int NUM_THREADS_TMA = NUM_THREADS + 32;   // one more warp issues the TMA loads
-constexpr long long SPIN_LIMIT_CYCLES = 2000000000LL;  // about one second
 
 struct Params {
   alignas(64) CUtensorMap tmA, tmA2, tmB, tmB2;   // TMA variants: tiles of A, of its addend (or its "lo" array), of B (and its "lo" array)
@@ -1431,7 +1431,7 @@ inline cudaError_t set_pair_attr() {
   return e;
 }
 // How many CTA pairs can be resident at once (per device, asked once).
-inline int pair_clusters(int sm_count) {
+int pair_clusters(int sm_count) {
   static int cached[64] = {};
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess) { cudaGetLastError(); return sm_count / 2; }
@@ -1565,7 +1565,7 @@ inline bool make_operand_map(CUtensorMap* map, const void* ptr, i64 rows, i64 K,
 }  // namespace umma
 
 // One-time set-up of the tensor-core kernels: opt in to their dynamic shared memory.
-inline int umma_configure() {
+int umma_configure() {
   using namespace umma;
   // function attributes belong to a device's context: once per device of this process
   static bool done_on[64] = {};
@@ -1621,19 +1621,10 @@ inline int umma_configure() {
   return DION_OK;
 }
 
-// Launches the product on the tensor cores if it qualifies.  Returns the number of
-// kernels launched (1, or 2 with a split-K reduction), 0 if this engine does not take
-// the product, or a negative DION_ERR_* code.
-// `variant` (test hook, 0 in the product): UMMA_VARIANT_* bits.
-enum : int {
-  UMMA_VARIANT_REGISTER_LOADS = 1,   // operands through registers instead of TMA
-  UMMA_VARIANT_WITHHOLD = 2,         // with register loads: withhold one producer arrival, 1 ms wait budget
-  UMMA_VARIANT_NO_PAIRS = 4          // single-CTA tiles where the product would take CTA pairs
-};
 constexpr i64 PAIR_MIN_ROWS = 512;   // smallest output height given to CTA pairs
 constexpr i64 PAIR_MIN_TRI = 2048;   // smallest lower-triangular output given to CTA pairs
-inline int umma_try_launch(const GemmArgs& g_in, int precision, int sm_count, float* part, i64 part_floats,
-                           int* status, cudaStream_t st, int variant = 0) {
+int umma_try_launch(const GemmArgs& g_in, int precision, int sm_count, float* part, i64 part_floats,
+                           int* status, cudaStream_t st, int variant) {
   using namespace umma;
   GemmArgs g = g_in;
   const bool d16 = g.ab16 != 0;      // bf16 operands in memory
@@ -1836,6 +1827,7 @@ inline int umma_try_launch(const GemmArgs& g_in, int precision, int sm_count, fl
     }
   }
   if (cudaGetLastError() != cudaSuccess) return DION_ERR_CUDA;
+  if (g.splits_out != nullptr) { *g.splits_out = splits; return 1; }      // (the caller sums the partial products itself)
   if (splits > 1) {
     const i64 total = g.M * g.N;
     int blocks = (int)((total + 255) / 256);
