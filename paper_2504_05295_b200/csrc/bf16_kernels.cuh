@@ -201,6 +201,19 @@ __global__ void __launch_bounds__(256) k_split_bf16_chain(const ChainPtrs srcs, 
                   copy != nullptr ? copy + b * ostride : nullptr);
 }
 
+// Dense fp32 copies of a chain's matrices (blockIdx.y; sources from a pointer table, 16-byte aligned rows, cols a multiple
+// of 4), `ostride` floats apart.
+__global__ void __launch_bounds__(256) k_copy_chain(const ChainPtrs srcs, i64 lds, i64 rows, i64 cols, float* __restrict__ out, i64 ostride) {
+  pdl_enter();
+  const float* __restrict__ src = reinterpret_cast<const float*>(srcs.p[blockIdx.y]);
+  out += (i64)blockIdx.y * ostride;
+  const i64 per_row = cols / 4, total = rows * per_row;
+  for (i64 e = (i64)blockIdx.x * blockDim.x + threadIdx.x; e < total; e += (i64)gridDim.x * blockDim.x) {
+    const i64 i = e / per_row, c = (e - i * per_row) * 4;
+    *reinterpret_cast<float4*>(out + i * cols + c) = *reinterpret_cast<const float4*>(src + i * lds + c);
+  }
+}
+
 // out = src with every value rounded to the nearest TF32 number (10 explicit mantissa bits, ties away
 // from zero), rows x cols (cols a multiple of 4, src rows 16-byte aligned), out dense.  The tensor core
 // truncates an fp32 operand to TF32 when it reads it; on pre-rounded values that truncation is exact, so a

@@ -443,7 +443,7 @@ __device__ __forceinline__ void potrf64(ctile_t L, ctile_t X, const Potrf64Set& 
 //
 // The right-looking form took one launch per 64 columns, ~21 us each, whatever the trailing work (r = 1024: 19 launches,
 // 440 us with the solve's products; now 230 us).  Bound by the chain of diagonal blocks, ~9 us each.  Here the chain
-// D_k -> L_{k+1,k} -> A_{k+1,k+1} -> D_{k+1} stays inside ONE CTA (the "runner" of its matrix: two 64^3 products on
+// D_k -> L_{k+1,k} -> A_{k+1,k+1} -> D_{k+1} stays inside ONE CTA (the "runner" of its matrix: two 64^3 products
 // and potrf64 per step), and every other tile is a task of a helper CTA, left-looking:
 //   L(i,k)    = (A_ik - sum_{j<k} L_ij L_kj^T) D_k^T                       i >= k + 3  (the runner makes i = k + 1)
 //   DIAG(k)   = A_kk - sum_{j<k-1} L_kj L_kj^T     for the runner's step k (it adds the last term); also makes L_{k,k-2}
@@ -455,8 +455,7 @@ __device__ __forceinline__ void potrf64(ctile_t L, ctile_t X, const Potrf64Set& 
 // (tiles of a row are finished in the order of k) and one for D; a consumer's thread 0 polls with acquire loads.
 // Helper tasks are handed out in the order of steps (the panel's a few steps behind the factor's), so a task only
 // ever waits for tasks handed out before it and for the runners, which are resident: the launch is cooperative.  Only the
-// preparations are handed out `ahead` steps early; they hold no more than half of the helpers.  And
-// every wait has a cycle limit (then DION_STATUS_TIMEOUT and os[OS_FAIL], and every CTA leaves).
+// preparations are handed out `ahead` steps early; they hold no more than half of the helpers.  Every wait has a cycle limit (then DION_STATUS_TIMEOUT and os[OS_FAIL], and every CTA leaves).
 // The last CTA to leave clears the counters for the next launch and evaluates the round (adaptive rounds).
 // ---------------------------------------------------------------------------------------------------------------
 enum : int { FLOW_TICKET = 0, FLOW_LEFT = 1, FLOW_ABORT = 2, FLOW_SM_BITS = 8, FLOW_SM_WORDS = 8, FLOW_HEAD_INTS = 32 };   // head of the control block

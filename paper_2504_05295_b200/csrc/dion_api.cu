@@ -61,7 +61,7 @@ struct Layout {
   i64 B32;                  // fp32 mode: M + G formed once per step (0: the products form it on the fly)
   i64 Psave;                // CholeskyQR2: the panel as the product wrote it, kept for the fallback (0: none)
   i64 fb_part, fb_h, fb_n;  // fallback kernel: partial dot products (SMs x r), their sums (r), partial norms (SMs)
-  i64 probe_y, probe_part;  // CholeskyQR2's orthogonality probe: U1 z (rows x NPROBE), partial U1^T (U1 z)
+  i64 probe_y, probe_part, probe_sums;  // CholeskyQR2's orthogonality probe: U1 z (rows x NPROBE), partial U1^T (U1 z), partial estimates
   i64 Bp;                   // fp32 mode, M + G in scratch: the same sum as a bf16 (hi, lo) pair (m x n x 2 bf16) for R; 0: none
   i64 Bh;                   // full rank: M + G as a scaled pair of half arrays for P (m x n x 2 halves), 0: none
   i64 pmax;                 // ... its partial maxima and the product's scale factor (like gmax)
@@ -126,6 +126,16 @@ void colnorm_plan(i64 rows, i64 r, int sm, int* chunks, i64* rows_per) {
   *rows_per = per;
   *chunks = (int)((rows + per - 1) / per);
 }
+
+// Row chunks of the probe's second pass: 32 rows (enough blocks to hide a block's few dependent loads; 4096 x 1024: 31 ->
+// 12 us against the 55 rows that one wave of blocks would take), more on tall panels (512 chunks of partial sums).
+void probe_plan(i64 rows, int* chunks, i64* rows_per) {
+  i64 per = (rows + 511) / 512;
+  if (per < 32) per = 32;
+  *rows_per = per;
+  *chunks = (int)((rows + per - 1) / per);
+}
+i64 probe_sums(i64 r) { return (r * NPROBE + PD_ENTRIES - 1) / PD_ENTRIES; }
 
 // fp32 mode on the tensor engine: M + G is formed once per step in scratch, as fp32 (4 bytes per element) and as a
 // bf16 (hi, lo) pair (4 bytes), and P, R and the error feedback read those.  Forming it inside the two products
@@ -216,7 +226,12 @@ Layout make_layout(const dion_ctx* c, i64 m, i64 n, i64 r) {
   if (L.Bp > 0 && (double)m * (double)n * (double)r >= P_PAIR_MIN_MNR) { L.Qc = o; o += align64(big * r); }
   L.S16 = o; o += align64(big * r);
   L.probe_y = o; o += align64(big * NPROBE);
-  L.probe_part = o; o += align64((i64)(L.cn_chunks + 1) * r * NPROBE);
+  {
+    int chunks; i64 per;
+    probe_plan(big, &chunks, &per);
+    L.probe_part = o; o += align64((i64)(chunks + 1) * r * NPROBE);
+    L.probe_sums = o; o += align64(probe_sums(r));
+  }
   if (may_fallback(c, m, n, r)) {
     L.Psave = o; o += align64(big * r);
     L.fb_part = o; o += align64((i64)c->sm_count * r);
@@ -664,7 +679,7 @@ int potrf_blocked(StepCtx& s, i64 r, int mode, const std::function<int(i64, i64)
 int probe(StepCtx& s, i64 off, i64 rows, i64 r, int phase) {
   dion_ctx* c = s.c;
   int chunks; i64 per;
-  colnorm_plan(rows, r, c->sm_count, &chunks, &per);
+  probe_plan(rows, &chunks, &per);
   const int* keep = (phase == PROBE_AFTER_REDO) ? (const int*)(s.os + OS_DONE) : nullptr;
   if (r % 4 == 0 && r >= 128) {
     i64 blocks = (rows + 31) / 32;          // a block of 8 warps takes 32 rows at a time
@@ -683,8 +698,8 @@ int probe(StepCtx& s, i64 off, i64 rows, i64 r, int phase) {
     launch_pdl(k_probe_w, dim3((unsigned)((r + 127) / 128), (unsigned)chunks, (unsigned)s.nb), dim3(128), 0, s.st,
                (const float*)(s.ws + off), r, rows, r, per, (const float*)(s.ws + s.L.probe_y), s.ws + s.L.probe_part, s.wstride, keep);
   DION_CHECK_LAUNCH(c);
-  launch_pdl(k_probe_decide, dim3((unsigned)s.nb), dim3(r >= 128 ? 1024 : 256), 0, s.st, (const float*)(s.ws + s.L.probe_part), chunks, r, s.os,
-             ORTH_TAU_F, c->dev_ints + 2, s.wstride, phase);
+  launch_pdl(k_probe_decide, dim3((unsigned)probe_sums(r), (unsigned)s.nb), dim3(PD_ENTRIES * PD_GROUPS), 0, s.st, (const float*)(s.ws + s.L.probe_part), chunks,
+             r, s.os, ORTH_TAU_F, c->dev_ints + 2, s.ws + s.L.probe_sums, s.wstride, phase);
   DION_CHECK_LAUNCH(c);
   return DION_OK;
 }
@@ -1565,6 +1580,24 @@ int step_batch(dion_ctx* c, const dion_matrix* const* list, int nb, float lr, cu
     }
     if (all_ok) { DION_TRY(split_chain(s, srcs, lds, qrow, r, s.L.S16, nullptr, s.L.Qc > 0 ? s.L.Qc : -1, &q_copied)); q_split = true; }
   }
+  // The other products of a chain read the callers' Q; dense copies of them in the scratch slices (S16, free until the
+  // error feedback) let one launch take the whole chain: 84 matrices of up to 768 x 3072 at r = 192 went through 147
+  // launches of a few tiles each, 1670 us.
+  bool q_dense = false;
+  if (nb > 1 && nb <= GEMM_TAB_MAX && c->chain_batch && b32 && !ppair && !p_half_ready && r % 4 == 0) {
+    bool all_ok = true;
+    for (int b = 0; b < nb; ++b) {
+      all_ok = all_ok && !((uintptr_t)list[b]->Q & 15) && list[b]->ldq == list[0]->ldq && list[b]->ldq % 4 == 0;
+      srcs[b] = (const float*)list[b]->Q;
+    }
+    if (all_ok) {
+      ChainPtrs t;
+      for (int b = 0; b < nb; ++b) t.p[b] = srcs[b];
+      launch_pdl(k_copy_chain, dim3((unsigned)grid_for(c, qrow * r / 4), (unsigned)nb), dim3(256), 0, st, t, list[0]->ldq, qrow, r, s.ws + s.L.S16, s.wstride);
+      DION_CHECK_LAUNCH(c);
+      q_dense = true;
+    }
+  }
   for (int b = 0; b < nb; ++b) {
     const dion_matrix* a = list[b];
     GemmArgs p = gemm_args();
@@ -1603,7 +1636,8 @@ int step_batch(dion_ctx* c, const dion_matrix* const* list, int nb, float lr, cu
       p.alpha_dev = s.W(b, s.L.pmax) + AMAX_PARTS;
     } else if (b32) {
       p.A = s.W(b, s.L.B32); p.a_si = tr ? 1 : n; p.a_sk = tr ? n : 1;
-      p.B = (const float*)a->Q; p.b_sk = a->ldq; p.b_sn = 1;
+      if (q_dense) { p.B = s.W(b, s.L.S16); p.b_sk = r; p.b_sn = 1; }
+      else { p.B = (const float*)a->Q; p.b_sk = a->ldq; p.b_sn = 1; }
     } else {
       p.A = (const float*)a->M; p.a_si = tr ? 1 : a->ldm; p.a_sk = tr ? a->ldm : 1;
       p.A2 = a->G; p.a2_si = tr ? 1 : a->ldg; p.a2_sk = tr ? a->ldg : 1; p.a2_mode = g_mode(a);
@@ -2474,7 +2508,7 @@ bool preload_kernels() {
   ok = ok && touch_kernel(k_gemm_simt<128, 128, 8, 8, 8>) && touch_kernel(k_gemm_simt<64, 64, 16, 4, 4>);
   ok = ok && touch_kernel(k_splitk_reduce) && touch_kernel(k_round_begin) && touch_kernel(k_chol_flow<true>);
   ok = ok && touch_kernel(k_chol_flow<false>) && touch_kernel(k_round_end) && touch_kernel(k_tiny_cholqr2);
-  ok = ok && touch_kernel(k_probe_y) && touch_kernel(k_probe_y4) && touch_kernel(k_probe_w) && touch_kernel(k_probe_decide) && touch_kernel(k_reset_rounds);
+  ok = ok && touch_kernel(k_probe_y) && touch_kernel(k_probe_y4) && touch_kernel(k_probe_w) && touch_kernel(k_probe_w4) && touch_kernel(k_probe_decide) && touch_kernel(k_reset_rounds);
   ok = ok && touch_kernel(k_orth_finish) && touch_kernel(k_cgs_fallback) && touch_kernel(k_copy_block);
   ok = ok && touch_kernel(k_colsumsq_partial) && touch_kernel(k_colnorm_apply) && touch_kernel(k_copy_panel);
   ok = ok && touch_kernel(k_latch_flag) && touch_kernel(k_finish_step) && touch_kernel(k_hh_reflector);

@@ -427,7 +427,7 @@ __global__ void __launch_bounds__(128) k_probe_w(const float* __restrict__ U, i6
   for (int p = 0; p < NPROBE; ++p) out[p] = acc[p];
 }
 
-// The same for r a multiple of 4: a thread takes four neighbouring columns (one 16-byte load per row, four rows'
+// The same for r a multiple of 4: a thread takes four neighbouring columns (one 16-byte load per row, eight rows'
 // loads in flight); every column's sum runs over the chunk's rows in the same order as above.
 // grid = (ceil(r/512), chunks, matrices).
 __global__ void __launch_bounds__(128) k_probe_w4(const float* __restrict__ U, i64 ld, i64 rows, i64 r,
@@ -445,7 +445,7 @@ __global__ void __launch_bounds__(128) k_probe_w4(const float* __restrict__ U, i
   for (int c = 0; c < 4; ++c)
 #pragma unroll
     for (int p = 0; p < NPROBE; ++p) acc[c][p] = 0.f;
-#pragma unroll 4
+#pragma unroll 8
   for (i64 i = i0; i < i1; ++i) {
     const float4 u4 = *reinterpret_cast<const float4*>(U + i * ld + j);
     const float4 y0 = *reinterpret_cast<const float4*>(Y + i * NPROBE);
@@ -467,42 +467,65 @@ __global__ void __launch_bounds__(128) k_probe_w4(const float* __restrict__ U, i
   }
 }
 
-// One block per matrix: est = sum_p |w_p - z_p|^2 / NPROBE (fixed summation order) into os[OS_MAXDEV] (float
-// bits); est <= tau_f^2 * r  ->  the panel is done (OS_DONE = 1: the rest of the second round is skipped).
+// est = sum_p |w_p - z_p|^2 / NPROBE (fixed summation order) into os[OS_MAXDEV] (float bits); est <= tau_f^2 * r  ->  the
+// panel is done (OS_DONE = 1: the rest of the second round is skipped).
 // Counts the rounds of the step that did work (1 or 2; with a recomputed panel 2 or 3).
 // phase PROBE_FAST (the round ran on a panel from the fast product): done -> OS_DONE = 1, else 0 (a failed pivot
 // too: the panel is recomputed before the fallback sees it); nothing is counted.  PROBE_AFTER_REDO: a panel that
 // passed PROBE_FAST keeps its decision (one round); otherwise its recomputed first round is judged.
+// grid = (ceil(r NPROBE / PD_ENTRIES), matrices): a block adds up the chunks of PD_ENTRIES (column, probe) entries, four
+// groups of threads a quarter of the chunks each; the last block of a matrix to arrive (os[OS_BARRIER], left at zero)
+// adds up the blocks' sums.  (One block per matrix took 81 us at r = 1024: a serial walk over 2.4 MB.)
 enum : int { PROBE_CHECK = 0, PROBE_FAST = 1, PROBE_AFTER_REDO = 2 };
-__global__ void __launch_bounds__(1024) k_probe_decide(const float* __restrict__ part, int chunks, i64 r,
-                                                      int* __restrict__ os, float tau_f,
-                                                      int* __restrict__ rounds_total, i64 wstride, int phase) {
+constexpr int PD_ENTRIES = 128, PD_GROUPS = 4;
+__global__ void __launch_bounds__(PD_ENTRIES * PD_GROUPS) k_probe_decide(const float* __restrict__ part, int chunks, i64 r, int* __restrict__ os,
+                                                                         float tau_f, int* __restrict__ rounds_total, float* __restrict__ sums,
+                                                                         i64 wstride, int phase) {
   pdl_enter();
-  part += (i64)blockIdx.x * wstride;
-  os += (i64)blockIdx.x * OS_SLOT_INTS;
+  part += (i64)blockIdx.y * wstride; sums += (i64)blockIdx.y * wstride;
+  os += (i64)blockIdx.y * OS_SLOT_INTS;
   if (phase == PROBE_AFTER_REDO && os[OS_DONE] != 0) {
-    if (threadIdx.x == 0) { os[OS_ROUNDS] = 1; atomicAdd(rounds_total, 1); }
+    if (threadIdx.x == 0 && blockIdx.x == 0) { os[OS_ROUNDS] = 1; atomicAdd(rounds_total, 1); }
     return;
   }
-  __shared__ float red[1024];
-  float e = 0.f;
-  // one (column, probe) entry per thread at a time: consecutive threads read consecutive words of a chunk's partials
-#pragma unroll 4       // (four entries' chunk sums advance together: their loads are independent)
-  for (i64 x = threadIdx.x; x < r * NPROBE; x += blockDim.x) {
-    float w = 0.f;
-#pragma unroll 8      // (eight chunks' loads in flight; the sum keeps its order)
-    for (int c = 0; c < chunks; ++c) w += part[(i64)c * r * NPROBE + x];
-    const float dlt = w - probe_sign(x / NPROBE, (int)(x % NPROBE));
-    e = fmaf(dlt, dlt, e);
+  __shared__ float red[PD_GROUPS][PD_ENTRIES];
+  __shared__ int s_last;
+  const int t = threadIdx.x % PD_ENTRIES, grp = threadIdx.x / PD_ENTRIES;
+  const i64 x = (i64)blockIdx.x * PD_ENTRIES + t;
+  const int per = (chunks + PD_GROUPS - 1) / PD_GROUPS, c0 = grp * per, c1 = min(chunks, c0 + per);
+  float w = 0.f;
+  if (x < r * NPROBE) {
+#pragma unroll 16      // (sixteen chunks' loads in flight; the sum keeps its order)
+    for (int c = c0; c < c1; ++c) w += part[(i64)c * r * NPROBE + x];
   }
-  red[threadIdx.x] = e;
+  red[grp][t] = w;
   __syncthreads();
-  for (int w = (int)blockDim.x / 2; w > 0; w >>= 1) {     // (the block size is a power of two)
-    if ((int)threadIdx.x < w) red[threadIdx.x] += red[threadIdx.x + w];
-    __syncthreads();
+  if (threadIdx.x < PD_ENTRIES) {
+    w = (red[0][t] + red[1][t]) + (red[2][t] + red[3][t]);
+    const float dlt = (x < r * NPROBE) ? w - probe_sign(x / NPROBE, (int)(x % NPROBE)) : 0.f;
+    red[0][t] = dlt * dlt;
   }
-  if (threadIdx.x == 0) {
-    const float est = red[0] / (float)NPROBE;
+  __syncthreads();
+  if (threadIdx.x < 32) {
+    float e = (red[0][t] + red[0][t + 32]) + (red[0][t + 64] + red[0][t + 96]);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) e += __shfl_xor_sync(0xffffffffu, e, o);
+    if (t == 0) {
+      sums[blockIdx.x] = e;
+      __threadfence();
+      s_last = (atomicAdd(&os[OS_BARRIER], 1) == (int)gridDim.x - 1) ? 1 : 0;
+    }
+  }
+  __syncthreads();
+  if (s_last == 0 || threadIdx.x >= 32) return;
+  __threadfence();
+  float e = 0.f;
+  for (int c = t; c < (int)gridDim.x; c += 32) e += __ldcg(sums + c);
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) e += __shfl_xor_sync(0xffffffffu, e, o);
+  if (t == 0) {
+    os[OS_BARRIER] = 0;
+    const float est = e / (float)NPROBE;
     os[OS_MAXDEV] = __float_as_int(est);
     const bool failed = os[OS_FAIL] != 0;       // a pivot of the first round failed: the fallback redoes the panel
     const bool done = !failed && (est <= tau_f * tau_f * (float)r);      // false for NaN
