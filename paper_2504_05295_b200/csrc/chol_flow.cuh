@@ -432,8 +432,8 @@ __device__ __forceinline__ void potrf64(ctile_t L, ctile_t X, const Potrf64Set& 
 //   L L^T = A (lower factor, below the block diagonal), D_k = L_kk^-1, and behind it, tile by tile
 //   and beside the rest of the factorization, either
 //     solve:    U = P L^-T for a panel P (rows x sz), or
-//     inverse:  L^-T of the square's diagonal squares of 512 (row-major, upper triangular, zeros below) for a solve by
-//               tensor-core products.
+//     inverse:  L^-T of the square (row-major, upper triangular; zeros below the diagonal as far as a product of 256-column
+//               tiles reads) for a solve by one tensor-core product, and its largest entry.
 // Pivots: with floor_rel == 0 a pivot that is <= 0 or not finite sets os[OS_FAIL] (and DION_STATUS_BREAKDOWN unless
 // `status` is null) and is replaced by 1, so that everything downstream stays finite.  With floor_rel > 0 (adaptive
 // rounds) a pivot below floor_rel times the column's entry of diag(A) is below the rounding noise of the Gram matrix:
@@ -463,7 +463,7 @@ constexpr int FLOW_CTL_INTS = 64 * 1024;      // ints of a context's control blo
 constexpr int FLOW_COMPUTE = 256;            // threads that compute ...
 constexpr int FLOW_SERVICE = 128;            // ... and the service warps of a runner (four: nothing else fits beside eight anyway)
 constexpr int FLOW_THREADS = FLOW_COMPUTE + FLOW_SERVICE;
-constexpr int FLOW_ISQ = 8;                   // tiles of the squares whose inverses are formed
+constexpr int FLOW_IZ = 4;                    // the inverse's rows are stored (as zeros below the diagonal) up to a multiple of this many tiles
 constexpr int FLOW_LAG = 2;                   // steps by which the panel's tasks follow the factor's
 
 struct FlowArgs {
@@ -478,7 +478,8 @@ struct FlowArgs {
   float* gdiag;             // r floats: diag of the whole Gram matrix, from the caller when gdiag_given (a later square of several), else written here
   int gdiag_given;
   const float* Pin;         // solve: panel rows x r (columns of the square start at o), else null
-  float* Pout;              // solve: the panel's result; inverse: L^-T in the place of the squares (leading dimension r)
+  float* Pout;              // solve: the panel's result; inverse: L^-T in the place of the square (leading dimension r)
+  float* xmax;              // inverse: its largest magnitude, wstride apart per matrix (or null)
   i64 rows;                 // panel rows
   i64 r, o, sz;
   float floor_rel;
@@ -489,6 +490,7 @@ struct FlowArgs {
   i64 wstride; int nb;
   int ahead;                // steps by which the preparations are handed out early (they take on every term since the first column)
   int exclusive;            // a runner has its SM to itself: the helper beside it leaves
+  int near;                 // a matrix whose OS_GOOD is 2 is left alone too (k_near_identity has formed its factor)
   int round_end;            // evaluate the adaptive round
   float good_rel, done_rel;
   int* rounds_total;
@@ -579,7 +581,11 @@ constexpr int FLOW_SMEM = 6 * CB * CLD * (int)sizeof(float);
 template <bool VEC>
 __global__ void __launch_bounds__(FLOW_THREADS, 1) k_chol_flow(const __grid_constant__ FlowArgs f) {
   pdl_enter();
-  if (f.nb == 1 && f.skips && f.os[OS_DONE] != 0) return;
+  auto skipped = [&](int b) -> bool {
+    const int* os = f.os + (i64)b * OS_SLOT_INTS;
+    return (f.skips && os[OS_DONE] != 0) || (f.near && os[OS_GOOD] == 2);
+  };
+  if ((f.skips || f.near) && __syncthreads_and((int)threadIdx.x >= f.nb || skipped((int)threadIdx.x))) return;      // (nb <= 64)
   extern __shared__ __align__(16) float flow_smem[];
   ctile_t SA[2] = {reinterpret_cast<ctile_t>(flow_smem), reinterpret_cast<ctile_t>(flow_smem + 2 * CB * CLD)};
   ctile_t SB[2] = {reinterpret_cast<ctile_t>(flow_smem + CB * CLD), reinterpret_cast<ctile_t>(flow_smem + 3 * CB * CLD)};
@@ -602,7 +608,8 @@ __global__ void __launch_bounds__(FLOW_THREADS, 1) k_chol_flow(const __grid_cons
   auto rowL = [&](int b, int i) { return ctl_of(b) + i; };
   auto prep = [&](int b, int k) { return ctl_of(b) + T + k; };
   auto doneD = [&](int b) { return ctl_of(b) + 2 * T; };
-  auto rowU = [&](int b, int I) { return ctl_of(b) + 2 * T + 1 + I; };
+  auto xmaxbits = [&](int b) { return ctl_of(b) + 2 * T + 1; };
+  auto rowU = [&](int b, int I) { return ctl_of(b) + 2 * T + 2 + I; };
   // entries of the square of matrix b's Gram matrix as the product left it: this thread's 16 of tile (i, k) (zeros
   // beyond the square) ...
   auto raw_tile = [&](int b, int i, int k, float (&v)[4][4]) {
@@ -678,7 +685,7 @@ __global__ void __launch_bounds__(FLOW_THREADS, 1) k_chol_flow(const __grid_cons
     // wait, load or fence is left on the chain but the barriers between the two.
     const int b = (int)blockIdx.x;
     int* os = f.os + (i64)b * OS_SLOT_INTS;
-    if (!(f.skips && os[OS_DONE] != 0)) {
+    if (!skipped(b)) {
       float* G = f.L + (i64)b * f.wstride;
       float* gdiag = f.gdiag + (i64)b * f.wstride;
       float* Dinv = f.Dinv + (i64)b * f.wstride;
@@ -805,7 +812,8 @@ __global__ void __launch_bounds__(FLOW_THREADS, 1) k_chol_flow(const __grid_cons
     nL = max(T - 3 - s, 0);
     nS = (s == 0) ? 2 * min(max(T - 2, 0), f.ahead + 1) : 2 * min(max(T - 2 - s - f.ahead, 0), 1);
     nP = 0;
-    if (s >= FLOW_LAG && s - FLOW_LAG < T) nP = solve ? NR : min(FLOW_ISQ, T - (s - FLOW_LAG) / FLOW_ISQ * FLOW_ISQ);
+    const int k = s - FLOW_LAG;
+    if (k >= 0 && k < T) nP = solve ? NR : min(T, k / FLOW_IZ * FLOW_IZ + FLOW_IZ);
   };
   auto fetch_task = [&](int ticket) -> FlowTask {
     FlowTask t;
@@ -824,7 +832,7 @@ __global__ void __launch_bounds__(FLOW_THREADS, 1) k_chol_flow(const __grid_cons
           t.type = FT_L; t.i = step + 3 + e; t.k = step;
         } else {
           t.type = FT_PANEL; t.k = step - FLOW_LAG;
-          t.i = e - nL + (solve ? 0 : t.k / FLOW_ISQ * FLOW_ISQ);
+          t.i = e - nL;
         }
         return t;
       }
@@ -844,7 +852,7 @@ __global__ void __launch_bounds__(FLOW_THREADS, 1) k_chol_flow(const __grid_cons
     const FlowTask t = s_task;
     if (t.type == FT_NONE) break;
     const int b = t.b;
-    if (f.skips && f.os[(i64)b * OS_SLOT_INTS + OS_DONE] != 0) { bar_named<1, FLOW_COMPUTE>(); continue; }
+    if (skipped(b)) { bar_named<1, FLOW_COMPUTE>(); continue; }
     float* G = f.L + (i64)b * f.wstride + f.o * ld + f.o;
     const float* Dk = ((t.type == FT_PANEL) ? f.Dinv : f.DinvP) + (i64)b * f.wstride + (i64)(f.o / CB + ((t.type == FT_SUB || t.type == FT_DIAG) ? t.k - 2 : t.k)) * (CB * CB);
     float* U = f.Pout + (i64)b * f.wstride + (solve ? f.o : f.o * ld + f.o);
@@ -969,6 +977,15 @@ __global__ void __launch_bounds__(FLOW_THREADS, 1) k_chol_flow(const __grid_cons
       st ^= 1;
     }
     if (!alive) break;
+    if (panel && !solve && f.xmax != nullptr) {      // (a maximum: the order of arrival does not matter)
+      float m = 0.f;
+#pragma unroll
+      for (int q = 0; q < 4; ++q)
+#pragma unroll
+        for (int x = 0; x < 4; ++x) m = fmaxf(m, fabsf(v[q][x]));
+      const unsigned u = __reduce_max_sync(0xffffffffu, __float_as_uint(m));
+      if ((tid & 31) == 0) atomicMax(xmaxbits(b), (int)u);
+    }
     if (prepares) store_tile(G + (i64)t.i * CB * ld + (i64)kw * CB, nrow, cols_of(kw), w);
     else store_tile((panel ? U : G) + (i64)t.i * CB * ld + (i64)t.k * CB, nrow, ncol, v);
     bar_named<1, FLOW_COMPUTE>();
@@ -992,11 +1009,15 @@ __global__ void __launch_bounds__(FLOW_THREADS, 1) k_chol_flow(const __grid_cons
   asm volatile("fence.acq_rel.gpu;" ::: "memory");
   const bool aborted = flow_ld(f.ctl + FLOW_ABORT) != 0;
   __syncthreads();
+  if (f.xmax != nullptr)
+    for (int b = tid; b < f.nb; b += FLOW_THREADS)
+      if (!skipped(b)) f.xmax[(i64)b * f.wstride] = __int_as_float(flow_ld(xmaxbits(b)));
+  __syncthreads();
   const int nints = FLOW_HEAD_INTS + f.nb * f.ctl_stride;
   for (int e = tid; e < nints; e += FLOW_THREADS) f.ctl[e] = 0;
   for (int b = tid; b < f.nb; b += FLOW_THREADS) {
     int* os = f.os + (i64)b * OS_SLOT_INTS;
-    if (f.skips && os[OS_DONE] != 0) continue;
+    if (skipped(b)) continue;
     if (aborted) { os[OS_FAIL] = 1; continue; }
     if (f.round_end == 0) continue;
     round_evaluate(os, f.good_rel, f.done_rel, f.rounds_total);

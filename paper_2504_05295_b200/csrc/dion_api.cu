@@ -46,8 +46,11 @@ constexpr double P_PAIR_MIN_MNR = 1.5e10;       // smallest m n r whose P = (M +
 constexpr i64 NBO_COLS = 512;  // = NBO, the outer block of the two-level Cholesky (defined below)
 
 // One launch of k_chol_flow factors Gram matrices up to this order; beyond it blocks of 512 columns.
-constexpr i64 FLOW_MAX_R = 2048;
-constexpr double FLOW_SOLVE_MAX = 6e9;          // largest rows r^2 whose panel that launch solves too
+constexpr i64 FLOW_MAX_R = 3072;
+constexpr double FLOW_SOLVE_MAX = 1.1e6;        // largest rows r whose panel that launch solves too
+constexpr i64 FLOW_SOLVE_MAX_TILES = 60000;     // ... in an adaptive round: most 64^3 products of its substitution
+constexpr float NEAR_MAX_DEF = 3e-3f;           // largest |P^T P - I|_F whose factor is taken as a series (k_near_identity): third-order error 3e-8
+constexpr i64 NEAR_MAX_BLOCKS = 512;
 constexpr int FLOW_EXCLUSIVE_MAX = 8;           // matrices of a chain up to which its runners get an SM each
 constexpr int FLOW_AHEAD_MAX = 16;              // steps by which its preparations are handed out early
 constexpr i64 FLOW_MAX_PANEL_TILES = 800;       // ... and most 64-row blocks of it (the control block holds 64 such matrices)
@@ -67,6 +70,8 @@ struct Layout {
   i64 pmax;                 // ... its partial maxima and the product's scale factor (like gmax)
   i64 SolveP, LfP, smax;    // blocked solves on half pairs (r > 512): pair of a rows x 512 right-hand side; pairs of a row block of
                             // the factor (512 x r) and of a diagonal inverse (512 x 512); partial maxima and scales
+  i64 XP;                   // scaled half pair of the inverse of the factor
+  i64 xmax;                 // largest magnitude of the factor's inverse, then the scale of the product with its pair
   i64 gmax;                 // Gram matrices on half pairs: AMAX_PARTS partial maxima of |P|, then 1 / scale^2
   i64 Qc;                   // fp32 mode, large matrices: dense fp32 copy of Q for the chain-wide recomputation of P (0: none)
   i64 S16;                  // fp32 mode: the bf16 (hi, lo) pair of the error feedback's second factor (max(m,n) x r x 2 bf16)
@@ -176,6 +181,7 @@ Layout make_layout(const dion_ctx* c, i64 m, i64 n, i64 r) {
   L.Gram = o; o += align64(r * r);
   L.Linv = o; o += align64(r * r);
   L.Tbuf = o; o += align64(r * r);
+  L.XP = o; o += align64(r <= FLOW_MAX_R ? r * r : 64);
   L.Dinv = o; o += align64(((r + NB - 1) / NB) * (i64)NB * NB);
   L.DinvP = o; o += align64(((r + NB - 1) / NB) * (i64)NB * NB);
   // split-K partials: the largest plain-store product of a step is max(m,n) x r
@@ -184,7 +190,7 @@ Layout make_layout(const dion_ctx* c, i64 m, i64 n, i64 r) {
   L.part_floats = pf;
   L.part = o; o += align64(pf);
   colnorm_plan(big, r, c->sm_count, &L.cn_chunks, &L.cn_rows);
-  L.cn_part = o; o += align64((i64)(L.cn_chunks + 1) * r);
+  L.cn_part = o; o += align64((i64)(L.cn_chunks + 1) * r + NEAR_MAX_BLOCKS);
   L.d = o; o += align64(r);
   L.gdiag = o; o += align64(r);
   L.scal = o; o += 64;
@@ -211,8 +217,9 @@ Layout make_layout(const dion_ctx* c, i64 m, i64 n, i64 r) {
   }
   L.Psave = L.fb_part = L.fb_h = L.fb_n = 0;
   L.gmax = o; o += align64(AMAX_PARTS + 64);
+  L.xmax = o; o += 64;
   L.SolveP = L.LfP = L.smax = 0;
-  if (r > NBO_COLS && (double)big * (double)r >= SOLVE_PAIR_MIN_PANEL) {
+  if (r > FLOW_MAX_R && (double)big * (double)r >= SOLVE_PAIR_MIN_PANEL) {
     L.SolveP = o; o += align64(big * NBO_COLS);
     L.LfP = o; o += align64(NBO_COLS * r + NBO_COLS * NBO_COLS);
     L.smax = o; o += align64(3 * (AMAX_PARTS + 64));
@@ -551,22 +558,25 @@ inline bool rm_precise(int mode) { return mode == RM_ADAPTIVE || mode == RM_FIRS
 // ints of the control block per matrix: progress of the rows of L and of the preparations, of D, of the panel's rows
 int flow_ctl_ints(i64 sz, i64 rows) {
   const i64 T = (sz + CB - 1) / CB, NR = (rows + CB - 1) / CB;
-  return (int)((2 * T + 1 + (NR > T ? NR : T) + 31) / 32 * 32);
+  return (int)((2 * T + 2 + (NR > T ? NR : T) + 31) / 32 * 32);
 }
-// Panels that the factorization's launch solves too (beside the factorization, on the FMA pipes: rows r^2 multiply-adds);
-// larger ones take tensor-core products behind it.  The rule looks at the shape alone (grouped calls compute what
-// single ones do).
-bool flow_solves(const StepCtx& s, i64 rows, i64 r) {
-  return (double)rows * (double)r * (double)r <= FLOW_SOLVE_MAX &&
-         (rows + CB - 1) / CB <= FLOW_MAX_PANEL_TILES;
+// Panels that the factorization's launch solves too, beside the factorization.  The rule looks at the shape alone (grouped
+// calls compute what single ones do).  CholeskyQR2: small panels; larger ones take one product behind it, before the
+// helpers' 64^3 products outlast the chain of diagonal blocks (more so with several matrices).  Adaptive rounds: up to the
+// number of tile products (~1.3 us of one SM each) that the blocked solve's tensor-core products would take as long for.
+bool flow_solves(const StepCtx& s, i64 rows, i64 r, bool adaptive) {
+  (void)s;
+  const i64 T = (r + CB - 1) / CB, NR = (rows + CB - 1) / CB;
+  if (r > FLOW_MAX_R || NR > FLOW_MAX_PANEL_TILES) return false;
+  return adaptive ? NR * T * (T + 1) / 2 <= FLOW_SOLVE_MAX_TILES : (double)rows * (double)r <= FLOW_SOLVE_MAX;
 }
 
 // One launch of the factorization (k_chol_flow) on the diagonal square [o, o + sz) of the Gram matrices, with either
-// the solve of the panel at pin_off into pout_off (rows > 0; the whole Gram matrix, o = 0 and sz = r) or the inverses of its
-// diagonal squares of 512 (transposed: L^-T, upper triangular) into L.Linv.  nsplit > 1: the Gram matrix is still the
-// product's partial sums (alpha_dev: their scale).
+// the solve of the panel at pin_off into pout_off (rows > 0; the whole Gram matrix, o = 0 and sz = r) or the inverse of its
+// factor (transposed: L^-T, upper triangular) into L.Linv.  nsplit > 1: the Gram matrix is still the
+// product's partial sums (alpha_dev: their scale).  near: see k_near_identity.
 int chol_flow(StepCtx& s, i64 r, i64 o, i64 sz, int mode, i64 pin_off, i64 pout_off, i64 rows, int nsplit, const float* alpha_dev,
-              bool round_end) {
+              bool round_end, bool near = false) {
   dion_ctx* c = s.c;
   const bool adaptive = (mode == RM_ADAPTIVE);
   FlowArgs f;
@@ -591,6 +601,8 @@ int chol_flow(StepCtx& s, i64 r, i64 o, i64 sz, int mode, i64 pin_off, i64 pout_
   f.ctl = c->flow_ctl;
   f.ctl_stride = flow_ctl_ints(sz, rows);
   f.wstride = s.wstride; f.nb = s.nb;
+  f.xmax = solve ? nullptr : s.ws + s.L.xmax;
+  f.near = near ? 1 : 0;
   f.round_end = (round_end && adaptive) ? 1 : 0;
   f.good_rel = GOOD_REL; f.done_rel = DONE_REL; f.rounds_total = c->dev_ints + 2;
   f.limit = umma::SPIN_LIMIT_CYCLES;
@@ -598,7 +610,7 @@ int chol_flow(StepCtx& s, i64 r, i64 o, i64 sz, int mode, i64 pin_off, i64 pout_
   // one runner per matrix; as many helpers as can be resident beside them, at most one per task
   i64 tasks = (T > 2) ? (T - 2) * (T - 3) / 2 + 2 * (T - 2) : 0;
   if (solve) tasks += NR * T;
-  else for (i64 k = 0; k < T; ++k) tasks += (T - k / FLOW_ISQ * FLOW_ISQ < FLOW_ISQ) ? T - k / FLOW_ISQ * FLOW_ISQ : FLOW_ISQ;
+  else for (i64 k = 0; k < T; ++k) tasks += (T < k / FLOW_IZ * FLOW_IZ + FLOW_IZ) ? T : k / FLOW_IZ * FLOW_IZ + FLOW_IZ;
   const i64 cap = (i64)flow_ctas_per_sm() * c->sm_count;
   i64 grid = s.nb + tasks * s.nb;
   if (grid > cap) grid = cap;
@@ -724,7 +736,7 @@ bool gram_on_pairs(const StepCtx& s, i64 rows, i64 r) {
 // adaptive: columns with negligible pivots are deflated, the round is skipped
 // once the panel is orthonormal, and the round statistics are evaluated at the end.
 int cholqr_round(StepCtx& s, i64 pin_off, i64 pout_off, i64 rows, i64 r, int mode, i64 gram_rows = 0,
-                 int probe_phase = PROBE_CHECK) {
+                 int probe_phase = PROBE_CHECK, int round = 0) {      // round: of the adaptive rounds
   // A skipped round leaves Pout untouched (the caller keeps using Pin).
   // gram_rows > 0: the Gram matrix is formed from the first gram_rows rows only (a sketch stacked on
   // top of the panel); the factor is applied to all rows
@@ -741,12 +753,13 @@ int cholqr_round(StepCtx& s, i64 pin_off, i64 pout_off, i64 rows, i64 r, int mod
   g.M = r; g.N = r; g.K = gram_rows > 0 ? gram_rows : rows;
   g.A = s.ws + pin_off; g.a_si = 1; g.a_sk = r;
   g.B = s.ws + pin_off; g.b_sk = r; g.b_sn = 1;
-  if (gram_rows == 0 && gram_on_pairs(s, rows, r)) {
-    // The Gram matrix of a tall panel on half pairs: the panel is scaled and split into Pout's buffer (free until
-    // the solve writes it) and the product takes three kind::f16 MMAs per K step instead of the three or four
+  const bool gpairs = gram_rows == 0 && gram_on_pairs(s, rows, r);
+  if (gpairs) {
+    // The Gram matrix of a tall panel on half pairs: the panel is scaled and split into S16 (free during the
+    // orthonormalization) and the product takes three kind::f16 MMAs per K step instead of the three or four
     // kind::tf32 ones; the same 22 significant bits.  1 / scale^2 reaches the epilogue through a device scalar.
     const int* sk = skips ? skip : nullptr;
-    __half* hi = reinterpret_cast<__half*>(s.ws + pout_off);
+    __half* hi = reinterpret_cast<__half*>(s.ws + s.L.S16);
     __half* lo = hi + rows * r;
     i64 parts = (rows * r / 4 + 2047) / 2048;
     if (parts > AMAX_PARTS) parts = AMAX_PARTS;
@@ -763,26 +776,81 @@ int cholqr_round(StepCtx& s, i64 pin_off, i64 pout_off, i64 rows, i64 r, int mod
     g.alpha_dev = s.ws + s.L.gmax + AMAX_PARTS; g.alpha_dev_stride = s.wstride;
   }
   g.C = s.ws + s.L.Gram; g.ldc = r; g.epi = EPI_STORE; g.tri = TRI_LOWER; g.skip_flag = skips ? skip : nullptr; g.precise = rm_precise(mode) ? 1 : 0;
-  const bool flow_all = r <= FLOW_MAX_R;      // the whole factorization in one launch
+  const bool in_flow = flow_solves(s, rows, r, adaptive);      // factorization and solve in one launch
+  const bool flow_all = in_flow || (!adaptive && r <= FLOW_MAX_R);      // at least the whole factorization
   int nsplit = 1;
   if (flow_all) g.splits_out = &nsplit;       // (which also adds up the partial products)
   DION_TRY(launch_gemm_chain(s, g));
   const float* part_scale = g.alpha_dev;
-  if (flow_all && flow_solves(s, rows, r))
-    return chol_flow(s, r, 0, r, mode, pin_off, pout_off, rows, nsplit, part_scale, true);
-  if (!flow_all) {
+  if (flow_all) {
+    // The panel's pair that the Gram matrix was formed from times the scaled half pair of L^-T, one product behind the
+    // factorization (22 significant bits in three kind::f16 MMAs; without a pair 3xTF32): CholeskyQR2 on large panels.
+    // The adaptive rounds solve by substitution instead: an explicit inverse costs a factor cond(L) of backward
+    // stability, and their panels are ill conditioned (2048^2 full rank, cond 1e7: Q off by 2.2e-2 against 3.5e-3).  Their
+    // finishing round has a factor near the identity, and where that is a short series (k_near_identity) the product
+    // replaces the factorization.
+    const NearSrc raw = {s.ws + s.L.Gram, s.ws + s.L.part, nsplit, part_scale};
+    i64 tiles = (r + 31) / 32 * ((r + 31) / 32) / 4;
+    if (tiles < 1) tiles = 1;
+    if (tiles > NEAR_MAX_BLOCKS) tiles = NEAR_MAX_BLOCKS;
+    const bool series = adaptive && gpairs && round > 0;      // (the first round is never the finishing one)
+    if (series) {
+      __half* eh = reinterpret_cast<__half*>(s.ws + s.L.Linv);
+      __half* fh = eh + r * r;
+      launch_pdl(k_near_identity, dim3((unsigned)tiles, (unsigned)s.nb), dim3(256), 0, s.st, raw, r, eh, fh, s.ws + s.L.xmax, s.ws + s.L.cn_part,
+                 s.os, NEAR_MAX_DEF, s.wstride);
+      DION_CHECK_LAUNCH(c);
+      GemmArgs q = gemm_args();      // S = Phi E, lower triangle
+      q.M = r; q.N = r; q.K = r;
+      q.ab16 = 1; q.f16 = 1;
+      q.A = (const float*)fh; q.a_si = r; q.a_sk = 1;
+      q.B = (const float*)eh; q.b_sk = 1; q.b_sn = r;
+      q.C = s.ws + s.L.Tbuf; q.ldc = r; q.epi = EPI_STORE; q.tri = TRI_LOWER; q.alpha = 1.f / (NEAR_SCALE * NEAR_SCALE);
+      q.skip_flag = s.os + OS_NOTNEAR;
+      s.no_split = true;      // (the split-K scratch holds the Gram matrix)
+      const int rc = launch_gemm_chain(s, q);
+      s.no_split = false;
+      DION_TRY(rc);
+    }
+    DION_TRY(chol_flow(s, r, 0, r, mode, pin_off, pout_off, in_flow ? rows : 0, nsplit, part_scale, in_flow, series));
+    if (in_flow && !series) return DION_OK;
+    const int* uskip = in_flow ? (const int*)(s.os + OS_NOTNEAR) : skip;
+    GemmArgs u = gemm_args();
+    u.M = rows; u.N = r; u.K = r;
+    if (gpairs) {
+      __half* ph = reinterpret_cast<__half*>(s.ws + s.L.S16);
+      __half* xh = reinterpret_cast<__half*>(s.ws + s.L.XP);
+      launch_pdl(k_split_f16_tri, dim3((unsigned)tiles, (unsigned)s.nb), dim3(256), 0, s.st, (const float*)(s.ws + s.L.Linv), r,
+                 (const float*)(s.ws + s.L.xmax), (const float*)(s.ws + s.L.gmax + AMAX_PARTS), xh, xh + r * r, s.ws + s.L.xmax + 1, s.wstride,
+                 uskip, raw, series ? (const float*)(s.ws + s.L.Tbuf) : (const float*)nullptr);
+      DION_CHECK_LAUNCH(c);
+      u.ab16 = 1; u.f16 = 1;
+      u.A = (const float*)ph; u.A16lo = ph + rows * r;
+      u.B = (const float*)xh; u.B16lo = xh + r * r;
+      u.alpha_dev = s.ws + s.L.xmax + 1; u.alpha_dev_stride = s.wstride;
+    } else {
+      u.A = s.ws + pin_off;
+      u.B = s.ws + s.L.Linv;
+    }
+    u.a_si = r; u.a_sk = 1; u.b_sk = r; u.b_sn = 1; u.klimit = 1;
+    u.C = s.ws + pout_off; u.ldc = r; u.epi = EPI_STORE; u.skip_flag = uskip;
+    DION_TRY(launch_gemm_chain(s, u));
+    if (series) {
+      launch_pdl(k_near_end, dim3((unsigned)s.nb), dim3(1), 0, s.st, s.os, c->dev_ints + 2);
+      DION_CHECK_LAUNCH(c);
+    }
+    return DION_OK;
+  } else {
     launch_pdl(k_round_begin, dim3((unsigned)(s.nb)), dim3(256), 0, s.st, s.ws + s.L.Gram, r, r, 0.f, s.ws + s.L.gdiag, s.ws + s.L.scal, s.os,
                                           skips ? 1 : 0, s.wstride, c->dev_ints);
     DION_CHECK_LAUNCH(c);
-  }
-  if (r > NBO) {
     // Pout_J = (Pin_J - sum_{K<J} Pout_K L_{J,K}^T) Linv_JJ^T, block columns J of 512.
     // The solves run with the plain 3xTF32 product: their rounding error enters U once (~1e-6),
     // whereas an error in the Gram matrix or its factor is amplified by the panel's conditioning.
     // Block column J needs row block J of the factor and the inverse of its diagonal square, both
     // final once the factorization has passed J: the solves run on a second stream beside the rest
     // of the factorization, whose serial 64-column chain leaves most SMs idle.
-    const float* Lm = s.ws + (flow_all ? s.L.Tbuf : s.L.Gram);     // the factor, lower
+    const float* Lm = s.ws + s.L.Gram;     // the factor, lower
     float* Wt = s.ws + (s.wt_off >= 0 ? s.wt_off : s.L.R);   // rows x 512 temporary (R is free during the orthonormalization)
     // On tall panels the two products of a block column run on scaled half pairs (22 significant bits in three
     // kind::f16 MMAs; 1024-k chains) like the Gram matrix: the right-hand side, the factor's row block and the
@@ -871,7 +939,7 @@ int cholqr_round(StepCtx& s, i64 pin_off, i64 pout_off, i64 rows, i64 r, int mod
       DION_TRY(launch_gemm_chain(s, v));
       return DION_OK;
     };
-    if (!flow_all && c->side != nullptr) {
+    if (c->side != nullptr) {
       cudaStream_t main_st = s.st;
       auto next_event = [&]() { cudaEvent_t e = c->side_ev[c->side_cursor]; c->side_cursor = (c->side_cursor + 1) % 32; return e; };
       const std::function<int(i64, i64)> after_block = [&](i64 J0, i64 sz) -> int {
@@ -886,23 +954,10 @@ int cholqr_round(StepCtx& s, i64 pin_off, i64 pout_off, i64 rows, i64 r, int mod
       cudaEvent_t e = next_event();   // join: the round ends when the last solve has finished
       if (cudaEventRecord(e, c->side) != cudaSuccess || cudaStreamWaitEvent(main_st, e, 0) != cudaSuccess) return DION_ERR_CUDA;
     } else {
-      if (flow_all) DION_TRY(chol_flow(s, r, 0, r, mode, 0, 0, 0, nsplit, part_scale, false));
-      else DION_TRY(potrf_blocked(s, r, mode, nullptr));
+      DION_TRY(potrf_blocked(s, r, mode, nullptr));
       for (i64 J0 = 0; J0 < r; J0 += NBO) DION_TRY(solve_block(J0, (r - J0 < NBO) ? (r - J0) : NBO));
     }
-    if (adaptive) {
-      launch_pdl(k_round_end, dim3((unsigned)(s.nb)), dim3(1), 0, s.st, s.os, GOOD_REL, DONE_REL, c->dev_ints + 2);
-      DION_CHECK_LAUNCH(c);
-    }
-    return DION_OK;
   }
-  DION_TRY(chol_flow(s, r, 0, r, mode, 0, 0, 0, nsplit, part_scale, false));
-  GemmArgs u = gemm_args();
-  u.M = rows; u.N = r; u.K = r;
-  u.A = s.ws + pin_off; u.a_si = r; u.a_sk = 1;
-  u.B = s.ws + s.L.Linv; u.b_sk = r; u.b_sn = 1; u.klimit = 1;
-  u.C = s.ws + pout_off; u.ldc = r; u.epi = EPI_STORE; u.skip_flag = skip;
-  DION_TRY(launch_gemm_chain(s, u));
   if (adaptive) {
     launch_pdl(k_round_end, dim3((unsigned)(s.nb)), dim3(1), 0, s.st, s.os, GOOD_REL, DONE_REL, c->dev_ints + 2);
     DION_CHECK_LAUNCH(c);
@@ -954,8 +1009,8 @@ int householder(StepCtx& s, float* A, float* V, i64 rows, i64 r, int b) {
 int adaptive_rounds(StepCtx& s, i64 off_a, i64 off_b, i64 rows, i64 r, i64 gram_rows) {
   static_assert(MAX_ROUNDS % 2 == 0, "the result must end in the first buffer");
   for (int it = 0; it < MAX_ROUNDS; it += 2) {
-    DION_TRY(cholqr_round(s, off_a, off_b, rows, r, RM_ADAPTIVE, gram_rows));
-    DION_TRY(cholqr_round(s, off_b, off_a, rows, r, RM_ADAPTIVE, gram_rows));
+    DION_TRY(cholqr_round(s, off_a, off_b, rows, r, RM_ADAPTIVE, gram_rows, PROBE_CHECK, it));
+    DION_TRY(cholqr_round(s, off_b, off_a, rows, r, RM_ADAPTIVE, gram_rows, PROBE_CHECK, it + 1));
   }
   {   // an odd number of rounds left the result in the second buffer
     dim3 grid((unsigned)grid_for(s.c, rows * r), (unsigned)s.nb);

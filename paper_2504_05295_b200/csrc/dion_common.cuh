@@ -73,7 +73,8 @@ enum : int {
   OS_ROUNDS = 5,    // rounds that did work
   OS_MAXDEV = 6,    // float bits: the estimate of |U1^T U1 - I|_F^2 of the CholeskyQR2 check
   OS_BARRIER = 7,   // arrival counter of the fallback kernel's grid-wide barriers (zero at the start of a step)
-  OS_SLOT_INTS = 8
+  OS_NOTNEAR = 8,   // adaptive rounds: the finishing round's factor is not the short series (k_near_identity)
+  OS_SLOT_INTS = 16
 };
 
 // Programmatic dependent launch (the small kernels of the serial Cholesky chain): lets the next

@@ -1,6 +1,8 @@
 // Small kernels of the orthonormalization (r x r factor work) and of ColNorm.
 #pragma once
 
+#include <cuda_fp16.h>
+
 #include "chol_flow.cuh"
 #include "dion_common.cuh"
 
@@ -272,6 +274,197 @@ __global__ void __launch_bounds__(TINY_THREADS) k_tiny_cholqr2(const float* __re
     const int i = e2 / r, c = e2 % r;
     Pout[(i64)i * r + c] = Ps[i * TINY_LD + c];
   }
+}
+
+// The finishing round of a panel that is orthonormal already but for a small defect E (its Gram matrix is I + E): the inverse
+// of its triangular factor, transposed, is a short series
+//   X = L^-T = I - Phi^T + Psi^T + O(E^3),  Phi = strictly lower part of E + half its diagonal,
+//   Psi = strictly lower part of S = Phi E, its diagonal (S_ii + Phi_ii^2) / 2
+// (from L L^T = I + E order by order).  Where |E|_F <= max_def and the last round was good (OS_GOOD == 1) this kernel
+// leaves scale x E and scale x Phi as IEEE half arrays for the product S (the second-order term needs few bits) and
+// sets OS_GOOD to 2: the factorization's launch then leaves the matrix alone and k_split_f16_tri puts X together.
+// (At r = 2048 that launch takes 390 us, this and the product 35.)  Else OS_NOTNEAR is set: the product is skipped.
+// Gram matrix: `part` (nsplit partial sums, times *alpha_dev) or G, lower triangle, r a multiple of 8.
+// grid = (blocks, matrices), 256 threads, a 32 x 32 tile at a time; sums: one float per block; OS_BARRIER as in k_probe_decide.
+struct NearSrc {
+  const float* G; const float* part; int nsplit; const float* alpha_dev;
+};
+__device__ __forceinline__ float4 near_load(const NearSrc& g, i64 wo, i64 r, i64 i, i64 j) {      // four entries of E + I
+  if (g.nsplit <= 1) return *reinterpret_cast<const float4*>(g.G + wo + i * r + j);
+  const float* p = g.part + wo + i * r + j;
+  float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
+  for (int q = 0; q < g.nsplit; ++q, p += r * r) {
+    const float4 v = *reinterpret_cast<const float4*>(p);
+    s.x += v.x; s.y += v.y; s.z += v.z; s.w += v.w;
+  }
+  const float a = (g.alpha_dev != nullptr) ? g.alpha_dev[wo] : 1.f;
+  return make_float4(s.x * a, s.y * a, s.z * a, s.w * a);
+}
+constexpr float NEAR_SCALE = 4096.f;
+__global__ void __launch_bounds__(256) k_near_identity(const NearSrc g, i64 r, __half* __restrict__ Eh, __half* __restrict__ Ph,
+                                                       float* __restrict__ xmax, float* __restrict__ sums, int* __restrict__ os, float max_def,
+                                                       i64 wstride) {
+  pdl_enter();
+  os += (i64)blockIdx.y * OS_SLOT_INTS;
+  if (os[OS_DONE] != 0 || os[OS_GOOD] != 1) {
+    if (blockIdx.x == 0 && threadIdx.x == 0) os[OS_NOTNEAR] = 1;
+    return;
+  }
+  const i64 wo = (i64)blockIdx.y * wstride;
+  Eh += 2 * wo; Ph += 2 * wo; xmax += wo; sums += wo;
+  __shared__ float T[32][33];
+  __shared__ float red[8];
+  __shared__ int s_last;
+  const int row = threadIdx.x >> 3, c4 = (threadIdx.x & 7) * 4, lane = threadIdx.x & 31;
+  const int n = (int)((r + 31) / 32);
+  float e2 = 0.f;
+  auto put = [&](__half* dst, const float (&v)[4]) {
+    __half2 a = __floats2half2_rn(NEAR_SCALE * v[0], NEAR_SCALE * v[1]), b = __floats2half2_rn(NEAR_SCALE * v[2], NEAR_SCALE * v[3]);
+    uint2 u;
+    u.x = *reinterpret_cast<uint32_t*>(&a); u.y = *reinterpret_cast<uint32_t*>(&b);
+    *reinterpret_cast<uint2*>(dst) = u;
+  };
+  for (i64 q = blockIdx.x; q < (i64)n * n; q += gridDim.x) {
+    const int ti = (int)(q / n), tj = (int)(q % n);
+    if (tj > ti) continue;
+    const i64 i = (i64)ti * 32 + row, j = (i64)tj * 32 + c4;
+    float e[4] = {0.f, 0.f, 0.f, 0.f}, ph[4];
+    if (i < r && j < r) {
+      const float4 v = near_load(g, wo, r, i, j);
+      e[0] = v.x; e[1] = v.y; e[2] = v.z; e[3] = v.w;
+    }
+#pragma unroll
+    for (int x = 0; x < 4; ++x) {
+      if (j + x > i) e[x] = 0.f;
+      if (j + x == i) e[x] -= 1.f;
+      if (i >= r || j >= r) e[x] = 0.f;
+      e2 = fmaf((i == j + x) ? e[x] : 2.f * e[x], e[x], e2);
+      ph[x] = (i == j + x) ? 0.5f * e[x] : e[x];
+      T[row][c4 + x] = e[x];
+    }
+    __syncthreads();
+    if (i < r && j < r) {
+      put(Ph + i * r + j, ph);
+      if (ti == tj) {
+        float f[4];
+#pragma unroll
+        for (int x = 0; x < 4; ++x) f[x] = (j + x > i) ? T[c4 + x][row] : e[x];
+        put(Eh + i * r + j, f);
+      } else {
+        put(Eh + i * r + j, e);
+      }
+    }
+    if (ti != tj) {      // the mirror tile (tj, ti)
+      const i64 mi = (i64)tj * 32 + row, mj = (i64)ti * 32 + c4;
+      if (mi < r && mj < r) {
+        float f[4];
+        const float z[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+        for (int x = 0; x < 4; ++x) f[x] = T[c4 + x][row];
+        put(Eh + mi * r + mj, f);
+        put(Ph + mi * r + mj, z);
+      }
+    }
+    __syncthreads();
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) e2 += __shfl_xor_sync(0xffffffffu, e2, o);
+  if (lane == 0) red[threadIdx.x >> 5] = e2;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    sums[blockIdx.x] = ((red[0] + red[1]) + (red[2] + red[3])) + ((red[4] + red[5]) + (red[6] + red[7]));
+    __threadfence();
+    s_last = (atomicAdd(&os[OS_BARRIER], 1) == (int)gridDim.x - 1) ? 1 : 0;
+  }
+  __syncthreads();
+  if (s_last == 0 || threadIdx.x >= 32) return;
+  __threadfence();
+  float t = 0.f;
+  for (int c = lane; c < (int)gridDim.x; c += 32) t += __ldcg(sums + c);
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+  if (lane == 0) {
+    os[OS_BARRIER] = 0;
+    os[OS_MAXDEV] = __float_as_int(t);
+    const bool near = t <= max_def * max_def;      // (false for NaN)
+    os[OS_NOTNEAR] = near ? 0 : 1;
+    if (near) {
+      *xmax = 1.f + max_def;
+      os[OS_GOOD] = 2;
+    }
+  }
+}
+
+// The scaled half pair of X = L^-T (n x n, upper triangular, n a multiple of 8) as far down each column as a product of
+// 256-column tiles reads: from src, or, with S given, put together from the Gram matrix and S (k_near_identity).
+// Scale as in k_split_f16_scaled from *amax, the largest magnitude.  *inv_out = 1 / scale, times the root of *other_sq (a power
+// of four: the square of the other operand's 1 / scale).  grid = (blocks, matrices), 256 threads, 32 x 32 tiles.
+__global__ void __launch_bounds__(256) k_split_f16_tri(const float* __restrict__ src, i64 n, const float* __restrict__ amax,
+                                                       const float* __restrict__ other_sq, __half* __restrict__ hi, __half* __restrict__ lo,
+                                                       float* __restrict__ inv_out, i64 wstride, const int* __restrict__ skip_flag,
+                                                       const NearSrc g, const float* __restrict__ S) {
+  pdl_enter();
+  if (skip_flag != nullptr && skip_flag[(i64)blockIdx.y * OS_SLOT_INTS] != 0) return;
+  const bool near = S != nullptr;
+  const i64 wo = (i64)blockIdx.y * wstride;
+  src += wo; hi += 2 * wo; lo += 2 * wo;
+  if (S != nullptr) S += wo;
+  const float m = amax[wo];
+  int ex = 14;                                   // amax = f 2^ex with f in [0.5, 1): scale 2^(14 - ex)
+  if (m > 0.f && m < 3.0e38f) frexpf(m, &ex);
+  if (ex < -100) ex = -100;
+  const float scale = ldexpf(1.f, 14 - ex);
+  if (blockIdx.x == 0 && threadIdx.x == 0) inv_out[wo] = ldexpf(1.f, ex - 14) * sqrtf(other_sq[wo]);
+  __shared__ float T[32][33];
+  const int row = threadIdx.x >> 3, c4 = (threadIdx.x & 7) * 4;
+  const int nt = (int)((n + 31) / 32);
+  for (i64 q = blockIdx.x; q < (i64)nt * nt; q += gridDim.x) {
+    const int tk = (int)(q / nt), tc = (int)(q % nt);      // tile of X: rows tk, columns tc
+    if (tk > tc / 8 * 8 + 7) continue;
+    const i64 k = (i64)tk * 32 + row, c = (i64)tc * 32 + c4;
+    float v[4] = {0.f, 0.f, 0.f, 0.f};
+    if (near) {
+      const i64 i = (i64)tc * 32 + row, j = (i64)tk * 32 + c4;      // the lower tile (tc, tk)
+      float4 e = make_float4(0.f, 0.f, 0.f, 0.f), s = e;
+      if (tk <= tc && i < n && j < n) {
+        e = near_load(g, wo, n, i, j);
+        s = *reinterpret_cast<const float4*>(S + i * n + j);
+      }
+      const float ev[4] = {e.x, e.y, e.z, e.w}, sv[4] = {s.x, s.y, s.z, s.w};
+#pragma unroll
+      for (int x = 0; x < 4; ++x) {
+        const float d = ev[x] - 1.f;
+        T[row][c4 + x] = (j + x < i) ? sv[x] - ev[x] : (j + x == i) ? 1.f - 0.5f * d + 0.5f * (sv[x] + 0.25f * d * d) : 0.f;
+      }
+      __syncthreads();
+#pragma unroll
+      for (int x = 0; x < 4; ++x) v[x] = T[c4 + x][row];
+      __syncthreads();
+    } else if (k < n && c < n) {
+      const float4 a = *reinterpret_cast<const float4*>(src + k * n + c);
+      v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w;
+    }
+    if (k >= n || c >= n) continue;
+    __half h[4], l[4];
+#pragma unroll
+    for (int x = 0; x < 4; ++x) {
+      const float y = scale * v[x];
+      h[x] = __float2half_rn(y);
+      l[x] = __float2half_rn(y - __half2float(h[x]));
+    }
+    *reinterpret_cast<uint2*>(hi + k * n + c) = *reinterpret_cast<const uint2*>(h);
+    *reinterpret_cast<uint2*>(lo + k * n + c) = *reinterpret_cast<const uint2*>(l);
+  }
+}
+
+// End of an adaptive round for the matrices that took the series (one thread per matrix).
+__global__ void k_near_end(int* __restrict__ os, int* __restrict__ rounds_total) {
+  pdl_enter();
+  os += (i64)blockIdx.x * OS_SLOT_INTS;
+  if (os[OS_DONE] != 0 || os[OS_GOOD] != 2) return;
+  os[OS_ROUNDS] += 1;
+  atomicAdd(rounds_total, 1);
+  os[OS_DONE] = 1;
 }
 
 // End of an adaptive round whose panel was solved by products behind the factorization (one thread per matrix).

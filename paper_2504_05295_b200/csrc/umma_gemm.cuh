@@ -628,6 +628,14 @@ k_gemm_umma(const __grid_constant__ Params p) {
   // item by item (every role reads the same flags, which no kernel writes while this one runs)
   const bool batched = p.g.batch2 > 1;
   if (!batched && p.g.skip_flag != nullptr && *p.g.skip_flag != 0) return;
+  if (batched && p.g.skip_flag != nullptr) {      // nothing to do when every matrix is flagged (a warp looks at 32 flags at a time)
+    bool all = true;
+    for (int b = 0; b < p.g.batch2 && all; b += 32) {
+      const int q = b + (int)(threadIdx.x & 31);
+      all = __all_sync(0xffffffffu, q >= p.g.batch2 || p.g.skip_flag[(i64)q * p.g.skip_stride] != 0);
+    }
+    if (all) return;
+  }
   auto skipped = [&](const Item& it) -> bool {
     return batched && p.g.skip_flag != nullptr && p.g.skip_flag[(i64)it.b * p.g.skip_stride] != 0;
   };
