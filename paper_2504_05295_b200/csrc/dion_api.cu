@@ -528,9 +528,11 @@ int flow_ctas_per_sm() {
 
 constexpr i64 NBO = NBO_COLS;  // outer block of the two-level Cholesky
 
-int grid_for(const dion_ctx* c, i64 total) {
+// Blocks of 256 threads for `total` items on each of nb matrices: at most one wave (eight per SM) over all of them.
+int grid_for(const dion_ctx* c, i64 total, int nb = 1) {
   i64 blocks = (total + 255) / 256;
-  if (blocks > 8 * (i64)c->sm_count) blocks = 8 * (i64)c->sm_count;
+  const i64 most = (8 * (i64)c->sm_count + nb - 1) / nb;
+  if (blocks > most) blocks = most;
   if (blocks < 1) blocks = 1;
   return (int)blocks;
 }
@@ -667,7 +669,7 @@ int potrf_blocked(StepCtx& s, i64 r, int mode, const std::function<int(i64, i64)
           if (cudaEventRecord(e, s.st) != cudaSuccess || cudaStreamWaitEvent(c->side, e, 0) != cudaSuccess) return DION_ERR_CUDA;
           cst = c->side;
         }
-        dim3 grid((unsigned)grid_for(c, rem * sz), (unsigned)s.nb);
+        dim3 grid((unsigned)grid_for(c, rem * sz, s.nb), (unsigned)s.nb);
         launch_pdl(k_copy_block, grid, dim3(256), 0, cst, ptmp, r, panel, r, rem, sz, skip, s.wstride);
         DION_CHECK_LAUNCH(c);
       }
@@ -699,7 +701,7 @@ int probe(StepCtx& s, i64 off, i64 rows, i64 r, int phase) {
     launch_pdl(k_probe_y4, dim3((unsigned)blocks, (unsigned)s.nb), dim3(256), (size_t)PY_SMEM, s.st, (const float*)(s.ws + off), r, rows, r,
                s.ws + s.L.probe_y, s.wstride, keep);
   } else {
-    launch_pdl(k_probe_y, dim3((unsigned)grid_for(c, rows * 32), (unsigned)s.nb), dim3(256), 0, s.st, (const float*)(s.ws + off), r,
+    launch_pdl(k_probe_y, dim3((unsigned)grid_for(c, rows * 32, s.nb), (unsigned)s.nb), dim3(256), 0, s.st, (const float*)(s.ws + off), r,
                rows, r, s.ws + s.L.probe_y, s.wstride, keep);
   }
   DION_CHECK_LAUNCH(c);
@@ -766,7 +768,7 @@ int cholqr_round(StepCtx& s, i64 pin_off, i64 pout_off, i64 rows, i64 r, int mod
     launch_pdl(k_absmax_partial, dim3((unsigned)parts, (unsigned)s.nb), dim3(256), 0, s.st, (const float*)(s.ws + pin_off), r, rows, r,
                s.ws + s.L.gmax, s.wstride, sk, (i64)OS_SLOT_INTS);
     DION_CHECK_LAUNCH(c);
-    launch_pdl(k_split_f16_scaled, dim3((unsigned)grid_for(c, rows * r / 8), (unsigned)s.nb), dim3(256), 0, s.st,
+    launch_pdl(k_split_f16_scaled, dim3((unsigned)grid_for(c, rows * r / 8, s.nb), (unsigned)s.nb), dim3(256), 0, s.st,
                (const float*)(s.ws + pin_off), r, rows, r, (const float*)(s.ws + s.L.gmax), (int)parts, hi, lo, s.ws + s.L.gmax + AMAX_PARTS,
                s.wstride, sk, (i64)OS_SLOT_INTS, -1.f, (const float*)nullptr);
     DION_CHECK_LAUNCH(c);
@@ -869,7 +871,7 @@ int cholqr_round(StepCtx& s, i64 pin_off, i64 pout_off, i64 rows, i64 r, int mod
                  (i64)OS_SLOT_INTS);
       DION_CHECK_LAUNCH(c);
       __half* hi = reinterpret_cast<__half*>(s.ws + out_off);
-      launch_pdl(k_split_f16_scaled, dim3((unsigned)grid_for(c, nrows * ncols / 8), (unsigned)s.nb), dim3(256), 0, s.st, src, ld, nrows, ncols,
+      launch_pdl(k_split_f16_scaled, dim3((unsigned)grid_for(c, nrows * ncols / 8, s.nb), (unsigned)s.nb), dim3(256), 0, s.st, src, ld, nrows, ncols,
                  (const float*)pm, (int)parts, hi, hi + nrows * ncols, pm + AMAX_PARTS, s.wstride, skip, (i64)OS_SLOT_INTS, other_inv, other_dev);
       DION_CHECK_LAUNCH(c);
       return DION_OK;
@@ -911,7 +913,7 @@ int cholqr_round(StepCtx& s, i64 pin_off, i64 pout_off, i64 rows, i64 r, int mod
       if (J0 + sz < r) {      // the new block column of Pout joins the pair (later block columns read it)
         ChainPtrs t;
         for (int b = 0; b < s.nb; ++b) t.p[b] = s.W(b, pout_off + J0);
-        launch_pdl(k_split_f16_fixed, dim3((unsigned)grid_for(c, rows * sz / 8), (unsigned)s.nb), dim3(256), 0, s.st, t, r, rows, sz,
+        launch_pdl(k_split_f16_fixed, dim3((unsigned)grid_for(c, rows * sz / 8, s.nb), (unsigned)s.nb), dim3(256), 0, s.st, t, r, rows, sz,
                    ldexpf(1.f, 6), pop + J0, pop + rows * r + J0, s.wstride, r, skip, (i64)OS_SLOT_INTS);
         DION_CHECK_LAUNCH(c);
       }
@@ -1013,7 +1015,7 @@ int adaptive_rounds(StepCtx& s, i64 off_a, i64 off_b, i64 rows, i64 r, i64 gram_
     DION_TRY(cholqr_round(s, off_b, off_a, rows, r, RM_ADAPTIVE, gram_rows, PROBE_CHECK, it + 1));
   }
   {   // an odd number of rounds left the result in the second buffer
-    dim3 grid((unsigned)grid_for(s.c, rows * r), (unsigned)s.nb);
+    dim3 grid((unsigned)grid_for(s.c, rows * r, s.nb), (unsigned)s.nb);
     launch_pdl(k_copy_panel, grid, dim3(256), 0, s.st, (const float*)(s.ws + off_b), r, s.ws + off_a, r, rows, r, (const int*)nullptr,
                (const int*)(s.os + OS_ROUNDS), s.wstride, 1);
     s.c->launches++;
@@ -1026,7 +1028,7 @@ int adaptive_rounds(StepCtx& s, i64 off_a, i64 off_b, i64 rows, i64 r, i64 gram_
 
 // The second round of CholeskyQR2, when it ran, went P0 -> P1: its result back to P0.
 int second_round_back(StepCtx& s, i64 rows, i64 r) {
-  dim3 grid((unsigned)grid_for(s.c, rows * r), (unsigned)s.nb);
+  dim3 grid((unsigned)grid_for(s.c, rows * r, s.nb), (unsigned)s.nb);
   launch_pdl(k_copy_panel, grid, dim3(256), 0, s.st, (const float*)(s.ws + s.L.P1), r, s.ws + s.L.P0, r, rows, r,
              (const int*)(s.os + OS_DONE), (const int*)nullptr, s.wstride, -1);
   DION_CHECK_LAUNCH(s.c);
@@ -1228,7 +1230,7 @@ int split_chain(StepCtx& s, const float* const* src, const i64* ld, i64 rows, i6
   dion_ctx* c = s.c;
   bool one = s.nb > 1 && s.nb <= GEMM_TAB_MAX && c->chain_batch;
   for (int b = 1; b < s.nb && one; ++b) one = ld[b] == ld[0];
-  const unsigned gx = (unsigned)grid_for(c, rows * cols / 8);
+  const unsigned gx = (unsigned)grid_for(c, rows * cols / 8, one ? s.nb : 1);
   if (one) {
     ChainPtrs t;
     for (int b = 0; b < s.nb; ++b) t.p[b] = src[b];
@@ -1257,7 +1259,7 @@ int round_chain(StepCtx& s, const float* const* src, const i64* ld, i64 rows, i6
   bool one = s.nb > 1 && s.nb <= GEMM_TAB_MAX && c->chain_batch;
   for (int b = 1; b < s.nb && one; ++b) one = ld[b] == ld[0];
   if (half_scale > 0.f) {
-    const unsigned g8 = (unsigned)grid_for(c, rows * cols / 8);
+    const unsigned g8 = (unsigned)grid_for(c, rows * cols / 8, one ? s.nb : 1);
     if (one) {
       ChainPtrs t;
       for (int b = 0; b < s.nb; ++b) t.p[b] = src[b];
@@ -1273,7 +1275,7 @@ int round_chain(StepCtx& s, const float* const* src, const i64* ld, i64 rows, i6
     }
     return DION_OK;
   }
-  const unsigned gx = (unsigned)grid_for(c, rows * cols / 4);
+  const unsigned gx = (unsigned)grid_for(c, rows * cols / 4, one ? s.nb : 1);
   if (one) {
     ChainPtrs t;
     for (int b = 0; b < s.nb; ++b) t.p[b] = src[b];
@@ -1390,7 +1392,7 @@ int form_sum_chain(StepCtx& s, const dion_matrix* const* list, bool pair) {
   const int g_mode = (a0->g_dtype == DION_BF16) ? ADD_BF16 : ADD_F32;
   __nv_bfloat16* bh = pair ? reinterpret_cast<__nv_bfloat16*>(s.ws + s.L.Bp) : nullptr;
   __nv_bfloat16* bl = pair ? bh + m * n : nullptr;
-  const dim3 grid((unsigned)grid_for(c, m * n / 4), (unsigned)s.nb);
+  const dim3 grid((unsigned)grid_for(c, m * n / 4, s.nb), (unsigned)s.nb);
   if (vec) launch_pdl(k_form_b32_chain<true>, grid, dim3(256), 0, s.st, Ms, a0->ldm, Gs, a0->ldg, g_mode, m, n, s.ws + s.L.B32, bh, bl, s.wstride);
   else launch_pdl(k_form_b32_chain<false>, grid, dim3(256), 0, s.st, Ms, a0->ldm, Gs, a0->ldg, g_mode, m, n, s.ws + s.L.B32, bh, bl, s.wstride);
   DION_CHECK_LAUNCH(c);
@@ -1613,14 +1615,14 @@ int step_batch(dion_ctx* c, const dion_matrix* const* list, int nb, float lr, cu
       launch_pdl(k_absmax_partial, dim3((unsigned)parts, (unsigned)nb), dim3(256), 0, st, (const float*)(s.ws + s.L.B32), n, m, n,
                  s.ws + s.L.pmax, s.wstride, (const int*)nullptr, (i64)0);
       DION_CHECK_LAUNCH(c);
-      launch_pdl(k_split_f16_scaled, dim3((unsigned)grid_for(c, m * n / 8), (unsigned)nb), dim3(256), 0, st,
+      launch_pdl(k_split_f16_scaled, dim3((unsigned)grid_for(c, m * n / 8, nb), (unsigned)nb), dim3(256), 0, st,
                  (const float*)(s.ws + s.L.B32), n, m, n, (const float*)(s.ws + s.L.pmax), (int)parts, bh, bh + m * n,
                  s.ws + s.L.pmax + AMAX_PARTS, s.wstride, (const int*)nullptr, (i64)0, ldexpf(1.f, -13), (const float*)nullptr);
       DION_CHECK_LAUNCH(c);
       ChainPtrs t;
       for (int b = 0; b < nb; ++b) t.p[b] = srcs[b];
       __half* qh = reinterpret_cast<__half*>(s.ws + s.L.S16);
-      launch_pdl(k_split_f16_fixed, dim3((unsigned)grid_for(c, qrow * r / 8), (unsigned)nb), dim3(256), 0, st, t, list[0]->ldq, qrow, r,
+      launch_pdl(k_split_f16_fixed, dim3((unsigned)grid_for(c, qrow * r / 8, nb), (unsigned)nb), dim3(256), 0, st, t, list[0]->ldq, qrow, r,
                  ldexpf(1.f, 13), qh, qh + qrow * r, s.wstride, (i64)0, (const int*)nullptr, (i64)0);
       DION_CHECK_LAUNCH(c);
       p_half_ready = true;
@@ -1648,7 +1650,7 @@ int step_batch(dion_ctx* c, const dion_matrix* const* list, int nb, float lr, cu
     if (all_ok) {
       ChainPtrs t;
       for (int b = 0; b < nb; ++b) t.p[b] = srcs[b];
-      launch_pdl(k_copy_chain, dim3((unsigned)grid_for(c, qrow * r / 4), (unsigned)nb), dim3(256), 0, st, t, list[0]->ldq, qrow, r, s.ws + s.L.S16, s.wstride);
+      launch_pdl(k_copy_chain, dim3((unsigned)grid_for(c, qrow * r / 4, nb), (unsigned)nb), dim3(256), 0, st, t, list[0]->ldq, qrow, r, s.ws + s.L.S16, s.wstride);
       DION_CHECK_LAUNCH(c);
       q_dense = true;
     }

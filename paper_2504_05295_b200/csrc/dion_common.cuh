@@ -86,6 +86,8 @@ __device__ __forceinline__ void pdl_enter() {
   asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 __device__ __forceinline__ float load_add(const void* p, i64 off, int mode) {
   if (mode == ADD_F32) return reinterpret_cast<const float*>(p)[off];
   if (mode == ADD_BF16) return __bfloat162float(reinterpret_cast<const __nv_bfloat16*>(p)[off]);

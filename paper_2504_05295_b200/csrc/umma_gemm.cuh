@@ -627,6 +627,7 @@ k_gemm_umma(const __grid_constant__ Params p) {
   // a launch over one matrix does nothing when that matrix's flag is set; a batched launch skips flagged matrices
   // item by item (every role reads the same flags, which no kernel writes while this one runs)
   const bool batched = p.g.batch2 > 1;
+  pdl_wait();      // (no early trigger: the next kernel's blocks would only take up threads and registers beside this one)
   if (!batched && p.g.skip_flag != nullptr && *p.g.skip_flag != 0) return;
   if (batched && p.g.skip_flag != nullptr) {      // nothing to do when every matrix is flagged (a warp looks at 32 flags at a time)
     bool all = true;
@@ -1330,12 +1331,23 @@ inline cudaError_t set_smem_attr() {
                               Cfg<BN, BF16, SPLIT, TMA, D16, CE, ONE, CG2, X2>::SMEM_BYTES);
 }
 
+// Launch of a single-CTA variant, with programmatic stream serialization like every other kernel of a step (pdl_enter).
+inline void launch_single(void (*kernel)(Params), const Params& p, int grid, int threads, int smem, cudaStream_t st) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)grid); cfg.blockDim = dim3((unsigned)threads); cfg.dynamicSmemBytes = (size_t)smem; cfg.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr; cfg.numAttrs = 1;
+  cudaLaunchKernelEx(&cfg, kernel, p);      // (the caller looks at cudaGetLastError)
+}
+
 // bf16 operand pairs
 template <int BN, bool A_MN, bool B_MN>
 inline void launch_x2_one(const Params& p, int grid, cudaStream_t st) {
   constexpr int smem = Cfg<BN, true, false, true, true, true, false, false, true>::SMEM_BYTES;
   constexpr int threads = Cfg<BN, true, false, true, true, true, false, false, true>::THREADS;
-  k_gemm_umma<BN, A_MN, B_MN, true, false, true, true, true, false, false, true><<<grid, threads, smem, st>>>(p);
+  launch_single(k_gemm_umma<BN, A_MN, B_MN, true, false, true, true, true, false, false, true>, p, grid, threads, smem, st);
 }
 template <int BN>
 inline void launch_x2(const Params& p, bool a_mn, bool b_mn, int grid, cudaStream_t st) {
@@ -1353,17 +1365,19 @@ inline cudaError_t set_x2_attr() {
 template <int BN, bool A_MN>
 inline void launch_x2s(const Params& p, int grid, cudaStream_t st) {
   using CF = Cfg<BN, true, true, true, true, true, false, false, true>;
-  k_gemm_umma<BN, A_MN, true, true, true, true, true, true, false, false, true><<<grid, CF::THREADS, CF::SMEM_BYTES, st>>>(p);
+  launch_single(k_gemm_umma<BN, A_MN, true, true, true, true, true, true, false, false, true>, p, grid, CF::THREADS, CF::SMEM_BYTES, st);
 }
 template <bool A_MN>
 inline cudaError_t launch_x2s_pair(const Params& p, int grid, cudaStream_t st) {
   using CF = Cfg<256, true, true, true, true, true, false, true, true>;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)grid); cfg.blockDim = dim3(CF::THREADS); cfg.dynamicSmemBytes = CF::SMEM_BYTES; cfg.stream = st;
-  cudaLaunchAttribute attr[1];
+  cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeClusterDimension;
   attr[0].val.clusterDim.x = 2; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
-  cfg.attrs = attr; cfg.numAttrs = 1;
+  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[1].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr; cfg.numAttrs = 2;
   return cudaLaunchKernelEx(&cfg, k_gemm_umma<256, A_MN, true, true, true, true, true, true, false, true, true>, p);
 }
 
@@ -1373,10 +1387,12 @@ inline cudaError_t launch_x2_pair_one(const Params& p, int grid, cudaStream_t st
   using CF = Cfg<256, true, false, true, true, true, false, true, true>;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)grid); cfg.blockDim = dim3(CF::THREADS); cfg.dynamicSmemBytes = CF::SMEM_BYTES; cfg.stream = st;
-  cudaLaunchAttribute attr[1];
+  cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeClusterDimension;
   attr[0].val.clusterDim.x = 2; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
-  cfg.attrs = attr; cfg.numAttrs = 1;
+  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[1].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr; cfg.numAttrs = 2;
   return cudaLaunchKernelEx(&cfg, k_gemm_umma<256, A_MN, B_MN, true, false, true, true, true, false, true, true>, p);
 }
 inline cudaError_t launch_x2_pair(const Params& p, bool a_mn, bool b_mn, int grid, cudaStream_t st) {
@@ -1396,10 +1412,12 @@ inline cudaError_t launch_d16_pair_one(const Params& p, int grid, cudaStream_t s
   using CF = Cfg<256, true, false, true, true, true, false, true, false>;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)grid); cfg.blockDim = dim3(CF::THREADS); cfg.dynamicSmemBytes = CF::SMEM_BYTES; cfg.stream = st;
-  cudaLaunchAttribute attr[1];
+  cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeClusterDimension;
   attr[0].val.clusterDim.x = 2; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
-  cfg.attrs = attr; cfg.numAttrs = 1;
+  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[1].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr; cfg.numAttrs = 2;
   return cudaLaunchKernelEx(&cfg, k_gemm_umma<256, A_MN, B_MN, true, false, true, true, true, false, true, false>, p);
 }
 inline cudaError_t launch_d16_pair(const Params& p, bool a_mn, bool b_mn, int grid, cudaStream_t st) {
@@ -1419,10 +1437,12 @@ inline cudaError_t launch_pair_one(const Params& p, int grid, cudaStream_t st) {
   constexpr int smem = Cfg<256, false, SPLIT, true, false, true, false, true>::SMEM_BYTES;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)grid); cfg.blockDim = dim3(NUM_THREADS_TMA); cfg.dynamicSmemBytes = smem; cfg.stream = st;
-  cudaLaunchAttribute attr[1];
+  cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeClusterDimension;
   attr[0].val.clusterDim.x = 2; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
-  cfg.attrs = attr; cfg.numAttrs = 1;
+  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[1].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr; cfg.numAttrs = 2;
   return cudaLaunchKernelEx(&cfg, k_gemm_umma<256, A_MN, B_MN, false, SPLIT, true, false, true, false, true>, p);
 }
 template <bool SPLIT>
@@ -1466,17 +1486,17 @@ int pair_clusters(int sm_count) {
 template <int BN>
 inline void launch_one(const Params& p, int grid, cudaStream_t st) {
   constexpr int smem = Cfg<BN, false, false, true, false, true, true>::SMEM_BYTES;
-  k_gemm_umma<BN, false, false, false, false, true, false, true, true><<<grid, NUM_THREADS_TMA, smem, st>>>(p);
+  launch_single(k_gemm_umma<BN, false, false, false, false, true, false, true, true>, p, grid, NUM_THREADS_TMA, smem, st);
 }
 
 template <int BN, bool BF16, bool SPLIT, bool TMA, bool D16 = false, bool CE = false>
 inline void launch_variant(const Params& p, bool a_mn, bool b_mn, int grid, cudaStream_t st) {
   constexpr int smem = Cfg<BN, BF16, SPLIT, TMA, D16, CE>::SMEM_BYTES;
   constexpr int threads = TMA ? NUM_THREADS_TMA : NUM_THREADS;
-  if (!a_mn && !b_mn) k_gemm_umma<BN, false, false, BF16, SPLIT, TMA, D16, CE><<<grid, threads, smem, st>>>(p);
-  else if (!a_mn && b_mn) k_gemm_umma<BN, false, true, BF16, SPLIT, TMA, D16, CE><<<grid, threads, smem, st>>>(p);
-  else if (a_mn && b_mn) k_gemm_umma<BN, true, true, BF16, SPLIT, TMA, D16, CE><<<grid, threads, smem, st>>>(p);
-  else k_gemm_umma<BN, true, false, BF16, SPLIT, TMA, D16, CE><<<grid, threads, smem, st>>>(p);
+  if (!a_mn && !b_mn) launch_single(k_gemm_umma<BN, false, false, BF16, SPLIT, TMA, D16, CE>, p, grid, threads, smem, st);
+  else if (!a_mn && b_mn) launch_single(k_gemm_umma<BN, false, true, BF16, SPLIT, TMA, D16, CE>, p, grid, threads, smem, st);
+  else if (a_mn && b_mn) launch_single(k_gemm_umma<BN, true, true, BF16, SPLIT, TMA, D16, CE>, p, grid, threads, smem, st);
+  else launch_single(k_gemm_umma<BN, true, false, BF16, SPLIT, TMA, D16, CE>, p, grid, threads, smem, st);
 }
 
 typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*, const cuuint64_t*,
@@ -1840,9 +1860,14 @@ int umma_try_launch(const GemmArgs& g_in, int precision, int sm_count, float* pa
     const i64 total = g.M * g.N;
     int blocks = (int)((total + 255) / 256);
     if (blocks > 8 * sm_count) blocks = 8 * sm_count;
-    k_splitk_reduce<<<dim3((unsigned)blocks, (unsigned)nbat), 256, 0, st>>>(part, splits, g.M, g.N, g.C, g.ldc, g.alpha, g.tri, 128, g.skip_flag,
-                                                                            nbat > 1 ? g.bs2 : 0, nbat > 1 ? g.skip_stride : 0, g.alpha_dev,
-                                                                            g.alpha_dev_stride);
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)blocks, (unsigned)nbat); cfg.blockDim = dim3(256); cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr; cfg.numAttrs = 1;
+    cudaLaunchKernelEx(&cfg, k_splitk_reduce, (const float*)part, splits, g.M, g.N, g.C, g.ldc, g.alpha, g.tri, 128, g.skip_flag,
+                       nbat > 1 ? g.bs2 : (i64)0, nbat > 1 ? g.skip_stride : (i64)0, g.alpha_dev, g.alpha_dev_stride);
     if (cudaGetLastError() != cudaSuccess) return DION_ERR_CUDA;
     return 2;
   }
