@@ -73,7 +73,8 @@ __global__ void __launch_bounds__(256) k_form_b16(const float* __restrict__ M, i
 template <bool VEC>
 __device__ __forceinline__ void form_b32_body(const float* __restrict__ M, i64 ldm, const void* __restrict__ G,
                                               i64 ldg, int g_mode, i64 rows, i64 cols, float* __restrict__ out,
-                                              __nv_bfloat16* __restrict__ hi, __nv_bfloat16* __restrict__ lo) {
+                                              __nv_bfloat16* __restrict__ hi, __nv_bfloat16* __restrict__ lo,
+                                              float* amax = nullptr) {      // amax (register, optional): largest magnitude seen by the thread
   const i64 per_row = cols / 4;
   const i64 total = rows * per_row;
   for (i64 e = (i64)blockIdx.x * blockDim.x + threadIdx.x; e < total; e += (i64)gridDim.x * blockDim.x) {
@@ -101,6 +102,7 @@ __device__ __forceinline__ void form_b32_body(const float* __restrict__ M, i64 l
       }
     }
     *reinterpret_cast<float4*>(out + i * cols + c) = v;
+    if (amax != nullptr) *amax = fmaxf(fmaxf(*amax, fmaxf(fabsf(v.x), fabsf(v.y))), fmaxf(fabsf(v.z), fabsf(v.w)));
     if (hi != nullptr) {
       const float h0 = __bfloat162float(__float2bfloat16_rn(v.x)), h1 = __bfloat162float(__float2bfloat16_rn(v.y));
       const float h2 = __bfloat162float(__float2bfloat16_rn(v.z)), h3 = __bfloat162float(__float2bfloat16_rn(v.w));
@@ -292,6 +294,25 @@ __global__ void __launch_bounds__(256) k_round_f16_chain(const ChainPtrs srcs, i
 // a fixed order; block 0 also writes 1 / scale^2, the factor that takes a Gram matrix of the pair back).
 // blockIdx.y: the matrix of a chain (arrays `wstride` floats apart); skip flags a state slot apart.
 constexpr int AMAX_PARTS = 512;
+__device__ __forceinline__ void block_max(float m, float* __restrict__ out) {      // 256 threads; out[blockIdx.x]
+  __shared__ float red[256];
+  red[threadIdx.x] = m;
+  __syncthreads();
+  for (int w = 128; w > 0; w >>= 1) {
+    if ((int)threadIdx.x < w) red[threadIdx.x] = fmaxf(red[threadIdx.x], red[threadIdx.x + w]);
+    __syncthreads();
+  }
+  if (threadIdx.x == 0) out[blockIdx.x] = red[0];
+}
+// M + G in fp32 and the blocks' largest magnitudes of it in one pass (the products on a scaled half pair of the sum).
+template <bool VEC>
+__global__ void __launch_bounds__(256) k_form_b32_amax(const float* __restrict__ M, i64 ldm, const void* __restrict__ G, i64 ldg, int g_mode,
+                                                       i64 rows, i64 cols, float* __restrict__ out, float* __restrict__ part) {
+  pdl_enter();
+  float m = 0.f;
+  form_b32_body<VEC>(M, ldm, G, ldg, g_mode, rows, cols, out, nullptr, nullptr, &m);
+  block_max(m, part);
+}
 __global__ void __launch_bounds__(256) k_absmax_partial(const float* __restrict__ src, i64 ld, i64 rows, i64 cols,
                                                         float* __restrict__ part, i64 wstride, const int* __restrict__ skip_flag,
                                                         i64 skip_stride) {
@@ -305,24 +326,18 @@ __global__ void __launch_bounds__(256) k_absmax_partial(const float* __restrict_
     const float4 a = *reinterpret_cast<const float4*>(src + i * ld + c);
     m = fmaxf(fmaxf(m, fmaxf(fabsf(a.x), fabsf(a.y))), fmaxf(fabsf(a.z), fabsf(a.w)));
   }
-  __shared__ float red[256];
-  red[threadIdx.x] = m;
-  __syncthreads();
-  for (int w = 128; w > 0; w >>= 1) {
-    if ((int)threadIdx.x < w) red[threadIdx.x] = fmaxf(red[threadIdx.x], red[threadIdx.x + w]);
-    __syncthreads();
-  }
-  if (threadIdx.x == 0) part[blockIdx.x] = red[0];
+  block_max(m, part);
 }
 // other_inv < 0: the scalar written is 1 / scale^2 (both operands of the product are this array); else
 // other_inv / scale (the other operand carries a fixed scale of its own), times *other_dev when that is given (the
-// other operand's own 1 / scale, written by its split; blockIdx.y entries wstride apart like everything else).
+// other operand's own 1 / scale, written by its split; blockIdx.y entries wstride apart like everything else).  own_inv
+// (optional): 1 / scale alone.
 __global__ void __launch_bounds__(256) k_split_f16_scaled(const float* __restrict__ src, i64 ld, i64 rows, i64 cols,
                                                           const float* __restrict__ part, int nparts,
                                                           __half* __restrict__ hi, __half* __restrict__ lo,
                                                           float* __restrict__ inv_scale2, i64 wstride,
                                                           const int* __restrict__ skip_flag, i64 skip_stride,
-                                                          float other_inv, const float* __restrict__ other_dev = nullptr) {
+                                                          float other_inv, const float* __restrict__ other_dev, float* __restrict__ own_inv) {
   pdl_enter();
   if (skip_flag != nullptr && skip_flag[(i64)blockIdx.y * skip_stride] != 0) return;
   src += (i64)blockIdx.y * wstride; part += (i64)blockIdx.y * wstride; inv_scale2 += (i64)blockIdx.y * wstride;
@@ -342,6 +357,7 @@ __global__ void __launch_bounds__(256) k_split_f16_scaled(const float* __restric
   if (amax > 0.f && amax < 3.0e38f) frexpf(amax, &ex);
   if (ex < -100) ex = -100;
   const float scale = ldexpf(1.f, 14 - ex);
+  if (blockIdx.x == 0 && threadIdx.x == 0 && own_inv != nullptr) own_inv[(i64)blockIdx.y * wstride] = ldexpf(1.f, ex - 14);
   if (blockIdx.x == 0 && threadIdx.x == 0)
     *inv_scale2 = (other_inv < 0.f) ? ldexpf(1.f, 2 * (ex - 14))
                                     : other_inv * ldexpf(1.f, ex - 14) * (other_dev != nullptr ? *other_dev : 1.f);

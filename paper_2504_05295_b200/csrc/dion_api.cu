@@ -40,6 +40,7 @@ constexpr float DONE_REL = 0.9f;          // smallest relative pivot of a round 
 constexpr i64 PART_CAP_FLOATS = (i64)16 << 20;  // split-K partial sums, at most 64 MiB
 constexpr double P_HALF_MIN_MNR = 4e9;          // smallest m n r whose full-rank P runs on scaled half pairs
 constexpr double SOLVE_PAIR_MIN_PANEL = 3e7;    // smallest rows x r whose blocked solves run on scaled half pairs
+constexpr i64 LAZY_PAIR_MIN_MNR = 50000000;     // smallest m n r whose Lazy-Dion step runs on scaled half pairs (2^25.6: 512 x 768 x 128)
 constexpr double GRAM_PAIR_MIN_FLOPS = 2e9;     // smallest rows r^2 whose Gram matrix runs on scaled half pairs
 constexpr double P_PAIR_MIN_MNR = 1.5e10;       // smallest m n r whose P = (M + G) Q runs on bf16 operand pairs first
 
@@ -70,6 +71,7 @@ struct Layout {
   i64 pmax;                 // ... its partial maxima and the product's scale factor (like gmax)
   i64 SolveP, LfP, smax;    // blocked solves on half pairs (r > 512): pair of a rows x 512 right-hand side; pairs of a row block of
                             // the factor (512 x r) and of a diagonal inverse (512 x 512); partial maxima and scales
+  i64 lz;                   // Lazy-Dion on half pairs: partial maxima, then the scales of its products (LZ_*)
   i64 XP;                   // scaled half pair of the inverse of the factor
   i64 xmax;                 // largest magnitude of the factor's inverse, then the scale of the product with its pair
   i64 gmax;                 // Gram matrices on half pairs: AMAX_PARTS partial maxima of |P|, then 1 / scale^2
@@ -218,6 +220,7 @@ Layout make_layout(const dion_ctx* c, i64 m, i64 n, i64 r) {
   L.Psave = L.fb_part = L.fb_h = L.fb_n = 0;
   L.gmax = o; o += align64(AMAX_PARTS + 64);
   L.xmax = o; o += 64;
+  L.lz = o; o += align64(8 * (i64)c->sm_count + 64);
   L.SolveP = L.LfP = L.smax = 0;
   if (r > FLOW_MAX_R && (double)big * (double)r >= SOLVE_PAIR_MIN_PANEL) {
     L.SolveP = o; o += align64(big * NBO_COLS);
@@ -770,7 +773,7 @@ int cholqr_round(StepCtx& s, i64 pin_off, i64 pout_off, i64 rows, i64 r, int mod
     DION_CHECK_LAUNCH(c);
     launch_pdl(k_split_f16_scaled, dim3((unsigned)grid_for(c, rows * r / 8, s.nb), (unsigned)s.nb), dim3(256), 0, s.st,
                (const float*)(s.ws + pin_off), r, rows, r, (const float*)(s.ws + s.L.gmax), (int)parts, hi, lo, s.ws + s.L.gmax + AMAX_PARTS,
-               s.wstride, sk, (i64)OS_SLOT_INTS, -1.f, (const float*)nullptr);
+               s.wstride, sk, (i64)OS_SLOT_INTS, -1.f, (const float*)nullptr, (float*)nullptr);
     DION_CHECK_LAUNCH(c);
     g.ab16 = 1; g.f16 = 1;
     g.A = reinterpret_cast<const float*>(hi); g.A16lo = lo;
@@ -872,7 +875,7 @@ int cholqr_round(StepCtx& s, i64 pin_off, i64 pout_off, i64 rows, i64 r, int mod
       DION_CHECK_LAUNCH(c);
       __half* hi = reinterpret_cast<__half*>(s.ws + out_off);
       launch_pdl(k_split_f16_scaled, dim3((unsigned)grid_for(c, nrows * ncols / 8, s.nb), (unsigned)s.nb), dim3(256), 0, s.st, src, ld, nrows, ncols,
-                 (const float*)pm, (int)parts, hi, hi + nrows * ncols, pm + AMAX_PARTS, s.wstride, skip, (i64)OS_SLOT_INTS, other_inv, other_dev);
+                 (const float*)pm, (int)parts, hi, hi + nrows * ncols, pm + AMAX_PARTS, s.wstride, skip, (i64)OS_SLOT_INTS, other_inv, other_dev, (float*)nullptr);
       DION_CHECK_LAUNCH(c);
       return DION_OK;
     };
@@ -1617,7 +1620,7 @@ int step_batch(dion_ctx* c, const dion_matrix* const* list, int nb, float lr, cu
       DION_CHECK_LAUNCH(c);
       launch_pdl(k_split_f16_scaled, dim3((unsigned)grid_for(c, m * n / 8, nb), (unsigned)nb), dim3(256), 0, st,
                  (const float*)(s.ws + s.L.B32), n, m, n, (const float*)(s.ws + s.L.pmax), (int)parts, bh, bh + m * n,
-                 s.ws + s.L.pmax + AMAX_PARTS, s.wstride, (const int*)nullptr, (i64)0, ldexpf(1.f, -13), (const float*)nullptr);
+                 s.ws + s.L.pmax + AMAX_PARTS, s.wstride, (const int*)nullptr, (i64)0, ldexpf(1.f, -13), (const float*)nullptr, (float*)nullptr);
       DION_CHECK_LAUNCH(c);
       ChainPtrs t;
       for (int b = 0; b < nb; ++b) t.p[b] = srcs[b];
@@ -1959,10 +1962,121 @@ int step_graph(dion_ctx* c, const dion_matrix* a, float lr, cudaStream_t st) {
   return DION_OK;
 }
 
+// Lazy-Dion on scaled half pairs (fp32 mode on the tensor engine; the shapes that keep M + G in scratch): M + G is formed once
+// per call, in fp32 for the error feedback and as a half pair for the products that read it, and every product takes three
+// kind::f16 MMAs per K step on pairs -- the 22 significant bits of the 3xTF32 products it replaces at twice their rate,
+// through the kernels with the deeper epilogue (4096^2, r = 256: W 128 -> 35 us + 50 of preparation, error feedback 141 -> 36,
+// weight update 85 -> 28).
+enum : int { LZ_B = 0, LZ_BQ = 1, LZ_Q = 2, LZ_A = 3, LZ_AQ = 4, LZ_SCALARS = 8 };      // floats behind the partial maxima: 1 / scale of
+                                                                                      // M + G, with Q's, Q's, the left factor's with another's
+bool lazy_on_pairs(const StepCtx& s, const dion_matrix* a) {
+  return s.tensor && s.L.B32 > 0 && s.L.Bp > 0 && a->r % 8 == 0 && a->m % 8 == 0 && a->n % 8 == 0 && a->m * a->n * a->r >= LAZY_PAIR_MIN_MNR &&
+         !((uintptr_t)a->X & 15) && a->ldx % 4 == 0 && !((uintptr_t)a->M & 15) && a->ldm % 4 == 0 && !((uintptr_t)a->Q & 15) && a->ldq % 4 == 0;
+}
+
+int lazy_pairs(StepCtx& s, const dion_matrix* a, float lr, int refresh) {
+  dion_ctx* c = s.c;
+  cudaStream_t st = s.st;
+  const i64 m = a->m, n = a->n, r = a->r;
+  const int gmode = (a->g_dtype == DION_BF16) ? ADD_BF16 : ADD_F32;
+  float* pm = s.ws + s.L.lz;
+  float* sc = pm + 8 * (i64)c->sm_count;
+  float* R = s.ws + s.L.R;
+  auto halves = [&](i64 off) { return reinterpret_cast<__half*>(s.ws + off); };
+  // the pair of a rows x cols array into scratch at `off`; scale slot `slot` (times slot `other`'s), `own`: its scale alone
+  auto pair_of = [&](const float* src, i64 ld, i64 rows, i64 cols, i64 off, int slot, int other, int own, bool have_max, i64 nparts) -> int {
+    if (!have_max) {
+      nparts = (rows * cols / 4 + 2047) / 2048;
+      if (nparts > AMAX_PARTS) nparts = AMAX_PARTS;
+      launch_pdl(k_absmax_partial, dim3((unsigned)nparts), dim3(256), 0, st, src, ld, rows, cols, pm, (i64)0, (const int*)nullptr, (i64)0);
+      DION_CHECK_LAUNCH(c);
+    }
+    launch_pdl(k_split_f16_scaled, dim3((unsigned)grid_for(c, rows * cols / 8)), dim3(256), 0, st, src, ld, rows, cols, (const float*)pm, (int)nparts,
+               halves(off), halves(off) + rows * cols, sc + slot, (i64)0, (const int*)nullptr, (i64)0, 1.f,
+               other >= 0 ? (const float*)(sc + other) : (const float*)nullptr, own >= 0 ? sc + own : (float*)nullptr);
+    DION_CHECK_LAUNCH(c);
+    return DION_OK;
+  };
+  auto product = [&](i64 M_, i64 N_, i64 K_, i64 a_off, i64 a_n, i64 a_si, i64 a_sk, i64 b_off, i64 b_n, i64 b_sk, i64 b_sn, int slot) {
+    GemmArgs g = gemm_args();
+    g.M = M_; g.N = N_; g.K = K_;
+    g.ab16 = 1; g.f16 = 1;
+    g.A = (const float*)halves(a_off); g.A16lo = halves(a_off) + a_n; g.a_si = a_si; g.a_sk = a_sk;
+    g.B = (const float*)halves(b_off); g.B16lo = halves(b_off) + b_n; g.b_sk = b_sk; g.b_sn = b_sn;
+    g.alpha_dev = sc + slot;
+    return g;
+  };
+  const bool vec = !((uintptr_t)a->G & ((a->g_dtype == DION_BF16) ? 7 : 15)) && a->ldg % 4 == 0;
+  const int fgrid = grid_for(c, m * n / 4);
+  float* sum = s.ws + s.L.B32;
+  if (vec) launch_pdl(k_form_b32_amax<true>, dim3((unsigned)fgrid), dim3(256), 0, st, (const float*)a->M, a->ldm, a->G, a->ldg, gmode, m, n, sum, pm);
+  else launch_pdl(k_form_b32_amax<false>, dim3((unsigned)fgrid), dim3(256), 0, st, (const float*)a->M, a->ldm, a->G, a->ldg, gmode, m, n, sum, pm);
+  DION_CHECK_LAUNCH(c);
+  DION_TRY(pair_of(sum, n, m, n, s.L.Bp, LZ_B, -1, -1, true, fgrid));
+  if (refresh) {
+    PhaseScope ps_orth(c, st, DION_PHASE_ORTH);
+    // T = (M + G) Q  (m x r), Z = (M + G)^T T (n x r), Q <- Orthonormalize(Z)
+    const int precise = (resolve_orth(c, r, (m < n) ? m : n) == DION_ORTH_SHIFTED3) ? 1 : 0;
+    DION_TRY(pair_of((const float*)a->Q, a->ldq, n, r, s.L.S16, LZ_BQ, LZ_B, -1, false, 0));
+    GemmArgs t = product(m, r, n, s.L.Bp, m * n, n, 1, s.L.S16, n * r, r, 1, LZ_BQ);
+    t.C = R; t.ldc = r; t.epi = EPI_STORE; t.precise = precise;
+    DION_TRY(launch_gemm(s, t));
+    DION_TRY(pair_of(R, r, m, r, s.L.P1, LZ_AQ, LZ_B, -1, false, 0));
+    const i64 pin_off = panel_offset(s, r, (m < n) ? m : n);
+    GemmArgs z = product(n, r, m, s.L.Bp, m * n, 1, n, s.L.P1, m * r, r, 1, LZ_AQ);
+    z.C = s.ws + pin_off; z.ldc = r; z.epi = EPI_STORE; z.precise = precise;
+    DION_TRY(launch_gemm(s, z));
+    i64 V_off = 0;
+    s.in_orth = true;
+    const int rc_orth = orthonormalize(s, n, r, (m < n) ? m : n, pin_off, &V_off);
+    s.in_orth = false;
+    DION_TRY(rc_orth);
+    launch_pdl(k_copy_panel, dim3((unsigned)grid_for(c, n * r)), dim3(256), 0, st, (const float*)(s.ws + V_off), r, (float*)a->Q, a->ldq, n, r,
+               (const int*)s.flag, (const int*)nullptr, (i64)0, -1);
+    DION_CHECK_LAUNCH(c);
+  }
+  {   // W = (M + G) Q
+  PhaseScope ps(c, st, DION_PHASE_P);
+  DION_TRY(pair_of((const float*)a->Q, a->ldq, n, r, s.L.S16, LZ_BQ, LZ_B, LZ_Q, false, 0));
+  GemmArgs w = product(m, r, n, s.L.Bp, m * n, n, 1, s.L.S16, n * r, r, 1, LZ_BQ);
+  w.C = R; w.ldc = r; w.epi = EPI_STORE;
+  DION_TRY(launch_gemm(s, w));
+  }
+  {   // M <- (M + G) - (1 - mu) W Q^T
+  PhaseScope ps(c, st, DION_PHASE_EF);
+  DION_TRY(pair_of(R, r, m, r, s.L.P1, LZ_AQ, LZ_Q, -1, false, 0));
+  GemmArgs e = product(m, n, r, s.L.P1, m * r, r, 1, s.L.S16, n * r, 1, r, LZ_AQ);
+  e.C = (float*)a->M; e.ldc = a->ldm; e.epi = EPI_C2_SUB; e.C2 = sum; e.ldc2 = n; e.c2_mode = ADD_F32;
+  e.alpha = 1.f - c->cfg.mu;
+  e.skip_flag = s.flag;
+  DION_TRY(launch_gemm(s, e));
+  }
+  {   // U = ColNorm(W)
+  PhaseScope ps(c, st, DION_PHASE_COLNORM);
+  DION_TRY(colnorm(s, 0, R, m, r, s.ws + s.L.P0, r, a->colnorm_out));
+  }
+  // X <- X - lr sqrt(m/n) U Q^T; U's columns have unit norm: its pair has a fixed scale
+  PhaseScope ps_x(c, st, DION_PHASE_X);
+  ChainPtrs t;
+  t.p[0] = s.ws + s.L.P0;
+  launch_pdl(k_split_f16_fixed, dim3((unsigned)grid_for(c, m * r / 8)), dim3(256), 0, st, t, r, m, r, ldexpf(1.f, 13), halves(s.L.P1), halves(s.L.P1) + m * r,
+             (i64)0, (i64)0, (const int*)nullptr, (i64)0);
+  DION_CHECK_LAUNCH(c);
+  GemmArgs x = product(m, n, r, s.L.P1, m * r, r, 1, s.L.S16, n * r, 1, r, LZ_Q);
+  x.C = (float*)a->X; x.ldc = a->ldx; x.epi = EPI_SUB;
+  x.alpha = ldexpf(lr * sqrtf((float)((double)m / (double)n)), -13);
+  x.skip_flag = s.flag;
+  DION_TRY(launch_gemm(s, x));
+  launch_pdl(k_finish_step, dim3(1), dim3(1), 0, st, (const int*)s.flag, c->dev_ints + 1);
+  DION_CHECK_LAUNCH(c);
+  return DION_OK;
+}
+
 // One Lazy-Dion step (Algorithm 6).
 int lazy_one(dion_ctx* c, const dion_matrix* a, float lr, int refresh, cudaStream_t st) {
   StepCtx s;
   DION_TRY(begin_step(c, a, 1, st, &s));
+  if (lazy_on_pairs(s, a)) return lazy_pairs(s, a, lr, refresh);
   const i64 m = a->m, n = a->n, r = a->r;
   const int gmode = (a->g_dtype == DION_BF16) ? ADD_BF16 : ADD_F32;
   float* P0 = s.ws + s.L.P0;
