@@ -20,7 +20,8 @@ int umma_configure();
 enum : int {
   UMMA_VARIANT_REGISTER_LOADS = 1,   // operands through registers instead of TMA
   UMMA_VARIANT_WITHHOLD = 2,         // with register loads: withhold one producer arrival, 1 ms wait budget
-  UMMA_VARIANT_NO_PAIRS = 4          // single-CTA tiles where the product would take CTA pairs
+  UMMA_VARIANT_NO_PAIRS = 4,         // single-CTA tiles where the product would take CTA pairs
+  UMMA_VARIANT_NO_TMA_EPI = 8        // register epilogue where the product would take the TMA epilogue
 };
 int umma_try_launch(const GemmArgs& g_in, int precision, int sm_count, float* part, i64 part_floats, int* status,
                     cudaStream_t st, int variant = 0);

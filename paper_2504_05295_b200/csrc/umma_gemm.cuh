@@ -66,6 +66,12 @@ struct Params {
   const void* c2tab[GEMM_TAB_MAX];
 };
 
+// The TMA epilogue's parameters: maps of the outputs (and second operands) of up to NB matrices.
+template <int NB>
+struct ParamsTE : Params {
+  alignas(64) CUtensorMap tmC[NB], tmC2[NB];
+};
+
 // ------------------------------------------------------------------ PTX wrappers
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
@@ -110,6 +116,12 @@ __device__ __forceinline__ void tma_load_3d_pair(uint32_t dst, const CUtensorMap
       "cp.async.bulk.tensor.3d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], [%5];" ::"r"(dst),
       "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(z), "r"(bar_cluster)
       : "memory");
+}
+// 2-D tiled TMA store from this CTA's shared memory (completes with the thread's bulk group)
+__device__ __forceinline__ void tma_store_2d(const CUtensorMap* map, uint32_t src, int x, int y) {
+  asm volatile("cp.async.bulk.tensor.2d.global.shared::cta.tile.bulk_group [%0, {%1, %2}], [%3];" ::"l"(reinterpret_cast<uint64_t>(map)), "r"(x),
+               "r"(y), "r"(src)
+               : "memory");
 }
 __device__ __forceinline__ uint32_t cluster_addr(uint32_t addr, uint32_t rank) {   // `addr` as seen in CTA `rank`
   uint32_t r;
@@ -551,7 +563,7 @@ struct TileMap {
 // ~1e-5 relative at 1.3 times the tensor time of one TF32 pass.  Used for the error-feedback product in fp32
 // mode, whose result enters M scaled by 1 - mu.
 template <int BN, bool BF16, bool SPLIT = false, bool TMA = false, bool D16 = false, bool CE = false, bool ONE = false,
-          bool CG2 = false, bool X2 = false>
+          bool CG2 = false, bool X2 = false, bool TE = false>
 struct Cfg {
   // BT: bf16 operands formed in shared memory from TMA-loaded fp32 tiles (K block of 32, as in
   // the fp32 TMA variant).  A stage then holds the raw fp32 tiles of A, of its fp32 addend and
@@ -568,11 +580,11 @@ struct Cfg {
                                         : (((BF16 && !X2) || ONE) ? 1 : 2) * (A_BYTES + B_BYTES);
   // D16: the producer warps have no conversion work and serve as epilogue warps too
   // (with operand pairs the stages leave room for 8 warps' epilogue tiles only)
-  static constexpr int EPI_WARPS = ((D16 && !X2) || ONE) ? NUM_EPI_WARPS + NUM_PROD_WARPS : NUM_EPI_WARPS;
+  static constexpr int EPI_WARPS = (((D16 && !X2) || ONE) && !TE) ? NUM_EPI_WARPS + NUM_PROD_WARPS : NUM_EPI_WARPS;
   // Operand pairs: nothing to convert and no room for more epilogue tiles, so the kernel runs without the producer
   // warps (10 warps in all); the registers they would hold go to the epilogue warps' loads in flight (DEEP).
   static constexpr bool DEEP = X2;
-  static constexpr int MMA_WARP = X2 ? NUM_EPI_WARPS : NUM_EPI_WARPS + NUM_PROD_WARPS;   // the warp that issues the MMAs
+  static constexpr int MMA_WARP = (X2 || TE) ? NUM_EPI_WARPS : NUM_EPI_WARPS + NUM_PROD_WARPS;   // the warp that issues the MMAs
   static constexpr int THREADS = (MMA_WARP + (TMA ? 2 : 1)) * 32;                         // ... then the TMA warp
   // CE (coalesced epilogue): an epilogue warp owns 32 rows x EPI_W columns of the tile and passes them
   // through a private shared-memory tile in passes of EPI_RPP rows (EPI_RPP * EPI_W = 1024 elements),
@@ -582,7 +594,9 @@ struct Cfg {
   static constexpr int EPI_W = 32 * (BN / 32) / (EPI_WARPS / 4);
   static constexpr int EPI_RPP = 1024 / EPI_W;
   static constexpr int EPI_TILE_FLOATS = EPI_RPP * (EPI_W + 4);
-  static constexpr int EPI_BYTES = CE ? EPI_WARPS * EPI_TILE_FLOATS * 4 : 0;
+  // TE (TMA epilogue): a ring of 128-row x 32-column slabs of C instead (see k_gemm_umma)
+  static constexpr int TE_RING = 6 * BM * 128;
+  static constexpr int EPI_BYTES = TE ? TE_RING : CE ? EPI_WARPS * EPI_TILE_FLOATS * 4 : 0;
   static constexpr int STAGES = CE ? (232448 - 1536 - EPI_BYTES) / STAGE_BYTES : (192 * 1024) / STAGE_BYTES;
   static constexpr int G16_BYTES = ((BF16 && !TMA) || D16 || CE) ? 0 : BM * 32 * 2;   // bf16 addend tile of the TMA variants (per stage)
   static constexpr int SMEM_BYTES = STAGES * (STAGE_BYTES + G16_BYTES) + EPI_BYTES + 1024 + 512;
@@ -604,10 +618,18 @@ struct Cfg {
 // TMA with bf16 operands: the same loads; the producer warps add, round to bf16 and write
 // the operand tiles the MMA reads (k-contiguous: rows of 64 bytes, 64-byte swizzle;
 // row-contiguous: 128-byte rows of 64 row indices, 128-byte swizzle); one MMA per K step.
+// TE (TMA epilogue; 16-bit arrays on CTA pairs, both operands k-contiguous, tiles of one accumulation chunk: the rank-r updates
+// C -= alpha A B^T, C = C2 - alpha A B^T and C = C + C2 - alpha A B^T).  At low rank such a product is a pass over C, and
+// through the register epilogue it was bound by that epilogue's instructions (16384^2, r = 256: 2760 per warp and tile, 606 us
+// of 333 at copy speed).  Here C (or C2, or both) comes by TMA in slabs of 128 rows x 32 columns into a ring of six
+// slabs, up to five ahead of their use and across tiles; the epilogue warps add the accumulator in place (a lane per row, 16
+// columns; the 128-byte swizzle keeps that free of bank conflicts) and one thread sends the slab out by TMA.  The same
+// operations per element as the other epilogues.  Paid for with operand stages: for K at which memory is the bound.
 template <int BN, bool A_MN, bool B_MN, bool BF16, bool SPLIT, bool TMA, bool D16 = false, bool CE = false, bool ONE = false,
-          bool CG2 = false, bool X2 = false>
-__global__ void __launch_bounds__((Cfg<BN, BF16, SPLIT, TMA, D16, CE, ONE, CG2, X2>::THREADS), 1)
-k_gemm_umma(const __grid_constant__ Params p) {
+          bool CG2 = false, bool X2 = false, bool TE = false, typename PT = Params>
+__global__ void __launch_bounds__((Cfg<BN, BF16, SPLIT, TMA, D16, CE, ONE, CG2, X2, TE>::THREADS), 1)
+k_gemm_umma(const __grid_constant__ PT p) {
+  static_assert(!TE || (D16 && CE && CG2 && !SPLIT && !A_MN && !B_MN), "TMA epilogue: 16-bit arrays on CTA pairs");
   static_assert(!X2 || (D16 && CE), "operand pairs are bf16 arrays");
   static_assert(!CG2 || (TMA && BN == 256 && ((!BF16 && !D16 && !ONE) || (D16 && CE))),
                 "CTA pairs: the fp32 TMA variants and the 16-bit array variants (single arrays or pairs), 256-column tiles");
@@ -615,7 +637,7 @@ k_gemm_umma(const __grid_constant__ Params p) {
   static_assert(!D16 || (BF16 && TMA), "bf16 operands in memory are loaded by TMA");
   static_assert(!CE || (TMA && (D16 || !BF16)), "the coalesced epilogue serves the bf16-array and the fp32 TMA variants");
   static_assert(!ONE || (TMA && CE && !BF16 && !SPLIT && !A_MN && !B_MN), "single pass: k-contiguous fp32 operands by TMA");
-  using C = Cfg<BN, BF16, SPLIT, TMA, D16, CE, ONE, CG2, X2>;
+  using C = Cfg<BN, BF16, SPLIT, TMA, D16, CE, ONE, CG2, X2, TE>;
   constexpr bool NOCONV = D16 || ONE;    // the operand tiles are what TMA writes: nothing to convert
   constexpr bool PAIRLOAD = CG2 && NOCONV;   // both CTAs' loads complete on the leader's barrier
   constexpr int BN_L = C::BN_L;
@@ -658,6 +680,7 @@ k_gemm_umma(const __grid_constant__ Params p) {
   volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(bars + 2 * STAGES + 5);
   volatile int* dead = reinterpret_cast<volatile int*>(bars + 2 * STAGES + 6);
   auto raw_bar = [&](int s) { return bar0 + 8u * (2 * STAGES + 7 + s); };   // TMA landed (TMA variant)
+  [[maybe_unused]] auto slab_bar = [&](int s) { return bar0 + 8u * (3 * STAGES + 7 + s); };   // a slab of C landed (TMA epilogue)
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 
@@ -669,6 +692,7 @@ k_gemm_umma(const __grid_constant__ Params p) {
     mbar_init(drain_bar, 1);
     // (pair without converters: the leader's "landed" barrier counts the bytes of both CTAs' tiles, see the TMA issuer)
     if (TMA) for (int s = 0; s < STAGES; ++s) mbar_init(raw_bar(s), 1);
+    if (TE) for (int s = 0; s < 6; ++s) mbar_init(slab_bar(s), 1);
     *dead = 0;
     fence_barrier_init();
   }
@@ -691,6 +715,120 @@ k_gemm_umma(const __grid_constant__ Params p) {
     // The K loop of a tile is therefore cut into chunks of p.kc K blocks; each chunk is
     // accumulated from zero in TMEM and added here, in fp32 round-to-nearest, to the
     // running result in global memory.
+    if constexpr (TE) {
+      const bool both = g.epi == EPI_ADD2_SUB;
+      const bool from_c2 = g.epi == EPI_C2_SUB;
+      const bool c2_16 = both && g.c2_mode == ADD_BF16;
+      const int nslots = both ? 3 : 6;
+      const uint32_t slot_bytes = both ? 2 * BM * 128 : BM * 128;      // C, then C2
+      const uint32_t ring = smem_base + STAGES * C::STAGE_BYTES;
+      const uint32_t load_bytes = BM * 128 + (both ? (c2_16 ? BM * 64 : BM * 128) : 0);
+      const int quad = warp & 3, half = warp >> 2;
+      const bool issuer = threadIdx.x == 0;
+      auto slabs_of = [&](const Item& it) -> int {      // slabs of this CTA's half of the tile that hold anything
+        if ((2 * (i64)it.mi + cta_rank) * BM >= g.M) return 0;
+        return (int)min((i64)(BN / 32), (g.N - (i64)it.ni * BN + 31) / 32);
+      };
+      // the issuer's walk over the slabs to load
+      int litem = worker, ls = 0, lns = 0, lq = 0;
+      Item lit;
+      auto find = [&]() {      // from litem on: the next item with slabs
+        for (; litem < p.num_items; litem += workers) {
+          lit = decode_item<BN, BKE, CG2>(p, litem);
+          if (!skipped(lit) && (lns = slabs_of(lit)) > 0) return;
+        }
+      };
+      auto load_next = [&]() {
+        if (litem >= p.num_items || *dead) return;
+        const int slot = lq % nslots;
+        const uint32_t dst = ring + (uint32_t)slot * slot_bytes, bar = slab_bar(slot);
+        const int x = lit.ni * BN + ls * 32, y = (2 * lit.mi + (int)cta_rank) * BM;
+        mbar_expect_tx(bar, load_bytes);
+        tma_load_2d(dst, from_c2 ? &p.tmC2[lit.b] : &p.tmC[lit.b], x, y, bar);
+        if (both) tma_load_2d(dst + BM * 128, &p.tmC2[lit.b], x, y, bar);
+        ++lq;
+        if (++ls == lns) { ls = 0; litem += workers; find(); }
+      };
+      if (issuer) {
+        find();
+        for (int s = 0; s + 1 < nslots; ++s) load_next();
+      }
+      int iter = 0, q = 0;
+      const int row = quad * 32 + lane;
+      const uint32_t swz = (uint32_t)(row & 7);
+      // (A wait that runs out marks the CTA dead; every warp still walks the same barriers, without waiting any more.)
+      for (int item = worker; item < p.num_items; item += workers) {
+        const Item it = decode_item<BN, BKE, CG2>(p, item);
+        if (skipped(it)) continue;
+        const int ns = slabs_of(it);
+        const int ab = iter % NBUF;
+        const uint32_t ph = (uint32_t)(iter / NBUF) & 1u;
+        ++iter;
+        const float f = -(g.alpha * (g.alpha_dev != nullptr ? __ldg(g.alpha_dev + (i64)it.b * g.alpha_dev_stride) : 1.f));
+        mbar_wait(accf_bar(ab), ph, dead, p.status, p.spin_limit, 64);
+        tc_fence_after();
+        for (int s = 0; s < ns; ++s, ++q) {
+          const int slot = q % nslots;
+          const uint32_t dst = ring + (uint32_t)slot * slot_bytes;
+          float acc[16];
+          tmem_ld16(tmem_base + (uint32_t)(ab * BN + s * 32 + half * 16) + ((uint32_t)(quad * 32) << 16), acc);
+          mbar_wait(slab_bar(slot), (uint32_t)(q / nslots) & 1u, dead, p.status, p.spin_limit);
+          const uint32_t rowp = dst + (uint32_t)row * 128u;
+#pragma unroll
+          for (int j = 0; j < 4; ++j) {
+            const uint32_t at = rowp + ((((uint32_t)(half * 4 + j)) ^ swz) << 4);
+            float4 c = lds128(at);
+            if (both) {
+              if (!c2_16) {
+                const float4 t = lds128(at + BM * 128);
+                c.x += t.x; c.y += t.y; c.z += t.z; c.w += t.w;
+              } else {      // rows of 64 bytes, 64-byte swizzle: four bf16 values, half of a 16-byte unit
+                const uint32_t unit = (uint32_t)(half * 2 + (j >> 1)) ^ ((uint32_t)(row >> 1) & 3u);
+                uint32_t w0, w1;
+                asm volatile("ld.shared.v2.b32 {%0, %1}, [%2];"
+                             : "=r"(w0), "=r"(w1) : "r"(dst + BM * 128 + (uint32_t)row * 64u + (unit << 4) + (uint32_t)(j & 1) * 8u) : "memory");
+                const __nv_bfloat162 lo = *reinterpret_cast<const __nv_bfloat162*>(&w0);
+                const __nv_bfloat162 hi = *reinterpret_cast<const __nv_bfloat162*>(&w1);
+                c.x += __low2float(lo); c.y += __high2float(lo); c.z += __low2float(hi); c.w += __high2float(hi);
+              }
+            }
+            sts128(at, make_float4(fmaf(f, acc[4 * j], c.x), fmaf(f, acc[4 * j + 1], c.y), fmaf(f, acc[4 * j + 2], c.z), fmaf(f, acc[4 * j + 3], c.w)));
+          }
+          fence_proxy_async();
+          if (s + 1 == ns) {      // the accumulator has been read
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) {
+              if (cta_rank != 0) mbar_arrive_remote_relaxed(acce_bar(ab), 0u);
+              else mbar_arrive(acce_bar(ab));
+            }
+          }
+          asm volatile("bar.sync 1, %0;" ::"n"(NUM_EPI_WARPS * 32) : "memory");
+          if (issuer && !*dead) {
+            tma_store_2d(&p.tmC[it.b], dst, it.ni * BN + s * 32, (2 * it.mi + (int)cta_rank) * BM);
+            asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+            // the next load goes where the slab before this one was: its store has to have read it
+            asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory");
+            load_next();
+          }
+        }
+        if (ns == 0) {
+          tc_fence_before();
+          __syncwarp();
+          if (lane == 0) {
+            if (cta_rank != 0) mbar_arrive_remote_relaxed(acce_bar(ab), 0u);
+            else mbar_arrive(acce_bar(ab));
+          }
+        }
+      }
+      if (issuer) {
+        asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
+        for (; q < lq; ++q) {      // (only after a wait ran out: loads still in flight)
+          const long long t0 = clock64();
+          while (!mbar_try_wait(slab_bar(q % nslots), (uint32_t)(q / nslots) & 1u) && clock64() - t0 < p.spin_limit) {}
+        }
+      }
+    } else {
     int iter = 0;
     bool alive = true;
     for (int item = worker; item < p.num_items && alive; item += workers) {
@@ -947,6 +1085,7 @@ k_gemm_umma(const __grid_constant__ Params p) {
           else mbar_arrive(acce_bar(ab));
         }
       }
+    }
     }
   } else if (warp < C::MMA_WARP) {
     // ------------------------------------------------------------ producers
@@ -1499,6 +1638,27 @@ inline void launch_variant(const Params& p, bool a_mn, bool b_mn, int grid, cuda
   else launch_single(k_gemm_umma<BN, true, false, BF16, SPLIT, TMA, D16, CE>, p, grid, threads, smem, st);
 }
 
+// the TMA epilogue (see k_gemm_umma): 16-bit arrays, single or pairs, on CTA pairs
+template <bool X2, int NB>
+inline cudaError_t launch_te(const ParamsTE<NB>& p, int grid, cudaStream_t st) {
+  using CF = Cfg<256, true, false, true, true, true, false, true, X2, true>;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)grid); cfg.blockDim = dim3(CF::THREADS); cfg.dynamicSmemBytes = CF::SMEM_BYTES; cfg.stream = st;
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = 2; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
+  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[1].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr; cfg.numAttrs = 2;
+  return cudaLaunchKernelEx(&cfg, k_gemm_umma<256, false, false, true, false, true, true, true, false, true, X2, true, ParamsTE<NB>>, p);
+}
+template <bool X2, int NB>
+inline cudaError_t set_te_attr() {
+  using CF = Cfg<256, true, false, true, true, true, false, true, X2, true>;
+  return cudaFuncSetAttribute(k_gemm_umma<256, false, false, true, false, true, true, true, false, true, X2, true, ParamsTE<NB>>,
+                              cudaFuncAttributeMaxDynamicSharedMemorySize, CF::SMEM_BYTES);
+}
+
 typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*, const cuuint64_t*,
                                   const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave, CUtensorMapSwizzle,
                                   CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
@@ -1561,6 +1721,33 @@ inline bool make_operand16_map(CUtensorMap* map, const void* ptr, i64 rows, i64 
                         CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                         CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   return r == CUDA_SUCCESS;
+}
+
+// Slabs of the TMA epilogue: 128 rows x 32 columns of an fp32 (128-byte swizzle) or bf16 (64-byte swizzle) array.
+inline bool make_slab_map(CUtensorMap* map, const void* ptr, i64 rows, i64 cols, i64 ld, bool bf16) {
+  EncodeTiledFn fn = encode_tiled_fn();
+  const i64 es = bf16 ? 2 : 4;
+  if (fn == nullptr || ((uintptr_t)ptr & 15) || (ld * es) % 16 != 0) return false;
+  const cuuint64_t gdim[2] = {(cuuint64_t)cols, (cuuint64_t)rows}, gstride[1] = {(cuuint64_t)(ld * es)};
+  const cuuint32_t box[2] = {32, BM}, estr[2] = {1, 1};
+  return fn(map, bf16 ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16 : CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, const_cast<void*>(ptr), gdim, gstride, box, estr,
+            CU_TENSOR_MAP_INTERLEAVE_NONE, bf16 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+            CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
+// Fills the maps of the TMA epilogue for the matrices of a launch; false: an array that a map cannot describe.
+template <int NB>
+inline bool te_maps(ParamsTE<NB>& q, const GemmArgs& g, int nbat) {
+  const bool c2 = g.epi != EPI_SUB, c2_16 = g.epi == EPI_ADD2_SUB && g.c2_mode == ADD_BF16;
+  for (int b = 0; b < nbat; ++b) {
+    const float* c = g.c_tab != nullptr ? g.c_tab[b] : g.C + (i64)b * g.bs2;
+    if (!make_slab_map(&q.tmC[b], c, g.M, g.N, g.ldc, false)) return false;
+    if (!c2) continue;
+    const void* t = g.c2_tab != nullptr ? g.c2_tab[b]
+                    : g.c2_batched      ? (const void*)(reinterpret_cast<const float*>(g.C2) + (i64)b * g.bs2) : g.C2;
+    if (!make_slab_map(&q.tmC2[b], t, g.M, g.N, g.ldc2, c2_16)) return false;
+  }
+  return true;
 }
 
 // The maps of fp32 operands are 3-D: the third coordinate is the matrix of a batched launch (`nbatch` matrices,
@@ -1640,6 +1827,10 @@ int umma_configure() {
   if (e == cudaSuccess) e = set_d16_pair_attr<false, true>();
   if (e == cudaSuccess) e = set_d16_pair_attr<true, true>();
   if (e == cudaSuccess) e = set_d16_pair_attr<true, false>();
+  if (e == cudaSuccess) e = set_te_attr<true, 1>();
+  if (e == cudaSuccess) e = set_te_attr<true, GEMM_TAB_MAX>();
+  if (e == cudaSuccess) e = set_te_attr<false, 1>();
+  if (e == cudaSuccess) e = set_te_attr<false, GEMM_TAB_MAX>();
   if (e == cudaSuccess) e = set_pair_attr<false, false>();
   if (e == cudaSuccess) e = set_pair_attr<false, true>();
   if (e == cudaSuccess) e = set_pair_attr<true, true>();
@@ -1651,6 +1842,10 @@ int umma_configure() {
 
 constexpr i64 PAIR_MIN_ROWS = 512;   // smallest output height given to CTA pairs
 constexpr i64 PAIR_MIN_TRI = 2048;   // smallest lower-triangular output given to CTA pairs
+// Largest K given to the TMA epilogue: operand pairs (two 64 KB stages left; at K = 1024 the error feedback of 14336 x 4096 took
+// 304 us against 262) and single arrays (four 32 KB stages; still ahead at 1024: 54.6 against 58.9 us at 4096^2).
+constexpr i64 TE_MAX_K_PAIRS = 512;
+constexpr i64 TE_MAX_K = 1024;
 int umma_try_launch(const GemmArgs& g_in, int precision, int sm_count, float* part, i64 part_floats,
                            int* status, cudaStream_t st, int variant) {
   using namespace umma;
@@ -1797,6 +1992,23 @@ int umma_try_launch(const GemmArgs& g_in, int precision, int sm_count, float* pa
   const int grid = cg2 ? 2 * (p.num_items < nclusters ? p.num_items : nclusters)
                        : (p.num_items < sm_count ? p.num_items : sm_count);
   const bool one = g.tf32x1 && !bf16 && tma && !a_mn && !b_mn && g.a2_mode == ADD_NONE && !g.precise && splits == 1;
+  // The TMA epilogue for rank-r updates whose tiles are one accumulation chunk, up to the K at which the tensor cores would miss
+  // the operand stages it costs.
+  if (cg2 && d16 && !a_mn && !b_mn && !g.precise && splits == 1 && g.tri == TRI_FULL && !g.klimit && p.nkb <= p.kc &&
+      (g.epi == EPI_SUB || g.epi == EPI_C2_SUB || g.epi == EPI_ADD2_SUB) && g.K <= (x2 ? TE_MAX_K_PAIRS : TE_MAX_K) &&
+      !(variant & UMMA_VARIANT_NO_TMA_EPI)) {
+    auto go = [&](auto& q) -> int {      // 1: launched, 0: not for this epilogue, < 0: error
+      static_cast<Params&>(q) = p;
+      if (!te_maps(q, g, nbat)) return 0;
+      const cudaError_t e = x2 ? launch_te<true>(q, grid, st) : launch_te<false>(q, grid, st);
+      if (e != cudaSuccess) { cudaGetLastError(); return DION_ERR_CUDA; }
+      return cudaGetLastError() == cudaSuccess ? 1 : DION_ERR_CUDA;
+    };
+    int rc;
+    if (nbat == 1) { ParamsTE<1> q; rc = go(q); }
+    else { ParamsTE<GEMM_TAB_MAX> q; rc = go(q); }
+    if (rc != 0) return rc;
+  }
   if (x2 && g.precise) {   // (built with split accumulators for B row-index contiguous: Gram matrices and P)
     if (!b_mn) return 0;
     if (cg2) {
