@@ -49,7 +49,7 @@ constexpr i64 NBO_COLS = 512;  // = NBO, the outer block of the two-level Choles
 // One launch of k_chol_flow factors Gram matrices up to this order; beyond it blocks of 512 columns.
 constexpr i64 FLOW_MAX_R = 3072;
 constexpr double FLOW_SOLVE_MAX = 1.1e6;        // largest rows r whose panel that launch solves too
-constexpr i64 FLOW_SOLVE_MAX_TILES = 60000;     // ... in an adaptive round: most 64^3 products of its substitution
+constexpr i64 FLOW_SOLVE_MAX_TILES = 40000;     // ... in an adaptive round: most 64^3 products of its substitution
 constexpr float NEAR_MAX_DEF = 3e-3f;           // largest |P^T P - I|_F whose factor is taken as a series (k_near_identity): third-order error 3e-8
 constexpr i64 NEAR_MAX_BLOCKS = 512;
 constexpr int FLOW_EXCLUSIVE_MAX = 8;           // matrices of a chain up to which its runners get an SM each
