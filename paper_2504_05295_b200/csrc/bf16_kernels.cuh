@@ -304,6 +304,12 @@ __device__ __forceinline__ void block_max(float m, float* __restrict__ out) {   
   }
   if (threadIdx.x == 0) out[blockIdx.x] = red[0];
 }
+// The exponent of the power of two that puts amax in [2^13, 2^14): amax = f 2^ex with f in [0.5, 1) gives 14 - ex.
+__device__ __forceinline__ int f16_scale_exponent(float amax) {
+  int ex = 14;
+  if (amax > 0.f && amax < 3.0e38f) frexpf(amax, &ex);
+  return 14 - (ex < -80 ? -80 : ex);
+}
 // M + G in fp32 and the blocks' largest magnitudes of it in one pass (the products on a scaled half pair of the sum).
 template <bool VEC>
 __global__ void __launch_bounds__(256) k_form_b32_amax(const float* __restrict__ M, i64 ldm, const void* __restrict__ G, i64 ldg, int g_mode,
@@ -312,6 +318,86 @@ __global__ void __launch_bounds__(256) k_form_b32_amax(const float* __restrict__
   float m = 0.f;
   form_b32_body<VEC>(M, ldm, G, ldg, g_mode, rows, cols, out, nullptr, nullptr, &m);
   block_max(m, part);
+}
+// The two launches that prepare a chain (blockIdx.y) of steps on half pairs: M + G in fp32 with the largest magnitudes of the sum
+// and of Q (Q is a right factor of the caller's making: nothing bounds its entries), then the scaled pairs of both.
+// part: gridDim.x maxima of the sum, then as many of Q.  16-byte accesses to Q where it allows them (qvec).
+template <bool VEC>
+__global__ void __launch_bounds__(256) k_form_sum_amax(const ChainPtrs Ms, i64 ldm, const ChainPtrs Gs, i64 ldg, int g_mode, i64 rows, i64 cols,
+                                                       const ChainPtrs Qs, i64 ldq, i64 qrows, i64 qcols, int qvec, float* __restrict__ out,
+                                                       float* __restrict__ part, i64 wstride) {
+  pdl_enter();
+  const i64 b = blockIdx.y;
+  part += b * wstride;
+  float m = 0.f, mq = 0.f;
+  form_b32_body<VEC>(reinterpret_cast<const float*>(Ms.p[b]), ldm, Gs.p[b], ldg, g_mode, rows, cols, out + b * wstride, nullptr, nullptr, &m);
+  const float* __restrict__ Q = reinterpret_cast<const float*>(Qs.p[b]);
+  const i64 per_row = qcols / 4, total = qrows * per_row;
+  for (i64 e = (i64)blockIdx.x * blockDim.x + threadIdx.x; e < total; e += (i64)gridDim.x * blockDim.x) {
+    const i64 i = e / per_row;
+    const float* q = Q + i * ldq + (e - i * per_row) * 4;
+    const float4 a = qvec ? *reinterpret_cast<const float4*>(q) : make_float4(q[0], q[1], q[2], q[3]);
+    mq = fmaxf(fmaxf(mq, fmaxf(fabsf(a.x), fabsf(a.y))), fmaxf(fabsf(a.z), fabsf(a.w)));
+  }
+  block_max(m, part);
+  __syncthreads();
+  block_max(mq, part + gridDim.x);
+}
+// A step's scalars: the factors that take the scales out of P, R and the error feedback; then R's block maxima.
+enum : int { HS_P = 0, HS_R = 1, HS_EF = 2, HS_MAX = 16 };
+constexpr int HS_U_BITS = 13;      // U's pair is scaled by 2^13 (entries at most 1)
+__global__ void __launch_bounds__(256) k_split_sum(const float* __restrict__ sum, i64 total_s, const ChainPtrs Qs, i64 ldq, i64 qrows,
+                                                   i64 qcols, int qvec, const float* __restrict__ part, int nparts,
+                                                   __half* __restrict__ sh, __half* __restrict__ qh, float* __restrict__ scal, i64 wstride) {
+  pdl_enter();
+  const i64 b = blockIdx.y;
+  sum += b * wstride; part += b * wstride; scal += b * wstride;
+  sh += 2 * b * wstride; qh += 2 * b * wstride;
+  const float* __restrict__ Q = reinterpret_cast<const float*>(Qs.p[b]);
+  __shared__ float red[2][256];
+  float m0 = 0.f, m1 = 0.f;
+  for (int e = threadIdx.x; e < nparts; e += 256) { m0 = fmaxf(m0, part[e]); m1 = fmaxf(m1, part[nparts + e]); }
+  red[0][threadIdx.x] = m0; red[1][threadIdx.x] = m1;
+  __syncthreads();
+  for (int w = 128; w > 0; w >>= 1) {
+    if ((int)threadIdx.x < w) {
+      red[0][threadIdx.x] = fmaxf(red[0][threadIdx.x], red[0][threadIdx.x + w]);
+      red[1][threadIdx.x] = fmaxf(red[1][threadIdx.x], red[1][threadIdx.x + w]);
+    }
+    __syncthreads();
+  }
+  const int es = f16_scale_exponent(red[0][0]), eq = f16_scale_exponent(red[1][0]);
+  if (blockIdx.x == 0 && threadIdx.x == 0) {
+    scal[HS_P] = ldexpf(1.f, -es) * ldexpf(1.f, -eq);
+    scal[HS_R] = ldexpf(1.f, -es - HS_U_BITS);
+  }
+  const float fs = ldexpf(1.f, es), fq = ldexpf(1.f, eq);
+  const i64 n8 = total_s / 8, qpr = qcols / 8, q8 = qrows * qpr;
+  for (i64 e = (i64)blockIdx.x * blockDim.x + threadIdx.x; e < n8 + q8; e += (i64)gridDim.x * blockDim.x) {
+    const bool of_q = e >= n8;
+    const i64 eo = of_q ? e - n8 : e;
+    float4 x, y;
+    if (!of_q) {
+      x = *reinterpret_cast<const float4*>(sum + eo * 8);
+      y = *reinterpret_cast<const float4*>(sum + eo * 8 + 4);
+    } else {
+      const i64 i = eo / qpr;
+      const float* q = Q + i * ldq + (eo - i * qpr) * 8;
+      x = qvec ? *reinterpret_cast<const float4*>(q) : make_float4(q[0], q[1], q[2], q[3]);
+      y = qvec ? *reinterpret_cast<const float4*>(q + 4) : make_float4(q[4], q[5], q[6], q[7]);
+    }
+    const float f = of_q ? fq : fs;
+    const float v[8] = {f * x.x, f * x.y, f * x.z, f * x.w, f * y.x, f * y.y, f * y.z, f * y.w};
+    __half h[8], l[8];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+      h[k] = __float2half_rn(v[k]);
+      l[k] = __float2half_rn(v[k] - __half2float(h[k]));
+    }
+    __half* hi = (of_q ? qh : sh) + eo * 8;
+    *reinterpret_cast<uint4*>(hi) = *reinterpret_cast<const uint4*>(h);
+    *reinterpret_cast<uint4*>(hi + (of_q ? qrows * qcols : total_s)) = *reinterpret_cast<const uint4*>(l);
+  }
 }
 __global__ void __launch_bounds__(256) k_absmax_partial(const float* __restrict__ src, i64 ld, i64 rows, i64 cols,
                                                         float* __restrict__ part, i64 wstride, const int* __restrict__ skip_flag,

@@ -11,6 +11,7 @@
 #include <vector>
 
 #include "bf16_kernels.cuh"
+#include "colnorm.cuh"
 #include "dion_common.cuh"
 #include "dion_internal.h"
 #include "orth_kernels.cuh"
@@ -41,6 +42,7 @@ constexpr i64 PART_CAP_FLOATS = (i64)16 << 20;  // split-K partial sums, at most
 constexpr double P_HALF_MIN_MNR = 4e9;          // smallest m n r whose full-rank P runs on scaled half pairs
 constexpr double SOLVE_PAIR_MIN_PANEL = 3e7;    // smallest rows x r whose blocked solves run on scaled half pairs
 constexpr i64 LAZY_PAIR_MIN_MNR = 50000000;     // smallest m n r whose Lazy-Dion step runs on scaled half pairs (2^25.6: 512 x 768 x 128)
+constexpr i64 HALF_PAIR_MIN_MNR = 50000000;     // ... and whose Dion step does (see step_on_half_pairs)
 constexpr double GRAM_PAIR_MIN_FLOPS = 2e9;     // smallest rows r^2 whose Gram matrix runs on scaled half pairs
 constexpr double P_PAIR_MIN_MNR = 1.5e10;       // smallest m n r whose P = (M + G) Q runs on bf16 operand pairs first
 
@@ -1179,49 +1181,69 @@ int orthonormalize(StepCtx& s, i64 rows, i64 r, i64 short_dim, i64 pin_off, i64*
   return DION_OK;
 }
 
-// ColNorm of matrix b's W (rows x r, ld = r) into `out`.
-int colnorm(StepCtx& s, int b, const float* W, i64 rows, i64 r, float* out, i64 ldo, float* d_out,
-            const int* skip = nullptr, i64 ldw = 0) {
-  if (ldw == 0) ldw = r;
+// Columns of W (rows x r) normalized into Q, for `per` matrices of the chain from b on: W (wstride apart), Q and d from pointer
+// tables.  x.kind != 0: the operands of the rank-r updates too (offsets in the scratch slices; see k_colnorm_apply).
+// sums != nullptr: the columns' sums of squares, given by the caller (sharded form).
+int colnorm_launch(StepCtx& s, int b, int per, const float* W, i64 ldw, i64 rows, i64 r, const ChainPtrs& Qs, i64 ldq, const ChainPtrs& ds,
+                   const int* skip, ColnormPairs x = ColnormPairs(), const float* sums = nullptr) {
   dion_ctx* c = s.c;
-  int chunks; i64 per;
-  colnorm_plan(rows, r, c->sm_count, &chunks, &per);
+  int chunks; i64 rpc;
+  colnorm_plan(rows, r, c->sm_count, &chunks, &rpc);
+  const dim3 grid((unsigned)((r + 127) / 128), (unsigned)chunks, (unsigned)per);
   float* part = s.W(b, s.L.cn_part);
-  dim3 grid((unsigned)((r + 127) / 128), (unsigned)chunks);
-  launch_pdl(k_colsumsq_partial, grid, dim3(128), 0, s.st, W, ldw, rows, r, per, part, (const int*)nullptr, (i64)0);
-  DION_CHECK_LAUNCH(c);
-  launch_pdl(k_colnorm_apply, grid, dim3(128), 0, s.st, W, ldw, rows, r, per, chunks, (const float*)part, c->cfg.eps, out, ldo,
-             s.W(b, s.L.d), d_out, c->dev_ints, skip != nullptr ? skip : (const int*)(s.OS(b) + OS_FAIL), (i64)0, ChainPtrs(), ChainPtrs());
+  const bool v4 = r % 4 == 0 && ldw % 4 == 0 && !((uintptr_t)W & 15);
+  float* amax = nullptr;
+  if (x.kind == CN_HALF) {
+    amax = s.W(b, s.L.lz) + HS_MAX;
+    x.amax = amax; x.scal = s.W(b, s.L.lz) + HS_EF;
+    x.nmax = (int)(grid.x * grid.y);
+  }
+  if (sums == nullptr) {
+    if (v4) launch_pdl(k_colsumsq_partial<true>, grid, dim3(CN_THREADS), 0, s.st, W, ldw, rows, r, rpc, part, amax, (const int*)nullptr, s.wstride);
+    else launch_pdl(k_colsumsq_partial<false>, grid, dim3(CN_THREADS), 0, s.st, W, ldw, rows, r, rpc, part, amax, (const int*)nullptr, s.wstride);
+    DION_CHECK_LAUNCH(c);
+  } else if (x.kind == CN_HALF) {
+    launch_pdl(k_absmax_partial, dim3((unsigned)x.nmax), dim3(256), 0, s.st, W, ldw, rows, r, amax, (i64)0, (const int*)nullptr, (i64)0);
+    DION_CHECK_LAUNCH(c);
+  }
+  int qvec = ldq % 4 == 0;
+  for (int k = 0; k < per; ++k) qvec = qvec && !((uintptr_t)Qs.p[k] & 15);
+  if (sums != nullptr) chunks = 1;
+  const float* sp = sums != nullptr ? sums : (const float*)part;
+  if (v4) launch_pdl(k_colnorm_apply<true>, grid, dim3(CN_THREADS), 0, s.st, W, ldw, rows, r, rpc, chunks, sp, c->cfg.eps, Qs, ldq, qvec, s.W(b, s.L.d), ds,
+                     c->dev_ints, skip, s.wstride, x);
+  else launch_pdl(k_colnorm_apply<false>, grid, dim3(CN_THREADS), 0, s.st, W, ldw, rows, r, rpc, chunks, sp, c->cfg.eps, Qs, ldq, qvec, s.W(b, s.L.d), ds,
+                  c->dev_ints, skip, s.wstride, x);
   DION_CHECK_LAUNCH(c);
   return DION_OK;
+}
+
+// ... of one matrix.
+int colnorm(StepCtx& s, int b, const float* W, i64 rows, i64 r, float* out, i64 ldo, float* d_out,
+            const int* skip = nullptr, ColnormPairs x = ColnormPairs(), const float* sums = nullptr) {
+  ChainPtrs Qs, ds;
+  Qs.p[0] = out; ds.p[0] = d_out;
+  return colnorm_launch(s, b, 1, W, r, rows, r, Qs, ldo, ds, skip != nullptr ? skip : (const int*)(s.OS(b) + OS_FAIL), x, sums);
 }
 
 // ---- elementwise kernels over a whole chain -------------------------------------------------------------------
 // Each helper makes ONE launch over the chain's matrices (blockIdx.y or .z) when their arrays share leading
 // dimensions and alignment, else one launch per matrix; outputs are in the scratch slices either way.
 
-// ColNorm of every matrix's R (scratch, rows x r dense) into its Q, d exported to colnorm_out.
-int colnorm_chain(StepCtx& s, const dion_matrix* const* list, i64 rows, i64 r) {
-  dion_ctx* c = s.c;
-  bool one = s.nb > 1 && s.nb <= GEMM_TAB_MAX && c->chain_batch;
-  for (int b = 1; b < s.nb && one; ++b) one = list[b]->ldq == list[0]->ldq;
-  if (!one) {
-    for (int b = 0; b < s.nb; ++b)
-      DION_TRY(colnorm(s, b, s.W(b, s.L.R), rows, r, (float*)list[b]->Q, list[b]->ldq, list[b]->colnorm_out));
-    return DION_OK;
+// ColNorm of every matrix's R (scratch, rows x r dense) into its Q, d exported to colnorm_out; kind, qh_off, qscale, pair_off: the
+// rank-r updates' operands beside it (offsets in the scratch slices).
+int colnorm_chain(StepCtx& s, const dion_matrix* const* list, i64 rows, i64 r, int kind = 0, i64 qh_off = 0, float qscale = 1.f, i64 pair_off = 0) {
+  bool one = s.nb <= GEMM_TAB_MAX && (s.nb == 1 || s.c->chain_batch);
+  for (int b = 1; b < s.nb && one; ++b)
+    one = list[b]->ldq == list[0]->ldq && ((uintptr_t)list[b]->Q & 15) == ((uintptr_t)list[0]->Q & 15);
+  const int per = one ? s.nb : 1;
+  for (int b = 0; b < s.nb; b += per) {
+    ChainPtrs Qs, ds;
+    for (int k = 0; k < per; ++k) { Qs.p[k] = list[b + k]->Q; ds.p[k] = list[b + k]->colnorm_out; }
+    ColnormPairs x = ColnormPairs();
+    x.kind = kind; x.qh = s.W(b, qh_off); x.qscale = qscale; x.hi = s.W(b, pair_off);
+    DION_TRY(colnorm_launch(s, b, per, s.W(b, s.L.R), r, rows, r, Qs, list[b]->ldq, ds, s.OS(b) + OS_FAIL, x));
   }
-  int chunks; i64 per;
-  colnorm_plan(rows, r, c->sm_count, &chunks, &per);
-  ChainPtrs Qs, ds;
-  for (int b = 0; b < s.nb; ++b) { Qs.p[b] = list[b]->Q; ds.p[b] = list[b]->colnorm_out; }
-  dim3 grid((unsigned)((r + 127) / 128), (unsigned)chunks, (unsigned)s.nb);
-  launch_pdl(k_colsumsq_partial, grid, dim3(128), 0, s.st, (const float*)(s.ws + s.L.R), r, rows, r, per, s.ws + s.L.cn_part,
-             (const int*)nullptr, s.wstride);
-  DION_CHECK_LAUNCH(c);
-  launch_pdl(k_colnorm_apply, grid, dim3(128), 0, s.st, (const float*)(s.ws + s.L.R), r, rows, r, per, chunks,
-             (const float*)(s.ws + s.L.cn_part), c->cfg.eps, (float*)nullptr, list[0]->ldq, s.ws + s.L.d, (float*)nullptr, c->dev_ints,
-             (const int*)(s.os + OS_FAIL), s.wstride, Qs, ds);
-  DION_CHECK_LAUNCH(c);
   return DION_OK;
 }
 
@@ -1249,6 +1271,21 @@ int split_chain(StepCtx& s, const float* const* src, const i64* ld, i64 rows, i6
     __nv_bfloat16* hi = reinterpret_cast<__nv_bfloat16*>(s.W(b, out_off));
     launch_pdl(k_split_bf16, dim3(gx), dim3(256), 0, s.st, src[b], ld[b], rows, cols, hi, hi + rows * cols,
                skip0 != nullptr ? skip0 + (i64)b * OS_SLOT_INTS : (const int*)nullptr);
+    DION_CHECK_LAUNCH(c);
+  }
+  return DION_OK;
+}
+
+// ... as a half pair scaled by 2^bits.
+int split_half_chain(StepCtx& s, const float* const* src, i64 ld, i64 rows, i64 cols, i64 out_off, int bits, const int* skip0) {
+  dion_ctx* c = s.c;
+  const int per = (s.nb <= GEMM_TAB_MAX && c->chain_batch) ? s.nb : 1;
+  for (int b = 0; b < s.nb; b += per) {
+    ChainPtrs t;
+    for (int k = 0; k < per; ++k) t.p[k] = src[b + k];
+    __half* hi = reinterpret_cast<__half*>(s.W(b, out_off));
+    launch_pdl(k_split_f16_fixed, dim3((unsigned)grid_for(c, rows * cols / 8, per), (unsigned)per), dim3(256), 0, s.st, t, ld, rows, cols, ldexpf(1.f, bits),
+               hi, hi + rows * cols, s.wstride, (i64)0, skip0 != nullptr ? skip0 + (i64)b * OS_SLOT_INTS : (const int*)nullptr, (i64)OS_SLOT_INTS);
     DION_CHECK_LAUNCH(c);
   }
   return DION_OK;
@@ -1354,6 +1391,53 @@ int begin_step(dion_ctx* c, const dion_matrix* a, int nb, cudaStream_t st, StepC
 // three); it is accurate to ~1e-5, which is what Q <- ColNorm(R) and the error feedback need of it.
 bool r_on_pairs(const StepCtx& s, i64 m, i64 n, i64 r) {
   return s.tensor && s.c->cfg.precision == DION_PREC_FP32 && s.L.B32 > 0 && s.L.Bp > 0 && m >= 128 && n >= 128 && r >= 64;
+}
+
+// The steps whose four products run on scaled half pairs (k_form_sum_amax): CholeskyQR2 panels between the smallest
+// product that pays for the second pass over M + G and the size from which P runs on the bf16 pairs that one pass makes.
+// M + G is read once more (from L2 where it fits), but P leaves the 3xTF32 form, whose converter warps bound it, for three
+// half MMAs per K step, U's pair also serves the weight update, and every result carries 22 bits (768^2 to 768 x 3072 at
+// r = 192, 72 matrices in one call: P 932 -> 516 us, R 420 -> 194 us with the unsplit chains, weight update 200 -> 173 us;
+// errors of Q and M 2 to 5 times smaller).  From P_PAIR_MIN_MNR on the second pass would be over HBM.
+// The rule looks at the shape alone, so that a grouped call computes what single calls compute.
+bool step_on_half_pairs(const StepCtx& s, i64 m, i64 n, i64 r, i64 short_dim) {
+  const i64 mnr = m * n * r;
+  return r_on_pairs(s, m, n, r) && s.L.Bh == 0 && mnr >= HALF_PAIR_MIN_MNR && (double)mnr < P_PAIR_MIN_MNR &&
+         resolve_orth_for(s.c, r, short_dim, s.list != nullptr) == DION_ORTH_CHOLQR2;
+}
+
+// M + G and the half pairs of it and of Q (in S16) for every matrix of the chain: in one pair of launches when they share
+// leading dimensions and alignment.
+int half_sum_chain(StepCtx& s, const dion_matrix* const* list, i64 qrow) {
+  dion_ctx* c = s.c;
+  const dion_matrix* a0 = list[0];
+  const i64 m = a0->m, n = a0->n, r = a0->r;
+  auto vec_ok = [](const dion_matrix* a) {
+    return !((uintptr_t)a->M & 15) && a->ldm % 4 == 0 &&
+           (a->g_dtype == DION_BF16 ? (!((uintptr_t)a->G & 7) && a->ldg % 4 == 0) : (!((uintptr_t)a->G & 15) && a->ldg % 4 == 0));
+  };
+  auto qvec_ok = [](const dion_matrix* a) { return !((uintptr_t)a->Q & 15) && a->ldq % 4 == 0; };
+  bool one = s.nb <= GEMM_TAB_MAX && (s.nb == 1 || c->chain_batch);
+  for (int b = 1; b < s.nb && one; ++b)
+    one = list[b]->ldm == a0->ldm && list[b]->ldg == a0->ldg && list[b]->g_dtype == a0->g_dtype && vec_ok(list[b]) == vec_ok(a0) &&
+          list[b]->ldq == a0->ldq && qvec_ok(list[b]) == qvec_ok(a0);
+  const int per = one ? s.nb : 1;
+  for (int b = 0; b < s.nb; b += per) {
+    const dion_matrix* a = list[b];
+    ChainPtrs Ms, Gs, Qs;
+    for (int k = 0; k < per; ++k) { Ms.p[k] = list[b + k]->M; Gs.p[k] = list[b + k]->G; Qs.p[k] = list[b + k]->Q; }
+    const int g_mode = (a->g_dtype == DION_BF16) ? ADD_BF16 : ADD_F32;
+    const dim3 fg((unsigned)grid_for(c, m * n / 4, per), (unsigned)per), sg((unsigned)grid_for(c, (m * n + qrow * r) / 8, per), (unsigned)per);
+    float* part = s.W(b, s.L.part);      // (the maxima are read before the products write their partial sums there)
+    const int qv = qvec_ok(a) ? 1 : 0;
+    if (vec_ok(a)) launch_pdl(k_form_sum_amax<true>, fg, dim3(256), 0, s.st, Ms, a->ldm, Gs, a->ldg, g_mode, m, n, Qs, a->ldq, qrow, r, qv, s.W(b, s.L.B32), part, s.wstride);
+    else launch_pdl(k_form_sum_amax<false>, fg, dim3(256), 0, s.st, Ms, a->ldm, Gs, a->ldg, g_mode, m, n, Qs, a->ldq, qrow, r, qv, s.W(b, s.L.B32), part, s.wstride);
+    DION_CHECK_LAUNCH(c);
+    launch_pdl(k_split_sum, sg, dim3(256), 0, s.st, (const float*)s.W(b, s.L.B32), m * n, Qs, a->ldq, qrow, r, qv, (const float*)part, (int)fg.x,
+               reinterpret_cast<__half*>(s.W(b, s.L.Bp)), reinterpret_cast<__half*>(s.W(b, s.L.S16)), s.W(b, s.L.lz), s.wstride);
+    DION_CHECK_LAUNCH(c);
+  }
+  return DION_OK;
 }
 
 // Forms M + G in scratch (fp32) and, when `pair`, as a bf16 pair beside it.
@@ -1499,13 +1583,15 @@ int ef_update(StepCtx& s, int b, const dion_matrix* a, const float* F1, i64 ld1,
 
 int x_update(StepCtx& s, int b, const dion_matrix* a, const float* F1, i64 ld1, const float* F2, i64 ld2, float* r1,
              float* r2, float alpha, const int* skip, const float* alpha_dev = nullptr, GemmArgs* defer = nullptr,
-             bool rounded = false) {   // rounded: r1 and r2 already hold the rounded factors
+             bool rounded = false, float s1 = 0.f, float s2 = 0.f) {   // rounded: r1 and r2 already hold the rounded factors,
+                                                                       // half arrays by the scales s1, s2 (0: half_scale's)
   dion_ctx* c = s.c;
   const i64 m = a->m, n = a->n, r = a->r;
   GemmArgs x = gemm_args();
   x.M = m; x.N = n; x.K = r;
   if (x_single_pass(s, a, F1, ld1, F2, ld2) && x_half(a)) {
-    const float s1 = half_scale(m), s2 = half_scale(n);
+    if (s1 == 0.f) s1 = half_scale(m);
+    if (s2 == 0.f) s2 = half_scale(n);
     if (!rounded) {
       launch_pdl(k_round_f16, dim3((unsigned)grid_for(c, m * r / 8)), dim3(256), 0, s.st, F1, ld1, m, r, s1, reinterpret_cast<__half*>(r1), skip);
       DION_CHECK_LAUNCH(c);
@@ -1590,6 +1676,7 @@ int step_batch(dion_ctx* c, const dion_matrix* const* list, int nb, float lr, cu
   const bool ppair = bpair && (double)m * (double)n * (double)r >= P_PAIR_MIN_MNR &&
                      resolve_orth_for(c, r, (m < n) ? m : n, s.list != nullptr) == DION_ORTH_CHOLQR2;
   bool any_pair = false;
+  const bool hstep = step_on_half_pairs(s, m, n, r, (m < n) ? m : n);
 
   // the large products: one GemmArgs per matrix, then one launch over the chain where that is possible
   std::vector<GemmArgs> group((size_t)nb);
@@ -1602,7 +1689,8 @@ int step_batch(dion_ctx* c, const dion_matrix* const* list, int nb, float lr, cu
   // elementwise preparation for the whole chain: M + G (and its pair), the pair of Q where P takes pairs
   const float* srcs[MAX_CHAIN];
   i64 lds[MAX_CHAIN];
-  if (b32) DION_TRY(form_sum_chain(s, list, bpair));
+  if (hstep) DION_TRY(half_sum_chain(s, list, qrow));
+  else if (b32) DION_TRY(form_sum_chain(s, list, bpair));
   const bool phalf = b32 && s.L.Bh > 0;
   bool p_half_ready = false;
   if (phalf) {      // the scaled half pairs of M + G and of Q, for the whole chain
@@ -1644,7 +1732,7 @@ int step_batch(dion_ctx* c, const dion_matrix* const* list, int nb, float lr, cu
   // error feedback) let one launch take the whole chain: 84 matrices of up to 768 x 3072 at r = 192 went through 147
   // launches of a few tiles each, 1670 us.
   bool q_dense = false;
-  if (nb > 1 && nb <= GEMM_TAB_MAX && c->chain_batch && b32 && !ppair && !p_half_ready && r % 4 == 0) {
+  if (nb > 1 && nb <= GEMM_TAB_MAX && c->chain_batch && b32 && !ppair && !hstep && !p_half_ready && r % 4 == 0) {
     bool all_ok = true;
     for (int b = 0; b < nb; ++b) {
       all_ok = all_ok && !((uintptr_t)list[b]->Q & 15) && list[b]->ldq == list[0]->ldq && list[b]->ldq % 4 == 0;
@@ -1687,6 +1775,13 @@ int step_batch(dion_ctx* c, const dion_matrix* const* list, int nb, float lr, cu
       p.A = (const float*)bh; p.A16lo = bh + m * n; p.a_si = tr ? 1 : n; p.a_sk = tr ? n : 1;
       p.B = (const float*)qh; p.B16lo = ql; p.b_sk = r; p.b_sn = 1;
       any_pair = true;
+    } else if (hstep) {
+      __half* bh = reinterpret_cast<__half*>(s.W(b, s.L.Bp));
+      __half* qh = reinterpret_cast<__half*>(s.W(b, s.L.S16));
+      p.ab16 = 1; p.f16 = 1;
+      p.A = (const float*)bh; p.A16lo = bh + m * n; p.a_si = tr ? 1 : n; p.a_sk = tr ? n : 1;
+      p.B = (const float*)qh; p.B16lo = qh + qrow * r; p.b_sk = r; p.b_sn = 1;
+      p.alpha_dev = s.W(b, s.L.lz) + HS_P;
     } else if (p_half_ready) {
       __half* bh = reinterpret_cast<__half*>(s.W(b, s.L.Bh));
       __half* qh = reinterpret_cast<__half*>(s.W(b, s.L.S16));
@@ -1742,11 +1837,12 @@ int step_batch(dion_ctx* c, const dion_matrix* const* list, int nb, float lr, cu
   {
   PhaseScope ps(c, st, DION_PHASE_R);
   const i64 other_off = (U_off == s.L.P0) ? s.L.P1 : s.L.P0;
-  if (!d16 && bpair) {   // U as a bf16 pair in the other panel buffer, for the whole chain
+  if (!d16 && bpair) {   // U as a pair in the other panel buffer, for the whole chain
     const float* srcs[MAX_CHAIN];
     i64 lds[MAX_CHAIN];
     for (int b = 0; b < nb; ++b) { srcs[b] = s.W(b, U_off); lds[b] = r; }
-    DION_TRY(split_chain(s, srcs, lds, prow, r, other_off, s.os + OS_FAIL));
+    if (hstep) DION_TRY(split_half_chain(s, srcs, r, prow, r, other_off, HS_U_BITS, s.os + OS_FAIL));
+    else DION_TRY(split_chain(s, srcs, lds, prow, r, other_off, s.os + OS_FAIL));
   }
   for (int b = 0; b < nb; ++b) {
     const dion_matrix* a = list[b];
@@ -1760,6 +1856,7 @@ int step_batch(dion_ctx* c, const dion_matrix* const* list, int nb, float lr, cu
     } else if (bpair) {
       // U as a bf16 pair in the other panel buffer (the error feedback reuses it)
       DION_TRY(r_pairs(s, b, a, tr, s.W(b, U_off), s.W(b, other_off), s.W(b, s.L.R), s.OS(b) + OS_FAIL, &group[b], true));
+      if (hstep) { group[b].f16 = 1; group[b].alpha_dev = s.W(b, s.L.lz) + HS_R; }      // (the same place and layout)
       continue;
     } else if (b32) {
       w.A = s.W(b, s.L.B32); w.a_si = tr ? n : 1; w.a_sk = tr ? 1 : n;
@@ -1773,6 +1870,29 @@ int step_batch(dion_ctx* c, const dion_matrix* const* list, int nb, float lr, cu
     group[b] = w;
   }
   DION_TRY(launch_gemm_group(s, group));
+  }
+
+  // Q <- ColNorm(R), and in the same pass the operands of the two rank-r updates that R and Q become (wherever every matrix of
+  // the chain takes them in that form): R's pair in S16, Q rounded in the save buffer of the panel, which nothing reads any more.
+  int cn_kind = 0;
+  {
+  PhaseScope ps(c, st, DION_PHASE_COLNORM);
+  if (d16) {
+    cn_kind = CN_ONE;
+  } else if (hstep) {
+    cn_kind = CN_HALF;
+  } else if (s.L.Psave > 0 && x_half(a0)) {
+    bool all = true;
+    for (int b = 0; b < nb; ++b) {
+      const dion_matrix* a = list[b];
+      const float* sum32 = b32 ? s.W(b, s.L.B32) : nullptr;
+      const float *Rf = s.W(b, s.L.R), *Uf = s.W(b, U_off), *Qf = (const float*)a->Q;
+      all = all && (tr ? ef_on_pairs(s, a, Rf, r, Uf, r, sum32) && x_single_pass(s, a, Qf, a->ldq, Uf, r)
+                       : ef_on_pairs(s, a, Uf, r, Rf, r, sum32) && x_single_pass(s, a, Uf, r, Qf, a->ldq));
+    }
+    if (all) cn_kind = CN_BF16;
+  }
+  DION_TRY(colnorm_chain(s, list, qrow, r, cn_kind, cn_kind == CN_ONE ? s.L.Q16 : s.L.Psave, half_scale(qrow), cn_kind == CN_ONE ? s.L.R16 : s.L.S16));
   }
 
   // M <- (M + G) - (1 - mu) U R^T   (transposed form: R U^T)
@@ -1789,9 +1909,9 @@ int step_batch(dion_ctx* c, const dion_matrix* const* list, int nb, float lr, cu
       all_pairs = all_pairs && (tr ? ef_on_pairs(s, list[b], s.W(b, s.L.R), r, s.W(b, U_off), r, sum32)
                                    : ef_on_pairs(s, list[b], s.W(b, U_off), r, s.W(b, s.L.R), r, sum32));
     }
-    if (all_pairs) {
+    if (all_pairs || cn_kind != 0) {
       for (int b = 0; b < nb; ++b) { srcs[b] = s.W(b, s.L.R); lds[b] = r; }
-      DION_TRY(split_chain(s, srcs, lds, qrow, r, s.L.S16, s.os + OS_FAIL));
+      if (cn_kind == 0) DION_TRY(split_chain(s, srcs, lds, qrow, r, s.L.S16, s.os + OS_FAIL));
       if (!bpair) {
         for (int b = 0; b < nb; ++b) srcs[b] = s.W(b, U_off);
         DION_TRY(split_chain(s, srcs, lds, prow, r, other_off, s.os + OS_FAIL));
@@ -1804,7 +1924,6 @@ int step_batch(dion_ctx* c, const dion_matrix* const* list, int nb, float lr, cu
     if (d16) {
       GemmArgs e = gemm_args();
       e.M = m; e.N = n; e.K = r;
-      DION_TRY(to_bf16(s.W(b, s.L.R), r, qrow, r, bf(b, s.L.R16)));
       e.ab16 = 1;
       e.A = (const float*)bf(b, tr ? s.L.R16 : s.L.U16); e.a_si = r; e.a_sk = 1;
       e.B = (const float*)bf(b, tr ? s.L.U16 : s.L.R16); e.b_sk = 1; e.b_sn = r;
@@ -1823,14 +1942,9 @@ int step_batch(dion_ctx* c, const dion_matrix* const* list, int nb, float lr, cu
     const float* sum32 = b32 ? s.W(b, s.L.B32) : nullptr;
     if (tr) DION_TRY(ef_update(s, b, a, Rf, r, Uf, r, sbuf, other, sum32, s.OS(b) + OS_FAIL, ef_split, bpair || ef_split, &group[b]));
     else DION_TRY(ef_update(s, b, a, Uf, r, Rf, r, other, sbuf, sum32, s.OS(b) + OS_FAIL, bpair || ef_split, ef_split, &group[b]));
+    if (hstep && group[b].ab16) { group[b].f16 = 1; group[b].alpha_dev = s.W(b, s.L.lz) + HS_EF; }
   }
   DION_TRY(launch_gemm_group(s, group));
-  }
-
-  // Q <- ColNorm(R)
-  {
-  PhaseScope ps(c, st, DION_PHASE_COLNORM);
-  DION_TRY(colnorm_chain(s, list, qrow, r));
   }
 
   // X <- X - lr sqrt(m/n) U Q^T   (transposed form: Q U^T)
@@ -1838,6 +1952,7 @@ int step_batch(dion_ctx* c, const dion_matrix* const* list, int nb, float lr, cu
   PhaseScope ps(c, st, DION_PHASE_X);
   const float x_alpha = (x_scale != nullptr) ? 1.f : lr * sqrtf((float)((double)m / (double)n));
   const i64 other_off = (U_off == s.L.P0) ? s.L.P1 : s.L.P0;
+  float u_half = 0.f;         // scale of U's half array when it is not half_scale's
   bool x_rounded = false;     // the rounded factors are made for the whole chain when every matrix takes the single pass
   if (!d16) {
     const float* srcs[MAX_CHAIN];
@@ -1851,9 +1966,12 @@ int step_batch(dion_ctx* c, const dion_matrix* const* list, int nb, float lr, cu
     if (all_one) {
       for (int b = 0; b < nb; ++b) { srcs[b] = s.W(b, U_off); lds[b] = r; }
       const bool half = x_half(a0);
-      DION_TRY(round_chain(s, srcs, lds, prow, r, other_off, s.os + OS_FAIL, half ? half_scale(prow) : 0.f));
-      for (int b = 0; b < nb; ++b) { srcs[b] = (const float*)list[b]->Q; lds[b] = list[b]->ldq; }
-      DION_TRY(round_chain(s, srcs, lds, qrow, r, s.L.R, s.os + OS_FAIL, half ? half_scale(qrow) : 0.f));
+      if (hstep && half) u_half = ldexpf(1.f, HS_U_BITS);      // the hi part of U's pair is that rounding
+      else DION_TRY(round_chain(s, srcs, lds, prow, r, other_off, s.os + OS_FAIL, half ? half_scale(prow) : 0.f));
+      if (cn_kind == 0) {
+        for (int b = 0; b < nb; ++b) { srcs[b] = (const float*)list[b]->Q; lds[b] = list[b]->ldq; }
+        DION_TRY(round_chain(s, srcs, lds, qrow, r, s.L.R, s.os + OS_FAIL, half ? half_scale(qrow) : 0.f));
+      }
       x_rounded = true;
     }
   }
@@ -1862,7 +1980,6 @@ int step_batch(dion_ctx* c, const dion_matrix* const* list, int nb, float lr, cu
     if (d16) {
       GemmArgs x = gemm_args();
       x.M = m; x.N = n; x.K = r;
-      DION_TRY(to_bf16((const float*)a->Q, a->ldq, qrow, r, bf(b, s.L.Q16)));
       x.ab16 = 1;
       x.A = (const float*)bf(b, tr ? s.L.Q16 : s.L.U16); x.a_si = r; x.a_sk = 1;
       x.B = (const float*)bf(b, tr ? s.L.U16 : s.L.Q16); x.b_sk = 1; x.b_sn = r;
@@ -1872,13 +1989,13 @@ int step_batch(dion_ctx* c, const dion_matrix* const* list, int nb, float lr, cu
       group[b] = x;
       continue;
     }
-    // the rounded copies of the single-pass form go to the other panel buffer and to R's, both free by now
+    // the rounded copies of the single-pass form: in the other panel buffer, and where the normalization put Q's or in R's (free)
     float* other = s.W(b, U_off == s.L.P0 ? s.L.P1 : s.L.P0);
-    float* rbuf = s.W(b, s.L.R);
+    float* rbuf = s.W(b, cn_kind != 0 && x_rounded ? s.L.Psave : s.L.R);
     const float* Uf = s.W(b, U_off);
     const float* Qf = (const float*)a->Q;
-    if (tr) DION_TRY(x_update(s, b, a, Qf, a->ldq, Uf, r, rbuf, other, x_alpha, s.OS(b) + OS_FAIL, x_scale, &group[b], x_rounded));
-    else DION_TRY(x_update(s, b, a, Uf, r, Qf, a->ldq, other, rbuf, x_alpha, s.OS(b) + OS_FAIL, x_scale, &group[b], x_rounded));
+    if (tr) DION_TRY(x_update(s, b, a, Qf, a->ldq, Uf, r, rbuf, other, x_alpha, s.OS(b) + OS_FAIL, x_scale, &group[b], x_rounded, 0.f, u_half));
+    else DION_TRY(x_update(s, b, a, Uf, r, Qf, a->ldq, other, rbuf, x_alpha, s.OS(b) + OS_FAIL, x_scale, &group[b], x_rounded, u_half, 0.f));
   }
   DION_TRY(launch_gemm_group(s, group));
   launch_pdl(k_finish_step, dim3((unsigned)(nb)), dim3(1), 0, st, s.flag, c->dev_ints + 1);
@@ -2370,6 +2487,47 @@ GemmArgs dp_b_product(const dion_matrix* a, bool transposed_b, const float* rhs,
   return g;
 }
 
+// The pieces of a step on half pairs (step_on_half_pairs) as calls of their own.  P = (M + G) Q:
+int half_project(StepCtx& s, const dion_matrix* a, float* P) {
+  const i64 m = a->m, n = a->n, r = a->r;
+  DION_TRY(half_sum_chain(s, &a, n));
+  const __half* bh = reinterpret_cast<const __half*>(s.ws + s.L.Bp);
+  const __half* qh = reinterpret_cast<const __half*>(s.ws + s.L.S16);
+  GemmArgs p = gemm_args();
+  p.M = m; p.N = r; p.K = n;
+  p.ab16 = 1; p.f16 = 1;
+  p.A = (const float*)bh; p.A16lo = bh + m * n; p.a_si = n; p.a_sk = 1;
+  p.B = (const float*)qh; p.B16lo = qh + n * r; p.b_sk = r; p.b_sn = 1;
+  p.alpha_dev = s.ws + s.L.lz + HS_P;
+  p.C = P; p.ldc = r; p.epi = EPI_STORE;
+  return launch_gemm(s, p, 0);
+}
+// W = (M + G)^T U:
+int half_factor(StepCtx& s, const dion_matrix* a, const float* U, float* W, const int* skip) {
+  const i64 m = a->m, r = a->r;
+  DION_TRY(half_sum_chain(s, &a, 0));
+  DION_TRY(split_half_chain(s, &U, r, m, r, s.L.P1, HS_U_BITS, skip));
+  GemmArgs w;
+  DION_TRY(r_pairs(s, 0, a, false, U, s.ws + s.L.P1, W, skip, &w, true));
+  w.f16 = 1; w.alpha_dev = s.ws + s.L.lz + HS_R;
+  return launch_gemm(s, w, 0);
+}
+// The error feedback, Q and the weight update (sums: see colnorm_launch; alpha: the update's factor):
+int half_finish(StepCtx& s, const dion_matrix* a, const float* U, const float* W, const float* sums, float alpha, const int* flag) {
+  const i64 m = a->m, n = a->n, r = a->r;
+  DION_TRY(split_half_chain(s, &U, r, m, r, s.L.P1, HS_U_BITS, flag));
+  ColnormPairs x = ColnormPairs();
+  x.kind = CN_HALF; x.qh = s.ws + s.L.P0; x.qscale = half_scale(n); x.hi = s.ws + s.L.S16;
+  DION_TRY(colnorm(s, 0, W, n, r, (float*)a->Q, a->ldq, a->colnorm_out, flag, x, sums));
+  GemmArgs e;
+  DION_TRY(ef_update(s, 0, a, U, r, W, r, s.ws + s.L.P1, s.ws + s.L.S16, nullptr, flag, true, true, &e));
+  if (e.ab16) { e.f16 = 1; e.alpha_dev = s.ws + s.L.lz + HS_EF; }
+  DION_TRY(launch_gemm(s, e, 0));
+  const bool rounded = x_single_pass(s, a, U, r, (const float*)a->Q, a->ldq) && x_half(a);
+  return x_update(s, 0, a, U, r, (const float*)a->Q, a->ldq, s.ws + s.L.P1, s.ws + s.L.P0, alpha, flag, nullptr, nullptr, rounded,
+                  rounded ? ldexpf(1.f, HS_U_BITS) : 0.f, 0.f);
+}
+
 }  // namespace
 
 int dion_dp_project(dion_ctx* ctx, const dion_matrix* a, float* P, int* dp_flag, void* cuda_stream) {
@@ -2378,6 +2536,7 @@ int dion_dp_project(dion_ctx* ctx, const dion_matrix* a, float* P, int* dp_flag,
   cudaStream_t st = (cudaStream_t)cuda_stream;
   DION_TRY(begin_step(ctx, a, 1, st, &s));
   if (cudaMemsetAsync(dp_flag, 0, sizeof(int), st) != cudaSuccess) return DION_ERR_CUDA;
+  if (step_on_half_pairs(s, a->m, a->n, a->r, (a->m < a->n) ? a->m : a->n)) return half_project(s, a, P);
   GemmArgs p = dp_b_product(a, false, (const float*)a->Q, P);
   p.b_sk = a->ldq;
   p.precise = (resolve_orth(ctx, a->r, (a->m < a->n) ? a->m : a->n) == DION_ORTH_SHIFTED3) ? 1 : 0;
@@ -2404,6 +2563,7 @@ int dion_dp_factor(dion_ctx* ctx, const dion_matrix* a, float* PU, float* W, int
   DION_CHECK_LAUNCH(ctx);
   launch_pdl(k_latch_flag, dim3((unsigned)(1)), dim3(1), 0, st, s.flag, dp_flag);      // a breakdown cancels dion_dp_finish
   DION_CHECK_LAUNCH(ctx);
+  if (step_on_half_pairs(s, m, n, r, (m < n) ? m : n)) return half_factor(s, a, PU, W, nullptr);
   if (r_on_pairs(s, m, n, r)) {       // as dion_step: W on the bf16 pairs of M + G and U
     DION_TRY(form_sum(s, 0, a, true));
     return r_pairs(s, 0, a, false, PU, s.ws + s.L.P1, W, nullptr);
@@ -2418,12 +2578,16 @@ int dion_dp_finish(dion_ctx* ctx, const dion_matrix* a, const float* U, const fl
   cudaStream_t st = (cudaStream_t)cuda_stream;
   DION_TRY(begin_step(ctx, a, 1, st, &s));
   const i64 m = a->m, n = a->n, r = a->r;
-  // M <- (M + G) - (1 - mu) U W^T, with this rank's M and G (as in dion_step)
-  DION_TRY(ef_update(s, 0, a, U, r, W, r, s.ws + s.L.P1, s.ws + s.L.S16, nullptr, dp_flag));
-  DION_TRY(colnorm(s, 0, W, n, r, (float*)a->Q, a->ldq, a->colnorm_out, dp_flag));
-  // X <- X - lr sqrt(m/n) U Q^T, as in dion_step (rounded copies in the two panel buffers of the scratch)
-  DION_TRY(x_update(s, 0, a, U, r, (const float*)a->Q, a->ldq, s.ws + s.L.P1, s.ws + s.L.R,
-                    lr * sqrtf((float)((double)m / (double)n)), dp_flag));
+  const float alpha = lr * sqrtf((float)((double)m / (double)n));
+  if (step_on_half_pairs(s, m, n, r, (m < n) ? m : n)) {
+    DION_TRY(half_finish(s, a, U, W, nullptr, alpha, dp_flag));
+  } else {
+    // M <- (M + G) - (1 - mu) U W^T, with this rank's M and G (as in dion_step)
+    DION_TRY(ef_update(s, 0, a, U, r, W, r, s.ws + s.L.P1, s.ws + s.L.S16, nullptr, dp_flag));
+    DION_TRY(colnorm(s, 0, W, n, r, (float*)a->Q, a->ldq, a->colnorm_out, dp_flag));
+    // X <- X - lr sqrt(m/n) U Q^T, as in dion_step (rounded copies in the two panel buffers of the scratch)
+    DION_TRY(x_update(s, 0, a, U, r, (const float*)a->Q, a->ldq, s.ws + s.L.P1, s.ws + s.L.R, alpha, dp_flag));
+  }
   launch_pdl(k_finish_step, dim3((unsigned)(1)), dim3(1), 0, st, dp_flag, ctx->dev_ints + 1);
   DION_CHECK_LAUNCH(ctx);
   return DION_OK;
@@ -2450,6 +2614,7 @@ int dion_shard_project(dion_ctx* ctx, const dion_matrix* a, int64_t n_total, flo
   cudaStream_t st = (cudaStream_t)cuda_stream;
   DION_TRY(begin_step(ctx, a, 1, st, &s));
   if (cudaMemsetAsync(flag, 0, sizeof(int), st) != cudaSuccess) return DION_ERR_CUDA;
+  if (step_on_half_pairs(s, a->m, a->n, a->r, (a->m < n_total) ? a->m : n_total)) return half_project(s, a, P);
   GemmArgs p = dp_b_product(a, false, (const float*)a->Q, P);
   p.b_sk = a->ldq;
   p.precise = (resolve_orth(ctx, a->r, (a->m < n_total) ? a->m : n_total) == DION_ORTH_SHIFTED3) ? 1 : 0;
@@ -2493,7 +2658,9 @@ int dion_shard_factor(dion_ctx* ctx, const dion_matrix* a, int64_t n_total, cons
   StepCtx s;
   cudaStream_t st = (cudaStream_t)cuda_stream;
   DION_TRY(begin_step(ctx, a, 1, st, &s));
-  if (r_on_pairs(s, a->m, a->n, a->r)) {       // as dion_step: W on the bf16 pairs of M + G and U
+  if (step_on_half_pairs(s, a->m, a->n, a->r, (a->m < n_total) ? a->m : n_total)) {
+    DION_TRY(half_factor(s, a, U, W, flag));
+  } else if (r_on_pairs(s, a->m, a->n, a->r)) {       // as dion_step: W on the bf16 pairs of M + G and U
     DION_TRY(form_sum(s, 0, a, true));
     DION_TRY(r_pairs(s, 0, a, false, U, s.ws + s.L.P1, W, flag));
   } else {
@@ -2504,10 +2671,16 @@ int dion_shard_factor(dion_ctx* ctx, const dion_matrix* a, int64_t n_total, cons
   int chunks; i64 per;
   colnorm_plan(a->n, a->r, ctx->sm_count, &chunks, &per);
   float* part = s.W(0, s.L.cn_part);
-  dim3 grid((unsigned)((a->r + 127) / 128), (unsigned)chunks);
-  launch_pdl(k_colsumsq_partial, grid, dim3(128), 0, st, (const float*)W, a->r, a->n, a->r, per, part, (const int*)flag, (i64)0);
-  DION_CHECK_LAUNCH(ctx);
-  launch_pdl(k_colsumsq_finish, dim3((unsigned)((a->r + 127) / 128)), dim3(128), 0, st, (const float*)part, chunks, a->r, colsumsq, flag);
+  const dim3 grid((unsigned)((a->r + 127) / 128), (unsigned)chunks);
+  if (a->r % 4 == 0) {
+    launch_pdl(k_colsumsq_partial<true>, grid, dim3(CN_THREADS), 0, st, (const float*)W, a->r, a->n, a->r, per, part, (float*)nullptr, flag, (i64)0);
+    DION_CHECK_LAUNCH(ctx);
+    launch_pdl(k_colsumsq_finish<true>, dim3(grid.x), dim3(CN_THREADS), 0, st, (const float*)part, chunks, a->r, colsumsq, flag);
+  } else {
+    launch_pdl(k_colsumsq_partial<false>, grid, dim3(CN_THREADS), 0, st, (const float*)W, a->r, a->n, a->r, per, part, (float*)nullptr, flag, (i64)0);
+    DION_CHECK_LAUNCH(ctx);
+    launch_pdl(k_colsumsq_finish<false>, dim3(grid.x), dim3(CN_THREADS), 0, st, (const float*)part, chunks, a->r, colsumsq, flag);
+  }
   DION_CHECK_LAUNCH(ctx);
   return DION_OK;
 }
@@ -2520,19 +2693,16 @@ int dion_shard_finish(dion_ctx* ctx, const dion_matrix* a, int64_t n_total, cons
   cudaStream_t st = (cudaStream_t)cuda_stream;
   DION_TRY(begin_step(ctx, a, 1, st, &s));
   const i64 m = a->m, n = a->n, r = a->r;
-  // M <- (M + G) - (1 - mu) U W^T on the shard's columns
-  DION_TRY(ef_update(s, 0, a, U, r, W, r, s.ws + s.L.P1, s.ws + s.L.S16, nullptr, flag));
-  {   // Q <- W / (sqrt(colsumsq) + eps): the squared column norms are the all-reduced ones (one "chunk")
-    int chunks; i64 per;
-    colnorm_plan(n, r, ctx->sm_count, &chunks, &per);
-    dim3 grid((unsigned)((r + 127) / 128), (unsigned)chunks);
-    launch_pdl(k_colnorm_apply, grid, dim3(128), 0, st, W, r, n, r, per, 1, colsumsq, ctx->cfg.eps, (float*)a->Q, a->ldq,
-               s.W(0, s.L.d), a->colnorm_out, ctx->dev_ints, (const int*)flag, (i64)0, ChainPtrs(), ChainPtrs());
-    DION_CHECK_LAUNCH(ctx);
+  const float alpha = lr * sqrtf((float)((double)m / (double)n_total));
+  if (step_on_half_pairs(s, m, n, r, (m < n_total) ? m : n_total)) {
+    DION_TRY(half_finish(s, a, U, W, colsumsq, alpha, flag));
+  } else {
+    // M <- (M + G) - (1 - mu) U W^T on the shard's columns; Q <- W / (sqrt(colsumsq) + eps) with the all-reduced squared norms
+    DION_TRY(ef_update(s, 0, a, U, r, W, r, s.ws + s.L.P1, s.ws + s.L.S16, nullptr, flag));
+    DION_TRY(colnorm(s, 0, W, n, r, (float*)a->Q, a->ldq, a->colnorm_out, flag, ColnormPairs(), colsumsq));
+    // X <- X - lr sqrt(m / n_total) U Q^T on the shard's columns
+    DION_TRY(x_update(s, 0, a, U, r, (const float*)a->Q, a->ldq, s.ws + s.L.P1, s.ws + s.L.R, alpha, flag));
   }
-  // X <- X - lr sqrt(m / n_total) U Q^T on the shard's columns
-  DION_TRY(x_update(s, 0, a, U, r, (const float*)a->Q, a->ldq, s.ws + s.L.P1, s.ws + s.L.R,
-                    lr * sqrtf((float)((double)m / (double)n_total)), flag));
   launch_pdl(k_finish_step, dim3(1), dim3(1), 0, st, flag, ctx->dev_ints + 1);
   DION_CHECK_LAUNCH(ctx);
   return DION_OK;
@@ -2681,7 +2851,8 @@ bool preload_kernels() {
   ok = ok && touch_kernel(k_chol_flow<false>) && touch_kernel(k_round_end) && touch_kernel(k_tiny_cholqr2);
   ok = ok && touch_kernel(k_probe_y) && touch_kernel(k_probe_y4) && touch_kernel(k_probe_w) && touch_kernel(k_probe_w4) && touch_kernel(k_probe_decide) && touch_kernel(k_reset_rounds);
   ok = ok && touch_kernel(k_orth_finish) && touch_kernel(k_cgs_fallback) && touch_kernel(k_copy_block);
-  ok = ok && touch_kernel(k_colsumsq_partial) && touch_kernel(k_colnorm_apply) && touch_kernel(k_copy_panel);
+  ok = ok && touch_kernel(k_colsumsq_partial<true>) && touch_kernel(k_colsumsq_partial<false>) &&
+       touch_kernel(k_colnorm_apply<true>) && touch_kernel(k_colnorm_apply<false>) && touch_kernel(k_copy_panel);
   ok = ok && touch_kernel(k_latch_flag) && touch_kernel(k_finish_step) && touch_kernel(k_hh_reflector);
   ok = ok && touch_kernel(k_hh_apply) && touch_kernel(k_set_identity) && touch_kernel(k_sign_fix);
   ok = ok && touch_kernel(k_form_b16<true>) && touch_kernel(k_form_b16<false>) && touch_kernel(k_form_b32<true>);

@@ -949,75 +949,6 @@ __global__ void k_copy_block(const float* __restrict__ src, i64 lds, float* __re
   }
 }
 
-// Partial sums of squares per column: part[chunk][j] = sum over the chunk's rows of R[i][j]^2.
-// grid = (ceil(r/128), chunks); 128 threads, one column each (coalesced rows).
-__global__ void __launch_bounds__(128) k_colsumsq_partial(const float* __restrict__ R, i64 ld, i64 n, i64 r,
-                                                          i64 rows_per_chunk, float* __restrict__ part,
-                                                          const int* __restrict__ skip_flag, i64 wstride) {
-  // blockIdx.z: the matrix of a chain (R and part wstride floats apart, skip flags a state slot apart)
-  pdl_enter();
-  if (skip_flag != nullptr && skip_flag[(i64)blockIdx.z * OS_SLOT_INTS] != 0) return;
-  R += (i64)blockIdx.z * wstride; part += (i64)blockIdx.z * wstride;
-  const i64 j = (i64)blockIdx.x * 128 + threadIdx.x;
-  if (j >= r) return;
-  const i64 i0 = (i64)blockIdx.y * rows_per_chunk;
-  const i64 i1 = min(n, i0 + rows_per_chunk);
-  float s = 0.f;
-  for (i64 i = i0; i < i1; ++i) {
-    const float v = R[i * ld + j];
-    s = fmaf(v, v, s);
-  }
-  part[(i64)blockIdx.y * r + j] = s;
-}
-
-// out[j] = sum over the chunks (in order) of part[chunk][j]: the squared column norms of a shard's rows,
-// handed to the caller for the all-reduce over the shards (1D-sharded Dion).
-__global__ void __launch_bounds__(128) k_colsumsq_finish(const float* __restrict__ part, int chunks, i64 r,
-                                                         float* __restrict__ out, const int* __restrict__ skip_flag) {
-  pdl_enter();
-  if (skip_flag != nullptr && *skip_flag != 0) return;
-  const i64 j = (i64)blockIdx.x * 128 + threadIdx.x;
-  if (j >= r) return;
-  float s = 0.f;
-  for (int c = 0; c < chunks; ++c) s += part[(i64)c * r + j];
-  out[j] = s;
-}
-
-// ColNorm: d_j = sqrt(sum of the partials in chunk order); Q[i][j] = R[i][j] / (d_j + eps).
-// Same grid as k_colsumsq_partial.  The chunk-0 blocks also export d.
-__global__ void __launch_bounds__(128) k_colnorm_apply(const float* __restrict__ R, i64 ldr, i64 n, i64 r,
-                                                       i64 rows_per_chunk, int chunks,
-                                                       const float* __restrict__ part, float eps,
-                                                       float* __restrict__ Q, i64 ldq,
-                                                       float* __restrict__ d_ws, float* __restrict__ d_out,
-                                                       int* __restrict__ status,
-                                                       const int* __restrict__ skip_flag, i64 wstride,
-                                                       const ChainPtrs Qs, const ChainPtrs ds) {
-  // wstride != 0: one launch over a chain (blockIdx.z): R, part and d_ws in the scratch slices, Q and d_out from
-  // the pointer tables
-  pdl_enter();
-  if (skip_flag != nullptr && skip_flag[(i64)blockIdx.z * OS_SLOT_INTS] != 0) return;
-  if (wstride != 0) {
-    R += (i64)blockIdx.z * wstride; part += (i64)blockIdx.z * wstride; d_ws += (i64)blockIdx.z * wstride;
-    Q = reinterpret_cast<float*>(const_cast<void*>(Qs.p[blockIdx.z]));
-    d_out = reinterpret_cast<float*>(const_cast<void*>(ds.p[blockIdx.z]));
-  }
-  const i64 j = (i64)blockIdx.x * 128 + threadIdx.x;
-  if (j >= r) return;
-  float s = 0.f;
-  for (int c = 0; c < chunks; ++c) s += part[(i64)c * r + j];
-  const float d = sqrtf(s);
-  if (blockIdx.y == 0) {
-    d_ws[j] = d;
-    if (d_out != nullptr) d_out[j] = d;
-    if (!isfinite(d)) atomicOr(status, DION_STATUS_NONFINITE);
-  }
-  const float inv = 1.f / (d + eps);
-  const i64 i0 = (i64)blockIdx.y * rows_per_chunk;
-  const i64 i1 = min(n, i0 + rows_per_chunk);
-  for (i64 i = i0; i < i1; ++i) Q[i * ldq + j] = R[i * ldr + j] * inv;
-}
-
 // Copies a rows x r panel (ld = ldv) into Q (ld = ldq) unless the step was flagged.
 // `only_if` (optional): the copy happens only when (*only_if & only_mask) != 0.
 __global__ void k_copy_panel(const float* __restrict__ V, i64 ldv, float* __restrict__ Q, i64 ldq,

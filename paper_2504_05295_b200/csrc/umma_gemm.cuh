@@ -846,6 +846,59 @@ k_gemm_umma(const __grid_constant__ PT p) {
       const i64 n0 = (i64)it.ni * BN;
       // (a device scalar: the learning rate under graph replay, or a matrix's own scale)
       const float alpha = g.alpha * (g.alpha_dev != nullptr ? __ldg(g.alpha_dev + (i64)it.b * g.alpha_dev_stride) : 1.f);
+      if constexpr (X2 && !SPLIT && CE) {
+        // Plain stores of operand pairs: the chunks of a tile are summed in registers (these variants run without the
+        // producer warps, so a lane has room for its row of W columns) and the tile is written once.
+        if (g.epi == EPI_STORE) {
+          constexpr int W = C::EPI_W, RPP = C::EPI_RPP, LPR = W / 4, RPI = 32 / LPR, TS = W + 4;
+          float run[W];
+#pragma unroll
+          for (int e = 0; e < W; ++e) run[e] = 0.f;
+          for (int kb = it.kb0; kb < it.kb1; kb += p.kc, ++iter) {
+            const int ab = iter % NBUF;
+            if (!mbar_wait(accf_bar(ab), (uint32_t)(iter / NBUF) & 1u, dead, p.status, p.spin_limit, 256)) { alive = false; break; }
+            tc_fence_after();
+#pragma unroll
+            for (int sl = 0; sl < W / 16; ++sl) {
+              float acc[16];
+              tmem_ld16(tmem_base + (uint32_t)(ab * BN + half * W + sl * 16) + ((uint32_t)(quad * 32) << 16), acc);
+#pragma unroll
+              for (int e = 0; e < 16; ++e) run[sl * 16 + e] += acc[e];
+            }
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) {
+              if (CG2 && cta_rank != 0) mbar_arrive_remote_relaxed(acce_bar(ab), 0u);
+              else mbar_arrive(acce_bar(ab));
+            }
+          }
+          if (!alive) break;
+          float* tb = epi_tiles + warp * C::EPI_TILE_FLOATS;
+          const i64 col = n0 + half * W + 4 * (lane % LPR);
+          const float f = p.splits > 1 ? 1.f : alpha;
+          float* const out = p.splits > 1 ? partb + (i64)it.ks * g.M * g.N : Cb;
+          const i64 ldo = p.splits > 1 ? g.N : g.ldc;
+#pragma unroll 1
+          for (int ps = 0; ps < 32 / RPP; ++ps) {
+            if (lane / RPP == ps) {
+#pragma unroll
+              for (int q = 0; q < W / 4; ++q)
+                *reinterpret_cast<float4*>(tb + (lane % RPP) * TS + 4 * q) =
+                    make_float4(f * run[4 * q], f * run[4 * q + 1], f * run[4 * q + 2], f * run[4 * q + 3]);
+            }
+            __syncwarp();
+#pragma unroll
+            for (int q = 0; q < RPP / RPI; ++q) {
+              const i64 row = (i64)it.mi * BM + quad * 32 + ps * RPP + RPI * q + lane / LPR;
+              if (row < g.M && col < g.N)
+                *reinterpret_cast<float4*>(out + row * ldo + col) =
+                    *reinterpret_cast<const float4*>(tb + (RPI * q + lane / LPR) * TS + 4 * (lane % LPR));
+            }
+            __syncwarp();
+          }
+          continue;
+        }
+      }
       for (int kb = it.kb0; kb < it.kb1; kb += p.kc, ++iter) {
         const bool first = (kb == it.kb0);
         const int ab = iter % NBUF;
@@ -1977,6 +2030,16 @@ int umma_try_launch(const GemmArgs& g_in, int precision, int sm_count, float* pa
   }
   p.kb_per_split = (p.nkb + splits - 1) / splits;
   splits = (p.nkb + p.kb_per_split - 1) / p.kb_per_split;   // no empty split
+  // 32 K blocks per accumulation chain: 1024 k (8e-6 relative error in fp32 mode, 1.4e-6 with
+  // split accumulators); 2048 k for bf16 operands loaded through registers
+  p.kc = (x2 && (g.precise || g.f16)) ? 16 : 32;   // (K blocks of 64 there: the same 1024 k per chain as the fp32 products)
+  // A chain whose tiles fill the chip needs no split: its K ranges become the accumulation chunks of one work item, which
+  // adds them in the order in which k_splitk_reduce would, so that the bits are those of a matrix of its own.
+  if (splits > 1 && x2 && !g.precise && p.kb_per_split <= p.kc && tiles * nbat >= workers_max * 3 / 4) {
+    p.kc = p.kb_per_split;
+    p.kb_per_split = p.nkb;
+    splits = 1;
+  }
   p.splits = splits;
   p.g.part = part;
   if (tiles * splits * nbat > 0x7fffffff) return 0;
@@ -1986,9 +2049,6 @@ int umma_try_launch(const GemmArgs& g_in, int precision, int sm_count, float* pa
   const bool withhold = (variant & UMMA_VARIANT_WITHHOLD) && !tma;
   p.spin_limit = withhold ? 2000000LL : SPIN_LIMIT_CYCLES;
   p.withhold_arrive = withhold ? 1 : 0;
-  // 32 K blocks per accumulation chain: 1024 k (8e-6 relative error in fp32 mode, 1.4e-6 with
-  // split accumulators); 2048 k for bf16 operands loaded through registers
-  p.kc = (x2 && (g.precise || g.f16)) ? 16 : 32;   // (K blocks of 64 there: the same 1024 k per chain as the fp32 products)
   const int grid = cg2 ? 2 * (p.num_items < nclusters ? p.num_items : nclusters)
                        : (p.num_items < sm_count ? p.num_items : sm_count);
   const bool one = g.tf32x1 && !bf16 && tma && !a_mn && !b_mn && g.a2_mode == ADD_NONE && !g.precise && splits == 1;
