@@ -24,7 +24,7 @@ __global__ void __launch_bounds__(256) k_form_b16(const float* __restrict__ M, i
   const i64 per_row = cols / 8;
   const i64 total = rows * per_row;
   for (i64 e = (i64)blockIdx.x * blockDim.x + threadIdx.x; e < total; e += (i64)gridDim.x * blockDim.x) {
-    const i64 i = e / per_row, c = (e - i * per_row) * 8;
+    const i64 i = row_of(e, per_row), c = (e - i * per_row) * 8;
     float v[8];
     const float* mp = M + i * ldm + c;
     if (VEC) {
@@ -70,6 +70,7 @@ __global__ void __launch_bounds__(256) k_form_b16(const float* __restrict__ M, i
 // error feedback read it.  One thread per 4 consecutive elements of a row; VEC as above.
 // hi / lo (optional, both or neither; cols a multiple of 8 then): the same sum as a pair of bf16 arrays, hi = bf16(sum),
 // lo = bf16(sum - hi), dense like out: the operand of the products that run on bf16 pairs.
+constexpr int FORM_BATCH = 4;
 template <bool VEC>
 __device__ __forceinline__ void form_b32_body(const float* __restrict__ M, i64 ldm, const void* __restrict__ G,
                                               i64 ldg, int g_mode, i64 rows, i64 cols, float* __restrict__ out,
@@ -77,31 +78,46 @@ __device__ __forceinline__ void form_b32_body(const float* __restrict__ M, i64 l
                                               float* amax = nullptr) {      // amax (register, optional): largest magnitude seen by the thread
   const i64 per_row = cols / 4;
   const i64 total = rows * per_row;
-  for (i64 e = (i64)blockIdx.x * blockDim.x + threadIdx.x; e < total; e += (i64)gridDim.x * blockDim.x) {
-    const i64 i = e / per_row, c = (e - i * per_row) * 4;
-    float4 v;
+  // (FORM_BATCH pieces in flight per thread: the sums' stores would keep the compiler from overlapping the loads)
+  const i64 stride = (i64)gridDim.x * blockDim.x;
+  for (i64 e0 = (i64)blockIdx.x * blockDim.x + threadIdx.x; e0 < total; e0 += FORM_BATCH * stride) {
+   float4 mv[FORM_BATCH], gv[FORM_BATCH];
+   i64 at[FORM_BATCH];
+#pragma unroll
+   for (int u = 0; u < FORM_BATCH; ++u) {
+    const i64 e = e0 + u * stride;
+    if (e >= total) break;
+    const i64 i = row_of(e, per_row), c = (e - i * per_row) * 4;
+    at[u] = i * cols + c;
     const float* mp = M + i * ldm + c;
-    if (VEC) v = __ldg(reinterpret_cast<const float4*>(mp));
-    else v = make_float4(mp[0], mp[1], mp[2], mp[3]);
+    if (VEC) mv[u] = __ldg(reinterpret_cast<const float4*>(mp));
+    else mv[u] = make_float4(mp[0], mp[1], mp[2], mp[3]);
     if (g_mode == ADD_F32) {
       const float* gp = reinterpret_cast<const float*>(G) + i * ldg + c;
-      float4 g;
-      if (VEC) g = __ldg(reinterpret_cast<const float4*>(gp));
-      else g = make_float4(gp[0], gp[1], gp[2], gp[3]);
-      v.x += g.x; v.y += g.y; v.z += g.z; v.w += g.w;
+      if (VEC) gv[u] = __ldg(reinterpret_cast<const float4*>(gp));
+      else gv[u] = make_float4(gp[0], gp[1], gp[2], gp[3]);
     } else if (g_mode == ADD_BF16) {
       const __nv_bfloat16* gp = reinterpret_cast<const __nv_bfloat16*>(G) + i * ldg + c;
       if (VEC) {
         const uint2 w = __ldg(reinterpret_cast<const uint2*>(gp));
-        const __nv_bfloat162 lo = *reinterpret_cast<const __nv_bfloat162*>(&w.x);
-        const __nv_bfloat162 hi = *reinterpret_cast<const __nv_bfloat162*>(&w.y);
-        v.x += __low2float(lo); v.y += __high2float(lo); v.z += __low2float(hi); v.w += __high2float(hi);
+        gv[u].x = __uint_as_float(w.x); gv[u].y = __uint_as_float(w.y);
       } else {
-        v.x += __bfloat162float(gp[0]); v.y += __bfloat162float(gp[1]);
-        v.z += __bfloat162float(gp[2]); v.w += __bfloat162float(gp[3]);
+        gv[u] = make_float4(__bfloat162float(gp[0]), __bfloat162float(gp[1]), __bfloat162float(gp[2]), __bfloat162float(gp[3]));
       }
     }
-    *reinterpret_cast<float4*>(out + i * cols + c) = v;
+   }
+#pragma unroll
+   for (int u = 0; u < FORM_BATCH; ++u) {
+    if (e0 + u * stride >= total) break;
+    float4 v = mv[u], g = gv[u];
+    if (VEC && g_mode == ADD_BF16) {      // (still the four bf16 values)
+      const uint32_t w0 = __float_as_uint(g.x), w1 = __float_as_uint(g.y);
+      const __nv_bfloat162 lo2 = *reinterpret_cast<const __nv_bfloat162*>(&w0);
+      const __nv_bfloat162 hi2 = *reinterpret_cast<const __nv_bfloat162*>(&w1);
+      g = make_float4(__low2float(lo2), __high2float(lo2), __low2float(hi2), __high2float(hi2));
+    }
+    if (g_mode != ADD_NONE) { v.x += g.x; v.y += g.y; v.z += g.z; v.w += g.w; }
+    *reinterpret_cast<float4*>(out + at[u]) = v;
     if (amax != nullptr) *amax = fmaxf(fmaxf(*amax, fmaxf(fabsf(v.x), fabsf(v.y))), fmaxf(fabsf(v.z), fabsf(v.w)));
     if (hi != nullptr) {
       const float h0 = __bfloat162float(__float2bfloat16_rn(v.x)), h1 = __bfloat162float(__float2bfloat16_rn(v.y));
@@ -109,13 +125,14 @@ __device__ __forceinline__ void form_b32_body(const float* __restrict__ M, i64 l
       uint2 oh, ol;
       oh.x = pack_bf16x2(h0, h1); oh.y = pack_bf16x2(h2, h3);
       ol.x = pack_bf16x2(v.x - h0, v.y - h1); ol.y = pack_bf16x2(v.z - h2, v.w - h3);
-      *reinterpret_cast<uint2*>(hi + i * cols + c) = oh;
-      *reinterpret_cast<uint2*>(lo + i * cols + c) = ol;
+      *reinterpret_cast<uint2*>(hi + at[u]) = oh;
+      *reinterpret_cast<uint2*>(lo + at[u]) = ol;
     }
+   }
   }
 }
 template <bool VEC>
-__global__ void __launch_bounds__(256) k_form_b32(const float* __restrict__ M, i64 ldm, const void* __restrict__ G,
+__global__ void __launch_bounds__(256, 3) k_form_b32(const float* __restrict__ M, i64 ldm, const void* __restrict__ G,
                                                   i64 ldg, int g_mode, i64 rows, i64 cols, float* __restrict__ out,
                                                   __nv_bfloat16* __restrict__ hi, __nv_bfloat16* __restrict__ lo) {
   pdl_enter();
@@ -124,7 +141,7 @@ __global__ void __launch_bounds__(256) k_form_b32(const float* __restrict__ M, i
 // The same for every matrix of a chain in one launch (blockIdx.y): the caller's M and G from pointer tables, the
 // outputs in the scratch slices, `ostride` floats apart.
 template <bool VEC>
-__global__ void __launch_bounds__(256) k_form_b32_chain(const ChainPtrs Ms, i64 ldm, const ChainPtrs Gs, i64 ldg, int g_mode,
+__global__ void __launch_bounds__(256, 3) k_form_b32_chain(const ChainPtrs Ms, i64 ldm, const ChainPtrs Gs, i64 ldg, int g_mode,
                                                         i64 rows, i64 cols, float* __restrict__ out,
                                                         __nv_bfloat16* __restrict__ hi, __nv_bfloat16* __restrict__ lo,
                                                         i64 ostride) {
@@ -143,7 +160,7 @@ __global__ void __launch_bounds__(256) k_to_bf16(const float* __restrict__ src, 
   const i64 per_row = cols / 8;
   const i64 total = rows * per_row;
   for (i64 e = (i64)blockIdx.x * blockDim.x + threadIdx.x; e < total; e += (i64)gridDim.x * blockDim.x) {
-    const i64 i = e / per_row, c = (e - i * per_row) * 8;
+    const i64 i = row_of(e, per_row), c = (e - i * per_row) * 8;
     const float4 a = *reinterpret_cast<const float4*>(src + i * lds + c);
     const float4 b = *(reinterpret_cast<const float4*>(src + i * lds + c) + 1);
     uint4 o;
@@ -162,7 +179,7 @@ __device__ __forceinline__ void split_bf16_body(const float* __restrict__ src, i
   const i64 per_row = cols / 8;
   const i64 total = rows * per_row;
   for (i64 e = (i64)blockIdx.x * blockDim.x + threadIdx.x; e < total; e += (i64)gridDim.x * blockDim.x) {
-    const i64 i = e / per_row, c = (e - i * per_row) * 8;
+    const i64 i = row_of(e, per_row), c = (e - i * per_row) * 8;
     const float4 a = *reinterpret_cast<const float4*>(src + i * lds + c);
     const float4 b = *(reinterpret_cast<const float4*>(src + i * lds + c) + 1);
     const float v[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
@@ -211,7 +228,7 @@ __global__ void __launch_bounds__(256) k_copy_chain(const ChainPtrs srcs, i64 ld
   out += (i64)blockIdx.y * ostride;
   const i64 per_row = cols / 4, total = rows * per_row;
   for (i64 e = (i64)blockIdx.x * blockDim.x + threadIdx.x; e < total; e += (i64)gridDim.x * blockDim.x) {
-    const i64 i = e / per_row, c = (e - i * per_row) * 4;
+    const i64 i = row_of(e, per_row), c = (e - i * per_row) * 4;
     *reinterpret_cast<float4*>(out + i * cols + c) = *reinterpret_cast<const float4*>(src + i * lds + c);
   }
 }
@@ -226,7 +243,7 @@ __device__ __forceinline__ void round_tf32_body(const float* __restrict__ src, i
   const i64 per_row = cols / 4;
   const i64 total = rows * per_row;
   for (i64 e = (i64)blockIdx.x * blockDim.x + threadIdx.x; e < total; e += (i64)gridDim.x * blockDim.x) {
-    const i64 i = e / per_row, c = (e - i * per_row) * 4;
+    const i64 i = row_of(e, per_row), c = (e - i * per_row) * 4;
     const float4 a = *reinterpret_cast<const float4*>(src + i * lds + c);
     uint4 o;
     asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(o.x) : "f"(a.x));
@@ -260,7 +277,7 @@ __device__ __forceinline__ void round_f16_body(const float* __restrict__ src, i6
   const i64 per_row = cols / 8;
   const i64 total = rows * per_row;
   for (i64 e = (i64)blockIdx.x * blockDim.x + threadIdx.x; e < total; e += (i64)gridDim.x * blockDim.x) {
-    const i64 i = e / per_row, c = (e - i * per_row) * 8;
+    const i64 i = row_of(e, per_row), c = (e - i * per_row) * 8;
     const float4 a = *reinterpret_cast<const float4*>(src + i * lds + c);
     const float4 b = *(reinterpret_cast<const float4*>(src + i * lds + c) + 1);
     __half2 h0 = __floats2half2_rn(scale * a.x, scale * a.y), h1 = __floats2half2_rn(scale * a.z, scale * a.w);
@@ -312,7 +329,7 @@ __device__ __forceinline__ int f16_scale_exponent(float amax) {
 }
 // M + G in fp32 and the blocks' largest magnitudes of it in one pass (the products on a scaled half pair of the sum).
 template <bool VEC>
-__global__ void __launch_bounds__(256) k_form_b32_amax(const float* __restrict__ M, i64 ldm, const void* __restrict__ G, i64 ldg, int g_mode,
+__global__ void __launch_bounds__(256, 3) k_form_b32_amax(const float* __restrict__ M, i64 ldm, const void* __restrict__ G, i64 ldg, int g_mode,
                                                        i64 rows, i64 cols, float* __restrict__ out, float* __restrict__ part) {
   pdl_enter();
   float m = 0.f;
@@ -323,7 +340,7 @@ __global__ void __launch_bounds__(256) k_form_b32_amax(const float* __restrict__
 // and of Q (Q is a right factor of the caller's making: nothing bounds its entries), then the scaled pairs of both.
 // part: gridDim.x maxima of the sum, then as many of Q.  16-byte accesses to Q where it allows them (qvec).
 template <bool VEC>
-__global__ void __launch_bounds__(256) k_form_sum_amax(const ChainPtrs Ms, i64 ldm, const ChainPtrs Gs, i64 ldg, int g_mode, i64 rows, i64 cols,
+__global__ void __launch_bounds__(256, 3) k_form_sum_amax(const ChainPtrs Ms, i64 ldm, const ChainPtrs Gs, i64 ldg, int g_mode, i64 rows, i64 cols,
                                                        const ChainPtrs Qs, i64 ldq, i64 qrows, i64 qcols, int qvec, float* __restrict__ out,
                                                        float* __restrict__ part, i64 wstride) {
   pdl_enter();
@@ -334,7 +351,7 @@ __global__ void __launch_bounds__(256) k_form_sum_amax(const ChainPtrs Ms, i64 l
   const float* __restrict__ Q = reinterpret_cast<const float*>(Qs.p[b]);
   const i64 per_row = qcols / 4, total = qrows * per_row;
   for (i64 e = (i64)blockIdx.x * blockDim.x + threadIdx.x; e < total; e += (i64)gridDim.x * blockDim.x) {
-    const i64 i = e / per_row;
+    const i64 i = row_of(e, per_row);
     const float* q = Q + i * ldq + (e - i * per_row) * 4;
     const float4 a = qvec ? *reinterpret_cast<const float4*>(q) : make_float4(q[0], q[1], q[2], q[3]);
     mq = fmaxf(fmaxf(mq, fmaxf(fabsf(a.x), fabsf(a.y))), fmaxf(fabsf(a.z), fabsf(a.w)));
@@ -381,7 +398,7 @@ __global__ void __launch_bounds__(256) k_split_sum(const float* __restrict__ sum
       x = *reinterpret_cast<const float4*>(sum + eo * 8);
       y = *reinterpret_cast<const float4*>(sum + eo * 8 + 4);
     } else {
-      const i64 i = eo / qpr;
+      const i64 i = row_of(eo, qpr);
       const float* q = Q + i * ldq + (eo - i * qpr) * 8;
       x = qvec ? *reinterpret_cast<const float4*>(q) : make_float4(q[0], q[1], q[2], q[3]);
       y = qvec ? *reinterpret_cast<const float4*>(q + 4) : make_float4(q[4], q[5], q[6], q[7]);
@@ -408,7 +425,7 @@ __global__ void __launch_bounds__(256) k_absmax_partial(const float* __restrict_
   const i64 per_row = cols / 4, total = rows * per_row;
   float m = 0.f;
   for (i64 e = (i64)blockIdx.x * blockDim.x + threadIdx.x; e < total; e += (i64)gridDim.x * blockDim.x) {
-    const i64 i = e / per_row, c = (e - i * per_row) * 4;
+    const i64 i = row_of(e, per_row), c = (e - i * per_row) * 4;
     const float4 a = *reinterpret_cast<const float4*>(src + i * ld + c);
     m = fmaxf(fmaxf(m, fmaxf(fabsf(a.x), fabsf(a.y))), fmaxf(fabsf(a.z), fabsf(a.w)));
   }
@@ -449,7 +466,7 @@ __global__ void __launch_bounds__(256) k_split_f16_scaled(const float* __restric
                                     : other_inv * ldexpf(1.f, ex - 14) * (other_dev != nullptr ? *other_dev : 1.f);
   const i64 per_row = cols / 8, total = rows * per_row;
   for (i64 e = (i64)blockIdx.x * blockDim.x + threadIdx.x; e < total; e += (i64)gridDim.x * blockDim.x) {
-    const i64 i = e / per_row, c = (e - i * per_row) * 8;
+    const i64 i = row_of(e, per_row), c = (e - i * per_row) * 8;
     const float4 a = *reinterpret_cast<const float4*>(src + i * ld + c);
     const float4 b = *(reinterpret_cast<const float4*>(src + i * ld + c) + 1);
     const float v[8] = {scale * a.x, scale * a.y, scale * a.z, scale * a.w, scale * b.x, scale * b.y, scale * b.z, scale * b.w};
@@ -480,7 +497,7 @@ __global__ void __launch_bounds__(256) k_split_f16_fixed(const ChainPtrs srcs, i
   hi += 2 * bm * ostride; lo += 2 * bm * ostride;
   const i64 per_row = cols / 8, total = rows * per_row;
   for (i64 e = (i64)blockIdx.x * blockDim.x + threadIdx.x; e < total; e += (i64)gridDim.x * blockDim.x) {
-    const i64 i = e / per_row, c = (e - i * per_row) * 8;
+    const i64 i = row_of(e, per_row), c = (e - i * per_row) * 8;
     const float4 a = *reinterpret_cast<const float4*>(src + i * lds + c);
     const float4 b = *(reinterpret_cast<const float4*>(src + i * lds + c) + 1);
     const float v[8] = {scale * a.x, scale * a.y, scale * a.z, scale * a.w, scale * b.x, scale * b.y, scale * b.z, scale * b.w};

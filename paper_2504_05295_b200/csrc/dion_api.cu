@@ -305,39 +305,68 @@ cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t s
   return cudaLaunchKernelEx(&cfg, kernel, args...);
 }
 
-// Launches one product on the fp32 FMA engine.
+// Products on the fp32 FMA engine.
+// Splits of K: a K step of 16 takes about as long as the latency of its loads whatever runs beside it, so a product of few tiles is
+// cut to two or three steps per block, up to two blocks per SM (1001 x 83 x 333 with the reduction: 28.6 -> 14 us).
+// Fewer where the next kernel adds the partial sums up itself (k_chol_flow).
+constexpr i64 SPLIT_MIN_K = 32;
+constexpr i64 SPLIT_MAX = 64;
+constexpr i64 SPLIT_MIN_K_DEFERRED = 128;
+constexpr i64 SIMT_THIN_N = 32;          // outputs of at most this many columns take 128 x 32 tiles
+constexpr i64 SIMT_WIDE_MIN_K = 96;      // updates of C below it are bound by C: 64 x 64 tiles, three blocks per SM
+
+// tabs != nullptr: the same product on nb matrices (operands from the tables, partial sums part_stride floats apart; outputs too
+// where the reduction follows).  Tiles and splits are those of one matrix: the same bits.
 int launch_gemm_simt(dion_ctx* c, GemmArgs g, cudaStream_t st, float* part, i64 part_floats,
-                     bool force64) {
+                     bool force64, const GemmTabs* tabs = nullptr, int nb = 1, i64 part_stride = 0) {
   if (g.M <= 0 || g.N <= 0) return DION_OK;
   const i64 t128 = ((g.M + 127) / 128) * ((g.N + 127) / 128) * g.batch * (g.batch2 > 1 ? g.batch2 : 1);
-  const bool use128 = !force64 && t128 >= c->sm_count;
-  const int BMN = use128 ? 128 : 64;
-  const i64 gm = (g.M + BMN - 1) / BMN, gn = (g.N + BMN - 1) / BMN;
+  const bool thin = !force64 && g.N <= SIMT_THIN_N && g.tri == TRI_FULL && !g.klimit;
+  const bool use128 = !force64 && !thin && t128 >= c->sm_count && (g.epi == EPI_STORE || g.K >= SIMT_WIDE_MIN_K);
+  const i64 bm = (use128 || thin) ? 128 : 64, bn = use128 ? 128 : thin ? 32 : 64;
+  const i64 gm = (g.M + bm - 1) / bm, gn = (g.N + bn - 1) / bn;
   int splits = 1;
   if (!use128 && !force64 && g.epi == EPI_STORE && g.batch == 1 && g.batch2 <= 1 && part != nullptr && g.alpha_dev == nullptr) {
     const i64 tiles = gm * gn;
     i64 want = (2 * (i64)c->sm_count + tiles - 1) / tiles;
-    const i64 kmax = g.K / 128;
+    const i64 kmax = g.K / SPLIT_MIN_K;
     if (want > kmax) want = kmax;
-    if (want > 64) want = 64;
+    if (want > SPLIT_MAX) want = SPLIT_MAX;
+    const i64 most = g.K / SPLIT_MIN_K_DEFERRED;
+    if (g.splits_out != nullptr && want > most) want = most;
     while (want > 1 && want * g.M * g.N > part_floats) --want;
-    if (want > 1) splits = (int)want;
+    if (want > 1) {
+      const i64 per = ((g.K + want - 1) / want + 15) / 16 * 16;      // as the kernel cuts K; no empty split
+      splits = (int)((g.K + per - 1) / per);
+    }
   }
+  // (a chain whose tiles fill the chip adds the splits up in the blocks instead of through memory)
+  int inner = 1;
+  if (tabs != nullptr && splits > 1 && g.splits_out == nullptr && gm * gn * nb >= 2 * c->sm_count) { inner = splits; splits = 1; }
   g.splits = splits;
   g.part = part;
   if (gm > 65535) return DION_ERR_UNSUPPORTED;
   if (g.batch2 < 1) g.batch2 = 1;
   if (splits > 1 && g.batch2 > 1) return DION_ERR_INVALID;
-  dim3 grid((unsigned)gn, (unsigned)gm, (unsigned)(splits > 1 ? splits : g.batch * g.batch2));
-  if (use128) launch_pdl(k_gemm_simt<128, 128, 8, 8, 8>, grid, dim3(256), 0, st, g);
-  else launch_pdl(k_gemm_simt<64, 64, 16, 4, 4>, grid, dim3(256), 0, st, g);
+  const dim3 grid((unsigned)gn, (unsigned)gm, (unsigned)(tabs != nullptr ? splits * nb : splits > 1 ? splits : g.batch * g.batch2));
+  if (tabs != nullptr) {
+    g.bs2 = part_stride;
+    if (use128) launch_pdl(k_gemm_simt<128, 128, 8, 8, 8, 1, GemmTabs>, grid, dim3(256), 0, st, g, *tabs, inner);
+    else if (thin) launch_pdl(k_gemm_simt<128, 32, 16, 4, 4, 2, GemmTabs>, grid, dim3(256), 0, st, g, *tabs, inner);
+    else launch_pdl(k_gemm_simt<64, 64, 16, 4, 4, 3, GemmTabs>, grid, dim3(256), 0, st, g, *tabs, inner);
+  } else {
+    if (use128) launch_pdl(k_gemm_simt<128, 128, 8, 8, 8, 1, NoTabs>, grid, dim3(256), 0, st, g, NoTabs(), 1);
+    else if (thin) launch_pdl(k_gemm_simt<128, 32, 16, 4, 4, 2, NoTabs>, grid, dim3(256), 0, st, g, NoTabs(), 1);
+    else launch_pdl(k_gemm_simt<64, 64, 16, 4, 4, 3, NoTabs>, grid, dim3(256), 0, st, g, NoTabs(), 1);
+  }
   DION_CHECK_LAUNCH(c);
   if (g.splits_out != nullptr) { *g.splits_out = splits; return DION_OK; }      // (the caller sums the partial products itself)
   if (splits > 1) {
-    const i64 total = g.M * g.N;
+    const i64 total = g.N % 4 == 0 ? (g.M * g.N + 3) / 4 : g.M * g.N;      // (four elements per thread where rows allow it)
     int blocks = (int)((total + 255) / 256);
     if (blocks > 8 * c->sm_count) blocks = 8 * c->sm_count;
-    launch_pdl(k_splitk_reduce, dim3((unsigned)(blocks)), dim3(256), 0, st, part, splits, g.M, g.N, g.C, g.ldc, g.alpha, g.tri, BMN, g.skip_flag, (i64)0, (i64)0, (const float*)nullptr, (i64)0);
+    launch_pdl(k_splitk_reduce, dim3((unsigned)blocks, (unsigned)nb), dim3(256), 0, st, part, splits, g.M, g.N, g.C, g.ldc, g.alpha, g.tri, (int)bm, g.skip_flag,
+               part_stride, nb > 1 ? g.skip_stride : (i64)0, (const float*)nullptr, (i64)0);
     DION_CHECK_LAUNCH(c);
   }
   return DION_OK;
@@ -441,6 +470,19 @@ int launch_gemm_chain(StepCtx& s, const GemmArgs& g, bool c2_ws = false) {
     if (rc > 0) { s.c->launches += rc; return DION_OK; }
     if (rc < 0) return rc;
   }
+  if (s.nb > 1 && s.nb <= GEMM_TAB_MAX && s.c->chain_batch && g.batch == 1 && g.batch2 <= 1 && g.alpha_dev == nullptr &&
+      s.c->cfg.engine != DION_ENGINE_TENSOR && !(s.tensor && umma_shape_ok(g, s.in_orth ? DION_PREC_FP32 : s.c->cfg.precision)) && !g.ab16) {
+    GemmTabs t;      // (shapes that only the FMA engine takes: one launch of it)
+    for (int m = 0; m < s.nb; ++m) {
+      const i64 o = (i64)m * s.wstride;
+      t.A[m] = g.A + o; t.B[m] = g.B + o; t.C[m] = g.C + o; t.A2[m] = g.A2;
+      t.C2[m] = g.C2 != nullptr && c2_ws ? (const void*)((const float*)g.C2 + o) : g.C2;
+    }
+    GemmArgs gb = g;
+    gb.skip_stride = OS_SLOT_INTS;
+    PhaseScope ps(s.c, s.st, s.in_orth ? DION_PHASE_ORTH_GEMM : -1);
+    return launch_gemm_simt(s.c, gb, s.st, s.no_split ? nullptr : s.W(0, s.L.part), s.L.part_floats, false, &t, s.nb, s.wstride);
+  }
   for (int m = 0; m < s.nb; ++m) {
     GemmArgs gm = for_matrix(s, g, m, true, true, true);
     if (c2_ws) gm.C2 = (const float*)gm.C2 + (i64)m * s.wstride;
@@ -459,22 +501,24 @@ int launch_gemm_group(StepCtx& s, const std::vector<GemmArgs>& v) {
   bool one = nb > 1 && nb <= GEMM_TAB_MAX && s.tensor && s.c->chain_batch;
   const GemmArgs& a = v[0];
   bool c_strided = true, c2_strided = true;
+  bool alike = nb > 1 && nb <= GEMM_TAB_MAX && s.c->chain_batch;      // the same product on every matrix, wherever its operands lie
   const i64 wb = s.wstride * 4;   // bytes between scratch slices
   auto at_stride = [&](const void* p0, const void* pb, int b) {
     return (p0 == nullptr && pb == nullptr) ||
            (p0 != nullptr && pb != nullptr && (const char*)pb - (const char*)p0 == (ptrdiff_t)((i64)b * wb));
   };
-  for (int b = 1; b < nb && one; ++b) {
+  for (int b = 1; b < nb && alike; ++b) {
     const GemmArgs& g = v[b];
-    one = g.M == a.M && g.N == a.N && g.K == a.K && g.a_si == a.a_si && g.a_sk == a.a_sk && g.a2_si == a.a2_si &&
-          g.a2_sk == a.a2_sk && g.a2_mode == a.a2_mode && g.b_sk == a.b_sk && g.b_sn == a.b_sn && g.ldc == a.ldc &&
-          g.epi == a.epi && g.ldc2 == a.ldc2 && g.c2_mode == a.c2_mode && g.alpha == a.alpha &&
-          (g.alpha_dev == a.alpha_dev || at_stride(a.alpha_dev, g.alpha_dev, b)) &&
-          g.batch == 1 && a.batch == 1 && g.tri == a.tri && g.klimit == a.klimit && g.precise == a.precise &&
-          g.ab16 == a.ab16 && g.f16 == a.f16 && g.tf32x1 == a.tf32x1 && at_stride(a.A, g.A, b) && at_stride(a.B, g.B, b) &&
-          at_stride(a.A2, g.A2, b) && at_stride(a.A16lo, g.A16lo, b) && at_stride(a.B16lo, g.B16lo, b) &&
-          ((a.skip_flag == nullptr && g.skip_flag == nullptr) ||
-           (a.skip_flag != nullptr && g.skip_flag == a.skip_flag + (i64)b * OS_SLOT_INTS));
+    alike = alike && g.M == a.M && g.N == a.N && g.K == a.K && g.a_si == a.a_si && g.a_sk == a.a_sk && g.a2_si == a.a2_si &&
+            g.a2_sk == a.a2_sk && g.a2_mode == a.a2_mode && g.b_sk == a.b_sk && g.b_sn == a.b_sn && g.ldc == a.ldc &&
+            g.epi == a.epi && g.ldc2 == a.ldc2 && g.c2_mode == a.c2_mode && g.alpha == a.alpha &&
+            (g.alpha_dev == a.alpha_dev || at_stride(a.alpha_dev, g.alpha_dev, b)) &&
+            g.batch == 1 && a.batch == 1 && g.tri == a.tri && g.klimit == a.klimit && g.precise == a.precise &&
+            g.ab16 == a.ab16 && g.f16 == a.f16 && g.tf32x1 == a.tf32x1 &&
+            ((a.skip_flag == nullptr && g.skip_flag == nullptr) ||
+             (a.skip_flag != nullptr && g.skip_flag == a.skip_flag + (i64)b * OS_SLOT_INTS));
+    one = one && alike && at_stride(a.A, g.A, b) && at_stride(a.B, g.B, b) && at_stride(a.A2, g.A2, b) && at_stride(a.A16lo, g.A16lo, b) &&
+          at_stride(a.B16lo, g.B16lo, b);
     c_strided = c_strided && at_stride(a.C, g.C, b);
     c2_strided = c2_strided && at_stride(a.C2, g.C2, b);
   }
@@ -497,6 +541,16 @@ int launch_gemm_group(StepCtx& s, const std::vector<GemmArgs>& v) {
                                    s.c->dev_ints, s.st);
     if (rc > 0) { s.c->launches += rc; return DION_OK; }
     if (rc < 0) return rc;
+  }
+  // (not for the tensor engine:) one launch of the FMA engine, with the operands' addresses in tables
+  if (alike && !a.ab16 && s.c->cfg.engine != DION_ENGINE_TENSOR && !(s.tensor && umma_shape_ok(a, s.in_orth ? DION_PREC_FP32 : s.c->cfg.precision)) && (c_strided || a.epi != EPI_STORE)) {
+    GemmTabs t;
+    for (int b = 0; b < nb; ++b) { t.A[b] = v[b].A; t.A2[b] = v[b].A2; t.B[b] = v[b].B; t.C[b] = v[b].C; t.C2[b] = v[b].C2; }
+    GemmArgs g = a;
+    g.skip_stride = OS_SLOT_INTS;
+    if (v[1].alpha_dev != a.alpha_dev) g.alpha_dev_stride = s.wstride;
+    PhaseScope ps(s.c, s.st, s.in_orth ? DION_PHASE_ORTH_GEMM : -1);
+    return launch_gemm_simt(s.c, g, s.st, s.no_split ? nullptr : s.W(0, s.L.part), s.L.part_floats, false, &t, nb, s.wstride);
   }
   for (int b = 0; b < nb; ++b) DION_TRY(launch_gemm(s, v[b], b));
   return DION_OK;
@@ -1209,10 +1263,13 @@ int colnorm_launch(StepCtx& s, int b, int per, const float* W, i64 ldw, i64 rows
   int qvec = ldq % 4 == 0;
   for (int k = 0; k < per; ++k) qvec = qvec && !((uintptr_t)Qs.p[k] & 15);
   if (sums != nullptr) chunks = 1;
+  i64 rpb = (rows * (i64)grid.x * per + 3 * c->sm_count - 1) / (3 * c->sm_count);      // three blocks per SM, all at once
+  if (rpb < 32) rpb = 32;
+  const dim3 agrid(grid.x, (unsigned)((rows + rpb - 1) / rpb), grid.z);
   const float* sp = sums != nullptr ? sums : (const float*)part;
-  if (v4) launch_pdl(k_colnorm_apply<true>, grid, dim3(CN_THREADS), 0, s.st, W, ldw, rows, r, rpc, chunks, sp, c->cfg.eps, Qs, ldq, qvec, s.W(b, s.L.d), ds,
+  if (v4) launch_pdl(k_colnorm_apply<true>, agrid, dim3(CN_THREADS), 0, s.st, W, ldw, rows, r, rpb, chunks, sp, c->cfg.eps, Qs, ldq, qvec, s.W(b, s.L.d), ds,
                      c->dev_ints, skip, s.wstride, x);
-  else launch_pdl(k_colnorm_apply<false>, grid, dim3(CN_THREADS), 0, s.st, W, ldw, rows, r, rpc, chunks, sp, c->cfg.eps, Qs, ldq, qvec, s.W(b, s.L.d), ds,
+  else launch_pdl(k_colnorm_apply<false>, agrid, dim3(CN_THREADS), 0, s.st, W, ldw, rows, r, rpb, chunks, sp, c->cfg.eps, Qs, ldq, qvec, s.W(b, s.L.d), ds,
                   c->dev_ints, skip, s.wstride, x);
   DION_CHECK_LAUNCH(c);
   return DION_OK;
@@ -2846,7 +2903,8 @@ bool touch_kernel(K kernel) {
 // tensor-core variants are covered by configure_kernels, which sets an attribute on each).
 bool preload_kernels() {
   bool ok = true;
-  ok = ok && touch_kernel(k_gemm_simt<128, 128, 8, 8, 8>) && touch_kernel(k_gemm_simt<64, 64, 16, 4, 4>);
+  ok = ok && touch_kernel(k_gemm_simt<128, 128, 8, 8, 8, 1, NoTabs>) && touch_kernel(k_gemm_simt<64, 64, 16, 4, 4, 3, NoTabs>) &&
+       touch_kernel(k_gemm_simt<128, 32, 16, 4, 4, 2, NoTabs>);
   ok = ok && touch_kernel(k_splitk_reduce) && touch_kernel(k_round_begin) && touch_kernel(k_chol_flow<true>);
   ok = ok && touch_kernel(k_chol_flow<false>) && touch_kernel(k_round_end) && touch_kernel(k_tiny_cholqr2);
   ok = ok && touch_kernel(k_probe_y) && touch_kernel(k_probe_y4) && touch_kernel(k_probe_w) && touch_kernel(k_probe_w4) && touch_kernel(k_probe_decide) && touch_kernel(k_reset_rounds);

@@ -32,6 +32,14 @@ constexpr int GEMM_TAB_MAX = 64;   // most matrices in one batched tensor-engine
 // Per-matrix pointers of a chain for the elementwise kernels that run once over all its matrices.
 struct ChainPtrs { const void* p[GEMM_TAB_MAX]; };
 
+#ifdef __CUDACC__
+// e / per_row: a 64-bit division is some eighty instructions, more than the rest of an elementwise pass over four elements;
+// indexes above 2^32 are rare.
+__device__ __forceinline__ i64 row_of(i64 e, i64 per_row) {
+  return ((e | per_row) >> 32) == 0 ? (i64)((uint32_t)e / (uint32_t)per_row) : e / per_row;
+}
+#endif
+
 struct GemmArgs {
   i64 M, N, K;
   const float* A; i64 a_si, a_sk;

@@ -944,7 +944,7 @@ __global__ void k_copy_block(const float* __restrict__ src, i64 lds, float* __re
   if (skip_flag != nullptr && skip_flag[(i64)blockIdx.y * OS_SLOT_INTS] != 0) return;
   const i64 total = rows * cols;
   for (i64 e = (i64)blockIdx.x * blockDim.x + threadIdx.x; e < total; e += (i64)gridDim.x * blockDim.x) {
-    const i64 i = e / cols, c = e % cols;
+    const i64 i = row_of(e, cols), c = e - i * cols;
     dst[i * ldd + c] = src[i * lds + c];
   }
 }
@@ -961,7 +961,7 @@ __global__ void k_copy_panel(const float* __restrict__ V, i64 ldv, float* __rest
   if (only_if != nullptr && (only_if[(i64)blockIdx.y * OS_SLOT_INTS] & only_mask) == 0) return;
   const i64 total = rows * r;
   for (i64 e = (i64)blockIdx.x * blockDim.x + threadIdx.x; e < total; e += (i64)gridDim.x * blockDim.x) {
-    const i64 i = e / r, c = e % r;
+    const i64 i = row_of(e, r), c = e - i * r;
     Q[i * ldq + c] = V[i * ldv + c];
   }
 }
@@ -1037,7 +1037,7 @@ __global__ void __launch_bounds__(256) k_hh_apply(float* __restrict__ T, i64 ldt
 __global__ void k_set_identity(float* __restrict__ U, i64 ld, i64 m, i64 r) {
   const i64 total = m * r;
   for (i64 e = (i64)blockIdx.x * blockDim.x + threadIdx.x; e < total; e += (i64)gridDim.x * blockDim.x) {
-    const i64 i = e / r, c = e % r;
+    const i64 i = row_of(e, r), c = e - i * r;
     U[i * ld + c] = (i == c) ? 1.f : 0.f;
   }
 }
@@ -1046,7 +1046,7 @@ __global__ void k_set_identity(float* __restrict__ U, i64 ld, i64 m, i64 r) {
 __global__ void k_sign_fix(float* __restrict__ U, i64 ld, i64 m, i64 r, const float* __restrict__ diag) {
   const i64 total = m * r;
   for (i64 e = (i64)blockIdx.x * blockDim.x + threadIdx.x; e < total; e += (i64)gridDim.x * blockDim.x) {
-    const i64 i = e / r, c = e % r;
+    const i64 i = row_of(e, r), c = e - i * r;
     if (diag[c] < 0.f) U[i * ld + c] = -U[i * ld + c];
   }
 }

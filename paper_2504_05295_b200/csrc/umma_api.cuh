@@ -13,6 +13,13 @@ int pair_clusters(int sm_count);
 // One-time set-up of the tensor-core kernels: opt in to their dynamic shared memory.
 int umma_configure();
 
+// Shapes the tensor engine may take (alignment decides the rest).
+inline bool umma_shape_ok(const GemmArgs& g, int precision) {
+  const int epc = (g.ab16 || precision == DION_PREC_BF16_OPERANDS) ? 8 : 4;
+  return g.M >= 128 && g.N >= 64 && g.K >= 64 && g.M % epc == 0 && g.N % epc == 0 && g.K % epc == 0;
+}
+
+
 // Launches the product on the tensor cores if it qualifies.  Returns the number of
 // kernels launched (1, or 2 with a split-K reduction), 0 if this engine does not take
 // the product, or a negative DION_ERR_* code.
