@@ -621,15 +621,25 @@ __global__ void __launch_bounds__(FLOW_THREADS, 1) k_chol_flow(const __grid_cons
     for (int j = 0; j < 4; ++j)
 #pragma unroll
       for (int x = 0; x < 4; ++x) v[j][x] = 0.f;
+    // (four partial sums' loads in flight: one after another, 16 partial sums of the first three tiles were 19 us of latency)
 #pragma unroll 1
-    for (int q = 0; q < n; ++q, p += ld * ld) {
+    for (int q = 0; q < n; q += 4, p += 4 * ld * ld) {
+      float w[4][4][4];
 #pragma unroll
-      for (int j = 0; j < 4; ++j)
+      for (int u = 0; u < 4; ++u)
 #pragma unroll
-        for (int x = 0; x < 4; ++x) {
-          const int dr = (x & 2) ? 8 : 0, dc = 16 * j + (x & 1);
-          if (dr < nr && dc < nc) v[j][x] += __ldcg(p + dr * ld + dc);
-        }
+        for (int j = 0; j < 4; ++j)
+#pragma unroll
+          for (int x = 0; x < 4; ++x) {
+            const int dr = (x & 2) ? 8 : 0, dc = 16 * j + (x & 1);
+            w[u][j][x] = (q + u < n && dr < nr && dc < nc) ? __ldcg(p + u * ld * ld + dr * ld + dc) : 0.f;
+          }
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+#pragma unroll
+          for (int x = 0; x < 4; ++x) v[j][x] += w[u][j][x];
     }
     if (f.part != nullptr && f.alpha_dev != nullptr) {
       const float al = f.alpha_dev[(i64)b * f.alpha_stride];

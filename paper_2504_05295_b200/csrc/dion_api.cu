@@ -308,12 +308,12 @@ cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t s
 // Products on the fp32 FMA engine.
 // Splits of K: a K step of 16 takes about as long as the latency of its loads whatever runs beside it, so a product of few tiles is
 // cut to two or three steps per block, up to two blocks per SM (1001 x 83 x 333 with the reduction: 28.6 -> 14 us).
-// Fewer where the next kernel adds the partial sums up itself (k_chol_flow).
+// Fewer where the next kernel adds the partial sums up itself (k_chol_flow: one CTA reads those of the first three tiles, which
+// costs it as much per split as a K step here).
 constexpr i64 SPLIT_MIN_K = 32;
 constexpr i64 SPLIT_MAX = 64;
-constexpr i64 SPLIT_MIN_K_DEFERRED = 128;
 constexpr i64 SIMT_THIN_N = 32;          // outputs of at most this many columns take 128 x 32 tiles
-constexpr i64 SIMT_WIDE_MIN_K = 96;      // updates of C below it are bound by C: 64 x 64 tiles, three blocks per SM
+constexpr i64 SIMT_WIDE_MIN_K = 96;      // updates of C below it are bound by C: 64 x 64 tiles
 
 // tabs != nullptr: the same product on nb matrices (operands from the tables, partial sums part_stride floats apart; outputs too
 // where the reduction follows).  Tiles and splits are those of one matrix: the same bits.
@@ -332,8 +332,7 @@ int launch_gemm_simt(dion_ctx* c, GemmArgs g, cudaStream_t st, float* part, i64 
     const i64 kmax = g.K / SPLIT_MIN_K;
     if (want > kmax) want = kmax;
     if (want > SPLIT_MAX) want = SPLIT_MAX;
-    const i64 most = g.K / SPLIT_MIN_K_DEFERRED;
-    if (g.splits_out != nullptr && want > most) want = most;
+    if (g.splits_out != nullptr) while (want > 1 && want * want * 16 > g.K) --want;
     while (want > 1 && want * g.M * g.N > part_floats) --want;
     if (want > 1) {
       const i64 per = ((g.K + want - 1) / want + 15) / 16 * 16;      // as the kernel cuts K; no empty split
@@ -353,11 +352,11 @@ int launch_gemm_simt(dion_ctx* c, GemmArgs g, cudaStream_t st, float* part, i64 
     g.bs2 = part_stride;
     if (use128) launch_pdl(k_gemm_simt<128, 128, 8, 8, 8, 1, GemmTabs>, grid, dim3(256), 0, st, g, *tabs, inner);
     else if (thin) launch_pdl(k_gemm_simt<128, 32, 16, 4, 4, 2, GemmTabs>, grid, dim3(256), 0, st, g, *tabs, inner);
-    else launch_pdl(k_gemm_simt<64, 64, 16, 4, 4, 3, GemmTabs>, grid, dim3(256), 0, st, g, *tabs, inner);
+    else launch_pdl(k_gemm_simt<64, 64, 16, 4, 4, 2, GemmTabs>, grid, dim3(256), 0, st, g, *tabs, inner);
   } else {
     if (use128) launch_pdl(k_gemm_simt<128, 128, 8, 8, 8, 1, NoTabs>, grid, dim3(256), 0, st, g, NoTabs(), 1);
     else if (thin) launch_pdl(k_gemm_simt<128, 32, 16, 4, 4, 2, NoTabs>, grid, dim3(256), 0, st, g, NoTabs(), 1);
-    else launch_pdl(k_gemm_simt<64, 64, 16, 4, 4, 3, NoTabs>, grid, dim3(256), 0, st, g, NoTabs(), 1);
+    else launch_pdl(k_gemm_simt<64, 64, 16, 4, 4, 2, NoTabs>, grid, dim3(256), 0, st, g, NoTabs(), 1);
   }
   DION_CHECK_LAUNCH(c);
   if (g.splits_out != nullptr) { *g.splits_out = splits; return DION_OK; }      // (the caller sums the partial products itself)
@@ -2903,7 +2902,7 @@ bool touch_kernel(K kernel) {
 // tensor-core variants are covered by configure_kernels, which sets an attribute on each).
 bool preload_kernels() {
   bool ok = true;
-  ok = ok && touch_kernel(k_gemm_simt<128, 128, 8, 8, 8, 1, NoTabs>) && touch_kernel(k_gemm_simt<64, 64, 16, 4, 4, 3, NoTabs>) &&
+  ok = ok && touch_kernel(k_gemm_simt<128, 128, 8, 8, 8, 1, NoTabs>) && touch_kernel(k_gemm_simt<64, 64, 16, 4, 4, 2, NoTabs>) &&
        touch_kernel(k_gemm_simt<128, 32, 16, 4, 4, 2, NoTabs>);
   ok = ok && touch_kernel(k_splitk_reduce) && touch_kernel(k_round_begin) && touch_kernel(k_chol_flow<true>);
   ok = ok && touch_kernel(k_chol_flow<false>) && touch_kernel(k_round_end) && touch_kernel(k_tiny_cholqr2);
