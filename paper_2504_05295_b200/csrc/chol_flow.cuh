@@ -630,9 +630,16 @@ __global__ void __launch_bounds__(FLOW_THREADS, 1) k_chol_flow(const __grid_cons
 #pragma unroll
         for (int j = 0; j < 4; ++j)
 #pragma unroll
-          for (int x = 0; x < 4; ++x) {
-            const int dr = (x & 2) ? 8 : 0, dc = 16 * j + (x & 1);
-            w[u][j][x] = (q + u < n && dr < nr && dc < nc) ? __ldcg(p + u * ld * ld + dr * ld + dc) : 0.f;
+          for (int h = 0; h < 2; ++h) {
+            const int dr = 8 * h, dc = 16 * j;
+            const float* e = p + u * ld * ld + dr * ld + dc;
+            if (VEC) {      // (cols is even; whole sectors: with single words the CTA moved twice the bytes)
+              const float2 t = (q + u < n && dr < nr && dc < nc) ? __ldcg(reinterpret_cast<const float2*>(e)) : make_float2(0.f, 0.f);
+              w[u][j][2 * h] = t.x; w[u][j][2 * h + 1] = t.y;
+            } else {
+              w[u][j][2 * h] = (q + u < n && dr < nr && dc < nc) ? __ldcg(e) : 0.f;
+              w[u][j][2 * h + 1] = (q + u < n && dr < nr && dc + 1 < nc) ? __ldcg(e + 1) : 0.f;
+            }
           }
 #pragma unroll
       for (int u = 0; u < 4; ++u)
@@ -656,9 +663,15 @@ __global__ void __launch_bounds__(FLOW_THREADS, 1) k_chol_flow(const __grid_cons
 #pragma unroll
     for (int j = 0; j < 4; ++j)
 #pragma unroll
-      for (int x = 0; x < 4; ++x) {
-        const int dr = (x & 2) ? 8 : 0, dc = 16 * j + (x & 1);
-        v[j][x] = (dr < nr && dc < nc) ? __ldcg(p + dr * ld + dc) : 0.f;
+      for (int h = 0; h < 2; ++h) {
+        const int dr = 8 * h, dc = 16 * j;
+        if (VEC) {
+          const float2 t = (dr < nr && dc < nc) ? __ldcg(reinterpret_cast<const float2*>(p + dr * ld + dc)) : make_float2(0.f, 0.f);
+          v[j][2 * h] = t.x; v[j][2 * h + 1] = t.y;
+        } else {
+          v[j][2 * h] = (dr < nr && dc < nc) ? __ldcg(p + dr * ld + dc) : 0.f;
+          v[j][2 * h + 1] = (dr < nr && dc + 1 < nc) ? __ldcg(p + dr * ld + dc + 1) : 0.f;
+        }
       }
   };
   auto store_tile = [&](float* p, int rows, int cols, const float (&v)[4][4]) {
