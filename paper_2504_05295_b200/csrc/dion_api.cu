@@ -140,7 +140,7 @@ void colnorm_plan(i64 rows, i64 r, int sm, int* chunks, i64* rows_per) {
 // 12 us against the 55 rows that one wave of blocks would take), more on tall panels (512 chunks of partial sums).
 void probe_plan(i64 rows, int* chunks, i64* rows_per) {
   i64 per = (rows + 511) / 512;
-  if (per < 32) per = 32;
+  per = (per + 31) / 32 * 32;
   *rows_per = per;
   *chunks = (int)((rows + per - 1) / per);
 }
@@ -559,6 +559,7 @@ int launch_gemm_group(StepCtx& s, const std::vector<GemmArgs>& v) {
 int configure_kernels() {
   if (umma_configure() != DION_OK) return DION_ERR_CUDA;
   if (cudaFuncSetAttribute(k_probe_y4, cudaFuncAttributeMaxDynamicSharedMemorySize, PY_SMEM) != cudaSuccess ||
+      cudaFuncSetAttribute(k_probe_fused, cudaFuncAttributeMaxDynamicSharedMemorySize, PF_SMEM_MAX) != cudaSuccess ||
       cudaFuncSetAttribute(k_chol_flow<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, FLOW_SMEM) != cudaSuccess ||
       cudaFuncSetAttribute(k_chol_flow<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, FLOW_SMEM) != cudaSuccess ||
       cudaFuncSetAttribute(k_tiny_cholqr2, cudaFuncAttributeMaxDynamicSharedMemorySize, tiny_cholqr2_smem(TINY_MAX_ROWS)) != cudaSuccess) {
@@ -753,22 +754,27 @@ int probe(StepCtx& s, i64 off, i64 rows, i64 r, int phase) {
   int chunks; i64 per;
   probe_plan(rows, &chunks, &per);
   const int* keep = (phase == PROBE_AFTER_REDO) ? (const int*)(s.os + OS_DONE) : nullptr;
-  if (r % 4 == 0 && r >= 128) {
-    i64 blocks = (rows + 31) / 32;          // a block of 8 warps takes 32 rows at a time
-    if (blocks > 2 * (i64)c->sm_count) blocks = 2 * (i64)c->sm_count;
-    launch_pdl(k_probe_y4, dim3((unsigned)blocks, (unsigned)s.nb), dim3(256), (size_t)PY_SMEM, s.st, (const float*)(s.ws + off), r, rows, r,
-               s.ws + s.L.probe_y, s.wstride, keep);
+  const float* U = s.ws + off;
+  if (r % 4 == 0 && r <= PF_MAX_R) {
+    int ct_log = 3;                         // threads by columns: 8 .. 256
+    while (4 << ct_log < r) ++ct_log;
+    const size_t smem = (size_t)(((r + 127) / 128 * 128) * NPROBE + PF_RED + 32 * NPROBE) * sizeof(float);
+    launch_pdl(k_probe_fused, dim3((unsigned)chunks, (unsigned)s.nb), dim3(256), smem, s.st, U, r, rows, r, per, s.ws + s.L.probe_part, s.wstride, keep, ct_log);
   } else {
-    launch_pdl(k_probe_y, dim3((unsigned)grid_for(c, rows * 32, s.nb), (unsigned)s.nb), dim3(256), 0, s.st, (const float*)(s.ws + off), r,
-               rows, r, s.ws + s.L.probe_y, s.wstride, keep);
+    if (r % 4 == 0) {
+      i64 blocks = (rows + 31) / 32;          // a block of 8 warps takes 32 rows at a time
+      if (blocks > 2 * (i64)c->sm_count) blocks = 2 * (i64)c->sm_count;
+      launch_pdl(k_probe_y4, dim3((unsigned)blocks, (unsigned)s.nb), dim3(256), (size_t)PY_SMEM, s.st, U, r, rows, r, s.ws + s.L.probe_y, s.wstride, keep);
+      DION_CHECK_LAUNCH(c);
+      launch_pdl(k_probe_w4, dim3((unsigned)((r / 4 + 127) / 128), (unsigned)chunks, (unsigned)s.nb), dim3(128), 0, s.st, U, r, rows, r, per,
+                 (const float*)(s.ws + s.L.probe_y), s.ws + s.L.probe_part, s.wstride, keep);
+    } else {
+      launch_pdl(k_probe_y, dim3((unsigned)grid_for(c, rows * 32, s.nb), (unsigned)s.nb), dim3(256), 0, s.st, U, r, rows, r, s.ws + s.L.probe_y, s.wstride, keep);
+      DION_CHECK_LAUNCH(c);
+      launch_pdl(k_probe_w, dim3((unsigned)((r + 127) / 128), (unsigned)chunks, (unsigned)s.nb), dim3(128), 0, s.st, U, r, rows, r, per,
+                 (const float*)(s.ws + s.L.probe_y), s.ws + s.L.probe_part, s.wstride, keep);
+    }
   }
-  DION_CHECK_LAUNCH(c);
-  if (r % 4 == 0)
-    launch_pdl(k_probe_w4, dim3((unsigned)((r / 4 + 127) / 128), (unsigned)chunks, (unsigned)s.nb), dim3(128), 0, s.st,
-               (const float*)(s.ws + off), r, rows, r, per, (const float*)(s.ws + s.L.probe_y), s.ws + s.L.probe_part, s.wstride, keep);
-  else
-    launch_pdl(k_probe_w, dim3((unsigned)((r + 127) / 128), (unsigned)chunks, (unsigned)s.nb), dim3(128), 0, s.st,
-               (const float*)(s.ws + off), r, rows, r, per, (const float*)(s.ws + s.L.probe_y), s.ws + s.L.probe_part, s.wstride, keep);
   DION_CHECK_LAUNCH(c);
   launch_pdl(k_probe_decide, dim3((unsigned)probe_sums(r), (unsigned)s.nb), dim3(PD_ENTRIES * PD_GROUPS), 0, s.st, (const float*)(s.ws + s.L.probe_part), chunks,
              r, s.os, ORTH_TAU_F, c->dev_ints + 2, s.ws + s.L.probe_sums, s.wstride, phase);
@@ -2906,7 +2912,7 @@ bool preload_kernels() {
        touch_kernel(k_gemm_simt<128, 32, 16, 4, 4, 2, NoTabs>);
   ok = ok && touch_kernel(k_splitk_reduce) && touch_kernel(k_round_begin) && touch_kernel(k_chol_flow<true>);
   ok = ok && touch_kernel(k_chol_flow<false>) && touch_kernel(k_round_end) && touch_kernel(k_tiny_cholqr2);
-  ok = ok && touch_kernel(k_probe_y) && touch_kernel(k_probe_y4) && touch_kernel(k_probe_w) && touch_kernel(k_probe_w4) && touch_kernel(k_probe_decide) && touch_kernel(k_reset_rounds);
+  ok = ok && touch_kernel(k_probe_fused) && touch_kernel(k_probe_y) && touch_kernel(k_probe_y4) && touch_kernel(k_probe_w) && touch_kernel(k_probe_w4) && touch_kernel(k_probe_decide) && touch_kernel(k_reset_rounds);
   ok = ok && touch_kernel(k_orth_finish) && touch_kernel(k_cgs_fallback) && touch_kernel(k_copy_block);
   ok = ok && touch_kernel(k_colsumsq_partial<true>) && touch_kernel(k_colsumsq_partial<false>) &&
        touch_kernel(k_colnorm_apply<true>) && touch_kernel(k_colnorm_apply<false>) && touch_kernel(k_copy_panel);

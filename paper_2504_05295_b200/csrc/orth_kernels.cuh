@@ -521,7 +521,7 @@ __global__ void __launch_bounds__(256) k_probe_y(const float* __restrict__ U, i6
   }
 }
 
-// The same for r a multiple of 4 (16-byte aligned rows): the +-1 entries of the probe vectors are hashed once per
+// The same for wider panels (r a multiple of 4 above PF_MAX_R; 16-byte aligned rows): the +-1 entries of the probe vectors are hashed once per
 // CTA and column block into a shared-memory table of floats instead of once per matrix element (the hash made the
 // plain kernel ALU bound at a seventh of HBM speed), and a warp takes four rows at a time so that one read of a
 // column's eight signs serves four elements.  Lane l owns columns 128 t + 4 l .. + 3 of a block of PY_COLS
@@ -620,7 +620,7 @@ __global__ void __launch_bounds__(128) k_probe_w(const float* __restrict__ U, i6
   for (int p = 0; p < NPROBE; ++p) out[p] = acc[p];
 }
 
-// The same for r a multiple of 4: a thread takes four neighbouring columns (one 16-byte load per row, eight rows'
+// The same for wide panels, r a multiple of 4: a thread takes four neighbouring columns (one 16-byte load per row, eight rows'
 // loads in flight); every column's sum runs over the chunk's rows in the same order as above.
 // grid = (ceil(r/512), chunks, matrices).
 __global__ void __launch_bounds__(128) k_probe_w4(const float* __restrict__ U, i64 ld, i64 rows, i64 r,
@@ -657,6 +657,113 @@ __global__ void __launch_bounds__(128) k_probe_w4(const float* __restrict__ U, i
   for (int c = 0; c < 4; ++c) {
     out[2 * c] = make_float4(acc[c][0], acc[c][1], acc[c][2], acc[c][3]);
     out[2 * c + 1] = make_float4(acc[c][4], acc[c][5], acc[c][6], acc[c][7]);
+  }
+}
+
+// Both passes in one launch for r a multiple of 4 up to PF_MAX_R: a block takes 32 rows at a time (they stay in L1 between the
+// passes), its warps four rows each for Y = U z, then (1 << ct_log) threads by four columns and the rest by row groups for
+// U^T Y.  Two launches read the panel twice from L2 and met in memory: 2048 x 128 14.5 us, 4096 x 1024 23 us (now 5 and 15 us).
+// grid = (chunks, matrices); part[chunk][j][p] as in k_probe_w.
+constexpr i64 PF_MAX_R = 1024;
+constexpr int PF_RED = 256 * 4 * NPROBE;      // floats: row groups x columns x probes
+constexpr int PF_SMEM_MAX = ((int)PF_MAX_R * NPROBE + PF_RED + 32 * NPROBE) * 4;
+__global__ void __launch_bounds__(256) k_probe_fused(const float* __restrict__ U, i64 ld, i64 rows, i64 r, i64 rows_per_chunk,
+                                                     float* __restrict__ part, i64 wstride, const int* __restrict__ keep, int ct_log) {
+  extern __shared__ __align__(16) float pf_smem[];
+  pdl_enter();
+  if (keep != nullptr && keep[(i64)blockIdx.y * OS_SLOT_INTS] != 0) return;   // this panel's decision stands
+  U += (i64)blockIdx.y * wstride; part += (i64)blockIdx.y * wstride;
+  float* ys = pf_smem;                             // [32][NPROBE]
+  float* red = ys + 32 * NPROBE;                   // [row group][column][probe]
+  float* sign = red + PF_RED;                      // (layout of k_probe_y4)
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nr = (int)r;
+  for (int e = threadIdx.x; e < nr * NPROBE; e += 256) {
+    const int col = e / NPROBE, pr = e % NPROBE;
+    sign[((((col >> 7) * 4 + (col & 3)) * 2 + (pr >> 2)) * 32 + ((col & 127) >> 2)) * 4 + (pr & 3)] = probe_sign(col, pr);
+  }
+  __syncthreads();
+  const int groups = 256 >> ct_log, per = 32 / groups;      // row groups, rows of each (groups <= 32)
+  const int j0 = 4 * ((int)threadIdx.x & ((1 << ct_log) - 1)), grp = (int)threadIdx.x >> ct_log;
+  float w[4][NPROBE];
+#pragma unroll
+  for (int c = 0; c < 4; ++c)
+#pragma unroll
+    for (int p = 0; p < NPROBE; ++p) w[c][p] = 0.f;
+  const i64 b0 = (i64)blockIdx.x * rows_per_chunk, b1 = min(rows, b0 + rows_per_chunk);
+  for (i64 ib = b0; ib < b1; ib += 32) {
+    float acc[4][NPROBE];
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+#pragma unroll
+      for (int p = 0; p < NPROBE; ++p) acc[q][p] = 0.f;
+    const i64 i0 = ib + 4 * warp;
+    for (int j = 4 * lane; j < nr; j += 128) {
+      float4 v[4];
+#pragma unroll
+      for (int q = 0; q < 4; ++q)
+        v[q] = (i0 + q < b1) ? *reinterpret_cast<const float4*>(U + (i0 + q) * ld + j) : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+      for (int cc = 0; cc < 4; ++cc) {
+        const float4* su = reinterpret_cast<const float4*>(sign) + (((j >> 7) * 4 + cc) * 2) * 32 + lane;
+        const float4 s0 = su[0], s1 = su[32];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          const float x = (cc == 0) ? v[q].x : (cc == 1) ? v[q].y : (cc == 2) ? v[q].z : v[q].w;
+          acc[q][0] = fmaf(x, s0.x, acc[q][0]); acc[q][1] = fmaf(x, s0.y, acc[q][1]);
+          acc[q][2] = fmaf(x, s0.z, acc[q][2]); acc[q][3] = fmaf(x, s0.w, acc[q][3]);
+          acc[q][4] = fmaf(x, s1.x, acc[q][4]); acc[q][5] = fmaf(x, s1.y, acc[q][5]);
+          acc[q][6] = fmaf(x, s1.z, acc[q][6]); acc[q][7] = fmaf(x, s1.w, acc[q][7]);
+        }
+      }
+    }
+    // the 32 sums of the warp (4 rows x 8 probes): lane l ends up with sum l (each step halves what a lane still holds)
+    float v32[32];
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+#pragma unroll
+      for (int p = 0; p < NPROBE; ++p) v32[q * NPROBE + p] = acc[q][p];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      const bool up = (lane & o) != 0;
+#pragma unroll
+      for (int k = 0; k < o; ++k) {
+        const float send = up ? v32[k] : v32[k + o], mine = up ? v32[k + o] : v32[k];
+        v32[k] = mine + __shfl_xor_sync(0xffffffffu, send, o);
+      }
+    }
+    ys[warp * 32 + lane] = v32[0];      // (row 4 warp + lane / 8, probe lane % 8)
+    __syncthreads();
+    if (j0 < nr) {
+#pragma unroll 4
+      for (int q = 0; q < per; ++q) {
+        const int i = grp * per + q;
+        if (ib + i >= b1) break;
+        const float4 u4 = *reinterpret_cast<const float4*>(U + (ib + i) * ld + j0);
+        const float4 y0 = *reinterpret_cast<const float4*>(ys + i * NPROBE), y1 = *reinterpret_cast<const float4*>(ys + i * NPROBE + 4);
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+          const float x = (c == 0) ? u4.x : (c == 1) ? u4.y : (c == 2) ? u4.z : u4.w;
+          w[c][0] = fmaf(x, y0.x, w[c][0]); w[c][1] = fmaf(x, y0.y, w[c][1]); w[c][2] = fmaf(x, y0.z, w[c][2]); w[c][3] = fmaf(x, y0.w, w[c][3]);
+          w[c][4] = fmaf(x, y1.x, w[c][4]); w[c][5] = fmaf(x, y1.y, w[c][5]); w[c][6] = fmaf(x, y1.z, w[c][6]); w[c][7] = fmaf(x, y1.w, w[c][7]);
+        }
+      }
+    }
+    __syncthreads();
+  }
+  if (j0 < nr) {
+    float4* out = reinterpret_cast<float4*>(groups > 1 ? red + ((grp << ct_log) * 4 + j0) * NPROBE : part + ((i64)blockIdx.x * r + j0) * NPROBE);
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+      out[2 * c] = make_float4(w[c][0], w[c][1], w[c][2], w[c][3]);
+      out[2 * c + 1] = make_float4(w[c][4], w[c][5], w[c][6], w[c][7]);
+    }
+  }
+  if (groups == 1) return;
+  __syncthreads();
+  for (int e = threadIdx.x; e < nr * NPROBE; e += 256) {
+    float s = 0.f;
+    for (int g = 0; g < groups; ++g) s += red[((g << ct_log) * 4) * NPROBE + e];
+    part[(i64)blockIdx.x * r * NPROBE + e] = s;
   }
 }
 
