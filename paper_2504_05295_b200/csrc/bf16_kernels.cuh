@@ -8,6 +8,11 @@
 
 namespace dion {
 
+// The first kernel of a step clears the state slots of the chain's matrices (blockIdx.y; a memset of its own was 2 us).
+__device__ __forceinline__ void clear_slot(int* slots) {
+  if (slots != nullptr && blockIdx.x == 0 && threadIdx.x < OS_SLOT_INTS) slots[blockIdx.y * OS_SLOT_INTS + threadIdx.x] = 0;
+}
+
 __device__ __forceinline__ uint32_t pack_bf16x2(float a, float b) {
   const __nv_bfloat162 v = __floats2bfloat162_rn(a, b);
   return *reinterpret_cast<const uint32_t*>(&v);
@@ -19,8 +24,9 @@ __device__ __forceinline__ uint32_t pack_bf16x2(float a, float b) {
 template <bool VEC>
 __global__ void __launch_bounds__(256) k_form_b16(const float* __restrict__ M, i64 ldm, const void* __restrict__ G,
                                                   i64 ldg, int g_mode, i64 rows, i64 cols,
-                                                  __nv_bfloat16* __restrict__ out) {
+                                                  __nv_bfloat16* __restrict__ out, int* __restrict__ slots) {
   pdl_enter();
+  clear_slot(slots);
   const i64 per_row = cols / 8;
   const i64 total = rows * per_row;
   for (i64 e = (i64)blockIdx.x * blockDim.x + threadIdx.x; e < total; e += (i64)gridDim.x * blockDim.x) {
@@ -134,8 +140,9 @@ __device__ __forceinline__ void form_b32_body(const float* __restrict__ M, i64 l
 template <bool VEC>
 __global__ void __launch_bounds__(256, 3) k_form_b32(const float* __restrict__ M, i64 ldm, const void* __restrict__ G,
                                                   i64 ldg, int g_mode, i64 rows, i64 cols, float* __restrict__ out,
-                                                  __nv_bfloat16* __restrict__ hi, __nv_bfloat16* __restrict__ lo) {
+                                                  __nv_bfloat16* __restrict__ hi, __nv_bfloat16* __restrict__ lo, int* __restrict__ slots) {
   pdl_enter();
+  clear_slot(slots);
   form_b32_body<VEC>(M, ldm, G, ldg, g_mode, rows, cols, out, hi, lo);
 }
 // The same for every matrix of a chain in one launch (blockIdx.y): the caller's M and G from pointer tables, the
@@ -144,8 +151,9 @@ template <bool VEC>
 __global__ void __launch_bounds__(256, 3) k_form_b32_chain(const ChainPtrs Ms, i64 ldm, const ChainPtrs Gs, i64 ldg, int g_mode,
                                                         i64 rows, i64 cols, float* __restrict__ out,
                                                         __nv_bfloat16* __restrict__ hi, __nv_bfloat16* __restrict__ lo,
-                                                        i64 ostride) {
+                                                        i64 ostride, int* __restrict__ slots) {
   pdl_enter();
+  clear_slot(slots);
   const i64 b = blockIdx.y;
   form_b32_body<VEC>(reinterpret_cast<const float*>(Ms.p[b]), ldm, Gs.p[b], ldg, g_mode, rows, cols, out + b * ostride,
                      hi != nullptr ? hi + 2 * b * ostride : nullptr, lo != nullptr ? lo + 2 * b * ostride : nullptr);
@@ -342,8 +350,9 @@ __global__ void __launch_bounds__(256, 3) k_form_b32_amax(const float* __restric
 template <bool VEC>
 __global__ void __launch_bounds__(256, 3) k_form_sum_amax(const ChainPtrs Ms, i64 ldm, const ChainPtrs Gs, i64 ldg, int g_mode, i64 rows, i64 cols,
                                                        const ChainPtrs Qs, i64 ldq, i64 qrows, i64 qcols, int qvec, float* __restrict__ out,
-                                                       float* __restrict__ part, i64 wstride) {
+                                                       float* __restrict__ part, i64 wstride, int* __restrict__ slots) {
   pdl_enter();
+  clear_slot(slots);
   const i64 b = blockIdx.y;
   part += b * wstride;
   float m = 0.f, mq = 0.f;

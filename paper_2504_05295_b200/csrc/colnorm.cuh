@@ -148,10 +148,14 @@ template <bool V4>
 __global__ void __launch_bounds__(CN_THREADS, 3) k_colnorm_apply(const float* __restrict__ R, i64 ldr, i64 n, i64 r, i64 rows_per_chunk, int chunks,
                                                               const float* __restrict__ part, float eps, const ChainPtrs Qs, i64 ldq, int qvec,
                                                               float* __restrict__ d_ws, const ChainPtrs ds, int* __restrict__ status,
-                                                              const int* __restrict__ skip_flag, i64 wstride, ColnormPairs x) {
+                                                              const int* __restrict__ skip_flag, i64 wstride, ColnormPairs x,
+                                                              int* __restrict__ skipped) {
   pdl_enter();
   const i64 b = blockIdx.z;
-  if (skip_flag != nullptr && skip_flag[b * OS_SLOT_INTS] != 0) return;
+  if (skip_flag != nullptr && skip_flag[b * OS_SLOT_INTS] != 0) {
+    if (threadIdx.x == 0 && blockIdx.x == 0 && blockIdx.y == 0) atomicAdd(skipped, 1);      // (once per step: the count of cancelled steps)
+    return;
+  }
   __shared__ float red[CN_WARPS][128];
   __shared__ float redm[CN_WARPS];
   R += b * wstride; part += b * wstride; d_ws += b * wstride;

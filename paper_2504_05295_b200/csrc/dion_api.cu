@@ -115,6 +115,7 @@ struct dion_ctx {
     int64_t launches;
     int index;            // its state slot and scalar
     uint64_t last_use;
+    float scale;          // the scalar's value on the device (NaN: none yet)
   };
   std::vector<GraphEntry> graphs;
   bool graphs_on = false;
@@ -1159,7 +1160,8 @@ i64 panel_offset(const StepCtx& s, i64 r, i64 short_dim) {
 }
 
 // The device-side fallback of CholeskyQR2 (k_cgs_fallback): one cooperative launch over the chain's matrices.
-int cgs_fallback(StepCtx& s, i64 pin_off, i64 pout_off, i64 rows, i64 r) {
+// second_off >= 0: where the second round, if it ran, left its result (copied to pout_off by the same launch).
+int cgs_fallback(StepCtx& s, i64 pin_off, i64 pout_off, i64 rows, i64 r, i64 second_off = -1) {
   dion_ctx* c = s.c;
   i64 G = rows / 8;
   if (G < 1) G = 1;
@@ -1175,7 +1177,8 @@ int cgs_fallback(StepCtx& s, i64 pin_off, i64 pout_off, i64 rows, i64 r) {
   i64 ld = r, wstride = s.wstride;
   int nb = s.nb;
   long long limit = umma::SPIN_LIMIT_CYCLES;
-  void* args[] = {&Pin, &U, &ld, &rows, &r, &part, &hvec, &npart, &os, &status, &fallbacks, &wstride, &nb, &limit};
+  const float* second = second_off >= 0 ? s.ws + second_off : nullptr;
+  void* args[] = {&Pin, &U, &ld, &rows, &r, &part, &hvec, &npart, &os, &status, &fallbacks, &wstride, &nb, &limit, &second};
   if (cudaLaunchCooperativeKernel((const void*)k_cgs_fallback, dim3((unsigned)G), dim3(256), args, 0, s.st) != cudaSuccess) {
     cudaGetLastError();
     return DION_ERR_CUDA;
@@ -1224,8 +1227,8 @@ int orthonormalize(StepCtx& s, i64 rows, i64 r, i64 short_dim, i64 pin_off, i64*
     if (rc == DION_OK) rc = cholqr_round(s, s.L.P0, s.L.P1, rows, r, RM_CHECKED, 0, redo ? PROBE_AFTER_REDO : PROBE_CHECK);
     s.quiet_fail = false;
     DION_TRY(rc);
-    DION_TRY(second_round_back(s, rows, r));
-    if (fb) DION_TRY(cgs_fallback(s, pin_off, s.L.P0, rows, r));   // else: the failed pivot was reported as a breakdown
+    if (fb) DION_TRY(cgs_fallback(s, pin_off, s.L.P0, rows, r, s.L.P1));      // (which also brings the second round's result back)
+    else DION_TRY(second_round_back(s, rows, r));                           // (the failed pivot was reported as a breakdown)
     *U_off = s.L.P0;
   } else if (mode == DION_ORTH_SHIFTED3) {
     DION_TRY(adaptive_rounds(s, s.L.P0, s.L.P1, rows, r, 0));
@@ -1273,9 +1276,9 @@ int colnorm_launch(StepCtx& s, int b, int per, const float* W, i64 ldw, i64 rows
   const dim3 agrid(grid.x, (unsigned)((rows + rpb - 1) / rpb), grid.z);
   const float* sp = sums != nullptr ? sums : (const float*)part;
   if (v4) launch_pdl(k_colnorm_apply<true>, agrid, dim3(CN_THREADS), 0, s.st, W, ldw, rows, r, rpb, chunks, sp, c->cfg.eps, Qs, ldq, qvec, s.W(b, s.L.d), ds,
-                     c->dev_ints, skip, s.wstride, x);
+                     c->dev_ints, skip, s.wstride, x, c->dev_ints + 1);
   else launch_pdl(k_colnorm_apply<false>, agrid, dim3(CN_THREADS), 0, s.st, W, ldw, rows, r, rpb, chunks, sp, c->cfg.eps, Qs, ldq, qvec, s.W(b, s.L.d), ds,
-                  c->dev_ints, skip, s.wstride, x);
+                  c->dev_ints, skip, s.wstride, x, c->dev_ints + 1);
   DION_CHECK_LAUNCH(c);
   return DION_OK;
 }
@@ -1427,7 +1430,7 @@ int validate(const dion_matrix* a, bool shard = false) {
   return DION_OK;
 }
 
-int begin_step(dion_ctx* c, const dion_matrix* a, int nb, cudaStream_t st, StepCtx* s, int fixed_slot = -1) {
+int begin_step(dion_ctx* c, const dion_matrix* a, int nb, cudaStream_t st, StepCtx* s, int fixed_slot = -1, bool clear = true) {
   s->c = c;
   s->st = st;
   s->L = make_layout(c, a->m, a->n, a->r);
@@ -1444,7 +1447,7 @@ int begin_step(dion_ctx* c, const dion_matrix* a, int nb, cudaStream_t st, StepC
   s->flag = s->os + OS_FAIL;
   s->tensor = (c->cfg.engine != DION_ENGINE_SIMT);
   s->in_orth = false;
-  if (cudaMemsetAsync(s->os, 0, sizeof(int) * OS_SLOT_INTS * nb, st) != cudaSuccess) return DION_ERR_CUDA;
+  if (clear && cudaMemsetAsync(s->os, 0, sizeof(int) * OS_SLOT_INTS * nb, st) != cudaSuccess) return DION_ERR_CUDA;
   return DION_OK;
 }
 
@@ -1470,7 +1473,7 @@ bool step_on_half_pairs(const StepCtx& s, i64 m, i64 n, i64 r, i64 short_dim) {
 
 // M + G and the half pairs of it and of Q (in S16) for every matrix of the chain: in one pair of launches when they share
 // leading dimensions and alignment.
-int half_sum_chain(StepCtx& s, const dion_matrix* const* list, i64 qrow) {
+int half_sum_chain(StepCtx& s, const dion_matrix* const* list, i64 qrow, bool clear = false) {
   dion_ctx* c = s.c;
   const dion_matrix* a0 = list[0];
   const i64 m = a0->m, n = a0->n, r = a0->r;
@@ -1492,8 +1495,8 @@ int half_sum_chain(StepCtx& s, const dion_matrix* const* list, i64 qrow) {
     const dim3 fg((unsigned)grid_for(c, m * n / 4, per), (unsigned)per), sg((unsigned)grid_for(c, (m * n + qrow * r) / 8, per), (unsigned)per);
     float* part = s.W(b, s.L.part);      // (the maxima are read before the products write their partial sums there)
     const int qv = qvec_ok(a) ? 1 : 0;
-    if (vec_ok(a)) launch_pdl(k_form_sum_amax<true>, fg, dim3(256), 0, s.st, Ms, a->ldm, Gs, a->ldg, g_mode, m, n, Qs, a->ldq, qrow, r, qv, s.W(b, s.L.B32), part, s.wstride);
-    else launch_pdl(k_form_sum_amax<false>, fg, dim3(256), 0, s.st, Ms, a->ldm, Gs, a->ldg, g_mode, m, n, Qs, a->ldq, qrow, r, qv, s.W(b, s.L.B32), part, s.wstride);
+    if (vec_ok(a)) launch_pdl(k_form_sum_amax<true>, fg, dim3(256), 0, s.st, Ms, a->ldm, Gs, a->ldg, g_mode, m, n, Qs, a->ldq, qrow, r, qv, s.W(b, s.L.B32), part, s.wstride, clear ? s.OS(b) : (int*)nullptr);
+    else launch_pdl(k_form_sum_amax<false>, fg, dim3(256), 0, s.st, Ms, a->ldm, Gs, a->ldg, g_mode, m, n, Qs, a->ldq, qrow, r, qv, s.W(b, s.L.B32), part, s.wstride, clear ? s.OS(b) : (int*)nullptr);
     DION_CHECK_LAUNCH(c);
     launch_pdl(k_split_sum, sg, dim3(256), 0, s.st, (const float*)s.W(b, s.L.B32), m * n, Qs, a->ldq, qrow, r, qv, (const float*)part, (int)fg.x,
                reinterpret_cast<__half*>(s.W(b, s.L.Bp)), reinterpret_cast<__half*>(s.W(b, s.L.S16)), s.W(b, s.L.lz), s.wstride);
@@ -1503,7 +1506,7 @@ int half_sum_chain(StepCtx& s, const dion_matrix* const* list, i64 qrow) {
 }
 
 // Forms M + G in scratch (fp32) and, when `pair`, as a bf16 pair beside it.
-int form_sum(StepCtx& s, int b, const dion_matrix* a, bool pair) {
+int form_sum(StepCtx& s, int b, const dion_matrix* a, bool pair, bool clear = false) {
   dion_ctx* c = s.c;
   const i64 m = a->m, n = a->n;
   const bool vec = !((uintptr_t)a->M & 15) && a->ldm % 4 == 0 &&
@@ -1513,14 +1516,14 @@ int form_sum(StepCtx& s, int b, const dion_matrix* a, bool pair) {
   const int grid = grid_for(c, m * n / 4);
   __nv_bfloat16* bh = pair ? reinterpret_cast<__nv_bfloat16*>(s.W(b, s.L.Bp)) : nullptr;
   __nv_bfloat16* bl = pair ? bh + m * n : nullptr;
-  if (vec) launch_pdl(k_form_b32<true>, grid, dim3(256), 0, s.st, (const float*)a->M, a->ldm, a->G, a->ldg, g_mode, m, n, s.W(b, s.L.B32), bh, bl);
-  else launch_pdl(k_form_b32<false>, grid, dim3(256), 0, s.st, (const float*)a->M, a->ldm, a->G, a->ldg, g_mode, m, n, s.W(b, s.L.B32), bh, bl);
+  if (vec) launch_pdl(k_form_b32<true>, grid, dim3(256), 0, s.st, (const float*)a->M, a->ldm, a->G, a->ldg, g_mode, m, n, s.W(b, s.L.B32), bh, bl, clear ? s.OS(b) : (int*)nullptr);
+  else launch_pdl(k_form_b32<false>, grid, dim3(256), 0, s.st, (const float*)a->M, a->ldm, a->G, a->ldg, g_mode, m, n, s.W(b, s.L.B32), bh, bl, clear ? s.OS(b) : (int*)nullptr);
   DION_CHECK_LAUNCH(c);
   return DION_OK;
 }
 
 // form_sum for every matrix of the chain: one launch when M and G share leading dimensions and alignment.
-int form_sum_chain(StepCtx& s, const dion_matrix* const* list, bool pair) {
+int form_sum_chain(StepCtx& s, const dion_matrix* const* list, bool pair, bool clear = false) {
   dion_ctx* c = s.c;
   const dion_matrix* a0 = list[0];
   auto vec_ok = [](const dion_matrix* a) {
@@ -1532,7 +1535,7 @@ int form_sum_chain(StepCtx& s, const dion_matrix* const* list, bool pair) {
   for (int b = 1; b < s.nb && one; ++b)
     one = list[b]->ldm == a0->ldm && list[b]->ldg == a0->ldg && list[b]->g_dtype == a0->g_dtype && vec_ok(list[b]) == vec;
   if (!one) {
-    for (int b = 0; b < s.nb; ++b) DION_TRY(form_sum(s, b, list[b], pair));
+    for (int b = 0; b < s.nb; ++b) DION_TRY(form_sum(s, b, list[b], pair, clear));
     return DION_OK;
   }
   const i64 m = a0->m, n = a0->n;
@@ -1542,8 +1545,8 @@ int form_sum_chain(StepCtx& s, const dion_matrix* const* list, bool pair) {
   __nv_bfloat16* bh = pair ? reinterpret_cast<__nv_bfloat16*>(s.ws + s.L.Bp) : nullptr;
   __nv_bfloat16* bl = pair ? bh + m * n : nullptr;
   const dim3 grid((unsigned)grid_for(c, m * n / 4, s.nb), (unsigned)s.nb);
-  if (vec) launch_pdl(k_form_b32_chain<true>, grid, dim3(256), 0, s.st, Ms, a0->ldm, Gs, a0->ldg, g_mode, m, n, s.ws + s.L.B32, bh, bl, s.wstride);
-  else launch_pdl(k_form_b32_chain<false>, grid, dim3(256), 0, s.st, Ms, a0->ldm, Gs, a0->ldg, g_mode, m, n, s.ws + s.L.B32, bh, bl, s.wstride);
+  if (vec) launch_pdl(k_form_b32_chain<true>, grid, dim3(256), 0, s.st, Ms, a0->ldm, Gs, a0->ldg, g_mode, m, n, s.ws + s.L.B32, bh, bl, s.wstride, clear ? s.os : (int*)nullptr);
+  else launch_pdl(k_form_b32_chain<false>, grid, dim3(256), 0, s.st, Ms, a0->ldm, Gs, a0->ldg, g_mode, m, n, s.ws + s.L.B32, bh, bl, s.wstride, clear ? s.os : (int*)nullptr);
   DION_CHECK_LAUNCH(c);
   return DION_OK;
 }
@@ -1694,7 +1697,7 @@ int step_batch(dion_ctx* c, const dion_matrix* const* list, int nb, float lr, cu
                const float* x_scale = nullptr, int fixed_slot = -1) {
   StepCtx s;
   const dion_matrix* a0 = list[0];
-  DION_TRY(begin_step(c, a0, nb, st, &s, fixed_slot));
+  DION_TRY(begin_step(c, a0, nb, st, &s, fixed_slot, false));      // (the state slots: by the kernel that forms M + G)
   const i64 m = a0->m, n = a0->n, r = a0->r;
   s.list = list;
   if (c->cfg.orth == DION_ORTH_RCQR) {
@@ -1751,8 +1754,9 @@ int step_batch(dion_ctx* c, const dion_matrix* const* list, int nb, float lr, cu
   // elementwise preparation for the whole chain: M + G (and its pair), the pair of Q where P takes pairs
   const float* srcs[MAX_CHAIN];
   i64 lds[MAX_CHAIN];
-  if (hstep) DION_TRY(half_sum_chain(s, list, qrow));
-  else if (b32) DION_TRY(form_sum_chain(s, list, bpair));
+  if (hstep) DION_TRY(half_sum_chain(s, list, qrow, true));
+  else if (b32) DION_TRY(form_sum_chain(s, list, bpair, true));
+  else if (!d16 && cudaMemsetAsync(s.os, 0, sizeof(int) * OS_SLOT_INTS * nb, st) != cudaSuccess) return DION_ERR_CUDA;
   const bool phalf = b32 && s.L.Bh > 0;
   bool p_half_ready = false;
   if (phalf) {      // the scaled half pairs of M + G and of Q, for the whole chain
@@ -1817,8 +1821,8 @@ int step_batch(dion_ctx* c, const dion_matrix* const* list, int nb, float lr, cu
                        (a->g_dtype == DION_BF16 ? (!((uintptr_t)a->G & 15) && a->ldg % 8 == 0)
                                                 : (!((uintptr_t)a->G & 15) && a->ldg % 4 == 0));
       const int grid = grid_for(c, m * n / 8);
-      if (vec) launch_pdl(k_form_b16<true>, grid, dim3(256), 0, st, (const float*)a->M, a->ldm, a->G, a->ldg, g_mode(a), m, n, bf(b, s.L.B16));
-      else launch_pdl(k_form_b16<false>, grid, dim3(256), 0, st, (const float*)a->M, a->ldm, a->G, a->ldg, g_mode(a), m, n, bf(b, s.L.B16));
+      if (vec) launch_pdl(k_form_b16<true>, grid, dim3(256), 0, st, (const float*)a->M, a->ldm, a->G, a->ldg, g_mode(a), m, n, bf(b, s.L.B16), s.OS(b));
+      else launch_pdl(k_form_b16<false>, grid, dim3(256), 0, st, (const float*)a->M, a->ldm, a->G, a->ldg, g_mode(a), m, n, bf(b, s.L.B16), s.OS(b));
       DION_CHECK_LAUNCH(c);
       DION_TRY(to_bf16((const float*)a->Q, a->ldq, qrow, r, bf(b, s.L.Q16)));
       p.ab16 = 1;
@@ -2060,8 +2064,6 @@ int step_batch(dion_ctx* c, const dion_matrix* const* list, int nb, float lr, cu
     else DION_TRY(x_update(s, b, a, Uf, r, Qf, a->ldq, other, rbuf, x_alpha, s.OS(b) + OS_FAIL, x_scale, &group[b], x_rounded, u_half, 0.f));
   }
   DION_TRY(launch_gemm_group(s, group));
-  launch_pdl(k_finish_step, dim3((unsigned)(nb)), dim3(1), 0, st, s.flag, c->dev_ints + 1);
-  DION_CHECK_LAUNCH(c);
   }
   return DION_OK;
 }
@@ -2130,14 +2132,19 @@ int step_graph(dion_ctx* c, const dion_matrix* a, float lr, cudaStream_t st) {
     const cudaError_t ie = cudaGraphInstantiate(&exec, graph, 0);
     cudaGraphDestroy(graph);
     if (ie != cudaSuccess || exec == nullptr) { cudaGetLastError(); c->graphs_on = false; return 1; }
-    c->graphs.push_back({*a, exec, nl, index, 0});
+    c->graphs.push_back({*a, exec, nl, index, 0, NAN});
     e = &c->graphs.back();
   }
   e->last_use = ++c->graph_clock;
-  k_set_scalar<<<1, 1, 0, st>>>(c->graph_scalars + e->index, lr * sqrtf((float)((double)a->m / (double)a->n)));
-  if (cudaGetLastError() != cudaSuccess) return DION_ERR_CUDA;
+  const float scale = lr * sqrtf((float)((double)a->m / (double)a->n));
+  if (!(e->scale == scale)) {      // (the learning rate changed)
+    k_set_scalar<<<1, 1, 0, st>>>(c->graph_scalars + e->index, scale);
+    if (cudaGetLastError() != cudaSuccess) return DION_ERR_CUDA;
+    e->scale = scale;
+    c->launches++;
+  }
   if (cudaGraphLaunch(e->exec, st) != cudaSuccess) { cudaGetLastError(); return DION_ERR_CUDA; }
-  c->launches += e->launches + 1;
+  c->launches += e->launches;
   return DION_OK;
 }
 
@@ -2246,8 +2253,6 @@ int lazy_pairs(StepCtx& s, const dion_matrix* a, float lr, int refresh) {
   x.alpha = ldexpf(lr * sqrtf((float)((double)m / (double)n)), -13);
   x.skip_flag = s.flag;
   DION_TRY(launch_gemm(s, x));
-  launch_pdl(k_finish_step, dim3(1), dim3(1), 0, st, (const int*)s.flag, c->dev_ints + 1);
-  DION_CHECK_LAUNCH(c);
   return DION_OK;
 }
 
@@ -2293,8 +2298,8 @@ int lazy_one(dion_ctx* c, const dion_matrix* a, float lr, int refresh, cudaStrea
     const bool vec = !((uintptr_t)a->M & 15) && a->ldm % 4 == 0 && !((uintptr_t)a->G & 15) &&
                      a->ldg % ((a->g_dtype == DION_BF16) ? 8 : 4) == 0;
     const dim3 grid((unsigned)grid_for(c, m * n / 8));
-    if (vec) launch_pdl(k_form_b16<true>, grid, dim3(256), 0, st, Mp, a->ldm, a->G, a->ldg, gmode, m, n, bf(s.L.B16));
-    else launch_pdl(k_form_b16<false>, grid, dim3(256), 0, st, Mp, a->ldm, a->G, a->ldg, gmode, m, n, bf(s.L.B16));
+    if (vec) launch_pdl(k_form_b16<true>, grid, dim3(256), 0, st, Mp, a->ldm, a->G, a->ldg, gmode, m, n, bf(s.L.B16), (int*)nullptr);
+    else launch_pdl(k_form_b16<false>, grid, dim3(256), 0, st, Mp, a->ldm, a->G, a->ldg, gmode, m, n, bf(s.L.B16), (int*)nullptr);
     DION_CHECK_LAUNCH(c);
   }
 
@@ -2380,8 +2385,6 @@ int lazy_one(dion_ctx* c, const dion_matrix* a, float lr, int refresh, cudaStrea
   x.alpha = lr * sqrtf((float)((double)m / (double)n));
   x.skip_flag = s.flag;
   DION_TRY(launch_gemm(s, x));
-  launch_pdl(k_finish_step, dim3((unsigned)(1)), dim3(1), 0, st, s.flag, c->dev_ints + 1);
-  DION_CHECK_LAUNCH(c);
   return DION_OK;
 }
 
@@ -2650,8 +2653,6 @@ int dion_dp_finish(dion_ctx* ctx, const dion_matrix* a, const float* U, const fl
     // X <- X - lr sqrt(m/n) U Q^T, as in dion_step (rounded copies in the two panel buffers of the scratch)
     DION_TRY(x_update(s, 0, a, U, r, (const float*)a->Q, a->ldq, s.ws + s.L.P1, s.ws + s.L.R, alpha, dp_flag));
   }
-  launch_pdl(k_finish_step, dim3((unsigned)(1)), dim3(1), 0, st, dp_flag, ctx->dev_ints + 1);
-  DION_CHECK_LAUNCH(ctx);
   return DION_OK;
 }
 
@@ -2765,8 +2766,6 @@ int dion_shard_finish(dion_ctx* ctx, const dion_matrix* a, int64_t n_total, cons
     // X <- X - lr sqrt(m / n_total) U Q^T on the shard's columns
     DION_TRY(x_update(s, 0, a, U, r, (const float*)a->Q, a->ldq, s.ws + s.L.P1, s.ws + s.L.R, alpha, flag));
   }
-  launch_pdl(k_finish_step, dim3(1), dim3(1), 0, st, flag, ctx->dev_ints + 1);
-  DION_CHECK_LAUNCH(ctx);
   return DION_OK;
 }
 
@@ -2916,7 +2915,7 @@ bool preload_kernels() {
   ok = ok && touch_kernel(k_orth_finish) && touch_kernel(k_cgs_fallback) && touch_kernel(k_copy_block);
   ok = ok && touch_kernel(k_colsumsq_partial<true>) && touch_kernel(k_colsumsq_partial<false>) &&
        touch_kernel(k_colnorm_apply<true>) && touch_kernel(k_colnorm_apply<false>) && touch_kernel(k_copy_panel);
-  ok = ok && touch_kernel(k_latch_flag) && touch_kernel(k_finish_step) && touch_kernel(k_hh_reflector);
+  ok = ok && touch_kernel(k_latch_flag) && touch_kernel(k_hh_reflector);
   ok = ok && touch_kernel(k_hh_apply) && touch_kernel(k_set_identity) && touch_kernel(k_sign_fix);
   ok = ok && touch_kernel(k_form_b16<true>) && touch_kernel(k_form_b16<false>) && touch_kernel(k_form_b32<true>);
   ok = ok && touch_kernel(k_form_b32<false>) && touch_kernel(k_to_bf16) && touch_kernel(k_round_tf32);

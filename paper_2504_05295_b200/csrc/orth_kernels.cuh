@@ -937,7 +937,7 @@ __global__ void __launch_bounds__(256) k_cgs_fallback(const float* __restrict__ 
                                                       i64 rows, i64 r, float* __restrict__ part, float* __restrict__ hvec,
                                                       float* __restrict__ npart, int* __restrict__ os_base,
                                                       int* __restrict__ status, int* __restrict__ fallbacks,
-                                                      i64 wstride, int nb, long long spin_limit) {
+                                                      i64 wstride, int nb, long long spin_limit, const float* __restrict__ second) {
   __shared__ float colj[CGS_MAX_ROWS_PER_CTA];
   __shared__ float red[9];
   __shared__ int s_dead;
@@ -949,7 +949,17 @@ __global__ void __launch_bounds__(256) k_cgs_fallback(const float* __restrict__ 
   const int nmy = (int)(i1 - i0);
   for (int b = 0; b < nb; ++b) {
     int* os = os_base + (i64)b * OS_SLOT_INTS;
-    if (os[OS_FAIL] == 0) continue;                 // written by an earlier launch: every CTA reads the same value
+    if (os[OS_FAIL] == 0) {                         // written by an earlier launch: every CTA reads the same value
+      if (second != nullptr && os[OS_DONE] == 0) {      // the second round ran: its result to where U is expected
+        const float* V = second + (i64)b * wstride;
+        float* Ub = U + (i64)b * wstride;
+        for (i64 e = (i64)c * 256 + tid; e < rows * r; e += (i64)G * 256) {
+          const i64 i = row_of(e, r), k = e - i * r;
+          Ub[i * ld + k] = V[i * r + k];
+        }
+      }
+      continue;
+    }
     const float* Pb = Pin + (i64)b * wstride;
     float* Ub = U + (i64)b * wstride;
     float* partb = part + (i64)b * wstride;
@@ -1077,12 +1087,6 @@ __global__ void k_copy_panel(const float* __restrict__ V, i64 ldv, float* __rest
 __global__ void k_latch_flag(const int* __restrict__ src, int* __restrict__ dst) {
   pdl_enter();
   if (*src != 0) *dst = 1;
-}
-
-// Counts a skipped step (breakdown) at the end of a step's launch chain.
-__global__ void k_finish_step(const int* __restrict__ step_flag, int* __restrict__ skipped) {
-  pdl_enter();
-  if (step_flag[(i64)blockIdx.x * OS_SLOT_INTS] != 0) atomicAdd(skipped, 1);
 }
 
 // ---------------------------------------------------------------------------

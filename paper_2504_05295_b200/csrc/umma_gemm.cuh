@@ -1905,7 +1905,6 @@ int umma_try_launch(const GemmArgs& g_in, int precision, int sm_count, float* pa
   GemmArgs g = g_in;
   const bool d16 = g.ab16 != 0;      // bf16 operands in memory
   const bool bf16 = d16 || (precision == DION_PREC_BF16_OPERANDS);
-  const int epc = bf16 ? 8 : 4;
   const int sm = d16 ? 8 : 4;        // stride granularity: 16 bytes
   if (g.batch != 1) return 0;
   // one launch over the matrices of a chain (same shape; operands, output and split-K scratch g.bs2 4-byte words
