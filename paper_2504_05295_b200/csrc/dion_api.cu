@@ -42,7 +42,6 @@ constexpr i64 PART_CAP_FLOATS = (i64)16 << 20;  // split-K partial sums, at most
 constexpr double P_HALF_MIN_MNR = 4e9;          // smallest m n r whose full-rank P runs on scaled half pairs
 constexpr double SOLVE_PAIR_MIN_PANEL = 3e7;    // smallest rows x r whose blocked solves run on scaled half pairs
 constexpr i64 LAZY_PAIR_MIN_MNR = 50000000;     // smallest m n r whose Lazy-Dion step runs on scaled half pairs (2^25.6: 512 x 768 x 128)
-constexpr i64 HALF_PAIR_MIN_MNR = 50000000;     // ... and whose Dion step does (see step_on_half_pairs)
 constexpr double GRAM_PAIR_MIN_FLOPS = 2e9;     // smallest rows r^2 whose Gram matrix runs on scaled half pairs
 constexpr double P_PAIR_MIN_MNR = 1.5e10;       // smallest m n r whose P = (M + G) Q runs on bf16 operand pairs first
 
@@ -1458,8 +1457,8 @@ bool r_on_pairs(const StepCtx& s, i64 m, i64 n, i64 r) {
   return s.tensor && s.c->cfg.precision == DION_PREC_FP32 && s.L.B32 > 0 && s.L.Bp > 0 && m >= 128 && n >= 128 && r >= 64;
 }
 
-// The steps whose four products run on scaled half pairs (k_form_sum_amax): CholeskyQR2 panels between the smallest
-// product that pays for the second pass over M + G and the size from which P runs on the bf16 pairs that one pass makes.
+// The steps whose four products run on scaled half pairs (k_form_sum_amax): CholeskyQR2 panels up to the size from which P
+// runs on the bf16 pairs that one pass over M + G makes.
 // M + G is read once more (from L2 where it fits), but P leaves the 3xTF32 form, whose converter warps bound it, for three
 // half MMAs per K step, U's pair also serves the weight update, and every result carries 22 bits (768^2 to 768 x 3072 at
 // r = 192, 72 matrices in one call: P 932 -> 516 us, R 420 -> 194 us with the unsplit chains, weight update 200 -> 173 us;
@@ -1467,7 +1466,7 @@ bool r_on_pairs(const StepCtx& s, i64 m, i64 n, i64 r) {
 // The rule looks at the shape alone, so that a grouped call computes what single calls compute.
 bool step_on_half_pairs(const StepCtx& s, i64 m, i64 n, i64 r, i64 short_dim) {
   const i64 mnr = m * n * r;
-  return r_on_pairs(s, m, n, r) && s.L.Bh == 0 && mnr >= HALF_PAIR_MIN_MNR && (double)mnr < P_PAIR_MIN_MNR &&
+  return r_on_pairs(s, m, n, r) && s.L.Bh == 0 && (double)mnr < P_PAIR_MIN_MNR &&
          resolve_orth_for(s.c, r, short_dim, s.list != nullptr) == DION_ORTH_CHOLQR2;
 }
 

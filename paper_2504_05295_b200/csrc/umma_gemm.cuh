@@ -1955,6 +1955,8 @@ int umma_try_launch(const GemmArgs& g_in, int precision, int sm_count, float* pa
              !(variant & (UMMA_VARIANT_REGISTER_LOADS | UMMA_VARIANT_NO_PAIRS)) && nclusters > 0 &&
              g.N >= 256 && g.M >= PAIR_MIN_ROWS && (g.tri != TRI_LOWER || g.N >= PAIR_MIN_TRI);
   int BN = ((g.tri == TRI_LOWER && !tri_wide && !cg2) || g.N < 256) ? 128 : 256;
+  // (a rank-r update of few tiles: its time is the epilogue of one tile; 256 x 512 in four tiles of 256 columns 12 us)
+  if (!cg2 && BN == 256 && g.epi != EPI_STORE && g.tri == TRI_FULL && ((g.M + BM - 1) / BM) * ((g.N + 255) / 256) * nbat * 2 <= sm_count) BN = 128;
   Params p;
   p.g = g;
   if (g.c_tab != nullptr) for (int b = 0; b < nbat; ++b) p.ctab[b] = g.c_tab[b];
