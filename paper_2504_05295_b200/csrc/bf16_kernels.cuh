@@ -335,15 +335,6 @@ __device__ __forceinline__ int f16_scale_exponent(float amax) {
   if (amax > 0.f && amax < 3.0e38f) frexpf(amax, &ex);
   return 14 - (ex < -80 ? -80 : ex);
 }
-// M + G in fp32 and the blocks' largest magnitudes of it in one pass (the products on a scaled half pair of the sum).
-template <bool VEC>
-__global__ void __launch_bounds__(256, 3) k_form_b32_amax(const float* __restrict__ M, i64 ldm, const void* __restrict__ G, i64 ldg, int g_mode,
-                                                       i64 rows, i64 cols, float* __restrict__ out, float* __restrict__ part) {
-  pdl_enter();
-  float m = 0.f;
-  form_b32_body<VEC>(M, ldm, G, ldg, g_mode, rows, cols, out, nullptr, nullptr, &m);
-  block_max(m, part);
-}
 // The two launches that prepare a chain (blockIdx.y) of steps on half pairs: M + G in fp32 with the largest magnitudes of the sum
 // and of Q (Q is a right factor of the caller's making: nothing bounds its entries), then the scaled pairs of both.
 // part: gridDim.x maxima of the sum, then as many of Q.  16-byte accesses to Q where it allows them (qvec).
@@ -370,7 +361,7 @@ __global__ void __launch_bounds__(256, 3) k_form_sum_amax(const ChainPtrs Ms, i6
   block_max(mq, part + gridDim.x);
 }
 // A step's scalars: the factors that take the scales out of P, R and the error feedback; then R's block maxima.
-enum : int { HS_P = 0, HS_R = 1, HS_EF = 2, HS_MAX = 16 };
+enum : int { HS_P = 0, HS_R = 1, HS_EF = 2, HS_Q = 3, HS_T = 4, HS_MAX = 16 };      // (HS_Q: 1 / scale of Q; HS_T: Lazy-Dion's left factor)
 constexpr int HS_U_BITS = 13;      // U's pair is scaled by 2^13 (entries at most 1)
 __global__ void __launch_bounds__(256) k_split_sum(const float* __restrict__ sum, i64 total_s, const ChainPtrs Qs, i64 ldq, i64 qrows,
                                                    i64 qcols, int qvec, const float* __restrict__ part, int nparts,
@@ -396,6 +387,7 @@ __global__ void __launch_bounds__(256) k_split_sum(const float* __restrict__ sum
   if (blockIdx.x == 0 && threadIdx.x == 0) {
     scal[HS_P] = ldexpf(1.f, -es) * ldexpf(1.f, -eq);
     scal[HS_R] = ldexpf(1.f, -es - HS_U_BITS);
+    scal[HS_Q] = ldexpf(1.f, -eq);
   }
   const float fs = ldexpf(1.f, es), fq = ldexpf(1.f, eq);
   const i64 n8 = total_s / 8, qpr = qcols / 8, q8 = qrows * qpr;

@@ -134,17 +134,20 @@ __global__ void __launch_bounds__(CN_THREADS) k_colsumsq_finish(const float* __r
 // What k_colnorm_apply writes beside Q (all optional; r a multiple of 8 then), per matrix of a chain in the scratch slices.
 struct ColnormPairs {
   int kind;                // 0: nothing, else what R becomes: CN_HALF or CN_BF16, a pair; CN_ONE, a bf16 array
-  void* qh; float qscale;  // Q as a half array, scaled (CN_ONE: as a bf16 array)
+  void* qh; float qscale;  // Q as a half array, scaled (CN_ONE: as a bf16 array) ...
+  int qpair;               // ... and what that leaves of it, n * r elements behind
   void* hi;                // R's array or pair: hi, then lo n * r elements behind it
   const float* amax; int nmax;   // CN_HALF: R's block maxima; its scale puts the largest magnitude in [2^13, 2^14)
-  float* scal;             // ... and the factor that takes the scales out of the product with U's pair
+  float* scal;             // ... and the factor that takes the scales out of the product with U's pair,
+  const float* other;      // or with another pair (optional: its 1 / scale)
 };
 enum : int { CN_HALF = 1, CN_BF16 = 2, CN_ONE = 3 };
 
 // d_j = sqrt(sum of the partials); Q[i][j] = R[i][j] / (d_j + eps).  Grid as for k_colsumsq_partial with row blocks of its own
 // (every block adds the chunks' sums up again, so a chain of many matrices takes fewer and larger ones: 48 of 768 x 192 in
 // blocks of 32 rows 47 us, 27 us now); the blocks of row block 0 also export d.  Q and d_out come from pointer tables; qvec: Q's rows are 16-byte aligned.
-template <bool V4>
+// QP: Q's half array is a pair (x.qpair).
+template <bool V4, bool QP>
 __global__ void __launch_bounds__(CN_THREADS, 3) k_colnorm_apply(const float* __restrict__ R, i64 ldr, i64 n, i64 r, i64 rows_per_chunk, int chunks,
                                                               const float* __restrict__ part, float eps, const ChainPtrs Qs, i64 ldq, int qvec,
                                                               float* __restrict__ d_ws, const ChainPtrs ds, int* __restrict__ status,
@@ -180,7 +183,7 @@ __global__ void __launch_bounds__(CN_THREADS, 3) k_colnorm_apply(const float* __
     for (int w = 1; w < CN_WARPS; ++w) m = fmaxf(m, redm[w]);
     const int e = f16_scale_exponent(m);
     rscale = ldexpf(1.f, e);
-    if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) x.scal[b * wstride] = ldexpf(1.f, -e - HS_U_BITS);
+    if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) x.scal[b * wstride] = x.other != nullptr ? ldexpf(1.f, -e) * x.other[b * wstride] : ldexpf(1.f, -e - HS_U_BITS);
   }
   float inv[4];
 #pragma unroll
@@ -209,8 +212,10 @@ __global__ void __launch_bounds__(CN_THREADS, 3) k_colnorm_apply(const float* __
     if (V4) {
       const i64 j = j0 + 4 * lane;
       if (j >= r) continue;
-      if (qvec) *reinterpret_cast<float4*>(Q + i * ldq + j) = make_float4(q[0], q[1], q[2], q[3]);
-      else {
+      if (Q == nullptr) {      // (only its half arrays are wanted)
+      } else if (qvec) {
+        *reinterpret_cast<float4*>(Q + i * ldq + j) = make_float4(q[0], q[1], q[2], q[3]);
+      } else {
 #pragma unroll
         for (int k = 0; k < 4; ++k) Q[i * ldq + j + k] = q[k];
       }
@@ -238,6 +243,13 @@ __global__ void __launch_bounds__(CN_THREADS, 3) k_colnorm_apply(const float* __
           if (x.kind == CN_ONE) { q16.x = pack_bf16x2(q[0], q[1]); q16.y = pack_bf16x2(q[2], q[3]); }
         }
         *reinterpret_cast<uint2*>(reinterpret_cast<uint16_t*>(x.qh) + at) = q16;
+        if constexpr (QP) {
+          const __half* qh = reinterpret_cast<const __half*>(&q16);
+          __half l[4];
+#pragma unroll
+          for (int k = 0; k < 4; ++k) l[k] = __float2half_rn(x.qscale * q[k] - __half2float(qh[k]));
+          *reinterpret_cast<uint2*>(reinterpret_cast<uint16_t*>(x.qh) + at + n * r) = *reinterpret_cast<const uint2*>(l);
+        }
         *reinterpret_cast<uint2*>(reinterpret_cast<uint16_t*>(x.hi) + at) = hi;
         if (x.kind != CN_ONE) *reinterpret_cast<uint2*>(reinterpret_cast<uint16_t*>(x.hi) + at + n * r) = lo;
       }

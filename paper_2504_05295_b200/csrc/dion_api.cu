@@ -1274,10 +1274,13 @@ int colnorm_launch(StepCtx& s, int b, int per, const float* W, i64 ldw, i64 rows
   if (rpb < 32) rpb = 32;
   const dim3 agrid(grid.x, (unsigned)((rows + rpb - 1) / rpb), grid.z);
   const float* sp = sums != nullptr ? sums : (const float*)part;
-  if (v4) launch_pdl(k_colnorm_apply<true>, agrid, dim3(CN_THREADS), 0, s.st, W, ldw, rows, r, rpb, chunks, sp, c->cfg.eps, Qs, ldq, qvec, s.W(b, s.L.d), ds,
-                     c->dev_ints, skip, s.wstride, x, c->dev_ints + 1);
-  else launch_pdl(k_colnorm_apply<false>, agrid, dim3(CN_THREADS), 0, s.st, W, ldw, rows, r, rpb, chunks, sp, c->cfg.eps, Qs, ldq, qvec, s.W(b, s.L.d), ds,
-                  c->dev_ints, skip, s.wstride, x, c->dev_ints + 1);
+  auto apply = [&](auto kernel) {
+    launch_pdl(kernel, agrid, dim3(CN_THREADS), 0, s.st, W, ldw, rows, r, rpb, chunks, sp, c->cfg.eps, Qs, ldq, qvec, s.W(b, s.L.d), ds,
+               c->dev_ints, skip, s.wstride, x, c->dev_ints + 1);
+  };
+  if (!v4) apply(k_colnorm_apply<false, false>);
+  else if (x.qpair != 0) apply(k_colnorm_apply<true, true>);
+  else apply(k_colnorm_apply<true, false>);
   DION_CHECK_LAUNCH(c);
   return DION_OK;
 }
@@ -2152,8 +2155,6 @@ int step_graph(dion_ctx* c, const dion_matrix* a, float lr, cudaStream_t st) {
 // kind::f16 MMAs per K step on pairs -- the 22 significant bits of the 3xTF32 products it replaces at twice their rate,
 // through the kernels with the deeper epilogue (4096^2, r = 256: W 128 -> 35 us + 50 of preparation, error feedback 141 -> 36,
 // weight update 85 -> 28).
-enum : int { LZ_B = 0, LZ_BQ = 1, LZ_Q = 2, LZ_A = 3, LZ_AQ = 4, LZ_SCALARS = 8 };      // floats behind the partial maxima: 1 / scale of
-                                                                                      // M + G, with Q's, Q's, the left factor's with another's
 bool lazy_on_pairs(const StepCtx& s, const dion_matrix* a) {
   return s.tensor && s.L.B32 > 0 && s.L.Bp > 0 && a->r % 8 == 0 && a->m % 8 == 0 && a->n % 8 == 0 && a->m * a->n * a->r >= LAZY_PAIR_MIN_MNR &&
          !((uintptr_t)a->X & 15) && a->ldx % 4 == 0 && !((uintptr_t)a->M & 15) && a->ldm % 4 == 0 && !((uintptr_t)a->Q & 15) && a->ldq % 4 == 0;
@@ -2163,22 +2164,19 @@ int lazy_pairs(StepCtx& s, const dion_matrix* a, float lr, int refresh) {
   dion_ctx* c = s.c;
   cudaStream_t st = s.st;
   const i64 m = a->m, n = a->n, r = a->r;
-  const int gmode = (a->g_dtype == DION_BF16) ? ADD_BF16 : ADD_F32;
-  float* pm = s.ws + s.L.lz;
-  float* sc = pm + 8 * (i64)c->sm_count;
+  float* sc = s.ws + s.L.lz;      // HS_*
   float* R = s.ws + s.L.R;
   auto halves = [&](i64 off) { return reinterpret_cast<__half*>(s.ws + off); };
-  // the pair of a rows x cols array into scratch at `off`; scale slot `slot` (times slot `other`'s), `own`: its scale alone
-  auto pair_of = [&](const float* src, i64 ld, i64 rows, i64 cols, i64 off, int slot, int other, int own, bool have_max, i64 nparts) -> int {
-    if (!have_max) {
-      nparts = (rows * cols / 4 + 2047) / 2048;
-      if (nparts > AMAX_PARTS) nparts = AMAX_PARTS;
-      launch_pdl(k_absmax_partial, dim3((unsigned)nparts), dim3(256), 0, st, src, ld, rows, cols, pm, (i64)0, (const int*)nullptr, (i64)0);
-      DION_CHECK_LAUNCH(c);
-    }
+  // the pair of a rows x cols array into scratch at `off`; slot: the scale factor of its product with M + G, own: of itself alone
+  auto pair_of = [&](const float* src, i64 ld, i64 rows, i64 cols, i64 off, int slot, int own) -> int {
+    i64 nparts = (rows * cols / 4 + 2047) / 2048;
+    if (nparts > AMAX_PARTS) nparts = AMAX_PARTS;
+    float* pm = s.ws + s.L.part;      // (read before the next product writes its partial sums there)
+    launch_pdl(k_absmax_partial, dim3((unsigned)nparts), dim3(256), 0, st, src, ld, rows, cols, pm, (i64)0, (const int*)nullptr, (i64)0);
+    DION_CHECK_LAUNCH(c);
     launch_pdl(k_split_f16_scaled, dim3((unsigned)grid_for(c, rows * cols / 8)), dim3(256), 0, st, src, ld, rows, cols, (const float*)pm, (int)nparts,
-               halves(off), halves(off) + rows * cols, sc + slot, (i64)0, (const int*)nullptr, (i64)0, 1.f,
-               other >= 0 ? (const float*)(sc + other) : (const float*)nullptr, own >= 0 ? sc + own : (float*)nullptr);
+               halves(off), halves(off) + rows * cols, sc + slot, (i64)0, (const int*)nullptr, (i64)0, ldexpf(1.f, HS_U_BITS),
+               (const float*)(sc + HS_R), own >= 0 ? sc + own : (float*)nullptr);
     DION_CHECK_LAUNCH(c);
     return DION_OK;
   };
@@ -2191,24 +2189,18 @@ int lazy_pairs(StepCtx& s, const dion_matrix* a, float lr, int refresh) {
     g.alpha_dev = sc + slot;
     return g;
   };
-  const bool vec = !((uintptr_t)a->G & ((a->g_dtype == DION_BF16) ? 7 : 15)) && a->ldg % 4 == 0;
-  const int fgrid = grid_for(c, m * n / 4);
   float* sum = s.ws + s.L.B32;
-  if (vec) launch_pdl(k_form_b32_amax<true>, dim3((unsigned)fgrid), dim3(256), 0, st, (const float*)a->M, a->ldm, a->G, a->ldg, gmode, m, n, sum, pm);
-  else launch_pdl(k_form_b32_amax<false>, dim3((unsigned)fgrid), dim3(256), 0, st, (const float*)a->M, a->ldm, a->G, a->ldg, gmode, m, n, sum, pm);
-  DION_CHECK_LAUNCH(c);
-  DION_TRY(pair_of(sum, n, m, n, s.L.Bp, LZ_B, -1, -1, true, fgrid));
+  DION_TRY(half_sum_chain(s, &a, n));      // M + G, its pair and Q's
   if (refresh) {
     PhaseScope ps_orth(c, st, DION_PHASE_ORTH);
     // T = (M + G) Q  (m x r), Z = (M + G)^T T (n x r), Q <- Orthonormalize(Z)
     const int precise = (resolve_orth(c, r, (m < n) ? m : n) == DION_ORTH_SHIFTED3) ? 1 : 0;
-    DION_TRY(pair_of((const float*)a->Q, a->ldq, n, r, s.L.S16, LZ_BQ, LZ_B, -1, false, 0));
-    GemmArgs t = product(m, r, n, s.L.Bp, m * n, n, 1, s.L.S16, n * r, r, 1, LZ_BQ);
+    GemmArgs t = product(m, r, n, s.L.Bp, m * n, n, 1, s.L.S16, n * r, r, 1, HS_P);
     t.C = R; t.ldc = r; t.epi = EPI_STORE; t.precise = precise;
     DION_TRY(launch_gemm(s, t));
-    DION_TRY(pair_of(R, r, m, r, s.L.P1, LZ_AQ, LZ_B, -1, false, 0));
+    DION_TRY(pair_of(R, r, m, r, s.L.P1, HS_T, -1));
     const i64 pin_off = panel_offset(s, r, (m < n) ? m : n);
-    GemmArgs z = product(n, r, m, s.L.Bp, m * n, 1, n, s.L.P1, m * r, r, 1, LZ_AQ);
+    GemmArgs z = product(n, r, m, s.L.Bp, m * n, 1, n, s.L.P1, m * r, r, 1, HS_T);
     z.C = s.ws + pin_off; z.ldc = r; z.epi = EPI_STORE; z.precise = precise;
     DION_TRY(launch_gemm(s, z));
     i64 V_off = 0;
@@ -2222,32 +2214,28 @@ int lazy_pairs(StepCtx& s, const dion_matrix* a, float lr, int refresh) {
   }
   {   // W = (M + G) Q
   PhaseScope ps(c, st, DION_PHASE_P);
-  DION_TRY(pair_of((const float*)a->Q, a->ldq, n, r, s.L.S16, LZ_BQ, LZ_B, LZ_Q, false, 0));
-  GemmArgs w = product(m, r, n, s.L.Bp, m * n, n, 1, s.L.S16, n * r, r, 1, LZ_BQ);
+  if (refresh) DION_TRY(pair_of((const float*)a->Q, a->ldq, n, r, s.L.S16, HS_P, HS_Q));
+  GemmArgs w = product(m, r, n, s.L.Bp, m * n, n, 1, s.L.S16, n * r, r, 1, HS_P);
   w.C = R; w.ldc = r; w.epi = EPI_STORE;
   DION_TRY(launch_gemm(s, w));
   }
+  {   // U = ColNorm(W), as a pair of fixed scale (unit-norm columns) in P0; W's pair in P1
+  PhaseScope ps(c, st, DION_PHASE_COLNORM);
+  ColnormPairs x = ColnormPairs();
+  x.kind = CN_HALF; x.qh = s.ws + s.L.P0; x.qscale = ldexpf(1.f, HS_U_BITS); x.qpair = 1; x.hi = s.ws + s.L.P1; x.other = sc + HS_Q;
+  DION_TRY(colnorm(s, 0, R, m, r, nullptr, r, a->colnorm_out, nullptr, x));
+  }
   {   // M <- (M + G) - (1 - mu) W Q^T
   PhaseScope ps(c, st, DION_PHASE_EF);
-  DION_TRY(pair_of(R, r, m, r, s.L.P1, LZ_AQ, LZ_Q, -1, false, 0));
-  GemmArgs e = product(m, n, r, s.L.P1, m * r, r, 1, s.L.S16, n * r, 1, r, LZ_AQ);
+  GemmArgs e = product(m, n, r, s.L.P1, m * r, r, 1, s.L.S16, n * r, 1, r, HS_EF);
   e.C = (float*)a->M; e.ldc = a->ldm; e.epi = EPI_C2_SUB; e.C2 = sum; e.ldc2 = n; e.c2_mode = ADD_F32;
   e.alpha = 1.f - c->cfg.mu;
   e.skip_flag = s.flag;
   DION_TRY(launch_gemm(s, e));
   }
-  {   // U = ColNorm(W)
-  PhaseScope ps(c, st, DION_PHASE_COLNORM);
-  DION_TRY(colnorm(s, 0, R, m, r, s.ws + s.L.P0, r, a->colnorm_out));
-  }
-  // X <- X - lr sqrt(m/n) U Q^T; U's columns have unit norm: its pair has a fixed scale
+  // X <- X - lr sqrt(m/n) U Q^T
   PhaseScope ps_x(c, st, DION_PHASE_X);
-  ChainPtrs t;
-  t.p[0] = s.ws + s.L.P0;
-  launch_pdl(k_split_f16_fixed, dim3((unsigned)grid_for(c, m * r / 8)), dim3(256), 0, st, t, r, m, r, ldexpf(1.f, 13), halves(s.L.P1), halves(s.L.P1) + m * r,
-             (i64)0, (i64)0, (const int*)nullptr, (i64)0);
-  DION_CHECK_LAUNCH(c);
-  GemmArgs x = product(m, n, r, s.L.P1, m * r, r, 1, s.L.S16, n * r, 1, r, LZ_Q);
+  GemmArgs x = product(m, n, r, s.L.P0, m * r, r, 1, s.L.S16, n * r, 1, r, HS_Q);
   x.C = (float*)a->X; x.ldc = a->ldx; x.epi = EPI_SUB;
   x.alpha = ldexpf(lr * sqrtf((float)((double)m / (double)n)), -13);
   x.skip_flag = s.flag;
@@ -2913,7 +2901,7 @@ bool preload_kernels() {
   ok = ok && touch_kernel(k_probe_fused) && touch_kernel(k_probe_y) && touch_kernel(k_probe_y4) && touch_kernel(k_probe_w) && touch_kernel(k_probe_w4) && touch_kernel(k_probe_decide) && touch_kernel(k_reset_rounds);
   ok = ok && touch_kernel(k_orth_finish) && touch_kernel(k_cgs_fallback) && touch_kernel(k_copy_block);
   ok = ok && touch_kernel(k_colsumsq_partial<true>) && touch_kernel(k_colsumsq_partial<false>) &&
-       touch_kernel(k_colnorm_apply<true>) && touch_kernel(k_colnorm_apply<false>) && touch_kernel(k_copy_panel);
+       touch_kernel(k_colnorm_apply<true, false>) && touch_kernel(k_colnorm_apply<false, false>) && touch_kernel(k_copy_panel);
   ok = ok && touch_kernel(k_latch_flag) && touch_kernel(k_hh_reflector);
   ok = ok && touch_kernel(k_hh_apply) && touch_kernel(k_set_identity) && touch_kernel(k_sign_fix);
   ok = ok && touch_kernel(k_form_b16<true>) && touch_kernel(k_form_b16<false>) && touch_kernel(k_form_b32<true>);
