@@ -325,7 +325,7 @@ int64_t dion_launch_count(const dion_ctx* ctx);
  * synchronisation is not acceptable.  dion_init and dion_step grow their scratch
  * with cudaMalloc; this call never does, and it needs no dion_ctx.  Its scratch
  * (the P/U panels, R, the Gram matrix and its factors, split-K partial sums, the
- * column norms and the step's flags) lives in an array of 24 MiB that is part of
+ * column norms and the step's flags) lives in an array of some 24 MiB that is part of
  * the library image, so every GPU that loads the library holds those 24 MiB until
  * the process exits.
  *

@@ -72,7 +72,7 @@ struct Layout {
   i64 pmax;                 // ... its partial maxima and the product's scale factor (like gmax)
   i64 SolveP, LfP, smax;    // blocked solves on half pairs (r > 512): pair of a rows x 512 right-hand side; pairs of a row block of
                             // the factor (512 x r) and of a diagonal inverse (512 x 512); partial maxima and scales
-  i64 lz;                   // Lazy-Dion on half pairs: partial maxima, then the scales of its products (LZ_*)
+  i64 lz;                   // steps on half pairs: the scales of their products (HS_*), then the block maxima of R
   i64 XP;                   // scaled half pair of the inverse of the factor
   i64 xmax;                 // largest magnitude of the factor's inverse, then the scale of the product with its pair
   i64 gmax;                 // Gram matrices on half pairs: AMAX_PARTS partial maxima of |P|, then 1 / scale^2
@@ -185,7 +185,8 @@ Layout make_layout(const dion_ctx* c, i64 m, i64 n, i64 r) {
   L.Gram = o; o += align64(r * r);
   L.Linv = o; o += align64(r * r);
   L.Tbuf = o; o += align64(r * r);
-  L.XP = o; o += align64(r <= FLOW_MAX_R ? r * r : 64);
+  const bool gpairs = (double)big * (double)r * (double)r >= GRAM_PAIR_MIN_FLOPS;      // Gram matrices may be formed on half pairs
+  L.XP = o; o += gpairs && r <= FLOW_MAX_R ? align64(r * r) : 0;
   L.Dinv = o; o += align64(((r + NB - 1) / NB) * (i64)NB * NB);
   L.DinvP = o; o += align64(((r + NB - 1) / NB) * (i64)NB * NB);
   // split-K partials: the largest plain-store product of a step is max(m,n) x r
@@ -194,7 +195,7 @@ Layout make_layout(const dion_ctx* c, i64 m, i64 n, i64 r) {
   L.part_floats = pf;
   L.part = o; o += align64(pf);
   colnorm_plan(big, r, c->sm_count, &L.cn_chunks, &L.cn_rows);
-  L.cn_part = o; o += align64((i64)(L.cn_chunks + 1) * r + NEAR_MAX_BLOCKS);
+  L.cn_part = o; o += align64((i64)(L.cn_chunks + 1) * r + (gpairs ? NEAR_MAX_BLOCKS : 0));
   L.d = o; o += align64(r);
   L.gdiag = o; o += align64(r);
   L.scal = o; o += 64;
@@ -222,7 +223,8 @@ Layout make_layout(const dion_ctx* c, i64 m, i64 n, i64 r) {
   L.Psave = L.fb_part = L.fb_h = L.fb_n = 0;
   L.gmax = o; o += align64(AMAX_PARTS + 64);
   L.xmax = o; o += 64;
-  L.lz = o; o += align64(8 * (i64)c->sm_count + 64);
+  L.lz = o;
+  if (sum_in_scratch(c, m, n, r)) o += align64(8 * (i64)c->sm_count + 64);
   L.SolveP = L.LfP = L.smax = 0;
   if (r > FLOW_MAX_R && (double)big * (double)r >= SOLVE_PAIR_MIN_PANEL) {
     L.SolveP = o; o += align64(big * NBO_COLS);
@@ -2865,7 +2867,8 @@ const char* dion_strerror(int code) {
 
 namespace {
 
-constexpr size_t NOALLOC_SCRATCH_BYTES = (size_t)24 << 20;  // 24 MiB, resident on every device that loads the library
+// 24 MiB and the factorization's counters and maxima, resident on every device that loads the library
+constexpr size_t NOALLOC_SCRATCH_BYTES = ((size_t)24 << 20) + 256 + 16 * 1024;
 constexpr size_t NOALLOC_INT_BYTES = 256;                   // status word, counters and one step slot
 constexpr size_t NOALLOC_CTL_BYTES = 16 * 1024;             // progress counters of the factorization
 constexpr int NOALLOC_MAX_DEVICES = 64;
