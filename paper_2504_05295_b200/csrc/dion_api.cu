@@ -731,7 +731,7 @@ int potrf_blocked(StepCtx& s, i64 r, int mode, const std::function<int(i64, i64)
           cst = c->side;
         }
         dim3 grid((unsigned)grid_for(c, rem * sz, s.nb), (unsigned)s.nb);
-        launch_pdl(k_copy_block, grid, dim3(256), 0, cst, ptmp, r, panel, r, rem, sz, skip, s.wstride);
+        launch_pdl(k_copy_block, grid, dim3(256), 0, cst, ptmp, r, panel, r, rem, sz, skip, s.wstride, (const int*)nullptr, (int*)nullptr);
         DION_CHECK_LAUNCH(c);
       }
       const float* lp = side_copy ? ptmp : panel;
@@ -1124,7 +1124,7 @@ int rcqr(StepCtx& s, i64 rows, i64 r) {
     g.C = stack; g.ldc = r; g.epi = EPI_STORE; g.precise = 1;
     DION_TRY(launch_gemm(s, g, b));
     dim3 grid((unsigned)grid_for(c, rows * r), 1);
-    launch_pdl(k_copy_block, grid, dim3(256), 0, s.st, (const float*)s.W(b, s.L.P0), r, stack + k * r, r, rows, r, nullptr, 0);
+    launch_pdl(k_copy_block, grid, dim3(256), 0, s.st, (const float*)s.W(b, s.L.P0), r, stack + k * r, r, rows, r, nullptr, 0, (const int*)nullptr, (int*)nullptr);
     DION_CHECK_LAUNCH(c);
   }
   s.wt_off = s.L.SkW;
@@ -2604,18 +2604,16 @@ int dion_dp_factor(dion_ctx* ctx, const dion_matrix* a, float* PU, float* W, int
   cudaStream_t st = (cudaStream_t)cuda_stream;
   DION_TRY(begin_step(ctx, a, 1, st, &s));
   const i64 m = a->m, n = a->n, r = a->r;
-  dim3 grid((unsigned)grid_for(ctx, m * r), 1);
+  dim3 grid((unsigned)grid_for(ctx, (m * r + 3) / 4), 1);
   const i64 pin_off = panel_offset(s, r, (m < n) ? m : n);
-  launch_pdl(k_copy_block, grid, dim3(256), 0, st, PU, r, s.ws + pin_off, r, m, r, nullptr, 0);
+  launch_pdl(k_copy_block, grid, dim3(256), 0, st, PU, r, s.ws + pin_off, r, m, r, nullptr, 0, (const int*)nullptr, (int*)nullptr);
   DION_CHECK_LAUNCH(ctx);
   i64 U_off = 0;
   s.in_orth = true;
   const int rc = orthonormalize(s, m, r, (m < n) ? m : n, pin_off, &U_off);
   s.in_orth = false;
   DION_TRY(rc);
-  launch_pdl(k_copy_block, grid, dim3(256), 0, st, s.ws + U_off, r, PU, r, m, r, nullptr, 0);
-  DION_CHECK_LAUNCH(ctx);
-  launch_pdl(k_latch_flag, dim3((unsigned)(1)), dim3(1), 0, st, s.flag, dp_flag);      // a breakdown cancels dion_dp_finish
+  launch_pdl(k_copy_block, grid, dim3(256), 0, st, s.ws + U_off, r, PU, r, m, r, nullptr, 0, (const int*)s.flag, dp_flag);      // (a breakdown cancels dion_dp_finish)
   DION_CHECK_LAUNCH(ctx);
   if (step_on_half_pairs(s, m, n, r, (m < n) ? m : n)) return half_factor(s, a, PU, W, nullptr);
   if (r_on_pairs(s, m, n, r)) {       // as dion_step: W on the bf16 pairs of M + G and U
@@ -2688,17 +2686,15 @@ int dion_orthonormalize(dion_ctx* ctx, int64_t m, int64_t r, int64_t n_total, fl
   DION_TRY(begin_step(ctx, &shape, 1, st, &s));
   const i64 sd = (m < n_total) ? m : n_total;
   const i64 pin_off = panel_offset(s, r, sd);
-  dim3 grid((unsigned)grid_for(ctx, m * r), 1);
-  launch_pdl(k_copy_block, grid, dim3(256), 0, st, (const float*)PU, r, s.ws + pin_off, r, m, r, nullptr, 0);
+  dim3 grid((unsigned)grid_for(ctx, (m * r + 3) / 4), 1);
+  launch_pdl(k_copy_block, grid, dim3(256), 0, st, (const float*)PU, r, s.ws + pin_off, r, m, r, nullptr, 0, (const int*)nullptr, (int*)nullptr);
   DION_CHECK_LAUNCH(ctx);
   i64 U_off = 0;
   s.in_orth = true;
   const int rc = orthonormalize(s, m, r, sd, pin_off, &U_off);
   s.in_orth = false;
   DION_TRY(rc);
-  launch_pdl(k_copy_block, grid, dim3(256), 0, st, (const float*)(s.ws + U_off), r, PU, r, m, r, nullptr, 0);
-  DION_CHECK_LAUNCH(ctx);
-  launch_pdl(k_latch_flag, dim3(1), dim3(1), 0, st, (const int*)s.flag, flag);
+  launch_pdl(k_copy_block, grid, dim3(256), 0, st, (const float*)(s.ws + U_off), r, PU, r, m, r, nullptr, 0, (const int*)s.flag, flag);
   DION_CHECK_LAUNCH(ctx);
   return DION_OK;
 }
@@ -2905,7 +2901,7 @@ bool preload_kernels() {
   ok = ok && touch_kernel(k_orth_finish) && touch_kernel(k_cgs_fallback) && touch_kernel(k_copy_block);
   ok = ok && touch_kernel(k_colsumsq_partial<true>) && touch_kernel(k_colsumsq_partial<false>) &&
        touch_kernel(k_colnorm_apply<true, false>) && touch_kernel(k_colnorm_apply<false, false>) && touch_kernel(k_copy_panel);
-  ok = ok && touch_kernel(k_latch_flag) && touch_kernel(k_hh_reflector);
+  ok = ok && touch_kernel(k_hh_reflector);
   ok = ok && touch_kernel(k_hh_apply) && touch_kernel(k_set_identity) && touch_kernel(k_sign_fix);
   ok = ok && touch_kernel(k_form_b16<true>) && touch_kernel(k_form_b16<false>) && touch_kernel(k_form_b32<true>);
   ok = ok && touch_kernel(k_form_b32<false>) && touch_kernel(k_to_bf16) && touch_kernel(k_round_tf32);

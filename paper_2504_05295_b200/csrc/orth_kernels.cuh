@@ -1053,17 +1053,32 @@ __global__ void __launch_bounds__(256) k_cgs_fallback(const float* __restrict__ 
   }
 }
 
-// Copies a rows x cols block between two matrices (leading dimensions lds, ldd).
-__global__ void k_copy_block(const float* __restrict__ src, i64 lds, float* __restrict__ dst, i64 ldd,
-                             i64 rows, i64 cols, const int* __restrict__ skip_flag, i64 wstride) {
-  pdl_enter();
-  src += (i64)blockIdx.y * wstride; dst += (i64)blockIdx.y * wstride;     // batched over blockIdx.y
-  if (skip_flag != nullptr && skip_flag[(i64)blockIdx.y * OS_SLOT_INTS] != 0) return;
-  const i64 total = rows * cols;
-  for (i64 e = (i64)blockIdx.x * blockDim.x + threadIdx.x; e < total; e += (i64)gridDim.x * blockDim.x) {
+// rows x cols from one matrix to another (four elements at a time where both allow it).
+__device__ __forceinline__ void copy_rows(const float* __restrict__ src, i64 lds, float* __restrict__ dst, i64 ldd, i64 rows, i64 cols) {
+  const i64 stride = (i64)gridDim.x * blockDim.x;
+  if (((cols | lds | ldd) & 3) == 0 && (((uintptr_t)src | (uintptr_t)dst) & 15) == 0) {
+    const i64 per_row = cols / 4;
+    for (i64 e = (i64)blockIdx.x * blockDim.x + threadIdx.x; e < rows * per_row; e += stride) {
+      const i64 i = row_of(e, per_row), c = (e - i * per_row) * 4;
+      *reinterpret_cast<float4*>(dst + i * ldd + c) = *reinterpret_cast<const float4*>(src + i * lds + c);
+    }
+    return;
+  }
+  for (i64 e = (i64)blockIdx.x * blockDim.x + threadIdx.x; e < rows * cols; e += stride) {
     const i64 i = row_of(e, cols), c = e - i * cols;
     dst[i * ldd + c] = src[i * lds + c];
   }
+}
+
+// Copies a rows x cols block between two matrices (leading dimensions lds, ldd).  latch_to (optional): set when *latch_from is (a
+// breakdown carried from one call of a multi-call step to the next).
+__global__ void k_copy_block(const float* __restrict__ src, i64 lds, float* __restrict__ dst, i64 ldd,
+                             i64 rows, i64 cols, const int* __restrict__ skip_flag, i64 wstride,
+                             const int* __restrict__ latch_from, int* __restrict__ latch_to) {
+  pdl_enter();
+  if (latch_to != nullptr && blockIdx.x == 0 && threadIdx.x == 0 && *latch_from != 0) *latch_to = 1;
+  if (skip_flag != nullptr && skip_flag[(i64)blockIdx.y * OS_SLOT_INTS] != 0) return;
+  copy_rows(src + (i64)blockIdx.y * wstride, lds, dst + (i64)blockIdx.y * wstride, ldd, rows, cols);     // batched over blockIdx.y
 }
 
 // Copies a rows x r panel (ld = ldv) into Q (ld = ldq) unless the step was flagged.
@@ -1076,17 +1091,7 @@ __global__ void k_copy_panel(const float* __restrict__ V, i64 ldv, float* __rest
   if (wstride != 0) Q += (i64)blockIdx.y * wstride;
   if (skip_flag != nullptr && skip_flag[(i64)blockIdx.y * OS_SLOT_INTS] != 0) return;
   if (only_if != nullptr && (only_if[(i64)blockIdx.y * OS_SLOT_INTS] & only_mask) == 0) return;
-  const i64 total = rows * r;
-  for (i64 e = (i64)blockIdx.x * blockDim.x + threadIdx.x; e < total; e += (i64)gridDim.x * blockDim.x) {
-    const i64 i = row_of(e, r), c = e - i * r;
-    Q[i * ldq + c] = V[i * ldv + c];
-  }
-}
-
-// *dst = 1 if *src != 0 (carries a breakdown from one call of a multi-call step to the next).
-__global__ void k_latch_flag(const int* __restrict__ src, int* __restrict__ dst) {
-  pdl_enter();
-  if (*src != 0) *dst = 1;
+  copy_rows(V, ldv, Q, ldq, rows, r);
 }
 
 // ---------------------------------------------------------------------------
