@@ -67,6 +67,7 @@ struct Layout {
   i64 Psave;                // CholeskyQR2: the panel as the product wrote it, kept for the fallback (0: none)
   i64 fb_part, fb_h, fb_n;  // fallback kernel: partial dot products (SMs x r), their sums (r), partial norms (SMs)
   i64 probe_y, probe_part, probe_sums;  // CholeskyQR2's orthogonality probe: U1 z (rows x NPROBE), partial U1^T (U1 z), partial estimates
+  i64 probe_cap;            // chunks that probe_part holds
   i64 Bp;                   // fp32 mode, M + G in scratch: the same sum as a bf16 (hi, lo) pair (m x n x 2 bf16) for R; 0: none
   i64 Bh;                   // full rank: M + G as a scaled pair of half arrays for P (m x n x 2 halves), 0: none
   i64 pmax;                 // ... its partial maxima and the product's scale factor (like gmax)
@@ -145,6 +146,15 @@ void probe_plan(i64 rows, int* chunks, i64* rows_per) {
   *chunks = (int)((rows + per - 1) / per);
 }
 i64 probe_sums(i64 r) { return (r * NPROBE + PD_ENTRIES - 1) / PD_ENTRIES; }
+
+// The plan is made for the long side when the scratch is laid out and for the panel's rows when it is used, and its chunks do
+// not grow with the rows: 16384 rows are 512 of them, 16448 are 257.  They are made larger until they fit what was laid out.
+void fit_chunks(i64 rows, i64 cap, i64 step, int* chunks, i64* rows_per) {
+  while (*chunks > cap) {
+    *rows_per += step;
+    *chunks = (int)((rows + *rows_per - 1) / *rows_per);
+  }
+}
 
 // fp32 mode on the tensor engine: M + G is formed once per step in scratch, as fp32 (4 bytes per element) and as a
 // bf16 (hi, lo) pair (4 bytes), and P, R and the error feedback read those.  Forming it inside the two products
@@ -243,7 +253,8 @@ Layout make_layout(const dion_ctx* c, i64 m, i64 n, i64 r) {
   {
     int chunks; i64 per;
     probe_plan(big, &chunks, &per);
-    L.probe_part = o; o += align64((i64)(chunks + 1) * r * NPROBE);
+    L.probe_cap = chunks + 1;
+    L.probe_part = o; o += align64(L.probe_cap * r * NPROBE);
     L.probe_sums = o; o += align64(probe_sums(r));
   }
   if (may_fallback(c, m, n, r)) {
@@ -254,6 +265,12 @@ Layout make_layout(const dion_ctx* c, i64 m, i64 n, i64 r) {
   }
   L.total = o;
   return L;
+}
+
+// The plan as a step with the layout L uses it.
+void probe_chunks(const Layout& L, i64 rows, int* chunks, i64* rows_per) {
+  probe_plan(rows, chunks, rows_per);
+  fit_chunks(rows, L.probe_cap, 32, chunks, rows_per);
 }
 
 void graphs_clear(dion_ctx* c);
@@ -754,7 +771,7 @@ int potrf_blocked(StepCtx& s, i64 r, int mode, const std::function<int(i64, i64)
 int probe(StepCtx& s, i64 off, i64 rows, i64 r, int phase) {
   dion_ctx* c = s.c;
   int chunks; i64 per;
-  probe_plan(rows, &chunks, &per);
+  probe_chunks(s.L, rows, &chunks, &per);
   const int* keep = (phase == PROBE_AFTER_REDO) ? (const int*)(s.os + OS_DONE) : nullptr;
   const float* U = s.ws + off;
   if (r % 4 == 0 && r <= PF_MAX_R) {
@@ -2989,6 +3006,20 @@ extern "C" int dion_debug_orth_measure(dion_ctx* ctx, void* cuda_stream, float* 
           cudaSuccess ||
       cudaStreamSynchronize(st) != cudaSuccess)
     return DION_ERR_CUDA;
+  return DION_OK;
+}
+
+// Test hook: chunks of the probe over a panel of `rows` rows in a step on (m, n, r), and those that its scratch holds.
+extern "C" int dion_debug_chunks(int64_t m, int64_t n, int64_t r, int64_t rows, int sm_count, int64_t out[2]) {
+  if (out == nullptr || m < 1 || n < 1 || r < 1 || rows < 1 || sm_count < 1) return DION_ERR_INVALID;
+  dion_ctx c;
+  dion_default_config(&c.cfg);
+  c.sm_count = sm_count;
+  const Layout L = make_layout(&c, m, n, r);
+  int chunks; i64 per;
+  probe_chunks(L, rows, &chunks, &per);
+  out[0] = chunks * per >= rows ? chunks : -1;
+  out[1] = (L.probe_sums - L.probe_part) / (r * NPROBE);
   return DION_OK;
 }
 
