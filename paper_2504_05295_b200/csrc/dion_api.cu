@@ -147,8 +147,9 @@ void probe_plan(i64 rows, int* chunks, i64* rows_per) {
 }
 i64 probe_sums(i64 r) { return (r * NPROBE + PD_ENTRIES - 1) / PD_ENTRIES; }
 
-// The plan is made for the long side when the scratch is laid out and for the panel's rows when it is used, and its chunks do
-// not grow with the rows: 16384 rows are 512 of them, 16448 are 257.  They are made larger until they fit what was laid out.
+// Both plans are made for the long side when the scratch is laid out and for the panel's or the right factor's rows when they
+// are used, and neither grows with the rows: 16384 rows are 512 chunks of the probe, 16448 are 257.  The chunks are made
+// larger until they fit what was laid out.
 void fit_chunks(i64 rows, i64 cap, i64 step, int* chunks, i64* rows_per) {
   while (*chunks > cap) {
     *rows_per += step;
@@ -205,7 +206,8 @@ Layout make_layout(const dion_ctx* c, i64 m, i64 n, i64 r) {
   L.part_floats = pf;
   L.part = o; o += align64(pf);
   colnorm_plan(big, r, c->sm_count, &L.cn_chunks, &L.cn_rows);
-  L.cn_part = o; o += align64((i64)(L.cn_chunks + 1) * r + (gpairs ? NEAR_MAX_BLOCKS : 0));
+  L.cn_chunks += 1;
+  L.cn_part = o; o += align64((i64)L.cn_chunks * r + (gpairs ? NEAR_MAX_BLOCKS : 0));
   L.d = o; o += align64(r);
   L.gdiag = o; o += align64(r);
   L.scal = o; o += 64;
@@ -267,10 +269,14 @@ Layout make_layout(const dion_ctx* c, i64 m, i64 n, i64 r) {
   return L;
 }
 
-// The plan as a step with the layout L uses it.
+// The plans as a step with the layout L uses them.
 void probe_chunks(const Layout& L, i64 rows, int* chunks, i64* rows_per) {
   probe_plan(rows, chunks, rows_per);
   fit_chunks(rows, L.probe_cap, 32, chunks, rows_per);
+}
+void colnorm_chunks(const dion_ctx* c, const Layout& L, i64 rows, i64 r, int* chunks, i64* rows_per) {
+  colnorm_plan(rows, r, c->sm_count, chunks, rows_per);
+  fit_chunks(rows, L.cn_chunks, 1, chunks, rows_per);
 }
 
 void graphs_clear(dion_ctx* c);
@@ -1268,7 +1274,7 @@ int colnorm_launch(StepCtx& s, int b, int per, const float* W, i64 ldw, i64 rows
                    const int* skip, ColnormPairs x = ColnormPairs(), const float* sums = nullptr) {
   dion_ctx* c = s.c;
   int chunks; i64 rpc;
-  colnorm_plan(rows, r, c->sm_count, &chunks, &rpc);
+  colnorm_chunks(c, s.L, rows, r, &chunks, &rpc);
   const dim3 grid((unsigned)((r + 127) / 128), (unsigned)chunks, (unsigned)per);
   float* part = s.W(b, s.L.cn_part);
   const bool v4 = r % 4 == 0 && ldw % 4 == 0 && !((uintptr_t)W & 15);
@@ -2734,7 +2740,7 @@ int dion_shard_factor(dion_ctx* ctx, const dion_matrix* a, int64_t n_total, cons
     DION_TRY(launch_gemm(s, w, 0));
   }
   int chunks; i64 per;
-  colnorm_plan(a->n, a->r, ctx->sm_count, &chunks, &per);
+  colnorm_chunks(ctx, s.L, a->n, a->r, &chunks, &per);
   float* part = s.W(0, s.L.cn_part);
   const dim3 grid((unsigned)((a->r + 127) / 128), (unsigned)chunks);
   if (a->r % 4 == 0) {
@@ -3009,17 +3015,20 @@ extern "C" int dion_debug_orth_measure(dion_ctx* ctx, void* cuda_stream, float* 
   return DION_OK;
 }
 
-// Test hook: chunks of the probe over a panel of `rows` rows in a step on (m, n, r), and those that its scratch holds.
-extern "C" int dion_debug_chunks(int64_t m, int64_t n, int64_t r, int64_t rows, int sm_count, int64_t out[2]) {
+// Test hook: row chunks of `rows` rows in a step on (m, n, r), and the chunks that its scratch holds.
+extern "C" int dion_debug_chunks(int64_t m, int64_t n, int64_t r, int64_t rows, int sm_count, int64_t out[4]) {
   if (out == nullptr || m < 1 || n < 1 || r < 1 || rows < 1 || sm_count < 1) return DION_ERR_INVALID;
   dion_ctx c;
   dion_default_config(&c.cfg);
   c.sm_count = sm_count;
   const Layout L = make_layout(&c, m, n, r);
   int chunks; i64 per;
-  probe_chunks(L, rows, &chunks, &per);
+  colnorm_chunks(&c, L, rows, r, &chunks, &per);
   out[0] = chunks * per >= rows ? chunks : -1;
-  out[1] = (L.probe_sums - L.probe_part) / (r * NPROBE);
+  out[1] = (L.d - L.cn_part - (L.XP < L.Dinv ? NEAR_MAX_BLOCKS : 0)) / r;
+  probe_chunks(L, rows, &chunks, &per);
+  out[2] = chunks * per >= rows ? chunks : -1;
+  out[3] = (L.probe_sums - L.probe_part) / (r * NPROBE);
   return DION_OK;
 }
 

@@ -43,9 +43,10 @@ int dion_debug_gemm(int engine, int precision, const dion_debug_gemm_args* args,
 struct dion_ctx;
 int dion_debug_orth_measure(struct dion_ctx* ctx, void* cuda_stream, float* estimate);
 
-/* Row chunks in which the orthogonality probe of a step on (m, n, r) walks a panel of `rows` rows (out[0]; -1: they do not
- * cover the rows), and the chunks that the scratch has room for (out[1]).  Needs no device. */
-int dion_debug_chunks(int64_t m, int64_t n, int64_t r, int64_t rows, int sm_count, int64_t out[2]);
+/* Row chunks in which a step on (m, n, r) walks `rows` rows, out[0] in the column normalization and out[2] in the
+ * orthogonality probe (-1: the chunks do not cover the rows), and the chunks that the scratch has room for, out[1] and
+ * out[3].  Needs no device. */
+int dion_debug_chunks(int64_t m, int64_t n, int64_t r, int64_t rows, int sm_count, int64_t out[4]);
 
 /* on = 0: the tensor-engine products of a grouped call's chain are launched matrix by matrix instead of once
  * over all matrices of the chain (the results must not depend on it). */

@@ -27,3 +27,27 @@ def test_the_probe_leaves_the_saved_panel_alone(long_side):
     # Gram-Schmidt twice in fp32: orthonormal to a few roundings per column, and U R = P to those of a column's sums
     assert (U.t() @ U - torch.eye(r, device="cuda", dtype=torch.float64)).abs().max().item() <= 1e-5
     assert ((U @ (U.t() @ D) - D).norm(dim=0) <= 1e-5 * D.norm(dim=0)).all()
+
+
+@pytest.mark.parametrize("m,n,r,transposed", [(9792, 9472, 148, False), (9472, 9792, 148, True), (4288, 4160, 520, False)])
+def test_the_column_sums_leave_the_sum_alone(m, n, r, transposed):
+    # A right factor of 9472 rows is 296 chunks of the column sums, a layout for 9792 rows holds 289: behind them lie the column
+    # norms and M + G, which the error feedback reads afterwards.
+    g = torch.Generator(device="cuda"); g.manual_seed(r)
+    rn = lambda *s: torch.randn(*s, generator=g, device="cuda")
+    X, M, G, Q = rn(m, n) * 0.02, rn(m, n) * 0.3, rn(m, n) * 0.1, rn(m if transposed else n, r)
+    Q /= Q.norm(dim=0)
+    B = (M + G).double()
+    Bt = B.t() if transposed else B
+    U, T = torch.linalg.qr(Bt @ Q.double())
+    U *= torch.sign(torch.diagonal(T))
+    R = Bt.t() @ U
+    Qr = R / R.norm(dim=0)
+    Mr = B - 0.05 * (R @ U.t() if transposed else U @ R.t())
+    d = torch.zeros(r, device="cuda")
+    with binding.Dion(mu=0.95) as opt:
+        opt.step(X, M, G, Q, 0.01, colnorm_out=d, transposed=transposed)
+        assert opt.get_status() == (0, 0)
+    # entry by entry: the library's 1e-4 of the largest one
+    for got, want in ((M, Mr), (Q, Qr), (d, R.norm(dim=0))):
+        assert (got.double() - want).abs().max().item() <= 1e-4 * want.abs().max().item()

@@ -11,7 +11,7 @@ def chunks():
     build.build()
     fn = ctypes.CDLL(binding.LIB_PATH).dion_debug_chunks
     fn.argtypes = [ctypes.c_int64] * 4 + [ctypes.c_int, ctypes.POINTER(ctypes.c_int64)]
-    out = (ctypes.c_int64 * 2)()
+    out = (ctypes.c_int64 * 4)()
 
     def call(m, n, r, rows, sms):
         assert fn(m, n, r, rows, sms, out) == 0
@@ -30,5 +30,15 @@ def test_probe_chunks_fit(chunks):
     for m, n in sides():
         for r in {1, min(m, n, 148), min(m, n, 1024)}:
             for rows in (m, n):
-                used, room = chunks(m, n, r, rows, 148)
+                used, room = chunks(m, n, r, rows, 148)[2:]
                 assert 0 < used <= room, (m, n, r, rows)
+
+
+def test_column_normalization_chunks_fit(chunks):
+    # 148 SMs, r = 148: 9472 rows (the right factor of 9792 x 9472) take 296 chunks of 32, 9792 take 288 of 34
+    for sms in (132, 148):
+        for m, n in sides():
+            for r in {1, min(m, n, 148), min(m, n, 520)}:
+                for rows in (m, n):
+                    used, room = chunks(m, n, r, rows, sms)[:2]
+                    assert 0 < used <= room, (m, n, r, rows, sms)
