@@ -115,7 +115,8 @@ struct dion_ctx {
     int64_t launches;
     int index;            // its state slot and scalar
     uint64_t last_use;
-    float scale;          // the scalar's value on the device (NaN: none yet)
+    float scale;          // the scalar's value on the device (NaN: not known)
+    bool recorded;        // a write of the scalar may be in a capture of the caller's: it changes behind the library's back
   };
   std::vector<GraphEntry> graphs;
   bool graphs_on = false;
@@ -2159,18 +2160,25 @@ int step_graph(dion_ctx* c, const dion_matrix* a, float lr, cudaStream_t st) {
     const cudaError_t ie = cudaGraphInstantiate(&exec, graph, 0);
     cudaGraphDestroy(graph);
     if (ie != cudaSuccess || exec == nullptr) { cudaGetLastError(); c->graphs_on = false; return 1; }
-    c->graphs.push_back({*a, exec, nl, index, 0, NAN});
+    c->graphs.push_back({*a, exec, nl, index, 0, NAN, false});
     e = &c->graphs.back();
   }
   e->last_use = ++c->graph_clock;
+  // The scalar is written when the rate changed (a launch of its own, 2 us).  What a stream that is being captured is given has not
+  // run and may run at any time later: nothing is concluded from it, and from then on every call writes.
+  cudaStreamCaptureStatus capturing = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(st, &capturing) != cudaSuccess) { cudaGetLastError(); capturing = cudaStreamCaptureStatusActive; }
+  if (capturing != cudaStreamCaptureStatusNone) e->recorded = true;
   const float scale = lr * sqrtf((float)((double)a->m / (double)a->n));
-  if (!(e->scale == scale)) {      // (the learning rate changed)
+  const bool written = !e->recorded && e->scale == scale;
+  e->scale = NAN;
+  if (!written) {
     k_set_scalar<<<1, 1, 0, st>>>(c->graph_scalars + e->index, scale);
     if (cudaGetLastError() != cudaSuccess) return DION_ERR_CUDA;
-    e->scale = scale;
     c->launches++;
   }
   if (cudaGraphLaunch(e->exec, st) != cudaSuccess) { cudaGetLastError(); return DION_ERR_CUDA; }
+  e->scale = scale;
   c->launches += e->launches;
   return DION_OK;
 }
