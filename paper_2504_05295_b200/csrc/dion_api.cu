@@ -2921,7 +2921,7 @@ bool touch_kernel(K kernel) {
 
 // With lazy module loading a kernel's code is loaded at its first use, which may allocate device memory.
 // Asking for the attributes of every kernel the launch chain can reach loads them all at set-up (the
-// tensor-core variants are covered by configure_kernels, which sets an attribute on each).
+// tensor-core variants and the reduction of their splits are covered by configure_kernels).
 bool preload_kernels() {
   bool ok = true;
   ok = ok && touch_kernel(k_gemm_simt<128, 128, 8, 8, 8, 1, NoTabs>) && touch_kernel(k_gemm_simt<64, 64, 16, 4, 4, 2, NoTabs>) &&
@@ -2936,7 +2936,7 @@ bool preload_kernels() {
   ok = ok && touch_kernel(k_hh_apply) && touch_kernel(k_set_identity) && touch_kernel(k_sign_fix);
   ok = ok && touch_kernel(k_form_b16<true>) && touch_kernel(k_form_b16<false>) && touch_kernel(k_form_b32<true>);
   ok = ok && touch_kernel(k_form_b32<false>) && touch_kernel(k_to_bf16) && touch_kernel(k_round_tf32);
-  ok = ok && touch_kernel(k_split_bf16);
+  ok = ok && touch_kernel(k_split_bf16) && touch_kernel(k_round_f16);
   return ok;
 }
 

@@ -1880,6 +1880,10 @@ int umma_configure() {
   if (e == cudaSuccess) e = set_d16_pair_attr<false, true>();
   if (e == cudaSuccess) e = set_d16_pair_attr<true, true>();
   if (e == cudaSuccess) e = set_d16_pair_attr<true, false>();
+  if (e == cudaSuccess) {      // (no attribute to set, but asking loads it: this unit's copy is the one the products launch)
+    cudaFuncAttributes fa;
+    e = cudaFuncGetAttributes(&fa, k_splitk_reduce);
+  }
   if (e == cudaSuccess) e = set_te_attr<true, 1>();
   if (e == cudaSuccess) e = set_te_attr<true, GEMM_TAB_MAX>();
   if (e == cudaSuccess) e = set_te_attr<false, 1>();
