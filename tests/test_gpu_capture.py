@@ -1,4 +1,6 @@
 """GPU: a step given to a stream that is being captured leaves later steps as they would have been without it."""
+import ctypes
+
 import pytest
 
 pytestmark = pytest.mark.gpu
@@ -6,6 +8,8 @@ torch = pytest.importorskip("torch")
 
 from helpers import MU  # noqa: E402
 from paper_2504_05295_b200 import binding  # noqa: E402
+
+THREAD_LOCAL = 1      # cudaStreamCaptureModeThreadLocal
 
 
 def problem(m, n, r):
@@ -18,6 +22,7 @@ def problem(m, n, r):
 def test_learning_rate_after_a_capture(rate):
     # a matrix small enough to be stepped by replaying a graph that reads the rate from memory; the runtime may refuse to
     # record that replay, and then nothing of the call has run
+    cudart = ctypes.CDLL("libcudart.so.12")
     rates = [0.01, 0.02, 0.01]
     X, M, G, Q = problem(512, 384, 64)
     with binding.Dion(mu=MU) as opt:
@@ -25,24 +30,30 @@ def test_learning_rate_after_a_capture(rate):
             opt.step(X, M, G, Q, lr)
         want = [t.clone() for t in (X, M, Q)]
     X, M, G, Q = problem(512, 384, 64)
+    side = torch.cuda.Stream()
+    graph, replay = ctypes.c_void_p(), ctypes.c_void_p()
     with binding.Dion(mu=MU) as opt:
         opt.step(X, M, G, Q, rates[0])
         torch.cuda.synchronize()
-        graph = torch.cuda.CUDAGraph()
+        assert cudart.cudaStreamBeginCapture(ctypes.c_void_p(side.cuda_stream), THREAD_LOCAL) == 0
         try:
-            with torch.cuda.graph(graph, capture_error_mode="thread_local"):
-                opt.step(X, M, G, Q, rate)
-        except RuntimeError:
-            graph = None
-        torch.cuda.synchronize()
+            opt.step(X, M, G, Q, rate, stream=side)
+            recorded = True
+        except binding.DionError:
+            recorded = False
+        recorded = cudart.cudaStreamEndCapture(ctypes.c_void_p(side.cuda_stream), ctypes.byref(graph)) == 0 and recorded
+        cudart.cudaGetLastError()
         for lr in rates[1:]:
             opt.step(X, M, G, Q, lr)
         assert opt.get_status() == (0, 0)
         for name, a, b in zip("XMQ", (X, M, Q), want):
             assert torch.equal(a, b), name
-        if graph is not None:      # the recorded step keeps its rate, and a direct step after it its own
+        if recorded:      # the recorded step keeps its rate, and a direct step after it its own
             Y = [t.clone() for t in (X, M, Q)]
-            graph.replay()
+            assert cudart.cudaGraphInstantiate(ctypes.byref(replay), graph, ctypes.c_ulonglong(0)) == 0
+            torch.cuda.synchronize()
+            assert cudart.cudaGraphLaunch(replay, ctypes.c_void_p(side.cuda_stream)) == 0
+            side.synchronize()
             opt.step(X, M, G, Q, rates[0])
             torch.cuda.synchronize()
             with binding.Dion(mu=MU) as other:
@@ -51,3 +62,5 @@ def test_learning_rate_after_a_capture(rate):
                 torch.cuda.synchronize()
             for name, a, b in zip("XMQ", (X, M, Q), Y):
                 assert torch.equal(a, b), name
+    # (the thread's own generator and allocator know nothing of the capture)
+    assert torch.isfinite(torch.randn(4, device="cuda")).all()
