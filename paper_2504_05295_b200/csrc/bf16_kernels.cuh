@@ -80,8 +80,7 @@ constexpr int FORM_BATCH = 4;
 template <bool VEC>
 __device__ __forceinline__ void form_b32_body(const float* __restrict__ M, i64 ldm, const void* __restrict__ G,
                                               i64 ldg, int g_mode, i64 rows, i64 cols, float* __restrict__ out,
-                                              __nv_bfloat16* __restrict__ hi, __nv_bfloat16* __restrict__ lo,
-                                              float* amax = nullptr) {      // amax (register, optional): largest magnitude seen by the thread
+                                              __nv_bfloat16* __restrict__ hi, __nv_bfloat16* __restrict__ lo) {
   const i64 per_row = cols / 4;
   const i64 total = rows * per_row;
   // (FORM_BATCH pieces in flight per thread: the sums' stores would keep the compiler from overlapping the loads)
@@ -124,7 +123,6 @@ __device__ __forceinline__ void form_b32_body(const float* __restrict__ M, i64 l
     }
     if (g_mode != ADD_NONE) { v.x += g.x; v.y += g.y; v.z += g.z; v.w += g.w; }
     *reinterpret_cast<float4*>(out + at[u]) = v;
-    if (amax != nullptr) *amax = fmaxf(fmaxf(*amax, fmaxf(fabsf(v.x), fabsf(v.y))), fmaxf(fabsf(v.z), fabsf(v.w)));
     if (hi != nullptr) {
       const float h0 = __bfloat162float(__float2bfloat16_rn(v.x)), h1 = __bfloat162float(__float2bfloat16_rn(v.y));
       const float h2 = __bfloat162float(__float2bfloat16_rn(v.z)), h3 = __bfloat162float(__float2bfloat16_rn(v.w));
@@ -335,9 +333,151 @@ __device__ __forceinline__ int f16_scale_exponent(float amax) {
   if (amax > 0.f && amax < 3.0e38f) frexpf(amax, &ex);
   return 14 - (ex < -80 ? -80 : ex);
 }
-// The two launches that prepare a chain (blockIdx.y) of steps on half pairs: M + G in fp32 with the largest magnitudes of the sum
-// and of Q (Q is a right factor of the caller's making: nothing bounds its entries), then the scaled pairs of both.
-// part: gridDim.x maxima of the sum, then as many of Q.  16-byte accesses to Q where it allows them (qvec).
+// ---- the range of an array ------------------------------------------------------------------------------------
+// The bits of a half pair are relative to the largest entry of its array: entries keep 22 of them down to 2^-17 of it, 17 at
+// 2^-22, 6 at 2^-33, while the three-term TF32 split (22 bits) and a bf16 pair (17) keep theirs at any magnitude.  So the pass
+// that finds the largest entry also looks for small ones that count: the largest entry of every piece, 128 neighbours of a row
+// or 8 of a column, and the smallest of those (pieces of zeros apart).  An array with a piece below 2^-18 of its largest
+// entry takes the 3xTF32 product where 22 bits are asked for (P), one with a piece below 2^-20 bf16 pairs instead of half pairs.
+// (A piece that large holds an entry near its rms for any spread of values but a difference of rows, columns or blocks:
+// Gaussian entries stay above 2^-8.)  512 x 768, r = 128, the lower rows 2^-24 of the upper ones: those of M off by 2.3e-5 on
+// half pairs throughout, 3.4e-7 now.
+constexpr int RANGE_ROWS = 8;
+constexpr float RANGE_P = 3.814697265625e-06f;        // 2^-18: 20 bits and more, below the error of the sums
+constexpr float RANGE_UPDATE = 9.5367431640625e-07f;  // 2^-20: as many as a bf16 pair
+struct Range {
+  float mx = 0.f;                  // largest magnitude
+  unsigned mn = 0x7f800000u;       // smallest of the pieces' largest (float bits: ordered like the values, none is negative)
+};
+__device__ __forceinline__ bool range_is_wide(float mx, float mn, float limit) {      // (also: beyond what the scale can bring back)
+  return mx > 0.f && (mn < mx * limit || mx < 8.3e-25f || !(mx < 3.0e38f));
+}
+// a lane's four entries of one row of a warp's piece (zeros where there are none); cm: its columns' largest so far
+__device__ __forceinline__ void range_row(Range& g, float4 v, float (&cm)[4]) {
+  const float a[4] = {fabsf(v.x), fabsf(v.y), fabsf(v.z), fabsf(v.w)};
+#pragma unroll
+  for (int k = 0; k < 4; ++k) cm[k] = fmaxf(cm[k], a[k]);
+  const float m = fmaxf(fmaxf(a[0], a[1]), fmaxf(a[2], a[3]));
+  g.mx = fmaxf(g.mx, m);
+  const unsigned u = __reduce_max_sync(0xffffffffu, __float_as_uint(m));
+  if (u != 0u) g.mn = min(g.mn, u);
+}
+__device__ __forceinline__ void range_cols(Range& g, const float (&cm)[4]) {
+#pragma unroll
+  for (int k = 0; k < 4; ++k) if (cm[k] > 0.f) g.mn = min(g.mn, __float_as_uint(cm[k]));
+}
+// the range of rows x cols (cols a multiple of 4), a warp per 8 x 128 piece; warp w of nw
+__device__ __forceinline__ void range_scan(Range& g, const float* __restrict__ src, i64 ld, i64 rows, i64 cols, bool vec, i64 w, i64 nw) {
+  const i64 nct = (cols + 127) / 128, pieces = (rows + RANGE_ROWS - 1) / RANGE_ROWS * nct;
+  const int lane = threadIdx.x & 31;
+  for (; w < pieces; w += nw) {
+    const i64 tr = row_of(w, nct), c = (w - tr * nct) * 128 + 4 * lane;
+    float cm[4] = {0.f, 0.f, 0.f, 0.f};
+    float4 v[RANGE_ROWS];
+#pragma unroll
+    for (int q = 0; q < RANGE_ROWS; ++q) {
+      const i64 i = tr * RANGE_ROWS + q;
+      const float* p = src + i * ld + c;
+      v[q] = make_float4(0.f, 0.f, 0.f, 0.f);
+      if (i < rows && c < cols) v[q] = vec ? *reinterpret_cast<const float4*>(p) : make_float4(p[0], p[1], p[2], p[3]);
+    }
+#pragma unroll
+    for (int q = 0; q < RANGE_ROWS; ++q) range_row(g, v[q], cm);
+    range_cols(g, cm);
+  }
+}
+// 256 threads: out[blockIdx.x] and out[gridDim.x + blockIdx.x]
+__device__ __forceinline__ void block_range(const Range& g, float* __restrict__ out) {
+  __shared__ unsigned red[2][8];
+  const unsigned m = __reduce_max_sync(0xffffffffu, __float_as_uint(g.mx)), n = __reduce_min_sync(0xffffffffu, g.mn);
+  if ((threadIdx.x & 31) == 0) { red[0][threadIdx.x >> 5] = m; red[1][threadIdx.x >> 5] = n; }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    unsigned x = red[0][0], y = red[1][0];
+#pragma unroll
+    for (int w = 1; w < 8; ++w) { x = max(x, red[0][w]); y = min(y, red[1][w]); }
+    out[blockIdx.x] = __uint_as_float(x); out[gridDim.x + blockIdx.x] = __uint_as_float(y);
+  }
+  __syncthreads();
+}
+// ... and over the blocks: every thread of 256 gets largest and smallest of n values each, at part and part + n.
+__device__ __forceinline__ void range_of_blocks(const float* __restrict__ part, int n, float& mx, float& mn) {
+  __shared__ unsigned red[2][8];
+  unsigned a = 0u, b = 0x7f800000u;
+  for (int e = threadIdx.x; e < n; e += 256) { a = max(a, __float_as_uint(part[e])); b = min(b, __float_as_uint(part[n + e])); }
+  a = __reduce_max_sync(0xffffffffu, a); b = __reduce_min_sync(0xffffffffu, b);
+  if ((threadIdx.x & 31) == 0) { red[0][threadIdx.x >> 5] = a; red[1][threadIdx.x >> 5] = b; }
+  __syncthreads();
+#pragma unroll
+  for (int w = 0; w < 8; ++w) { a = max(a, red[0][w]); b = min(b, red[1][w]); }
+  mx = __uint_as_float(a); mn = __uint_as_float(b);
+  __syncthreads();
+}
+// The ranges of arrays from a table (blockIdx.y; 16-byte aligned rows), of rows0 or, from the second on, rows1 rows: gridDim.x
+// blocks' partial results `stride` floats apart.
+__global__ void __launch_bounds__(256) k_range_partial(const ChainPtrs srcs, i64 ld, i64 rows0, i64 rows1, i64 cols, float* __restrict__ part,
+                                                       i64 stride, const int* __restrict__ skip_flag, i64 skip_stride) {
+  pdl_enter();
+  if (skip_flag != nullptr && skip_flag[(i64)blockIdx.y * skip_stride] != 0) return;
+  Range g;
+  range_scan(g, reinterpret_cast<const float*>(srcs.p[blockIdx.y]), ld, blockIdx.y == 0 ? rows0 : rows1, cols, true,
+             (i64)blockIdx.x * 8 + (threadIdx.x >> 5), (i64)gridDim.x * 8);
+  block_range(g, part + (i64)blockIdx.y * stride);
+}
+// M + G into `out` (dense), 4 rows of a warp's 8 x 128 piece at a time, and its range.  VEC as for k_form_b32.
+template <bool VEC>
+__device__ __forceinline__ void form_sum_range(Range& g, const float* __restrict__ M, i64 ldm, const void* __restrict__ G, i64 ldg, int g_mode,
+                                               i64 rows, i64 cols, float* __restrict__ out) {
+  const i64 nct = (cols + 127) / 128, pieces = (rows + RANGE_ROWS - 1) / RANGE_ROWS * nct;
+  const int lane = threadIdx.x & 31;
+  for (i64 w = (i64)blockIdx.x * 8 + (threadIdx.x >> 5); w < pieces; w += (i64)gridDim.x * 8) {
+    const i64 tr = row_of(w, nct), c = (w - tr * nct) * 128 + 4 * lane;
+    float cm[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+    for (int h = 0; h < RANGE_ROWS; h += FORM_BATCH) {
+      float4 mv[FORM_BATCH], gv[FORM_BATCH];
+#pragma unroll
+      for (int u = 0; u < FORM_BATCH; ++u) {
+        const i64 i = tr * RANGE_ROWS + h + u;
+        mv[u] = gv[u] = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (i >= rows || c >= cols) continue;
+        const float* mp = M + i * ldm + c;
+        mv[u] = VEC ? __ldg(reinterpret_cast<const float4*>(mp)) : make_float4(mp[0], mp[1], mp[2], mp[3]);
+        if (g_mode == ADD_F32) {
+          const float* gp = reinterpret_cast<const float*>(G) + i * ldg + c;
+          gv[u] = VEC ? __ldg(reinterpret_cast<const float4*>(gp)) : make_float4(gp[0], gp[1], gp[2], gp[3]);
+        } else if (g_mode == ADD_BF16) {
+          const __nv_bfloat16* gp = reinterpret_cast<const __nv_bfloat16*>(G) + i * ldg + c;
+          if (VEC) {
+            const uint2 t = __ldg(reinterpret_cast<const uint2*>(gp));
+            gv[u].x = __uint_as_float(t.x); gv[u].y = __uint_as_float(t.y);
+          } else {
+            gv[u] = make_float4(__bfloat162float(gp[0]), __bfloat162float(gp[1]), __bfloat162float(gp[2]), __bfloat162float(gp[3]));
+          }
+        }
+      }
+#pragma unroll
+      for (int u = 0; u < FORM_BATCH; ++u) {
+        const i64 i = tr * RANGE_ROWS + h + u;
+        float4 v = mv[u], a = gv[u];
+        if (VEC && g_mode == ADD_BF16) {      // (still the four bf16 values)
+          const uint32_t w0 = __float_as_uint(a.x), w1 = __float_as_uint(a.y);
+          a = make_float4(__uint_as_float(w0 << 16), __uint_as_float(w0 & 0xffff0000u), __uint_as_float(w1 << 16), __uint_as_float(w1 & 0xffff0000u));
+        }
+        if (g_mode != ADD_NONE) { v.x += a.x; v.y += a.y; v.z += a.z; v.w += a.w; }
+        if (i < rows && c < cols) *reinterpret_cast<float4*>(out + i * cols + c) = v;
+        range_row(g, v, cm);
+      }
+    }
+    range_cols(g, cm);
+  }
+}
+// The two launches that prepare a chain (blockIdx.y) of steps on half pairs: M + G in fp32 with the ranges of the sum and of Q
+// (Q is a right factor of the caller's making: nothing bounds its entries), then the scaled pairs of both -- or, where the ranges
+// say so, a dense fp32 copy of Q for the 3xTF32 product that then forms P, and the sum as a bf16 pair, with which R and the
+// error feedback run at the same speed.
+// part: gridDim.x partial ranges of the sum (maxima, then minima), then as many of Q.  16-byte accesses to Q where it allows
+// them (qvec).
 template <bool VEC>
 __global__ void __launch_bounds__(256, 3) k_form_sum_amax(const ChainPtrs Ms, i64 ldm, const ChainPtrs Gs, i64 ldg, int g_mode, i64 rows, i64 cols,
                                                        const ChainPtrs Qs, i64 ldq, i64 qrows, i64 qcols, int qvec, float* __restrict__ out,
@@ -346,48 +486,61 @@ __global__ void __launch_bounds__(256, 3) k_form_sum_amax(const ChainPtrs Ms, i6
   clear_slot(slots);
   const i64 b = blockIdx.y;
   part += b * wstride;
-  float m = 0.f, mq = 0.f;
-  form_b32_body<VEC>(reinterpret_cast<const float*>(Ms.p[b]), ldm, Gs.p[b], ldg, g_mode, rows, cols, out + b * wstride, nullptr, nullptr, &m);
-  const float* __restrict__ Q = reinterpret_cast<const float*>(Qs.p[b]);
-  const i64 per_row = qcols / 4, total = qrows * per_row;
-  for (i64 e = (i64)blockIdx.x * blockDim.x + threadIdx.x; e < total; e += (i64)gridDim.x * blockDim.x) {
-    const i64 i = row_of(e, per_row);
-    const float* q = Q + i * ldq + (e - i * per_row) * 4;
-    const float4 a = qvec ? *reinterpret_cast<const float4*>(q) : make_float4(q[0], q[1], q[2], q[3]);
-    mq = fmaxf(fmaxf(mq, fmaxf(fabsf(a.x), fabsf(a.y))), fmaxf(fabsf(a.z), fabsf(a.w)));
-  }
-  block_max(m, part);
-  __syncthreads();
-  block_max(mq, part + gridDim.x);
+  Range g, gq;
+  form_sum_range<VEC>(g, reinterpret_cast<const float*>(Ms.p[b]), ldm, Gs.p[b], ldg, g_mode, rows, cols, out + b * wstride);
+  // (from the last warp down: the first ones have a piece of the sum more)
+  range_scan(gq, reinterpret_cast<const float*>(Qs.p[b]), ldq, qrows, qcols, qvec != 0, (i64)gridDim.x * 8 - 1 - ((i64)blockIdx.x * 8 + (threadIdx.x >> 5)),
+             (i64)gridDim.x * 8);
+  block_range(g, part);
+  block_range(gq, part + 2 * gridDim.x);
 }
 // A step's scalars: the factors that take the scales out of P, R and the error feedback; then R's block maxima.
 enum : int { HS_P = 0, HS_R = 1, HS_EF = 2, HS_Q = 3, HS_T = 4, HS_MAX = 16 };      // (HS_Q: 1 / scale of Q; HS_T: Lazy-Dion's left factor)
 constexpr int HS_U_BITS = 13;      // U's pair is scaled by 2^13 (entries at most 1)
+// eight values as a pair: half values scaled by f (a power of two), or bf16 values as they are
+__device__ __forceinline__ void pair_of_8(const float (&x)[8], float f, bool bf16, uint4& hi, uint4& lo) {
+  if (!bf16) {
+    __half h[8], l[8];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+      h[k] = __float2half_rn(f * x[k]);
+      l[k] = __float2half_rn(f * x[k] - __half2float(h[k]));
+    }
+    hi = *reinterpret_cast<const uint4*>(h); lo = *reinterpret_cast<const uint4*>(l);
+  } else {
+    uint32_t h[4], l[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      h[k] = pack_bf16x2(x[2 * k], x[2 * k + 1]);
+      l[k] = pack_bf16x2(x[2 * k] - __uint_as_float(h[k] << 16), x[2 * k + 1] - __uint_as_float(h[k] & 0xffff0000u));
+    }
+    hi = make_uint4(h[0], h[1], h[2], h[3]); lo = make_uint4(l[0], l[1], l[2], l[3]);
+  }
+}
+// os (optional: without it the ranges are not looked at): state slots; qd (optional): the dense copy of Q.
 __global__ void __launch_bounds__(256) k_split_sum(const float* __restrict__ sum, i64 total_s, const ChainPtrs Qs, i64 ldq, i64 qrows,
                                                    i64 qcols, int qvec, const float* __restrict__ part, int nparts,
-                                                   __half* __restrict__ sh, __half* __restrict__ qh, float* __restrict__ scal, i64 wstride) {
+                                                   __half* __restrict__ sh, __half* __restrict__ qh, float* __restrict__ qd,
+                                                   float* __restrict__ scal, int* __restrict__ os, i64 wstride) {
   pdl_enter();
   const i64 b = blockIdx.y;
   sum += b * wstride; part += b * wstride; scal += b * wstride;
   sh += 2 * b * wstride; qh += 2 * b * wstride;
   const float* __restrict__ Q = reinterpret_cast<const float*>(Qs.p[b]);
-  __shared__ float red[2][256];
-  float m0 = 0.f, m1 = 0.f;
-  for (int e = threadIdx.x; e < nparts; e += 256) { m0 = fmaxf(m0, part[e]); m1 = fmaxf(m1, part[nparts + e]); }
-  red[0][threadIdx.x] = m0; red[1][threadIdx.x] = m1;
-  __syncthreads();
-  for (int w = 128; w > 0; w >>= 1) {
-    if ((int)threadIdx.x < w) {
-      red[0][threadIdx.x] = fmaxf(red[0][threadIdx.x], red[0][threadIdx.x + w]);
-      red[1][threadIdx.x] = fmaxf(red[1][threadIdx.x], red[1][threadIdx.x + w]);
-    }
-    __syncthreads();
-  }
-  const int es = f16_scale_exponent(red[0][0]), eq = f16_scale_exponent(red[1][0]);
+  float m0, n0, m1, n1;
+  range_of_blocks(part, nparts, m0, n0);
+  range_of_blocks(part + 2 * nparts, nparts, m1, n1);
+  const bool wide = os != nullptr && range_is_wide(m0, n0, RANGE_UPDATE);
+  const bool p32 = os != nullptr && (range_is_wide(m0, n0, RANGE_P) || range_is_wide(m1, n1, RANGE_P));
+  const int es = f16_scale_exponent(m0), eq = f16_scale_exponent(m1);
   if (blockIdx.x == 0 && threadIdx.x == 0) {
     scal[HS_P] = ldexpf(1.f, -es) * ldexpf(1.f, -eq);
-    scal[HS_R] = ldexpf(1.f, -es - HS_U_BITS);
+    scal[HS_R] = wide ? 1.f : ldexpf(1.f, -es - HS_U_BITS);
     scal[HS_Q] = ldexpf(1.f, -eq);
+    if (os != nullptr) {
+      int* o = os + b * OS_SLOT_INTS;
+      o[OS_WIDE] = wide ? 1 : 0; o[OS_P32] = p32 ? 1 : 0; o[OS_PHALF] = p32 ? 0 : 1;
+    }
   }
   const float fs = ldexpf(1.f, es), fq = ldexpf(1.f, eq);
   const i64 n8 = total_s / 8, qpr = qcols / 8, q8 = qrows * qpr;
@@ -403,18 +556,18 @@ __global__ void __launch_bounds__(256) k_split_sum(const float* __restrict__ sum
       const float* q = Q + i * ldq + (eo - i * qpr) * 8;
       x = qvec ? *reinterpret_cast<const float4*>(q) : make_float4(q[0], q[1], q[2], q[3]);
       y = qvec ? *reinterpret_cast<const float4*>(q + 4) : make_float4(q[4], q[5], q[6], q[7]);
+      if (p32 && qd != nullptr) {
+        *reinterpret_cast<float4*>(qd + b * wstride + eo * 8) = x;
+        *reinterpret_cast<float4*>(qd + b * wstride + eo * 8 + 4) = y;
+        continue;
+      }
     }
-    const float f = of_q ? fq : fs;
-    const float v[8] = {f * x.x, f * x.y, f * x.z, f * x.w, f * y.x, f * y.y, f * y.z, f * y.w};
-    __half h[8], l[8];
-#pragma unroll
-    for (int k = 0; k < 8; ++k) {
-      h[k] = __float2half_rn(v[k]);
-      l[k] = __float2half_rn(v[k] - __half2float(h[k]));
-    }
+    const float v[8] = {x.x, x.y, x.z, x.w, y.x, y.y, y.z, y.w};
+    uint4 h, l;
+    pair_of_8(v, of_q ? fq : fs, wide && !of_q, h, l);
     __half* hi = (of_q ? qh : sh) + eo * 8;
-    *reinterpret_cast<uint4*>(hi) = *reinterpret_cast<const uint4*>(h);
-    *reinterpret_cast<uint4*>(hi + (of_q ? qrows * qcols : total_s)) = *reinterpret_cast<const uint4*>(l);
+    *reinterpret_cast<uint4*>(hi) = h;
+    *reinterpret_cast<uint4*>(hi + (of_q ? qrows * qcols : total_s)) = l;
   }
 }
 __global__ void __launch_bounds__(256) k_absmax_partial(const float* __restrict__ src, i64 ld, i64 rows, i64 cols,
@@ -485,31 +638,39 @@ __global__ void __launch_bounds__(256) k_split_f16_scaled(const float* __restric
 // hi = half(scale x), lo = half(scale x - hi) with a scale given by the caller (a power of two; for arrays whose
 // entries are bounded, like the unit-norm columns of Q).  Sources from a pointer table (blockIdx.y), outputs
 // `ostride` floats apart.
-// ldo: leading dimension of the outputs (0: dense).
+// ldo: leading dimension of the outputs (0: dense).  wide (optional, a state slot apart): flagged matrices get a bf16 pair.
+// one (optional, dense): half(scale x) either way.
 __global__ void __launch_bounds__(256) k_split_f16_fixed(const ChainPtrs srcs, i64 lds, i64 rows, i64 cols, float scale,
                                                          __half* __restrict__ hi, __half* __restrict__ lo, i64 ostride,
-                                                         i64 ldo = 0, const int* __restrict__ skip_flag = nullptr,
-                                                         i64 skip_stride = 0) {
+                                                         i64 ldo, const int* __restrict__ skip_flag, i64 skip_stride,
+                                                         const int* __restrict__ wide, __half* __restrict__ one) {
   pdl_enter();
   const i64 bm = blockIdx.y;
   if (skip_flag != nullptr && skip_flag[bm * skip_stride] != 0) return;
   if (ldo == 0) ldo = cols;
   const float* __restrict__ src = reinterpret_cast<const float*>(srcs.p[bm]);
   hi += 2 * bm * ostride; lo += 2 * bm * ostride;
+  if (one != nullptr) one += 2 * bm * ostride;
+  const bool bf16 = wide != nullptr && wide[bm * OS_SLOT_INTS] != 0;
   const i64 per_row = cols / 8, total = rows * per_row;
   for (i64 e = (i64)blockIdx.x * blockDim.x + threadIdx.x; e < total; e += (i64)gridDim.x * blockDim.x) {
     const i64 i = row_of(e, per_row), c = (e - i * per_row) * 8;
     const float4 a = *reinterpret_cast<const float4*>(src + i * lds + c);
     const float4 b = *(reinterpret_cast<const float4*>(src + i * lds + c) + 1);
-    const float v[8] = {scale * a.x, scale * a.y, scale * a.z, scale * a.w, scale * b.x, scale * b.y, scale * b.z, scale * b.w};
-    __half h[8], l[8];
+    const float v[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
+    uint4 h, l;
+    pair_of_8(v, scale, bf16, h, l);
+    *reinterpret_cast<uint4*>(hi + i * ldo + c) = h;
+    *reinterpret_cast<uint4*>(lo + i * ldo + c) = l;
+    if (one != nullptr) {
+      if (bf16) {
+        __half t[8];
 #pragma unroll
-    for (int q = 0; q < 8; ++q) {
-      h[q] = __float2half_rn(v[q]);
-      l[q] = __float2half_rn(v[q] - __half2float(h[q]));
+        for (int k = 0; k < 8; ++k) t[k] = __float2half_rn(scale * v[k]);
+        h = *reinterpret_cast<const uint4*>(t);
+      }
+      *reinterpret_cast<uint4*>(one + i * cols + c) = h;
     }
-    *reinterpret_cast<uint4*>(hi + i * ldo + c) = *reinterpret_cast<const uint4*>(h);
-    *reinterpret_cast<uint4*>(lo + i * ldo + c) = *reinterpret_cast<const uint4*>(l);
   }
 }
 

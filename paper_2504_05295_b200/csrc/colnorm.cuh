@@ -140,6 +140,9 @@ struct ColnormPairs {
   const float* amax; int nmax;   // CN_HALF: R's block maxima; its scale puts the largest magnitude in [2^13, 2^14)
   float* scal;             // ... and the factor that takes the scales out of the product with U's pair,
   const float* other;      // or with another pair (optional: its 1 / scale)
+  int* os;                 // CN_HALF, optional: state slots; the pair of a matrix whose OS_WIDE is set is a bf16 pair.  With
+  const float* range;      // `range` the flag is set here: ranges (k_range_partial) of R and, behind them, of U, of
+  int nrange;              // this many blocks
 };
 enum : int { CN_HALF = 1, CN_BF16 = 2, CN_ONE = 3 };
 
@@ -177,13 +180,25 @@ __global__ void __launch_bounds__(CN_THREADS, 3) k_colnorm_apply(const float* __
   float s[4];
   cn_sum_chunks<V4>(part, chunks, j0, r, red, s);      // (its barrier also covers redm)
   float rscale = 1.f;
+  bool bf16 = x.kind == CN_BF16;
   if (x.kind == CN_HALF) {
     m = redm[0];
 #pragma unroll
     for (int w = 1; w < CN_WARPS; ++w) m = fmaxf(m, redm[w]);
+    if (x.range != nullptr) {      // (U's scale is 2^13, its entries are at most 1)
+      float mw, nw, mu, nu;
+      range_of_blocks(x.range, x.nrange, mw, nw);
+      range_of_blocks(x.range + 2 * x.nrange, x.nrange, mu, nu);
+      m = mw;
+      bf16 = range_is_wide(mw, nw, RANGE_UPDATE) || nu < RANGE_UPDATE;
+      if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) x.os[OS_WIDE] = bf16 ? 1 : 0;
+    } else if (x.os != nullptr) {
+      bf16 = x.os[b * OS_SLOT_INTS + OS_WIDE] != 0;
+    }
     const int e = f16_scale_exponent(m);
     rscale = ldexpf(1.f, e);
-    if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) x.scal[b * wstride] = x.other != nullptr ? ldexpf(1.f, -e) * x.other[b * wstride] : ldexpf(1.f, -e - HS_U_BITS);
+    if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0)
+      x.scal[b * wstride] = bf16 ? 1.f : x.other != nullptr ? ldexpf(1.f, -e) * x.other[b * wstride] : ldexpf(1.f, -e - HS_U_BITS);
   }
   float inv[4];
 #pragma unroll
@@ -225,7 +240,7 @@ __global__ void __launch_bounds__(CN_THREADS, 3) k_colnorm_apply(const float* __
 #pragma unroll
         for (int k = 0; k < 4; ++k) h[k] = __float2half_rn(x.qscale * q[k]);
         uint2 q16 = *reinterpret_cast<const uint2*>(h), hi, lo;
-        if (x.kind == CN_HALF) {
+        if (x.kind == CN_HALF && !bf16) {
           __half l[4];
 #pragma unroll
           for (int k = 0; k < 4; ++k) {

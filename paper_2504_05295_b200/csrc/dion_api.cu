@@ -474,6 +474,7 @@ GemmArgs for_matrix(const StepCtx& s, GemmArgs g, int b, bool a_ws, bool b_ws, b
   if (b_ws && g.B16lo != nullptr) g.B16lo = (const char*)g.B16lo + 4 * o;
   if (g.alpha_dev != nullptr) g.alpha_dev += (i64)b * g.alpha_dev_stride;
   if (g.skip_flag != nullptr) g.skip_flag += (i64)b * OS_SLOT_INTS;
+  if (g.wide_flag != nullptr) g.wide_flag += (i64)b * OS_SLOT_INTS;
   return g;
 }
 
@@ -541,7 +542,9 @@ int launch_gemm_group(StepCtx& s, const std::vector<GemmArgs>& v) {
             g.batch == 1 && a.batch == 1 && g.tri == a.tri && g.klimit == a.klimit && g.precise == a.precise &&
             g.ab16 == a.ab16 && g.f16 == a.f16 && g.tf32x1 == a.tf32x1 &&
             ((a.skip_flag == nullptr && g.skip_flag == nullptr) ||
-             (a.skip_flag != nullptr && g.skip_flag == a.skip_flag + (i64)b * OS_SLOT_INTS));
+             (a.skip_flag != nullptr && g.skip_flag == a.skip_flag + (i64)b * OS_SLOT_INTS)) &&
+            ((a.wide_flag == nullptr && g.wide_flag == nullptr) ||
+             (a.wide_flag != nullptr && g.wide_flag == a.wide_flag + (i64)b * OS_SLOT_INTS));
     one = one && alike && at_stride(a.A, g.A, b) && at_stride(a.B, g.B, b) && at_stride(a.A2, g.A2, b) && at_stride(a.A16lo, g.A16lo, b) &&
           at_stride(a.B16lo, g.B16lo, b);
     c_strided = c_strided && at_stride(a.C, g.C, b);
@@ -1004,7 +1007,7 @@ int cholqr_round(StepCtx& s, i64 pin_off, i64 pout_off, i64 rows, i64 r, int mod
         ChainPtrs t;
         for (int b = 0; b < s.nb; ++b) t.p[b] = s.W(b, pout_off + J0);
         launch_pdl(k_split_f16_fixed, dim3((unsigned)grid_for(c, rows * sz / 8, s.nb), (unsigned)s.nb), dim3(256), 0, s.st, t, r, rows, sz,
-                   ldexpf(1.f, 6), pop + J0, pop + rows * r + J0, s.wstride, r, skip, (i64)OS_SLOT_INTS);
+                   ldexpf(1.f, 6), pop + J0, pop + rows * r + J0, s.wstride, r, skip, (i64)OS_SLOT_INTS, (const int*)nullptr, (__half*)nullptr);
         DION_CHECK_LAUNCH(c);
       }
       return DION_OK;
@@ -1281,16 +1284,16 @@ int colnorm_launch(StepCtx& s, int b, int per, const float* W, i64 ldw, i64 rows
   const bool v4 = r % 4 == 0 && ldw % 4 == 0 && !((uintptr_t)W & 15);
   float* amax = nullptr;
   if (x.kind == CN_HALF) {
-    amax = s.W(b, s.L.lz) + HS_MAX;
-    x.amax = amax; x.scal = s.W(b, s.L.lz) + HS_EF;
-    x.nmax = (int)(grid.x * grid.y);
+    x.scal = s.W(b, s.L.lz) + HS_EF;
+    if (x.range == nullptr) {
+      amax = s.W(b, s.L.lz) + HS_MAX;
+      x.amax = amax;
+      x.nmax = (int)(grid.x * grid.y);
+    }
   }
   if (sums == nullptr) {
     if (v4) launch_pdl(k_colsumsq_partial<true>, grid, dim3(CN_THREADS), 0, s.st, W, ldw, rows, r, rpc, part, amax, (const int*)nullptr, s.wstride);
     else launch_pdl(k_colsumsq_partial<false>, grid, dim3(CN_THREADS), 0, s.st, W, ldw, rows, r, rpc, part, amax, (const int*)nullptr, s.wstride);
-    DION_CHECK_LAUNCH(c);
-  } else if (x.kind == CN_HALF) {
-    launch_pdl(k_absmax_partial, dim3((unsigned)x.nmax), dim3(256), 0, s.st, W, ldw, rows, r, amax, (i64)0, (const int*)nullptr, (i64)0);
     DION_CHECK_LAUNCH(c);
   }
   int qvec = ldq % 4 == 0;
@@ -1335,6 +1338,7 @@ int colnorm_chain(StepCtx& s, const dion_matrix* const* list, i64 rows, i64 r, i
     for (int k = 0; k < per; ++k) { Qs.p[k] = list[b + k]->Q; ds.p[k] = list[b + k]->colnorm_out; }
     ColnormPairs x = ColnormPairs();
     x.kind = kind; x.qh = s.W(b, qh_off); x.qscale = qscale; x.hi = s.W(b, pair_off);
+    if (kind == CN_HALF) x.os = s.OS(b);
     DION_TRY(colnorm_launch(s, b, per, s.W(b, s.L.R), r, rows, r, Qs, list[b]->ldq, ds, s.OS(b) + OS_FAIL, x));
   }
   return DION_OK;
@@ -1369,8 +1373,9 @@ int split_chain(StepCtx& s, const float* const* src, const i64* ld, i64 rows, i6
   return DION_OK;
 }
 
-// ... as a half pair scaled by 2^bits.
-int split_half_chain(StepCtx& s, const float* const* src, i64 ld, i64 rows, i64 cols, i64 out_off, int bits, const int* skip0) {
+// ... as a half pair scaled by 2^bits, or a bf16 pair where a matrix's range is wide (OS_WIDE).  one_off >= 0: the half array
+// alone too, whichever pair it is.
+int split_half_chain(StepCtx& s, const float* const* src, i64 ld, i64 rows, i64 cols, i64 out_off, int bits, const int* skip0, i64 one_off) {
   dion_ctx* c = s.c;
   const int per = (s.nb <= GEMM_TAB_MAX && c->chain_batch) ? s.nb : 1;
   for (int b = 0; b < s.nb; b += per) {
@@ -1378,7 +1383,8 @@ int split_half_chain(StepCtx& s, const float* const* src, i64 ld, i64 rows, i64 
     for (int k = 0; k < per; ++k) t.p[k] = src[b + k];
     __half* hi = reinterpret_cast<__half*>(s.W(b, out_off));
     launch_pdl(k_split_f16_fixed, dim3((unsigned)grid_for(c, rows * cols / 8, per), (unsigned)per), dim3(256), 0, s.st, t, ld, rows, cols, ldexpf(1.f, bits),
-               hi, hi + rows * cols, s.wstride, (i64)0, skip0 != nullptr ? skip0 + (i64)b * OS_SLOT_INTS : (const int*)nullptr, (i64)OS_SLOT_INTS);
+               hi, hi + rows * cols, s.wstride, (i64)0, skip0 != nullptr ? skip0 + (i64)b * OS_SLOT_INTS : (const int*)nullptr, (i64)OS_SLOT_INTS,
+               (const int*)(s.OS(b) + OS_WIDE), one_off >= 0 ? reinterpret_cast<__half*>(s.W(b, one_off)) : (__half*)nullptr);
     DION_CHECK_LAUNCH(c);
   }
   return DION_OK;
@@ -1500,8 +1506,9 @@ bool step_on_half_pairs(const StepCtx& s, i64 m, i64 n, i64 r, i64 short_dim) {
 }
 
 // M + G and the half pairs of it and of Q (in S16) for every matrix of the chain: in one pair of launches when they share
-// leading dimensions and alignment.
-int half_sum_chain(StepCtx& s, const dion_matrix* const* list, i64 qrow, bool clear = false) {
+// leading dimensions and alignment.  ranges: matrices of wide range are flagged and get what the other formats need instead
+// (Q dense in P1, a bf16 pair of the sum).
+int half_sum_chain(StepCtx& s, const dion_matrix* const* list, i64 qrow, bool clear, bool ranges) {
   dion_ctx* c = s.c;
   const dion_matrix* a0 = list[0];
   const i64 m = a0->m, n = a0->n, r = a0->r;
@@ -1520,17 +1527,33 @@ int half_sum_chain(StepCtx& s, const dion_matrix* const* list, i64 qrow, bool cl
     ChainPtrs Ms, Gs, Qs;
     for (int k = 0; k < per; ++k) { Ms.p[k] = list[b + k]->M; Gs.p[k] = list[b + k]->G; Qs.p[k] = list[b + k]->Q; }
     const int g_mode = (a->g_dtype == DION_BF16) ? ADD_BF16 : ADD_F32;
-    const dim3 fg((unsigned)grid_for(c, m * n / 4, per), (unsigned)per), sg((unsigned)grid_for(c, (m * n + qrow * r) / 8, per), (unsigned)per);
-    float* part = s.W(b, s.L.part);      // (the maxima are read before the products write their partial sums there)
+    const i64 pieces = (m + RANGE_ROWS - 1) / RANGE_ROWS * ((n + 127) / 128);
+    const dim3 fg((unsigned)grid_for(c, 32 * pieces, per), (unsigned)per), sg((unsigned)grid_for(c, (m * n + qrow * r) / 8, per), (unsigned)per);
+    float* part = s.W(b, s.L.part);      // (the ranges are read before the products write their partial sums there)
     const int qv = qvec_ok(a) ? 1 : 0;
     if (vec_ok(a)) launch_pdl(k_form_sum_amax<true>, fg, dim3(256), 0, s.st, Ms, a->ldm, Gs, a->ldg, g_mode, m, n, Qs, a->ldq, qrow, r, qv, s.W(b, s.L.B32), part, s.wstride, clear ? s.OS(b) : (int*)nullptr);
     else launch_pdl(k_form_sum_amax<false>, fg, dim3(256), 0, s.st, Ms, a->ldm, Gs, a->ldg, g_mode, m, n, Qs, a->ldq, qrow, r, qv, s.W(b, s.L.B32), part, s.wstride, clear ? s.OS(b) : (int*)nullptr);
     DION_CHECK_LAUNCH(c);
     launch_pdl(k_split_sum, sg, dim3(256), 0, s.st, (const float*)s.W(b, s.L.B32), m * n, Qs, a->ldq, qrow, r, qv, (const float*)part, (int)fg.x,
-               reinterpret_cast<__half*>(s.W(b, s.L.Bp)), reinterpret_cast<__half*>(s.W(b, s.L.S16)), s.W(b, s.L.lz), s.wstride);
+               reinterpret_cast<__half*>(s.W(b, s.L.Bp)), reinterpret_cast<__half*>(s.W(b, s.L.S16)), s.W(b, s.L.P1), s.W(b, s.L.lz),
+               ranges ? s.OS(b) : (int*)nullptr, s.wstride);
     DION_CHECK_LAUNCH(c);
   }
   return DION_OK;
+}
+
+// P = (M + G) Q of a matrix of a step on half pairs, where its range is wide: the 3xTF32 product of the fp32 sum and the dense
+// copy of Q.  (Launched behind the product on half pairs; each of the two finds itself flagged for the other's matrices.)
+GemmArgs wide_p(const StepCtx& s, int b, const dion_matrix* a, bool tr, float* P) {
+  const i64 n = a->n, r = a->r;
+  GemmArgs p = gemm_args();
+  p.M = tr ? n : a->m; p.N = r; p.K = tr ? a->m : n;
+  p.A = s.W(b, s.L.B32); p.a_si = tr ? 1 : n; p.a_sk = tr ? n : 1;
+  p.B = s.W(b, s.L.P1); p.b_sk = r; p.b_sn = 1;
+  p.C = P; p.ldc = r; p.epi = EPI_STORE;
+  p.skip_flag = s.OS(b) + OS_PHALF;
+  p.precise = 1;      // (as accurate as the half pairs are on a narrow range: 1.4e-6; 8e-6 without)
+  return p;
 }
 
 // Forms M + G in scratch (fp32) and, when `pair`, as a bf16 pair beside it.
@@ -1782,7 +1805,7 @@ int step_batch(dion_ctx* c, const dion_matrix* const* list, int nb, float lr, cu
   // elementwise preparation for the whole chain: M + G (and its pair), the pair of Q where P takes pairs
   const float* srcs[MAX_CHAIN];
   i64 lds[MAX_CHAIN];
-  if (hstep) DION_TRY(half_sum_chain(s, list, qrow, true));
+  if (hstep) DION_TRY(half_sum_chain(s, list, qrow, true, true));
   else if (b32) DION_TRY(form_sum_chain(s, list, bpair, true));
   else if (!d16 && cudaMemsetAsync(s.os, 0, sizeof(int) * OS_SLOT_INTS * nb, st) != cudaSuccess) return DION_ERR_CUDA;
   const bool phalf = b32 && s.L.Bh > 0;
@@ -1808,7 +1831,7 @@ int step_batch(dion_ctx* c, const dion_matrix* const* list, int nb, float lr, cu
       for (int b = 0; b < nb; ++b) t.p[b] = srcs[b];
       __half* qh = reinterpret_cast<__half*>(s.ws + s.L.S16);
       launch_pdl(k_split_f16_fixed, dim3((unsigned)grid_for(c, qrow * r / 8, nb), (unsigned)nb), dim3(256), 0, st, t, list[0]->ldq, qrow, r,
-                 ldexpf(1.f, 13), qh, qh + qrow * r, s.wstride, (i64)0, (const int*)nullptr, (i64)0);
+                 ldexpf(1.f, 13), qh, qh + qrow * r, s.wstride, (i64)0, (const int*)nullptr, (i64)0, (const int*)nullptr, (__half*)nullptr);
       DION_CHECK_LAUNCH(c);
       p_half_ready = true;
     }
@@ -1876,6 +1899,7 @@ int step_batch(dion_ctx* c, const dion_matrix* const* list, int nb, float lr, cu
       p.A = (const float*)bh; p.A16lo = bh + m * n; p.a_si = tr ? 1 : n; p.a_sk = tr ? n : 1;
       p.B = (const float*)qh; p.B16lo = qh + qrow * r; p.b_sk = r; p.b_sn = 1;
       p.alpha_dev = s.W(b, s.L.lz) + HS_P;
+      p.skip_flag = s.OS(b) + OS_P32;
     } else if (p_half_ready) {
       __half* bh = reinterpret_cast<__half*>(s.W(b, s.L.Bh));
       __half* qh = reinterpret_cast<__half*>(s.W(b, s.L.S16));
@@ -1898,10 +1922,16 @@ int step_batch(dion_ctx* c, const dion_matrix* const* list, int nb, float lr, cu
     group[b] = p;
   }
   DION_TRY(launch_gemm_group(s, group));
+  if (hstep) {
+    for (int b = 0; b < nb; ++b) group[b] = wide_p(s, b, list[b], tr, s.W(b, pin_off));
+    DION_TRY(launch_gemm_group(s, group));
+  }
   }
 
   // U = Orthonormalize(P)
   i64 U_off = 0;
+  // (steps on half pairs: U as a half array for the weight update, behind Q's in the panel's save buffer, free by then)
+  const i64 u_one = s.L.Psave + ((m > n) ? m : n) * r / 2;
   {
   PhaseScope ps(c, st, DION_PHASE_ORTH);
   const std::function<int()> redo = [&]() -> int {
@@ -1935,7 +1965,7 @@ int step_batch(dion_ctx* c, const dion_matrix* const* list, int nb, float lr, cu
     const float* srcs[MAX_CHAIN];
     i64 lds[MAX_CHAIN];
     for (int b = 0; b < nb; ++b) { srcs[b] = s.W(b, U_off); lds[b] = r; }
-    if (hstep) DION_TRY(split_half_chain(s, srcs, r, prow, r, other_off, HS_U_BITS, s.os + OS_FAIL));
+    if (hstep) DION_TRY(split_half_chain(s, srcs, r, prow, r, other_off, HS_U_BITS, s.os + OS_FAIL, u_one));
     else DION_TRY(split_chain(s, srcs, lds, prow, r, other_off, s.os + OS_FAIL));
   }
   for (int b = 0; b < nb; ++b) {
@@ -1950,7 +1980,7 @@ int step_batch(dion_ctx* c, const dion_matrix* const* list, int nb, float lr, cu
     } else if (bpair) {
       // U as a bf16 pair in the other panel buffer (the error feedback reuses it)
       DION_TRY(r_pairs(s, b, a, tr, s.W(b, U_off), s.W(b, other_off), s.W(b, s.L.R), s.OS(b) + OS_FAIL, &group[b], true));
-      if (hstep) { group[b].f16 = 1; group[b].alpha_dev = s.W(b, s.L.lz) + HS_R; }      // (the same place and layout)
+      if (hstep) { group[b].f16 = 1; group[b].wide_flag = s.OS(b) + OS_WIDE; group[b].alpha_dev = s.W(b, s.L.lz) + HS_R; }      // (the same place and layout)
       continue;
     } else if (b32) {
       w.A = s.W(b, s.L.B32); w.a_si = tr ? n : 1; w.a_sk = tr ? 1 : n;
@@ -2036,7 +2066,7 @@ int step_batch(dion_ctx* c, const dion_matrix* const* list, int nb, float lr, cu
     const float* sum32 = b32 ? s.W(b, s.L.B32) : nullptr;
     if (tr) DION_TRY(ef_update(s, b, a, Rf, r, Uf, r, sbuf, other, sum32, s.OS(b) + OS_FAIL, ef_split, bpair || ef_split, &group[b]));
     else DION_TRY(ef_update(s, b, a, Uf, r, Rf, r, other, sbuf, sum32, s.OS(b) + OS_FAIL, bpair || ef_split, ef_split, &group[b]));
-    if (hstep && group[b].ab16) { group[b].f16 = 1; group[b].alpha_dev = s.W(b, s.L.lz) + HS_EF; }
+    if (hstep && group[b].ab16) { group[b].f16 = 1; group[b].wide_flag = s.OS(b) + OS_WIDE; group[b].alpha_dev = s.W(b, s.L.lz) + HS_EF; }
   }
   DION_TRY(launch_gemm_group(s, group));
   }
@@ -2060,7 +2090,7 @@ int step_batch(dion_ctx* c, const dion_matrix* const* list, int nb, float lr, cu
     if (all_one) {
       for (int b = 0; b < nb; ++b) { srcs[b] = s.W(b, U_off); lds[b] = r; }
       const bool half = x_half(a0);
-      if (hstep && half) u_half = ldexpf(1.f, HS_U_BITS);      // the hi part of U's pair is that rounding
+      if (hstep && half) u_half = ldexpf(1.f, HS_U_BITS);      // (made beside U's pair)
       else DION_TRY(round_chain(s, srcs, lds, prow, r, other_off, s.os + OS_FAIL, half ? half_scale(prow) : 0.f));
       if (cn_kind == 0) {
         for (int b = 0; b < nb; ++b) { srcs[b] = (const float*)list[b]->Q; lds[b] = list[b]->ldq; }
@@ -2084,7 +2114,7 @@ int step_batch(dion_ctx* c, const dion_matrix* const* list, int nb, float lr, cu
       continue;
     }
     // the rounded copies of the single-pass form: in the other panel buffer, and where the normalization put Q's or in R's (free)
-    float* other = s.W(b, U_off == s.L.P0 ? s.L.P1 : s.L.P0);
+    float* other = s.W(b, u_half > 0.f ? u_one : U_off == s.L.P0 ? s.L.P1 : s.L.P0);
     float* rbuf = s.W(b, cn_kind != 0 && x_rounded ? s.L.Psave : s.L.R);
     const float* Uf = s.W(b, U_off);
     const float* Qf = (const float*)a->Q;
@@ -2223,7 +2253,7 @@ int lazy_pairs(StepCtx& s, const dion_matrix* a, float lr, int refresh) {
     return g;
   };
   float* sum = s.ws + s.L.B32;
-  DION_TRY(half_sum_chain(s, &a, n));      // M + G, its pair and Q's
+  DION_TRY(half_sum_chain(s, &a, n, false, false));      // M + G, its pair and Q's
   if (refresh) {
     PhaseScope ps_orth(c, st, DION_PHASE_ORTH);
     // T = (M + G) Q  (m x r), Z = (M + G)^T T (n x r), Q <- Orthonormalize(Z)
@@ -2575,7 +2605,7 @@ GemmArgs dp_b_product(const dion_matrix* a, bool transposed_b, const float* rhs,
 // The pieces of a step on half pairs (step_on_half_pairs) as calls of their own.  P = (M + G) Q:
 int half_project(StepCtx& s, const dion_matrix* a, float* P) {
   const i64 m = a->m, n = a->n, r = a->r;
-  DION_TRY(half_sum_chain(s, &a, n));
+  DION_TRY(half_sum_chain(s, &a, n, false, true));
   const __half* bh = reinterpret_cast<const __half*>(s.ws + s.L.Bp);
   const __half* qh = reinterpret_cast<const __half*>(s.ws + s.L.S16);
   GemmArgs p = gemm_args();
@@ -2585,31 +2615,43 @@ int half_project(StepCtx& s, const dion_matrix* a, float* P) {
   p.B = (const float*)qh; p.B16lo = qh + n * r; p.b_sk = r; p.b_sn = 1;
   p.alpha_dev = s.ws + s.L.lz + HS_P;
   p.C = P; p.ldc = r; p.epi = EPI_STORE;
-  return launch_gemm(s, p, 0);
+  p.skip_flag = s.os + OS_P32;
+  DION_TRY(launch_gemm(s, p, 0));
+  return launch_gemm(s, wide_p(s, 0, a, false, P), 0);
 }
 // W = (M + G)^T U:
 int half_factor(StepCtx& s, const dion_matrix* a, const float* U, float* W, const int* skip) {
   const i64 m = a->m, r = a->r;
-  DION_TRY(half_sum_chain(s, &a, 0));
-  DION_TRY(split_half_chain(s, &U, r, m, r, s.L.P1, HS_U_BITS, skip));
+  DION_TRY(half_sum_chain(s, &a, 0, false, true));
+  DION_TRY(split_half_chain(s, &U, r, m, r, s.L.P1, HS_U_BITS, skip, -1));
   GemmArgs w;
   DION_TRY(r_pairs(s, 0, a, false, U, s.ws + s.L.P1, W, skip, &w, true));
-  w.f16 = 1; w.alpha_dev = s.ws + s.L.lz + HS_R;
+  w.f16 = 1; w.wide_flag = s.os + OS_WIDE; w.alpha_dev = s.ws + s.L.lz + HS_R;
   return launch_gemm(s, w, 0);
 }
-// The error feedback, Q and the weight update (sums: see colnorm_launch; alpha: the update's factor):
+// The error feedback, Q and the weight update (sums: see colnorm_launch; alpha: the update's factor).  M + G is not formed
+// here: whether the error feedback's factors are half or bf16 pairs is decided by their own ranges.
 int half_finish(StepCtx& s, const dion_matrix* a, const float* U, const float* W, const float* sums, float alpha, const int* flag) {
+  dion_ctx* c = s.c;
   const i64 m = a->m, n = a->n, r = a->r;
-  DION_TRY(split_half_chain(s, &U, r, m, r, s.L.P1, HS_U_BITS, flag));
+  ChainPtrs t;
+  t.p[0] = W; t.p[1] = U;
   ColnormPairs x = ColnormPairs();
-  x.kind = CN_HALF; x.qh = s.ws + s.L.P0; x.qscale = half_scale(n); x.hi = s.ws + s.L.S16;
+  const i64 pieces = (((m > n) ? m : n) + RANGE_ROWS - 1) / RANGE_ROWS * ((r + 127) / 128);
+  x.nrange = grid_for(c, 32 * pieces, 2);
+  float* range = s.ws + s.L.part;
+  launch_pdl(k_range_partial, dim3((unsigned)x.nrange, 2), dim3(256), 0, s.st, t, r, n, m, r, range, (i64)2 * x.nrange, (const int*)nullptr, (i64)0);
+  DION_CHECK_LAUNCH(c);
+  const i64 u_one = s.L.P0 + ((m > n) ? m : n) * r / 2;      // (behind Q's half array)
+  x.kind = CN_HALF; x.qh = s.ws + s.L.P0; x.qscale = half_scale(n); x.hi = s.ws + s.L.S16; x.os = s.os; x.range = range;
   DION_TRY(colnorm(s, 0, W, n, r, (float*)a->Q, a->ldq, a->colnorm_out, flag, x, sums));
+  DION_TRY(split_half_chain(s, &U, r, m, r, s.L.P1, HS_U_BITS, flag, u_one));
   GemmArgs e;
   DION_TRY(ef_update(s, 0, a, U, r, W, r, s.ws + s.L.P1, s.ws + s.L.S16, nullptr, flag, true, true, &e));
-  if (e.ab16) { e.f16 = 1; e.alpha_dev = s.ws + s.L.lz + HS_EF; }
+  if (e.ab16) { e.f16 = 1; e.wide_flag = s.os + OS_WIDE; e.alpha_dev = s.ws + s.L.lz + HS_EF; }
   DION_TRY(launch_gemm(s, e, 0));
   const bool rounded = x_single_pass(s, a, U, r, (const float*)a->Q, a->ldq) && x_half(a);
-  return x_update(s, 0, a, U, r, (const float*)a->Q, a->ldq, s.ws + s.L.P1, s.ws + s.L.P0, alpha, flag, nullptr, nullptr, rounded,
+  return x_update(s, 0, a, U, r, (const float*)a->Q, a->ldq, s.ws + (rounded ? u_one : s.L.P1), s.ws + s.L.P0, alpha, flag, nullptr, nullptr, rounded,
                   rounded ? ldexpf(1.f, HS_U_BITS) : 0.f, 0.f);
 }
 

@@ -65,7 +65,8 @@ struct GemmArgs {
   int ab16;                      // tensor engine only: A and B point to bf16 arrays (strides in elements), no addend
   const void* A16lo;             // with ab16: A and B are PAIRS of bf16 arrays, x ~ hi + lo (A, B point to the "hi" arrays, these
   const void* B16lo;             // to the "lo" arrays of the same shape and strides): three bf16 MMAs per K step, ~1e-5 relative
-  int f16;                       // with ab16 (no pairs): the arrays hold IEEE half values instead of bf16 (11 significant bits)
+  int f16;                       // with ab16: the arrays hold IEEE half values instead of bf16 (11 significant bits)
+  const int* wide_flag;          // with f16, optional: the arrays of a matrix whose flag is set hold bf16 after all (OS_WIDE; OS_SLOT_INTS apart)
   int* splits_out;               // HOST, optional: a product that splits K leaves its partial sums unreduced and reports their number here
   int tf32x1;                    // tensor engine, fp32 mode: the operands' values fit TF32 already (k_round_tf32): one MMA
                                  // per K step instead of the three-term split.  Ignored by the FMA engine.
@@ -82,6 +83,9 @@ enum : int {
   OS_MAXDEV = 6,    // float bits: the estimate of |U1^T U1 - I|_F^2 of the CholeskyQR2 check
   OS_BARRIER = 7,   // arrival counter of the fallback kernel's grid-wide barriers (zero at the start of a step)
   OS_NOTNEAR = 8,   // adaptive rounds: the finishing round's factor is not the short series (k_near_identity)
+  OS_WIDE = 9,      // steps on half pairs: the range of M + G is so wide that a bf16 pair holds more (see k_form_sum_amax)
+  OS_P32 = 10,      // ... the range of M + G or of Q is too wide for P on half pairs; it comes from the 3xTF32 product,
+  OS_PHALF = 11,    // ... or is not: the skip flags of the two products that form P
   OS_SLOT_INTS = 16
 };
 

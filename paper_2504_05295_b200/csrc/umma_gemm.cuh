@@ -1400,7 +1400,10 @@ k_gemm_umma(const __grid_constant__ PT p) {
   } else {
     // ------------------------------------------------------------ MMA issuer (CTA pair: the leader only)
     if (lane == 0 && (!CG2 || cta_rank == 0)) {
-      const uint32_t idesc = make_idesc(BF16, A_MN, B_MN, BN, CG2 ? 2 * BM : BM, BF16 && p.g.f16 != 0);
+      auto holds_half = [&](int b) {
+        return BF16 && p.g.f16 != 0 && (!X2 || p.g.wide_flag == nullptr || p.g.wide_flag[(i64)b * OS_SLOT_INTS] == 0);
+      };
+      uint32_t idesc = make_idesc(BF16, A_MN, B_MN, BN, CG2 ? 2 * BM : BM, holds_half(0));
       const uint32_t lbo = BKE * 128;
       constexpr uint32_t A_KSTEP = A_MN ? (BF16 ? 2048u : 1024u) : 32u;   // bytes per UMMA K step
       constexpr uint32_t B_KSTEP = B_MN ? (BF16 ? 2048u : 1024u) : 32u;
@@ -1411,6 +1414,7 @@ k_gemm_umma(const __grid_constant__ PT p) {
       for (int item = worker; item < p.num_items && alive; item += workers) {
         const Item it = decode_item<BN, BKE, CG2>(p, item);
         if (skipped(it)) continue;
+        if (X2 && batched && p.g.wide_flag != nullptr) idesc = make_idesc(BF16, A_MN, B_MN, BN, CG2 ? 2 * BM : BM, holds_half(it.b));
         for (int kbc = it.kb0; kbc < it.kb1 && alive; kbc += p.kc, ++iter) {   // one accumulation chunk
         const int kbc1 = min(it.kb1, kbc + p.kc);
         const int ab = iter % NBUF;
