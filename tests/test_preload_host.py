@@ -10,7 +10,7 @@ ELSEWHERE = {
     "k_set_scalar": "graph replay of dion_step",
     "k_copy_chain": "chains", "k_form_b32_chain": "chains", "k_round_f16_chain": "chains", "k_round_tf32_chain": "chains",
     "k_split_bf16_chain": "chains", "k_colsumsq_finish": "sharded calls",
-    "k_form_sum_amax": "M + G in scratch", "k_split_sum": "M + G in scratch", "k_split_f16_fixed": "M + G in scratch",
+    "k_range_partial": "M + G in scratch", "k_form_sum_amax": "M + G in scratch", "k_split_sum": "M + G in scratch", "k_split_f16_fixed": "M + G in scratch",
     "k_absmax_partial": "panels of 2e9 operations", "k_split_f16_scaled": "panels of 2e9 operations",
     "k_split_f16_tri": "panels of 2e9 operations", "k_near_identity": "panels of 2e9 operations",
     "k_near_end": "panels of 2e9 operations",
