@@ -589,27 +589,41 @@ __global__ void __launch_bounds__(256) k_absmax_partial(const float* __restrict_
 // other_inv / scale (the other operand carries a fixed scale of its own), times *other_dev when that is given (the
 // other operand's own 1 / scale, written by its split; blockIdx.y entries wstride apart like everything else).  own_inv
 // (optional): 1 / scale alone.
+// os (optional; part holds ranges then: k_range_partial): state slots; the flag u = "wide, or os[in]" (in < 0: wide) goes to
+// os[use32] and its opposite to os[usehalf] (both optional, < 0).
 __global__ void __launch_bounds__(256) k_split_f16_scaled(const float* __restrict__ src, i64 ld, i64 rows, i64 cols,
                                                           const float* __restrict__ part, int nparts,
                                                           __half* __restrict__ hi, __half* __restrict__ lo,
                                                           float* __restrict__ inv_scale2, i64 wstride,
                                                           const int* __restrict__ skip_flag, i64 skip_stride,
-                                                          float other_inv, const float* __restrict__ other_dev, float* __restrict__ own_inv) {
+                                                          float other_inv, const float* __restrict__ other_dev, float* __restrict__ own_inv,
+                                                          int* __restrict__ os, int in, int use32, int usehalf) {
   pdl_enter();
   if (skip_flag != nullptr && skip_flag[(i64)blockIdx.y * skip_stride] != 0) return;
   src += (i64)blockIdx.y * wstride; part += (i64)blockIdx.y * wstride; inv_scale2 += (i64)blockIdx.y * wstride;
   if (other_dev != nullptr) other_dev += (i64)blockIdx.y * wstride;
   hi += 2 * (i64)blockIdx.y * wstride; lo += 2 * (i64)blockIdx.y * wstride;
-  __shared__ float red[256];
-  float m = 0.f;
-  for (int e = threadIdx.x; e < nparts; e += 256) m = fmaxf(m, part[e]);
-  red[threadIdx.x] = m;
-  __syncthreads();
-  for (int w = 128; w > 0; w >>= 1) {
-    if ((int)threadIdx.x < w) red[threadIdx.x] = fmaxf(red[threadIdx.x], red[threadIdx.x + w]);
+  float amax, mn = 0.f;
+  if (os != nullptr) {
+    range_of_blocks(part, nparts, amax, mn);
+  } else {
+    __shared__ float red[256];
+    float m = 0.f;
+    for (int e = threadIdx.x; e < nparts; e += 256) m = fmaxf(m, part[e]);
+    red[threadIdx.x] = m;
     __syncthreads();
+    for (int w = 128; w > 0; w >>= 1) {
+      if ((int)threadIdx.x < w) red[threadIdx.x] = fmaxf(red[threadIdx.x], red[threadIdx.x + w]);
+      __syncthreads();
+    }
+    amax = red[0];
   }
-  const float amax = red[0];
+  if (os != nullptr && blockIdx.x == 0 && threadIdx.x == 0) {
+    os += (i64)blockIdx.y * OS_SLOT_INTS;
+    const bool u = range_is_wide(amax, mn, RANGE_P) || (in >= 0 && os[in] != 0);
+    if (use32 >= 0) os[use32] = u ? 1 : 0;
+    if (usehalf >= 0) os[usehalf] = u ? 0 : 1;
+  }
   int ex = 14;                                   // amax = f 2^ex with f in [0.5, 1): scale 2^(14 - ex)
   if (amax > 0.f && amax < 3.0e38f) frexpf(amax, &ex);
   if (ex < -100) ex = -100;

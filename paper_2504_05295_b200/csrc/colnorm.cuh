@@ -142,7 +142,8 @@ struct ColnormPairs {
   const float* other;      // or with another pair (optional: its 1 / scale)
   int* os;                 // CN_HALF, optional: state slots; the pair of a matrix whose OS_WIDE is set is a bf16 pair.  With
   const float* range;      // `range` the flag is set here: ranges (k_range_partial) of R and, behind them, of U, of
-  int nrange;              // this many blocks
+  int nrange;              // this many blocks.  With qpair (Lazy-Dion) the flag is OS_P32 instead: U goes to qh as it is, in fp32,
+                           // and OS_USE32 and OS_USEHALF are set for the updates (both when the step is cancelled)
 };
 enum : int { CN_HALF = 1, CN_BF16 = 2, CN_ONE = 3 };
 
@@ -159,7 +160,10 @@ __global__ void __launch_bounds__(CN_THREADS, 3) k_colnorm_apply(const float* __
   pdl_enter();
   const i64 b = blockIdx.z;
   if (skip_flag != nullptr && skip_flag[b * OS_SLOT_INTS] != 0) {
-    if (threadIdx.x == 0 && blockIdx.x == 0 && blockIdx.y == 0) atomicAdd(skipped, 1);      // (once per step: the count of cancelled steps)
+    if (threadIdx.x == 0 && blockIdx.x == 0 && blockIdx.y == 0) {
+      atomicAdd(skipped, 1);      // (once per step: the count of cancelled steps)
+      if (QP && x.os != nullptr) x.os[b * OS_SLOT_INTS + OS_USE32] = x.os[b * OS_SLOT_INTS + OS_USEHALF] = 1;
+    }
     return;
   }
   __shared__ float red[CN_WARPS][128];
@@ -192,13 +196,19 @@ __global__ void __launch_bounds__(CN_THREADS, 3) k_colnorm_apply(const float* __
       m = mw;
       bf16 = range_is_wide(mw, nw, RANGE_UPDATE) || nu < RANGE_UPDATE;
       if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) x.os[OS_WIDE] = bf16 ? 1 : 0;
-    } else if (x.os != nullptr) {
+    } else if (!QP && x.os != nullptr) {
       bf16 = x.os[b * OS_SLOT_INTS + OS_WIDE] != 0;
     }
     const int e = f16_scale_exponent(m);
     rscale = ldexpf(1.f, e);
     if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0)
       x.scal[b * wstride] = bf16 ? 1.f : x.other != nullptr ? ldexpf(1.f, -e) * x.other[b * wstride] : ldexpf(1.f, -e - HS_U_BITS);
+  }
+  bool use32 = false;
+  if (QP && x.os != nullptr) {
+    int* os = x.os + b * OS_SLOT_INTS;
+    use32 = os[OS_P32] != 0;
+    if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) { os[OS_USE32] = use32 ? 1 : 0; os[OS_USEHALF] = use32 ? 0 : 1; }
   }
   float inv[4];
 #pragma unroll
@@ -234,7 +244,9 @@ __global__ void __launch_bounds__(CN_THREADS, 3) k_colnorm_apply(const float* __
 #pragma unroll
         for (int k = 0; k < 4; ++k) Q[i * ldq + j + k] = q[k];
       }
-      if (x.kind != 0) {
+      if (QP && use32) {
+        *reinterpret_cast<float4*>(reinterpret_cast<float*>(x.qh) + b * wstride + i * r + j) = make_float4(q[0], q[1], q[2], q[3]);
+      } else if (x.kind != 0) {
         const i64 at = 2 * b * wstride + i * r + j;
         __half h[4];
 #pragma unroll

@@ -863,7 +863,7 @@ int cholqr_round(StepCtx& s, i64 pin_off, i64 pout_off, i64 rows, i64 r, int mod
     DION_CHECK_LAUNCH(c);
     launch_pdl(k_split_f16_scaled, dim3((unsigned)grid_for(c, rows * r / 8, s.nb), (unsigned)s.nb), dim3(256), 0, s.st,
                (const float*)(s.ws + pin_off), r, rows, r, (const float*)(s.ws + s.L.gmax), (int)parts, hi, lo, s.ws + s.L.gmax + AMAX_PARTS,
-               s.wstride, sk, (i64)OS_SLOT_INTS, -1.f, (const float*)nullptr, (float*)nullptr);
+               s.wstride, sk, (i64)OS_SLOT_INTS, -1.f, (const float*)nullptr, (float*)nullptr, (int*)nullptr, 0, 0, 0);
     DION_CHECK_LAUNCH(c);
     g.ab16 = 1; g.f16 = 1;
     g.A = reinterpret_cast<const float*>(hi); g.A16lo = lo;
@@ -965,7 +965,7 @@ int cholqr_round(StepCtx& s, i64 pin_off, i64 pout_off, i64 rows, i64 r, int mod
       DION_CHECK_LAUNCH(c);
       __half* hi = reinterpret_cast<__half*>(s.ws + out_off);
       launch_pdl(k_split_f16_scaled, dim3((unsigned)grid_for(c, nrows * ncols / 8, s.nb), (unsigned)s.nb), dim3(256), 0, s.st, src, ld, nrows, ncols,
-                 (const float*)pm, (int)parts, hi, hi + nrows * ncols, pm + AMAX_PARTS, s.wstride, skip, (i64)OS_SLOT_INTS, other_inv, other_dev, (float*)nullptr);
+                 (const float*)pm, (int)parts, hi, hi + nrows * ncols, pm + AMAX_PARTS, s.wstride, skip, (i64)OS_SLOT_INTS, other_inv, other_dev, (float*)nullptr, (int*)nullptr, 0, 0, 0);
       DION_CHECK_LAUNCH(c);
       return DION_OK;
     };
@@ -1825,7 +1825,7 @@ int step_batch(dion_ctx* c, const dion_matrix* const* list, int nb, float lr, cu
       DION_CHECK_LAUNCH(c);
       launch_pdl(k_split_f16_scaled, dim3((unsigned)grid_for(c, m * n / 8, nb), (unsigned)nb), dim3(256), 0, st,
                  (const float*)(s.ws + s.L.B32), n, m, n, (const float*)(s.ws + s.L.pmax), (int)parts, bh, bh + m * n,
-                 s.ws + s.L.pmax + AMAX_PARTS, s.wstride, (const int*)nullptr, (i64)0, ldexpf(1.f, -13), (const float*)nullptr, (float*)nullptr);
+                 s.ws + s.L.pmax + AMAX_PARTS, s.wstride, (const int*)nullptr, (i64)0, ldexpf(1.f, -13), (const float*)nullptr, (float*)nullptr, (int*)nullptr, 0, 0, 0);
       DION_CHECK_LAUNCH(c);
       ChainPtrs t;
       for (int b = 0; b < nb; ++b) t.p[b] = srcs[b];
@@ -2223,49 +2223,69 @@ bool lazy_on_pairs(const StepCtx& s, const dion_matrix* a) {
          !((uintptr_t)a->X & 15) && a->ldx % 4 == 0 && !((uintptr_t)a->M & 15) && a->ldm % 4 == 0 && !((uintptr_t)a->Q & 15) && a->ldq % 4 == 0;
 }
 
+//
+// Where the ranges of M + G, Q or T are too wide for that (k_form_sum_amax), the 3xTF32 product of the fp32 operands takes its
+// place: every product is two launches, of which the state slot skips one.
 int lazy_pairs(StepCtx& s, const dion_matrix* a, float lr, int refresh) {
   dion_ctx* c = s.c;
   cudaStream_t st = s.st;
   const i64 m = a->m, n = a->n, r = a->r;
   float* sc = s.ws + s.L.lz;      // HS_*
   float* R = s.ws + s.L.R;
+  float* sum = s.ws + s.L.B32;
+  const float* Q = (const float*)a->Q;
   auto halves = [&](i64 off) { return reinterpret_cast<__half*>(s.ws + off); };
-  // the pair of a rows x cols array into scratch at `off`; slot: the scale factor of its product with M + G, own: of itself alone
-  auto pair_of = [&](const float* src, i64 ld, i64 rows, i64 cols, i64 off, int slot, int own) -> int {
+  // the pair of a rows x cols array into scratch at `off`; slot: the scale factor of its product with M + G, own: of itself
+  // alone; the flags of the products that read it
+  auto pair_of = [&](const float* src, i64 ld, i64 rows, i64 cols, i64 off, int slot, int own, int use32, int usehalf) -> int {
     i64 nparts = (rows * cols / 4 + 2047) / 2048;
     if (nparts > AMAX_PARTS) nparts = AMAX_PARTS;
     float* pm = s.ws + s.L.part;      // (read before the next product writes its partial sums there)
-    launch_pdl(k_absmax_partial, dim3((unsigned)nparts), dim3(256), 0, st, src, ld, rows, cols, pm, (i64)0, (const int*)nullptr, (i64)0);
+    ChainPtrs t;
+    t.p[0] = src;
+    launch_pdl(k_range_partial, dim3((unsigned)nparts), dim3(256), 0, st, t, ld, rows, rows, cols, pm, (i64)0, (const int*)nullptr, (i64)0);
     DION_CHECK_LAUNCH(c);
     launch_pdl(k_split_f16_scaled, dim3((unsigned)grid_for(c, rows * cols / 8)), dim3(256), 0, st, src, ld, rows, cols, (const float*)pm, (int)nparts,
                halves(off), halves(off) + rows * cols, sc + slot, (i64)0, (const int*)nullptr, (i64)0, ldexpf(1.f, HS_U_BITS),
-               (const float*)(sc + HS_R), own >= 0 ? sc + own : (float*)nullptr);
+               (const float*)(sc + HS_R), own >= 0 ? sc + own : (float*)nullptr, s.os, (int)OS_P32, use32, usehalf);
     DION_CHECK_LAUNCH(c);
     return DION_OK;
   };
-  auto product = [&](i64 M_, i64 N_, i64 K_, i64 a_off, i64 a_n, i64 a_si, i64 a_sk, i64 b_off, i64 b_n, i64 b_sk, i64 b_sn, int slot) {
+  // a product: on the pairs at a_off and b_off, or of A and B (the same shapes, leading dimensions lda and ldb; ta, tb: transposed)
+  auto product = [&](GemmArgs g, i64 a_off, const float* A, i64 lda, bool ta, i64 b_off, const float* B, i64 ldb, bool tb, int slot, float half_alpha,
+                     int use32, int usehalf) -> int {
+    const i64 ac = ta ? g.M : g.K, bc = tb ? g.K : g.N;      // columns of the arrays
+    GemmArgs h = g;
+    h.ab16 = 1; h.f16 = 1;
+    h.A = (const float*)halves(a_off); h.A16lo = halves(a_off) + g.M * g.K; h.a_si = ta ? 1 : ac; h.a_sk = ta ? ac : 1;
+    h.B = (const float*)halves(b_off); h.B16lo = halves(b_off) + g.K * g.N; h.b_sk = tb ? 1 : bc; h.b_sn = tb ? bc : 1;
+    h.alpha = g.alpha * half_alpha; h.alpha_dev = sc + slot;
+    h.skip_flag = s.os + use32;
+    DION_TRY(launch_gemm(s, h));
+    g.A = A; g.a_si = ta ? 1 : lda; g.a_sk = ta ? lda : 1;
+    g.B = B; g.b_sk = tb ? 1 : ldb; g.b_sn = tb ? ldb : 1;
+    g.skip_flag = s.os + usehalf;
+    if (g.epi == EPI_STORE) g.precise = 1;
+    return launch_gemm(s, g);
+  };
+  auto shape = [&](i64 M_, i64 N_, i64 K_, float* C, i64 ldc, int epi) {
     GemmArgs g = gemm_args();
-    g.M = M_; g.N = N_; g.K = K_;
-    g.ab16 = 1; g.f16 = 1;
-    g.A = (const float*)halves(a_off); g.A16lo = halves(a_off) + a_n; g.a_si = a_si; g.a_sk = a_sk;
-    g.B = (const float*)halves(b_off); g.B16lo = halves(b_off) + b_n; g.b_sk = b_sk; g.b_sn = b_sn;
-    g.alpha_dev = sc + slot;
+    g.M = M_; g.N = N_; g.K = K_; g.C = C; g.ldc = ldc; g.epi = epi;
     return g;
   };
-  float* sum = s.ws + s.L.B32;
-  DION_TRY(half_sum_chain(s, &a, n, false, false));      // M + G, its pair and Q's
+  DION_TRY(half_sum_chain(s, &a, n, false, true));      // M + G, its pair and Q's
   if (refresh) {
     PhaseScope ps_orth(c, st, DION_PHASE_ORTH);
     // T = (M + G) Q  (m x r), Z = (M + G)^T T (n x r), Q <- Orthonormalize(Z)
     const int precise = (resolve_orth(c, r, (m < n) ? m : n) == DION_ORTH_SHIFTED3) ? 1 : 0;
-    GemmArgs t = product(m, r, n, s.L.Bp, m * n, n, 1, s.L.S16, n * r, r, 1, HS_P);
-    t.C = R; t.ldc = r; t.epi = EPI_STORE; t.precise = precise;
-    DION_TRY(launch_gemm(s, t));
-    DION_TRY(pair_of(R, r, m, r, s.L.P1, HS_T, -1));
+    GemmArgs t = shape(m, r, n, R, r, EPI_STORE);
+    t.precise = precise;
+    DION_TRY(product(t, s.L.Bp, sum, n, false, s.L.S16, Q, a->ldq, false, HS_P, 1.f, OS_P32, OS_PHALF));
+    DION_TRY(pair_of(R, r, m, r, s.L.P1, HS_T, -1, OS_USE32, OS_USEHALF));
     const i64 pin_off = panel_offset(s, r, (m < n) ? m : n);
-    GemmArgs z = product(n, r, m, s.L.Bp, m * n, 1, n, s.L.P1, m * r, r, 1, HS_T);
-    z.C = s.ws + pin_off; z.ldc = r; z.epi = EPI_STORE; z.precise = precise;
-    DION_TRY(launch_gemm(s, z));
+    GemmArgs z = shape(n, r, m, s.ws + pin_off, r, EPI_STORE);
+    z.precise = precise;
+    DION_TRY(product(z, s.L.Bp, sum, n, true, s.L.P1, R, r, false, HS_T, 1.f, OS_USE32, OS_USEHALF));
     i64 V_off = 0;
     s.in_orth = true;
     const int rc_orth = orthonormalize(s, n, r, (m < n) ? m : n, pin_off, &V_off);
@@ -2277,33 +2297,27 @@ int lazy_pairs(StepCtx& s, const dion_matrix* a, float lr, int refresh) {
   }
   {   // W = (M + G) Q
   PhaseScope ps(c, st, DION_PHASE_P);
-  if (refresh) DION_TRY(pair_of((const float*)a->Q, a->ldq, n, r, s.L.S16, HS_P, HS_Q));
-  GemmArgs w = product(m, r, n, s.L.Bp, m * n, n, 1, s.L.S16, n * r, r, 1, HS_P);
-  w.C = R; w.ldc = r; w.epi = EPI_STORE;
-  DION_TRY(launch_gemm(s, w));
+  if (refresh) DION_TRY(pair_of(Q, a->ldq, n, r, s.L.S16, HS_P, HS_Q, OS_P32, OS_PHALF));
+  DION_TRY(product(shape(m, r, n, R, r, EPI_STORE), s.L.Bp, sum, n, false, s.L.S16, Q, a->ldq, false, HS_P, 1.f, OS_P32, OS_PHALF));
   }
-  {   // U = ColNorm(W), as a pair of fixed scale (unit-norm columns) in P0; W's pair in P1
+  {   // U = ColNorm(W), as a pair of fixed scale (unit-norm columns) or in fp32, in P0; W's pair in P1
   PhaseScope ps(c, st, DION_PHASE_COLNORM);
   ColnormPairs x = ColnormPairs();
-  x.kind = CN_HALF; x.qh = s.ws + s.L.P0; x.qscale = ldexpf(1.f, HS_U_BITS); x.qpair = 1; x.hi = s.ws + s.L.P1; x.other = sc + HS_Q;
+  x.kind = CN_HALF; x.qh = s.ws + s.L.P0; x.qscale = ldexpf(1.f, HS_U_BITS); x.qpair = 1; x.hi = s.ws + s.L.P1; x.other = sc + HS_Q; x.os = s.os;
   DION_TRY(colnorm(s, 0, R, m, r, nullptr, r, a->colnorm_out, nullptr, x));
   }
   {   // M <- (M + G) - (1 - mu) W Q^T
   PhaseScope ps(c, st, DION_PHASE_EF);
-  GemmArgs e = product(m, n, r, s.L.P1, m * r, r, 1, s.L.S16, n * r, 1, r, HS_EF);
-  e.C = (float*)a->M; e.ldc = a->ldm; e.epi = EPI_C2_SUB; e.C2 = sum; e.ldc2 = n; e.c2_mode = ADD_F32;
+  GemmArgs e = shape(m, n, r, (float*)a->M, a->ldm, EPI_C2_SUB);
+  e.C2 = sum; e.ldc2 = n; e.c2_mode = ADD_F32;
   e.alpha = 1.f - c->cfg.mu;
-  e.skip_flag = s.flag;
-  DION_TRY(launch_gemm(s, e));
+  DION_TRY(product(e, s.L.P1, R, r, false, s.L.S16, Q, a->ldq, true, HS_EF, 1.f, OS_USE32, OS_USEHALF));
   }
   // X <- X - lr sqrt(m/n) U Q^T
   PhaseScope ps_x(c, st, DION_PHASE_X);
-  GemmArgs x = product(m, n, r, s.L.P0, m * r, r, 1, s.L.S16, n * r, 1, r, HS_Q);
-  x.C = (float*)a->X; x.ldc = a->ldx; x.epi = EPI_SUB;
-  x.alpha = ldexpf(lr * sqrtf((float)((double)m / (double)n)), -13);
-  x.skip_flag = s.flag;
-  DION_TRY(launch_gemm(s, x));
-  return DION_OK;
+  GemmArgs x = shape(m, n, r, (float*)a->X, a->ldx, EPI_SUB);
+  x.alpha = lr * sqrtf((float)((double)m / (double)n));
+  return product(x, s.L.P0, s.ws + s.L.P0, r, false, s.L.S16, Q, a->ldq, true, HS_Q, ldexpf(1.f, -HS_U_BITS), OS_USE32, OS_USEHALF);
 }
 
 // One Lazy-Dion step (Algorithm 6).

@@ -130,3 +130,50 @@ def test_zero_rows_and_columns_are_no_wide_range():
         assert opt.get_status() == (0, 0)
     assert off(Q, Qr) <= 2e-6
     assert torch.equal(M[100:300], torch.zeros_like(M[100:300])) and torch.equal(Q[7:40], torch.zeros_like(Q[7:40]))
+
+
+@pytest.mark.parametrize("refresh", [True, False])
+@pytest.mark.parametrize("m,n,r", [(640, 768, 128), (1288, 648, 136)])
+@pytest.mark.parametrize("axis,exponent", CASES)
+def test_lazy_step(m, n, r, refresh, axis, exponent):
+    X, M, G, Q = problem(m, n, r, axis, exponent)
+    at = block(axis, m, n)
+    if not refresh:      # the factor of an earlier refresh
+        Q = torch.linalg.qr(Q)[0].contiguous()
+    B, X0, Qr = M.double() + G.double(), X.double(), Q.double()
+    if refresh:
+        Qr, T = torch.linalg.qr(B.t() @ (B @ Qr))
+        Qr = Qr * torch.sign(torch.diagonal(T))
+    W = B @ Qr
+    low, dX = W @ Qr.t(), LR * math.sqrt(m / n) * (W / W.norm(dim=0)) @ Qr.t()
+    with binding.Dion(mu=MU) as opt:
+        opt.lazy_step(X, M, G, Q, LR, refresh=refresh)
+        assert opt.get_status() == (0, 0)
+    # products of 22 significant bits and chains of at most 1024 terms (8e-6), three in a row on a well-conditioned panel
+    assert off(((B - M.double()) / (1 - MU))[at], low[at]) <= 4e-5 + 1e-6 / (1 - MU)
+    assert off(M[at], (B - (1 - MU) * low)[at]) <= 2e-6
+    assert ((X.double() - X0 + dX)[at]).norm() <= 4e-5 * dX[at].norm() + 2.0 ** -24 * X0[at].norm()
+    rows = slice(n // 2, None) if axis == "cols" else slice(None)
+    assert off(Q[rows], Qr[rows]) <= 4e-5
+
+
+def test_lazy_step_of_graded_columns_and_of_a_breakdown():
+    m, n, r = 512, 768, 128
+    # T = (M + G) Q with columns 2^-24 of others: only Z has to see them
+    X, M, G, Q = problem(m, n, r, "none", 0)
+    Q[:, r // 2:] *= 2.0 ** -24
+    B = M.double() + G.double()
+    want, T = torch.linalg.qr(B.t() @ (B @ Q.double()))
+    with binding.Dion(mu=MU) as opt:
+        opt.lazy_step(X, M, G, Q, LR, refresh=True)
+        assert opt.get_status() == (0, 0)
+        assert off(Q, want * torch.sign(torch.diagonal(T))) <= 4e-5
+        # a panel of rank one less than its width cancels the step, on either kind of product
+        for exponent in (0, -30):
+            X, M, G, Q = problem(m, n, r, "rows", exponent)
+            Q[:, 5] = Q[:, 3]
+            before = [t.clone() for t in (X, M, Q)]
+            opt.lazy_step(X, M, G, Q, LR, refresh=True)
+            assert opt.get_status() == (binding.STATUS_BREAKDOWN, 1)
+            for a, b in zip(before, (X, M, Q)):
+                assert torch.equal(a, b)
