@@ -204,7 +204,9 @@ __device__ __forceinline__ void potrf64_setup(Potrf64Set& st, float g0, float g1
   for (int h = 0; h < 2; ++h) {
     const float g = (h ? g1 : g0) * s2;
     const float fl = floor_rel * g;
-    const float alt = (fl > 0.f && fl < inf) ? fl : 1.f;      // zero or non-finite column: unit pivot
+    // Zero or non-finite column: unit pivot, of the block as it was before the scale.  (A column whose entries are beyond the
+    // panel's pair has a zero here; it comes back in a later round only if nothing divides it by the others' norm.)
+    const float alt = (fl > 0.f && fl < inf) ? fl : s2;
     st.gd[lane + 32 * h] = g;
     st.floor[lane + 32 * h] = fl;
     st.alt_inv[lane + 32 * h] = rsqrtf(alt);

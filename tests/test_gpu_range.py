@@ -177,3 +177,19 @@ def test_lazy_step_of_graded_columns_and_of_a_breakdown():
             assert opt.get_status() == (binding.STATUS_BREAKDOWN, 1)
             for a, b in zip(before, (X, M, Q)):
                 assert torch.equal(a, b)
+
+
+@pytest.mark.parametrize("exponent", [-37, -38, -40, -42])
+def test_adaptive_rounds_of_columns_beyond_the_pair(exponent):
+    # At 2^-38 of the others a column's half pair is a few odd bits or zero, and so is its entry of the Gram matrix: the first round
+    # leaves it as it is, the next one sees it beside columns of norm 1.  The split lies inside a block of 64 columns.
+    rows, r = 4096, 1032
+    g = torch.Generator(device="cuda"); g.manual_seed(r)
+    P = torch.randn(rows, r, generator=g, device="cuda")
+    P[:, r // 2:] *= 2.0 ** exponent
+    want, T = torch.linalg.qr(P.double())
+    flag = torch.zeros(1, dtype=torch.int32, device="cuda")
+    with binding.Dion() as opt:
+        opt.orthonormalize(rows, r, rows, P, flag)
+        assert opt.get_status() == (0, 0) and int(flag.item()) == 0
+    assert off(P, want * torch.sign(torch.diagonal(T))) <= 4e-5      # 22 bits, chains of at most 1024 terms, twice
