@@ -858,12 +858,14 @@ int cholqr_round(StepCtx& s, i64 pin_off, i64 pout_off, i64 rows, i64 r, int mod
     __half* lo = hi + rows * r;
     i64 parts = (rows * r / 4 + 2047) / 2048;
     if (parts > AMAX_PARTS) parts = AMAX_PARTS;
-    launch_pdl(k_absmax_partial, dim3((unsigned)parts, (unsigned)s.nb), dim3(256), 0, s.st, (const float*)(s.ws + pin_off), r, rows, r,
-               s.ws + s.L.gmax, s.wstride, sk, (i64)OS_SLOT_INTS);
+    float* range = s.ws + s.L.part;      // (read before the product writes its partial sums there)
+    ChainPtrs t;
+    for (int b = 0; b < s.nb; ++b) t.p[b] = s.W(b, pin_off);
+    launch_pdl(k_range_partial, dim3((unsigned)parts, (unsigned)s.nb), dim3(256), 0, s.st, t, r, rows, rows, r, range, s.wstride, sk, (i64)OS_SLOT_INTS);
     DION_CHECK_LAUNCH(c);
     launch_pdl(k_split_f16_scaled, dim3((unsigned)grid_for(c, rows * r / 8, s.nb), (unsigned)s.nb), dim3(256), 0, s.st,
-               (const float*)(s.ws + pin_off), r, rows, r, (const float*)(s.ws + s.L.gmax), (int)parts, hi, lo, s.ws + s.L.gmax + AMAX_PARTS,
-               s.wstride, sk, (i64)OS_SLOT_INTS, -1.f, (const float*)nullptr, (float*)nullptr, (int*)nullptr, 0, 0, 0);
+               (const float*)(s.ws + pin_off), r, rows, r, (const float*)range, (int)parts, hi, lo, s.ws + s.L.gmax + AMAX_PARTS,
+               s.wstride, sk, (i64)OS_SLOT_INTS, -1.f, (const float*)nullptr, (float*)nullptr, s.os, -1, (int)OS_PANEL_WIDE, -1);
     DION_CHECK_LAUNCH(c);
     g.ab16 = 1; g.f16 = 1;
     g.A = reinterpret_cast<const float*>(hi); g.A16lo = lo;
@@ -912,24 +914,28 @@ int cholqr_round(StepCtx& s, i64 pin_off, i64 pout_off, i64 rows, i64 r, int mod
     const int* uskip = in_flow ? (const int*)(s.os + OS_NOTNEAR) : skip;
     GemmArgs u = gemm_args();
     u.M = rows; u.N = r; u.K = r;
+    u.a_si = r; u.a_sk = 1; u.b_sk = r; u.b_sn = 1; u.klimit = 1;
+    u.C = s.ws + pout_off; u.ldc = r; u.epi = EPI_STORE; u.skip_flag = uskip;
+    u.A = s.ws + pin_off;
+    u.B = s.ws + s.L.Linv;
     if (gpairs) {
       __half* ph = reinterpret_cast<__half*>(s.ws + s.L.S16);
       __half* xh = reinterpret_cast<__half*>(s.ws + s.L.XP);
       launch_pdl(k_split_f16_tri, dim3((unsigned)tiles, (unsigned)s.nb), dim3(256), 0, s.st, (const float*)(s.ws + s.L.Linv), r,
                  (const float*)(s.ws + s.L.xmax), (const float*)(s.ws + s.L.gmax + AMAX_PARTS), xh, xh + r * r, s.ws + s.L.xmax + 1, s.wstride,
-                 uskip, raw, series ? (const float*)(s.ws + s.L.Tbuf) : (const float*)nullptr);
+                 uskip, raw, series ? (const float*)(s.ws + s.L.Tbuf) : (const float*)nullptr, series ? (int*)nullptr : s.os);
       DION_CHECK_LAUNCH(c);
-      u.ab16 = 1; u.f16 = 1;
-      u.A = (const float*)ph; u.A16lo = ph + rows * r;
-      u.B = (const float*)xh; u.B16lo = xh + r * r;
-      u.alpha_dev = s.ws + s.L.xmax + 1; u.alpha_dev_stride = s.wstride;
-    } else {
-      u.A = s.ws + pin_off;
-      u.B = s.ws + s.L.Linv;
+      GemmArgs h = u;
+      h.ab16 = 1; h.f16 = 1;
+      h.A = (const float*)ph; h.A16lo = ph + rows * r;
+      h.B = (const float*)xh; h.B16lo = xh + r * r;
+      h.alpha_dev = s.ws + s.L.xmax + 1; h.alpha_dev_stride = s.wstride;
+      if (!series) h.skip_flag = s.os + OS_USE32;
+      DION_TRY(launch_gemm_chain(s, h));
+      u.precise = 1;      // (as accurate as the pairs are on a narrow range)
+      u.skip_flag = s.os + OS_USEHALF;
     }
-    u.a_si = r; u.a_sk = 1; u.b_sk = r; u.b_sn = 1; u.klimit = 1;
-    u.C = s.ws + pout_off; u.ldc = r; u.epi = EPI_STORE; u.skip_flag = uskip;
-    DION_TRY(launch_gemm_chain(s, u));
+    if (!series) DION_TRY(launch_gemm_chain(s, u));
     if (series) {
       launch_pdl(k_near_end, dim3((unsigned)s.nb), dim3(1), 0, s.st, s.os, c->dev_ints + 2);
       DION_CHECK_LAUNCH(c);

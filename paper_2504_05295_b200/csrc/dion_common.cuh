@@ -86,8 +86,9 @@ enum : int {
   OS_WIDE = 9,      // steps on half pairs: the range of M + G is so wide that a bf16 pair holds more (see k_form_sum_amax)
   OS_P32 = 10,      // ... the range of M + G or of Q is too wide for P on half pairs; it comes from the 3xTF32 product,
   OS_PHALF = 11,    // ... or is not: the skip flags of the two products that form P
-  OS_USE32 = 12,    // the same pair of skip flags for a product further on (Lazy-Dion: Z, then the two updates)
-  OS_USEHALF = 13,
+  OS_USE32 = 12,    // the same pair of skip flags for a product further on (the panel times the inverse of its factor;
+  OS_USEHALF = 13,  // Lazy-Dion: Z, the two updates)
+  OS_PANEL_WIDE = 14,   // the range of the panel of a round is too wide for a product on its pair
   OS_SLOT_INTS = 16
 };
 

@@ -3,6 +3,7 @@
 
 #include <cuda_fp16.h>
 
+#include "bf16_kernels.cuh"
 #include "chol_flow.cuh"
 #include "dion_common.cuh"
 
@@ -284,6 +285,7 @@ __global__ void __launch_bounds__(TINY_THREADS) k_tiny_cholqr2(const float* __re
 // leaves scale x E and scale x Phi as IEEE half arrays for the product S (the second-order term needs few bits) and
 // sets OS_GOOD to 2: the factorization's launch then leaves the matrix alone and k_split_f16_tri puts X together.
 // (At r = 2048 that launch takes 390 us, this and the product 35.)  Else OS_NOTNEAR is set: the product is skipped.
+// A panel whose range is too wide for its pair (OS_PANEL_WIDE) is solved by substitution instead.
 // Gram matrix: `part` (nsplit partial sums, times *alpha_dev) or G, lower triangle, r a multiple of 8.
 // grid = (blocks, matrices), 256 threads, a 32 x 32 tile at a time; sums: one float per block; OS_BARRIER as in k_probe_decide.
 struct NearSrc {
@@ -306,7 +308,7 @@ __global__ void __launch_bounds__(256) k_near_identity(const NearSrc g, i64 r, _
                                                        i64 wstride) {
   pdl_enter();
   os += (i64)blockIdx.y * OS_SLOT_INTS;
-  if (os[OS_DONE] != 0 || os[OS_GOOD] != 1) {
+  if (os[OS_DONE] != 0 || os[OS_GOOD] != 1 || os[OS_PANEL_WIDE] != 0) {
     if (blockIdx.x == 0 && threadIdx.x == 0) os[OS_NOTNEAR] = 1;
     return;
   }
@@ -399,17 +401,30 @@ __global__ void __launch_bounds__(256) k_near_identity(const NearSrc g, i64 r, _
 // 256-column tiles reads: from src, or, with S given, put together from the Gram matrix and S (k_near_identity).
 // Scale as in k_split_f16_scaled from *amax, the largest magnitude.  *inv_out = 1 / scale, times the root of *other_sq (a power
 // of four: the square of the other operand's 1 / scale).  grid = (blocks, matrices), 256 threads, 32 x 32 tiles.
+// os (optional): state slots; OS_USE32 and OS_USEHALF say which product takes the panel to U: the one on the pairs, or the
+// 3xTF32 one where the panel or the columns of X (its diagonal: no column's largest entry is smaller) spread over more than the
+// pairs hold (see k_form_sum_amax); neither when the round is skipped.
 __global__ void __launch_bounds__(256) k_split_f16_tri(const float* __restrict__ src, i64 n, const float* __restrict__ amax,
                                                        const float* __restrict__ other_sq, __half* __restrict__ hi, __half* __restrict__ lo,
                                                        float* __restrict__ inv_out, i64 wstride, const int* __restrict__ skip_flag,
-                                                       const NearSrc g, const float* __restrict__ S) {
+                                                       const NearSrc g, const float* __restrict__ S, int* __restrict__ os) {
   pdl_enter();
-  if (skip_flag != nullptr && skip_flag[(i64)blockIdx.y * OS_SLOT_INTS] != 0) return;
+  if (os != nullptr) os += (i64)blockIdx.y * OS_SLOT_INTS;
+  if (skip_flag != nullptr && skip_flag[(i64)blockIdx.y * OS_SLOT_INTS] != 0) {
+    if (os != nullptr && blockIdx.x == 0 && threadIdx.x == 0) os[OS_USE32] = os[OS_USEHALF] = 1;
+    return;
+  }
   const bool near = S != nullptr;
   const i64 wo = (i64)blockIdx.y * wstride;
   src += wo; hi += 2 * wo; lo += 2 * wo;
   if (S != nullptr) S += wo;
   const float m = amax[wo];
+  if (os != nullptr && blockIdx.x == 0) {
+    bool u = os[OS_PANEL_WIDE] != 0;
+    for (i64 i = threadIdx.x; i < n; i += 256) u = u || fabsf(src[i * n + i]) < m * RANGE_P;
+    u = __syncthreads_or(u) != 0;
+    if (threadIdx.x == 0) { os[OS_USE32] = u ? 1 : 0; os[OS_USEHALF] = u ? 0 : 1; }
+  }
   int ex = 14;                                   // amax = f 2^ex with f in [0.5, 1): scale 2^(14 - ex)
   if (m > 0.f && m < 3.0e38f) frexpf(m, &ex);
   if (ex < -100) ex = -100;

@@ -193,3 +193,21 @@ def test_adaptive_rounds_of_columns_beyond_the_pair(exponent):
         opt.orthonormalize(rows, r, rows, P, flag)
         assert opt.get_status() == (0, 0) and int(flag.item()) == 0
     assert off(P, want * torch.sign(torch.diagonal(T))) <= 4e-5      # 22 bits, chains of at most 1024 terms, twice
+
+
+@pytest.mark.parametrize("axis,exponent", CASES)
+@pytest.mark.parametrize("rows,r,short", [(4096, 768, 4096), (4104, 1024, 4104), (4096, 1032, 4096), (8192, 512, 2048)])
+def test_panel(rows, r, short, axis, exponent):
+    # panels whose Gram matrix, and the product that takes them to U, run on half pairs (the third: adaptive rounds)
+    g = torch.Generator(device="cuda"); g.manual_seed(r)
+    P = torch.randn(rows, r, generator=g, device="cuda")
+    at = block(axis, rows, r)
+    P[at] *= 2.0 ** exponent
+    want, T = torch.linalg.qr(P.double())
+    want *= torch.sign(torch.diagonal(T))
+    flag = torch.zeros(1, dtype=torch.int32, device="cuda")
+    with binding.Dion() as opt:
+        opt.orthonormalize(rows, r, short, P, flag)
+        assert opt.get_status() == (0, 0) and int(flag.item()) == 0
+    # 22 bits, chains of at most 1024 terms, twice; condition at most 3
+    assert off(P[at], want[at]) <= 4e-5
