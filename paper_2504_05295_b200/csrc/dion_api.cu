@@ -43,6 +43,8 @@ constexpr double P_HALF_MIN_MNR = 4e9;          // smallest m n r whose full-ran
 constexpr double SOLVE_PAIR_MIN_PANEL = 3e7;    // smallest rows x r whose blocked solves run on scaled half pairs
 constexpr i64 LAZY_PAIR_MIN_MNR = 50000000;     // smallest m n r whose Lazy-Dion step runs on scaled half pairs (2^25.6: 512 x 768 x 128)
 constexpr double GRAM_PAIR_MIN_FLOPS = 2e9;     // smallest rows r^2 whose Gram matrix runs on scaled half pairs
+constexpr i64 WIDE_P_WHOLE_K = 1024;            // K up to which the P of a wide range (wide_p) is not split: a tile's K loop is short, and the
+                                                // reduction would be one more launch that nearly always finds itself skipped (2 us)
 constexpr double P_PAIR_MIN_MNR = 1.5e10;       // smallest m n r whose P = (M + G) Q runs on bf16 operand pairs first
 
 constexpr i64 NBO_COLS = 512;  // = NBO, the outer block of the two-level Cholesky (defined below)
@@ -1930,7 +1932,10 @@ int step_batch(dion_ctx* c, const dion_matrix* const* list, int nb, float lr, cu
   DION_TRY(launch_gemm_group(s, group));
   if (hstep) {
     for (int b = 0; b < nb; ++b) group[b] = wide_p(s, b, list[b], tr, s.W(b, pin_off));
-    DION_TRY(launch_gemm_group(s, group));
+    s.no_split = qrow <= WIDE_P_WHOLE_K;
+    const int rc_wide = launch_gemm_group(s, group);
+    s.no_split = false;
+    DION_TRY(rc_wide);
   }
   }
 
@@ -2637,7 +2642,10 @@ int half_project(StepCtx& s, const dion_matrix* a, float* P) {
   p.C = P; p.ldc = r; p.epi = EPI_STORE;
   p.skip_flag = s.os + OS_P32;
   DION_TRY(launch_gemm(s, p, 0));
-  return launch_gemm(s, wide_p(s, 0, a, false, P), 0);
+  s.no_split = n <= WIDE_P_WHOLE_K;
+  const int rc = launch_gemm(s, wide_p(s, 0, a, false, P), 0);
+  s.no_split = false;
+  return rc;
 }
 // W = (M + G)^T U:
 int half_factor(StepCtx& s, const dion_matrix* a, const float* U, float* W, const int* skip) {
