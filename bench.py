@@ -11,9 +11,10 @@ in one process, each for the same --steps / --warmup, building and freeing one a
   llama405b  one Llama-3-405B-shaped block at rank fractions 1/4 and 1/16, bf16 gradients (one dion_step_grouped call)
   llama8b    Llama-3-8B-shaped list, 224 matrices, bf16 gradients, rank fraction 1/4 (ONE dion_step_grouped call)
 
-The top-level metric is the device time of the llama8b step in milliseconds (lower is better);
-every workload's record, with its own roofline, end-to-end time and per-case table, is under
-"workloads".  --workload NAME times that workload alone.
+The top-level metric is the device time of the llama8b step in milliseconds (lower is better).  The
+result line on stdout is kept short: per workload its time, end-to-end time, launches, clocks and
+roofline fraction under "workloads"; the full records, with the per-case and per-phase tables and
+the notes, go to stderr before it, one JSON line each.  --workload NAME times that workload alone.
 
   python bench.py [--gpus N] [--steps K] [--warmup W]          # this library
   python bench.py --impl reference ...                          # float64 CPU oracle, bounded samples
@@ -45,7 +46,10 @@ FFMA_PEAK_TFLOPS = 148 * 128 * 2 * 1.965e9 / 1e12     # 148 SMs x 128 FMA lanes 
 # DRAM bytes (read + write, ncu dram__bytes_*.sum) of the contraction kernel's four large launches over their
 # algorithmic bytes, one ratio per way the kernel is fed.  `roofline.traffic` is the algorithmic bytes of each
 # case times the ratio of its variant: a scaled figure, not a per-run counter (traffic grows in proportion to
-# the matrix sizes).  Each entry names the capture it came from.
+# the matrix sizes).  Each entry names the capture it came from.  The captures are of the register epilogue and, in fp32
+# mode, of bf16 pairs; the TMA epilogue moves the same tiles (8192^2 r=256, fp32 mode: P 281 + R 278 + error feedback 520
+# + X 483 MB = 0.63 of the model's 2.48 GB, some of a 268 MB array
+# staying in L2) and half pairs are as large as bf16 pairs.
 TRAFFIC_RATIOS = {
     # M + G kept in scratch: P, R and the error feedback read 4 bytes per element where the algorithmic model
     # counts M and G (the elementwise pass that forms the sum is another kernel)
@@ -763,10 +767,10 @@ def workload_record(wid, cases, grouped, args, peaks, binding, ms_step, e2e_ms, 
                                "ten consecutive dion_step calls per step" if reps_per_step > 1 else
                                "one dion_step call per matrix per step"),
                       "engine": ["auto", "simt", "tensor"][args.engine],
-                      "precision": ["fp32 (Orthonormalize 3xTF32; R, the error feedback and, on large matrices, P on bf16 "
-                                    "(hi, lo) pairs, 16 significant bits, where M + G is kept in scratch, P recomputed in "
-                                    "3xTF32 when the orthogonality probe asks; the X update one pass on factors rounded to "
-                                    "IEEE half (11 significant bits); FMA for ragged shapes)", "bf16 operands"][args.precision],
+                      "precision": ["fp32 (where M + G is kept in scratch: P, R and the error feedback on scaled IEEE half pairs, "
+                                    "22 significant bits, below m n r = 1.5e10, from there on on bf16 pairs, 16 bits, P recomputed "
+                                    "in 3xTF32 when the orthogonality probe asks; the X update one pass on factors rounded to "
+                                    "IEEE half (11 bits); FMA for ragged shapes)", "bf16 operands"][args.precision],
                       "orth": ["auto", "cholqr2", "shifted3", "householder", "rcqr"][args.orth],
                       "sync": ("compressed data-parallel sync: P and W all-reduced (mean) over the ranks"
                                if args.sync == "dp" else "none (independent replicas)"),
@@ -787,6 +791,42 @@ def workload_record(wid, cases, grouped, args, peaks, binding, ms_step, e2e_ms, 
         rec["us_per_dion_step"] = ms_step * 1e3 / reps_per_step
         rec["launches_per_dion_step"] = launches / args.steps / reps_per_step
     return rec
+
+
+def rounded(v):
+    """Six significant digits in every float of a record."""
+    if isinstance(v, float):
+        return float(f"{v:.6g}")
+    if isinstance(v, dict):
+        return {k: rounded(x) for k, x in v.items()}
+    if isinstance(v, (list, tuple)):
+        return [rounded(x) for x in v]
+    return v
+
+
+def result_line(records, top, peaks, tf32_measured, cpu, dtype, world):
+    """The one line on stdout: the headline workload's record without its tables and notes, and a few figures of each
+    workload."""
+    rec = records[top]
+    roof_keys = ("bound", "achieved", "peak", "unit", "frac", "traffic", "kernel", "ms_per_step", "share_of_step", "launches_per_step")
+    roof = {k: rec["roofline"].get(k) for k in roof_keys}
+
+    def brief(r):
+        out = {"value": r["value"], "steps": r["steps"], "e2e": r["e2e"], "gpu_launches": r["gpu_launches"],
+               "roofline_frac": r["roofline"]["frac"], "roofline_bound": r["roofline"]["bound"],
+               "clocks": {k: r["clocks"].get(k) for k in ("sm_mhz", "sm_max_mhz", "reasons")} if r["clocks"] else None,
+               "l2": r["config"]["l2"], "device_status": r["device_status"]}
+        return out | {k: r[k] for k in ("us_per_dion_step", "launches_per_dion_step") if k in r}
+
+    return rounded({
+        "metric": METRIC, "value": rec["value"], "unit": UNIT, "n_gpus": world, "steps": rec["steps"], "warmup": rec["warmup"],
+        "ms_per_step": rec["value"], "higher_is_better": False, "scaling": "weak", "vs_baseline": None, "dtype": dtype,
+        "data": "synthetic", "config": {k: v for k, v in rec["config"].items() if k != "precision"}, "e2e": rec["e2e"],
+        "gpu_launches": rec["gpu_launches"], "clocks": rec["clocks"], "roofline": roof,
+        "phases_ms": {p: v["ms"] for p, v in rec["phases"].items()}, "cpu_baseline": cpu, "device_status": rec["device_status"],
+        "peaks": {"hbm_gbs": peaks["hbm_gbs"], "bf16_tflops_sustained": peaks["bf16_sustained"],
+                  "tf32_single_pass_measured_tflops": tf32_measured, "source": peaks["source"]},
+        "workloads": {w: brief(r) for w, r in records.items()}})
 
 
 def run_ours(args):
@@ -842,21 +882,10 @@ def run_ours(args):
                          "the workload when it has several); value = their summed host time",
                "gpu_ms_same_cases": records[top].get("sample_gpu_ms")}
 
-    rec = records[top]
-    peaks = ctx["peaks"]
-    line = {"metric": METRIC, "value": rec["value"], "unit": UNIT, "n_gpus": world, "steps": args.steps,
-            "warmup": args.warmup, "ms_per_step": rec["value"], "higher_is_better": False, "scaling": "weak",
-            "vs_baseline": None, "dtype": "bf16" if args.precision == binding.PREC_BF16_OPERANDS else "f32",
-            "data": "synthetic", "config": rec["config"], "cases": rec["cases"], "phases": rec["phases"],
-            "roofline": rec["roofline"], "cpu_baseline": cpu, "e2e": rec["e2e"], "gpu_launches": rec["gpu_launches"],
-            "clocks": rec["clocks"], "device_status": rec["device_status"],
-            "peaks": {"hbm_gbs": peaks["hbm_gbs"], "bf16_tflops_sustained": peaks["bf16_sustained"],
-                      "tf32_assumed_tflops": 0.5 * peaks["bf16_sustained"],
-                      "tf32_single_pass_measured_tflops": tf32_measured, "source": peaks["source"],
-                      "tf32_note": "measured: this library's single-pass TF32 contraction on 8192^3 (burst, best of 5); "
-                                   "the roofline fractions use the assumed figure"},
-            "workloads": {w: {k: v for k, v in r.items() if k != "sample_gpu_ms"} for w, r in records.items()}}
-    print(json.dumps(line))
+    for r in records.values():
+        print(json.dumps(rounded({k: v for k, v in r.items() if k != "sample_gpu_ms"})), file=sys.stderr)
+    dtype = "bf16" if args.precision == binding.PREC_BF16_OPERANDS else "f32"
+    print(json.dumps(result_line(records, top, ctx["peaks"], tf32_measured, cpu, dtype, world)), flush=True)
     if world > 1:
         dist.destroy_process_group()
 

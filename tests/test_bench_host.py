@@ -100,3 +100,28 @@ def test_reference_arm_prints_one_json_line():
     assert line["e2e"]["h2d_bytes_per_step"] == 0 and line["vs_baseline"] is None
     # the value is a timing of the sample; the flop-scaled figure has its own field
     assert line["value"] == line["workloads"]["custom"]["value"] and line["projected_ms"] >= line["value"] * 0.999
+
+
+def test_result_line_is_short_enough_to_be_read_whole():
+    from types import SimpleNamespace
+    from paper_2504_05295_b200 import binding
+    args = SimpleNamespace(orth=0, form="standard", lazy=0, precision=0, engine=0, steps=20, warmup=5, sync="replicas")
+    peaks = {"hbm_gbs": 6556.8, "bf16_burst": 1620.3, "bf16_sustained": 1395.1, "source": "measured"}
+    clocks = {"sm_mhz": 1335.0, "sm_max_mhz": 1965.0, "reasons": ["sw_power_cap"], "samples": 309, "note": "x" * 200}
+    records = {}
+    for wid in bench.ALL_WORKLOADS:
+        cases = bench.parse_cases("", inputs, wid)
+        grouped = wid.startswith("llama")
+        ms = {p: 1000.0 / 7.0 for p in binding.PHASES}
+        records[wid] = bench.workload_record(wid, cases, grouped, args, peaks, binding, 100.0 / 3.0, 200.0 / 3.0, 3, 1, 10 ** 10, 10 ** 6, 5540,
+                                             clocks, ms, {p: 100 for p in binding.PHASES}, [1.0 / 3.0] * len(cases), [1] * len(cases),
+                                             10 ** 10, (0, 0, 0, 0), 10 if wid == "config1" else 1, 1, 0)
+    cpu = {"value": 3500.0 / 3.0, "unit": "ms", "cores": 64, "kind": "oracle", "sample": "y" * 300, "gpu_ms_same_cases": 1.0 / 3.0}
+    line = bench.result_line(records, bench.HEADLINE, peaks, 600.0 / 7.0, cpu, "f32", 1)
+    text = json.dumps(line)
+    assert len(text) < 7000, len(text)
+    for key in ("metric", "value", "unit", "n_gpus", "steps", "warmup", "ms_per_step", "higher_is_better", "scaling", "vs_baseline", "dtype",
+                "data", "config", "e2e", "gpu_launches", "clocks"):
+        assert key in line
+    assert line["value"] == 33.3333 and line["e2e"]["h2d_bytes_per_step"] == 10 ** 10 and set(line["workloads"]) == set(bench.ALL_WORKLOADS)
+    assert line["config"]["workload_id"] == "llama8b" and line["clocks"]["reasons"] == ["sw_power_cap"]
