@@ -1,9 +1,9 @@
 """Builds the CUDA library (``libdion_b200.so``) in-tree with nvcc for sm_100a.
 
-Run as ``true`` or through
-``__graft_entry__.build()``.  nvcc cross-compiles, so no GPU is needed.  The
-translation units are compiled side by side; an object is reused while none of
-the files it includes is newer.
+Run as ``python -m paper_2504_05295_b200.build`` (``-f`` compiles everything, ``-v`` does and shows
+ptxas's report) or through ``__graft_entry__.build()``.  nvcc cross-compiles, so no GPU is needed.
+The translation units are compiled side by side; an object is reused while none of the files it
+includes is newer.
 """
 from __future__ import annotations
 
