@@ -28,8 +28,8 @@ def reference(X, M, G, Q, lr, mu, transposed):
     return X - lr * math.sqrt(X.shape[0] / X.shape[1]) * Lx, B - (1 - mu) * L, Qn
 
 
-# 64 x (the smallest m n r that takes them), column counts beside the tiles' 64, 128, 192 and 256, odd row tiles, G in bf16
-SIZES = [(512, 1536, 64, False), (768, 1000, 72, False), (1000, 768, 136, True), (776, 1544, 128, False), (2056, 768, 192, False),
+# the smallest shapes that take them, column counts beside the tiles' 64, 128, 192 and 256, odd row tiles, G in bf16
+SIZES = [(256, 256, 64, False), (256, 264, 64, False), (264, 256, 64, True), (512, 1536, 64, False), (768, 1000, 72, False), (1000, 768, 136, True), (776, 1544, 128, False), (2056, 768, 192, False),
          (1032, 1040, 248, True), (1096, 1032, 256, False)]
 
 
