@@ -61,11 +61,15 @@ typedef enum { DION_F32 = 0, DION_BF16 = 1 } dion_dtype;
  * DION_PREC_FP32:           X, M and Q stay within 1e-4 (relative, Frobenius) of the rule evaluated in float64
  *                           wherever the rule itself is that well determined.  On the FMA engine every product is
  *                           fp32.  On the tensor cores each product runs at the cheapest arithmetic that keeps
- *                           the bound: P with 22 significant bits (3-term TF32 split), or, on large matrices, with
- *                           16 bits first (pairs of bf16 arrays) and again with 22 when the orthonormalization's
- *                           probe finds the panel ill conditioned; R and U R^T with 16 bits (bf16 pairs, ~1e-5 of
- *                           the product; U R^T enters M scaled by 1 - mu); U Q^T with 11 bits on factors rounded
- *                           to nearest (3e-4 of the update, 3e-6 of X).
+ *                           the bound.  Matrices with m n r below 1.5e10 whose orthonormalization is CholeskyQR2 (and
+ *                           Lazy-Dion steps): P, R and U R^T on scaled pairs of IEEE half arrays, 22 significant bits
+ *                           relative to an operand's largest entry.  Where a row, a column or a block lies so far below
+ *                           the rest that a pair would hold less of it (2^-18 for P, 2^-20 for the others, found on the
+ *                           device), P takes the three-term TF32 split, R and U R^T bf16 pairs: 22 and 16 bits at any
+ *                           magnitude.  Larger matrices: P with 16 bits first (bf16 pairs) and again with 22 (TF32 split)
+ *                           when the orthonormalization's probe finds the panel ill conditioned; R and U R^T with 16
+ *                           bits (~1e-5 of the product; U R^T enters M scaled by 1 - mu).  At higher rank P carries 22
+ *                           bits.  U Q^T: 11 bits on factors rounded to nearest (3e-4 of the update, 3e-6 of X).
  * DION_PREC_BF16_OPERANDS:  operands rounded to bf16 (M + G is added in fp32, then rounded); 3e-2 on X, M, Q.
  * The products inside Orthonormalize carry 22 significant bits in both modes.          */
 typedef enum { DION_PREC_FP32 = 0, DION_PREC_BF16_OPERANDS = 1 } dion_precision;
@@ -195,7 +199,7 @@ int dion_init(dion_ctx** out, const dion_config* cfg);
  * unchanged and DION_STATUS_BREAKDOWN is latched.
  *
  * Small matrices (up to 2048 x 2048 elements, r <= 512, fp32 mode on the tensor engine) are launch bound: a
- * step is a chain of ~30 short kernels.  For these the chain is captured into a CUDA graph the first time a
+ * step is a chain of 12 to 30 short kernels.  For these the chain is captured into a CUDA graph the first time a
  * descriptor is seen (same pointers, shapes and leading dimensions; the capture runs on a stream of the
  * context, so `cuda_stream` may be the legacy default stream) and later calls with that descriptor replay the
  * graph on `cuda_stream`; lr reaches it through a device scalar, so it may change from call to call.  Up to 64

@@ -443,8 +443,10 @@ __device__ __forceinline__ void potrf64(ctile_t L, ctile_t X, const Potrf64Set& 
 // column never reaches the trailing matrix and the factor stays nonsingular; a later round finishes the job.
 // A diagonal entry of A that is not finite means a NaN or Inf in M, G or Q: os[OS_FAIL] and DION_STATUS_NONFINITE.
 //
-// The right-looking form took one launch per 64 columns, ~21 us each, whatever the trailing work (r = 1024: 19 launches,
-// 440 us with the solve's products; now 230 us).  Bound by the chain of diagonal blocks, ~9 us each.  Here the chain
+// The right-looking form took one launch per 64 columns, ~21 us each, whatever the trailing work (r = 1024: 19 launches, 440 us
+// with the solve's products; now 160 us and one product).  Bound by the chain of diagonal blocks, ~8.5 us each: under ncu at
+// r = 1024 160 us at 1.85 GHz, 9 % of the SMs' issue slots, 0.4 % of DRAM, 18.5 of a warp's 25 cycles per instruction at barriers
+// (the runner's service warps, and helpers without a task).  Here the chain
 // D_k -> L_{k+1,k} -> A_{k+1,k+1} -> D_{k+1} stays inside ONE CTA (the "runner" of its matrix: two 64^3 products
 // and potrf64 per step), and every other tile is a task of a helper CTA, left-looking:
 //   L(i,k)    = (A_ik - sum_{j<k} L_ij L_kj^T) D_k^T                       i >= k + 3  (the runner makes i = k + 1)

@@ -49,9 +49,14 @@ constexpr double P_PAIR_MIN_MNR = 1.5e10;       // smallest m n r whose P = (M +
 
 constexpr i64 NBO_COLS = 512;  // = NBO, the outer block of the two-level Cholesky (defined below)
 
-// One launch of k_chol_flow factors Gram matrices up to this order; beyond it blocks of 512 columns.
+// One launch of k_chol_flow factors Gram matrices up to this order; beyond it blocks of 512 columns, whose products are on the
+// tensor cores.  Orthonormalization of rows x r in us, one launch against blocks: 8192 x 1536 547, 741; 8192 x 2048 827, 1047;
+// 12288 x 3072 2121, 2148; 16384 x 3584 3156, 2904; 16384 x 4096 4014, 3296.
 constexpr i64 FLOW_MAX_R = 3072;
-constexpr double FLOW_SOLVE_MAX = 1.1e6;        // largest rows r whose panel that launch solves too
+// Largest rows r whose panel that launch solves too, against the product with the inverse behind it; in us, the launch's own
+// solve first: 1024 x 256 98, 121; 4096 x 256 121, 143; 8192 x 256 137, 152; 4096 x 512 168, 187; 4096 x 1024 352, 298.  (One
+// matrix by itself would have the line near 3e6; the helpers of a chain have as many panels to solve as it has matrices.)
+constexpr double FLOW_SOLVE_MAX = 1.1e6;
 constexpr i64 FLOW_SOLVE_MAX_TILES = 40000;     // ... in an adaptive round: most 64^3 products of its substitution
 constexpr float NEAR_MAX_DEF = 3e-3f;           // largest |P^T P - I|_F whose factor is taken as a series (k_near_identity): third-order error 3e-8
 constexpr i64 NEAR_MAX_BLOCKS = 512;
@@ -337,7 +342,8 @@ cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t s
 // Splits of K: a K step of 16 takes about as long as the latency of its loads whatever runs beside it, so a product of few tiles is
 // cut to two or three steps per block, up to two blocks per SM (1001 x 83 x 333 with the reduction: 28.6 -> 14 us).
 // Fewer where the next kernel adds the partial sums up itself (k_chol_flow: one CTA reads those of the first three tiles, which
-// costs it as much per split as a K step here).
+// costs it as much per split as a K step here: with the square of the splits kept to K / 16, orthonormalizing 1001 x 83 takes 87
+// us and 1030 x 190 127, with every split 99 and 148).
 constexpr i64 SPLIT_MIN_K = 32;
 constexpr i64 SPLIT_MAX = 64;
 constexpr i64 SIMT_THIN_N = 32;          // outputs of at most this many columns take 128 x 32 tiles
@@ -1189,7 +1195,7 @@ int resolve_orth_for(const dion_ctx* c, i64 r, i64 short_dim, bool has_sketches)
 }
 
 // Where the product that forms the panel writes it: CholeskyQR2 reads it from the save buffer (round one goes
-// Psave -> P1, round two P1 -> P0), so that the panel is still there if a pivot fails; every other mode works in P0.
+// Psave -> P0, round two P0 -> P1), so that the panel is still there if a pivot fails; every other mode works in P0.
 i64 panel_offset(const StepCtx& s, i64 r, i64 short_dim) {
   const bool cq2 = resolve_orth_for(s.c, r, short_dim, s.list != nullptr) == DION_ORTH_CHOLQR2;
   return (cq2 && s.L.Psave > 0) ? s.L.Psave : s.L.P0;
@@ -2157,7 +2163,7 @@ bool same_matrix(const dion_matrix& x, const dion_matrix& y) {
          x.sketch_rows == y.sketch_rows && x.ld_sketch == y.ld_sketch;
 }
 
-// A step on a small matrix is a chain of ~30 launches that take longer to issue than to run.  Such steps are
+// A step on a small matrix is a chain of 12 to 30 launches that take longer to issue than to run.  Such steps are
 // captured once (on the context's own stream: the caller's may be the legacy stream, which cannot capture) and
 // replayed as one graph launch into the caller's stream.
 bool graph_eligible(const dion_ctx* c, const dion_matrix* a) {

@@ -62,9 +62,9 @@ constexpr int TINY_MAX_ROWS = 512;
 constexpr int TINY_THREADS = 512;      // (128 registers a thread: potrf64 keeps an 8 x 8 piece in them)
 // Row strides (floats) that keep the fragment loads of the two products off each other's banks: a lane reads
 // (row ft, column fg) of the panel for the Gram matrix (stride = 8 mod 32: no conflict) and (row fg, column ft)
-// of it (two-way) and of the inverse (copied to stride = 4 mod 32: none) for U.
+// of it and of the inverse (both two-way) for U.
 constexpr int TINY_LD = NB + 8;
-constexpr int TINY_BLK = CB * CLD;          // floats of a 64 x 64 tile (row stride = 4 mod 32: none for the inverse)
+constexpr int TINY_BLK = CB * CLD;          // floats of a 64 x 64 tile (row stride = 8 mod 32)
 inline int tiny_rows_pad(i64 rows) { return (int)((rows + 15) / 16 * 16); }
 inline int tiny_cholqr2_smem(i64 rows) {    // panel (rows padded to 16), L, X, red, what potrf64 needs beside them
   return (int)sizeof(float) * (tiny_rows_pad(rows) * TINY_LD + 2 * TINY_BLK + TINY_THREADS) + (int)(sizeof(Potrf64Set) + sizeof(Potrf64Aux));
@@ -679,7 +679,7 @@ __global__ void __launch_bounds__(128) k_probe_w4(const float* __restrict__ U, i
 // passes), its warps four rows each for Y = U z, then (1 << ct_log) threads by four columns and the rest by row groups for
 // U^T Y.  Two launches read the panel twice from L2 and met in memory: 2048 x 128 14.5 us, 4096 x 1024 23 us (now 5 and 15 us).
 // grid = (chunks, matrices); part[chunk][j][p] as in k_probe_w.
-constexpr i64 PF_MAX_R = 1024;
+constexpr i64 PF_MAX_R = 1024;      // 256 threads by four columns
 constexpr int PF_RED = 256 * 4 * NPROBE;      // floats: row groups x columns x probes
 constexpr int PF_SMEM_MAX = ((int)PF_MAX_R * NPROBE + PF_RED + 32 * NPROBE) * 4;
 __global__ void __launch_bounds__(256) k_probe_fused(const float* __restrict__ U, i64 ld, i64 rows, i64 r, i64 rows_per_chunk,
