@@ -434,8 +434,9 @@ __device__ __forceinline__ void potrf64(ctile_t L, ctile_t X, const Potrf64Set& 
 //   L L^T = A (lower factor, below the block diagonal), D_k = L_kk^-1, and behind it, tile by tile
 //   and beside the rest of the factorization, either
 //     solve:    U = P L^-T for a panel P (rows x sz), or
-//     inverse:  L^-T of the square (row-major, upper triangular; zeros below the diagonal as far as a product of 256-column
-//               tiles reads) for a solve by one tensor-core product, and its largest entry.
+//     inverse:  L^-T of the square (row-major, upper triangular; zeros below the diagonal, of the whole Gram matrix as far as a
+//               product of 256-column tiles reads, of a smaller square everywhere) for a solve by tensor-core products, and
+//               its largest entry.
 // Pivots: with floor_rel == 0 a pivot that is <= 0 or not finite sets os[OS_FAIL] (and DION_STATUS_BREAKDOWN unless
 // `status` is null) and is replaced by 1, so that everything downstream stays finite.  With floor_rel > 0 (adaptive
 // rounds) a pivot below floor_rel times the column's entry of diag(A) is below the rounding noise of the Gram matrix:
@@ -468,6 +469,11 @@ constexpr int FLOW_COMPUTE = 256;            // threads that compute ...
 constexpr int FLOW_SERVICE = 128;            // ... and the service warps of a runner (four: nothing else fits beside eight anyway)
 constexpr int FLOW_THREADS = FLOW_COMPUTE + FLOW_SERVICE;
 constexpr int FLOW_IZ = 4;                    // the inverse's rows are stored (as zeros below the diagonal) up to a multiple of this many tiles
+// rows of tiles of column k of the inverse that are written (whole: of a square whose largest entry is looked for afterwards)
+__host__ __device__ __forceinline__ int flow_inverse_rows(int T, int k, bool whole) {
+  const int n = k / FLOW_IZ * FLOW_IZ + FLOW_IZ;
+  return (whole || n > T) ? T : n;
+}
 constexpr int FLOW_LAG = 2;                   // steps by which the panel's tasks follow the factor's
 
 struct FlowArgs {
@@ -840,7 +846,7 @@ __global__ void __launch_bounds__(FLOW_THREADS, 1) k_chol_flow(const __grid_cons
     nS = (s == 0) ? 2 * min(max(T - 2, 0), f.ahead + 1) : 2 * min(max(T - 2 - s - f.ahead, 0), 1);
     nP = 0;
     const int k = s - FLOW_LAG;
-    if (k >= 0 && k < T) nP = solve ? NR : min(T, k / FLOW_IZ * FLOW_IZ + FLOW_IZ);
+    if (k >= 0 && k < T) nP = solve ? NR : flow_inverse_rows(T, k, f.sz < f.r);
   };
   auto fetch_task = [&](int ticket) -> FlowTask {
     FlowTask t;

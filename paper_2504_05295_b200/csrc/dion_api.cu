@@ -708,7 +708,7 @@ int chol_flow(StepCtx& s, i64 r, i64 o, i64 sz, int mode, i64 pin_off, i64 pout_
   // one runner per matrix; as many helpers as can be resident beside them, at most one per task
   i64 tasks = (T > 2) ? (T - 2) * (T - 3) / 2 + 2 * (T - 2) : 0;
   if (solve) tasks += NR * T;
-  else for (i64 k = 0; k < T; ++k) tasks += (T < k / FLOW_IZ * FLOW_IZ + FLOW_IZ) ? T : k / FLOW_IZ * FLOW_IZ + FLOW_IZ;
+  else for (i64 k = 0; k < T; ++k) tasks += flow_inverse_rows((int)T, (int)k, sz < r);
   const i64 cap = (i64)flow_ctas_per_sm() * c->sm_count;
   i64 grid = s.nb + tasks * s.nb;
   if (grid > cap) grid = cap;

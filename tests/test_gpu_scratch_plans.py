@@ -51,3 +51,24 @@ def test_the_column_sums_leave_the_sum_alone(m, n, r, transposed):
     # entry by entry: the library's 1e-4 of the largest one
     for got, want in ((M, Mr), (Q, Qr), (d, R.norm(dim=0))):
         assert (got.double() - want).abs().max().item() <= 1e-4 * want.abs().max().item()
+
+
+def test_what_an_earlier_call_left_in_the_scratch_does_not_matter():
+    # Blocked solves (r > 3072) on half pairs scale the inverses of 512-column squares by their largest entry: below the diagonal
+    # there must be zeros, not the saved panel of an earlier call of another shape, which lies where the inverses go.
+    g = torch.Generator(device="cuda"); g.manual_seed(1)
+    rows, r = 14336, 3584
+    P = torch.randn(rows, r, generator=g, device="cuda")
+    big = torch.randn(73728, 512, generator=g, device="cuda") * 1e15
+    flag = torch.zeros(1, dtype=torch.int32, device="cuda")
+    outs = []
+    for before in (False, True):
+        U = P.clone()
+        with binding.Dion(workspace_bytes=6 << 30) as opt:
+            if before:
+                opt.orthonormalize(73728, 512, 73728, big, flag)
+                assert opt.get_status() == (0, 0)
+            opt.orthonormalize(rows, r, rows, U, flag)
+            assert opt.get_status() == (0, 0) and opt.fallbacks() == 0
+        outs.append(U)
+    assert torch.equal(outs[0], outs[1])
