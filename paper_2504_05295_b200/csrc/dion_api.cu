@@ -61,6 +61,10 @@ constexpr i64 FLOW_SOLVE_MAX_TILES = 40000;     // ... in an adaptive round: mos
 constexpr float NEAR_MAX_DEF = 3e-3f;           // largest |P^T P - I|_F whose factor is taken as a series (k_near_identity): third-order error 3e-8
 constexpr i64 NEAR_MAX_BLOCKS = 512;
 constexpr int FLOW_EXCLUSIVE_MAX = 8;           // matrices of a chain up to which its runners get an SM each
+// Partial sums of the Gram product that it adds up itself.  One CTA reads those of the first three tiles; from there on a launch over
+// all SMs reduces them first (4096 x 256, 32 splits: orthonormalization 120.8 -> 101.5 us, 2048 x 128, 16 splits: 82.0 -> 75.5;
+// 1001 x 83, 7 splits: 86.7 -> 87.1, left in the launch).
+constexpr int FLOW_MAX_SPLITS = 8;
 constexpr int FLOW_AHEAD_MAX = 16;              // steps by which its preparations are handed out early
 constexpr i64 FLOW_MAX_PANEL_TILES = 800;       // ... and most 64-row blocks of it (the control block holds 64 such matrices)
 
@@ -210,6 +214,14 @@ Layout make_layout(const dion_ctx* c, i64 m, i64 n, i64 r) {
   L.DinvP = o; o += align64(((r + NB - 1) / NB) * (i64)NB * NB);
   // split-K partials: the largest plain-store product of a step is max(m,n) x r
   i64 pf = 4 * (i64)c->sm_count * 64 * 64;
+  // ... and enough for as many splits as give every SM work: 148 tiles of 64 x 64 held two splits of a 4096 x 256 product, which
+  // left more than half of the chip idle (from 4096^2: 50 us with two, 37 with four).  The fixed scratch keeps its size: what fits it is
+  // what fitted before.
+  if (c->form_sum) {
+    const i64 need[4] = {umma_split_floats(m, r, n, false, c->sm_count), umma_split_floats(n, r, m, false, c->sm_count),
+                         umma_split_floats(r, r, big, true, c->sm_count), pf};
+    for (i64 f : need) if (f > pf) pf = f;
+  }
   if (pf > PART_CAP_FLOATS) pf = PART_CAP_FLOATS;
   L.part_floats = pf;
   L.part = o; o += align64(pf);
@@ -393,7 +405,10 @@ int launch_gemm_simt(dion_ctx* c, GemmArgs g, cudaStream_t st, float* part, i64 
     else launch_pdl(k_gemm_simt<64, 64, 16, 4, 4, 2, NoTabs>, grid, dim3(256), 0, st, g, NoTabs(), 1);
   }
   DION_CHECK_LAUNCH(c);
-  if (g.splits_out != nullptr) { *g.splits_out = splits; return DION_OK; }      // (the caller sums the partial products itself)
+  if (g.splits_out != nullptr) {      // (the caller sums that many partial products itself)
+    if (splits <= *g.splits_out) { *g.splits_out = splits; return DION_OK; }
+    *g.splits_out = 1;
+  }
   if (splits > 1) {
     const i64 total = g.N % 4 == 0 ? (g.M * g.N + 3) / 4 : g.M * g.N;      // (four elements per thread where rows allow it)
     int blocks = (int)((total + 255) / 256);
@@ -883,8 +898,8 @@ int cholqr_round(StepCtx& s, i64 pin_off, i64 pout_off, i64 rows, i64 r, int mod
   g.C = s.ws + s.L.Gram; g.ldc = r; g.epi = EPI_STORE; g.tri = TRI_LOWER; g.skip_flag = skips ? skip : nullptr; g.precise = rm_precise(mode) ? 1 : 0;
   const bool in_flow = flow_solves(s, rows, r, adaptive);      // factorization and solve in one launch
   const bool flow_all = in_flow || (!adaptive && r <= FLOW_MAX_R);      // at least the whole factorization
-  int nsplit = 1;
-  if (flow_all) g.splits_out = &nsplit;       // (which also adds up the partial products)
+  int nsplit = flow_all ? FLOW_MAX_SPLITS : 1;
+  if (flow_all) g.splits_out = &nsplit;       // (which also adds up a few partial products)
   DION_TRY(launch_gemm_chain(s, g));
   const float* part_scale = g.alpha_dev;
   if (flow_all) {

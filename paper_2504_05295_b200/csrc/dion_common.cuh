@@ -67,7 +67,7 @@ struct GemmArgs {
   const void* B16lo;             // to the "lo" arrays of the same shape and strides): three bf16 MMAs per K step, ~1e-5 relative
   int f16;                       // with ab16: the arrays hold IEEE half values instead of bf16 (11 significant bits)
   const int* wide_flag;          // with f16, optional: the arrays of a matrix whose flag is set hold bf16 after all (OS_WIDE; OS_SLOT_INTS apart)
-  int* splits_out;               // HOST, optional: a product that splits K leaves its partial sums unreduced and reports their number here
+  int* splits_out;               // HOST, optional: a product that splits K leaves up to so many partial sums unreduced; their number on return
   int tf32x1;                    // tensor engine, fp32 mode: the operands' values fit TF32 already (k_round_tf32): one MMA
                                  // per K step instead of the three-term split.  Ignored by the FMA engine.
 };

@@ -30,6 +30,26 @@ enum : int {
   UMMA_VARIANT_NO_PAIRS = 4,         // single-CTA tiles where the product would take CTA pairs
   UMMA_VARIANT_NO_TMA_EPI = 8        // register epilogue where the product would take the TMA epilogue
 };
+
+// K splits of a plain-store product of few tiles: enough for every worker (CTA, or pair of CTAs) to have an item, at least four
+// K blocks each.
+constexpr i64 UMMA_MAX_SPLITS = 32;
+inline i64 umma_split_count(i64 tiles, i64 workers, i64 nkb) {
+  i64 want = workers / tiles;
+  if (want > nkb / 4) want = nkb / 4;
+  return want > UMMA_MAX_SPLITS ? UMMA_MAX_SPLITS : want < 1 ? 1 : want;
+}
+constexpr i64 UMMA_PAIR_MIN_ROWS = 512;   // smallest output height given to CTA pairs
+constexpr i64 UMMA_PAIR_MIN_TRI = 2048;   // smallest lower-triangular output given to CTA pairs
+// Floats of partial sums that the splits of an M x N product take (an upper bound over the operand types).
+inline i64 umma_split_floats(i64 M, i64 N, i64 K, bool tri, int sm_count) {
+  if (M < 128 || N < 64) return 0;
+  const bool pairs = N >= 256 && M >= UMMA_PAIR_MIN_ROWS && (!tri || N >= UMMA_PAIR_MIN_TRI);
+  const i64 tm = pairs ? 256 : 128, tn = (N < 256 || (tri && !pairs)) ? 128 : 256;
+  const i64 nM = (M + tm - 1) / tm, nN = (N + tn - 1) / tn, tiles = tri ? nM * (nM + 1) / 2 : nM * nN;
+  const i64 splits = umma_split_count(tiles, pairs ? sm_count / 2 : sm_count, K / 32);
+  return splits > 1 ? splits * M * N : 0;
+}
 int umma_try_launch(const GemmArgs& g_in, int precision, int sm_count, float* part, i64 part_floats, int* status,
                     cudaStream_t st, int variant = 0);
 

@@ -1901,8 +1901,6 @@ int umma_configure() {
   return DION_OK;
 }
 
-constexpr i64 PAIR_MIN_ROWS = 512;   // smallest output height given to CTA pairs
-constexpr i64 PAIR_MIN_TRI = 2048;   // smallest lower-triangular output given to CTA pairs
 // Largest K given to the TMA epilogue: operand pairs (two 64 KB stages left; at K = 1024 the error feedback of 14336 x 4096 took
 // 304 us against 262) and single arrays (four 32 KB stages; still ahead at 1024: 54.6 against 58.9 us at 4096^2).
 constexpr i64 TE_MAX_K_PAIRS = 512;
@@ -1961,7 +1959,7 @@ int umma_try_launch(const GemmArgs& g_in, int precision, int sm_count, float* pa
   // (Not the single-pass TF32 product, which only ragged shapes still take.)
   bool cg2 = ((!bf16 && !g.tf32x1 && g.a2_mode != ADD_BF16) || d16) &&
              !(variant & (UMMA_VARIANT_REGISTER_LOADS | UMMA_VARIANT_NO_PAIRS)) && nclusters > 0 &&
-             g.N >= 256 && g.M >= PAIR_MIN_ROWS && (g.tri != TRI_LOWER || g.N >= PAIR_MIN_TRI);
+             g.N >= 256 && g.M >= UMMA_PAIR_MIN_ROWS && (g.tri != TRI_LOWER || g.N >= UMMA_PAIR_MIN_TRI);
   int BN = ((g.tri == TRI_LOWER && !tri_wide && !cg2) || g.N < 256) ? 128 : 256;
   // (a rank-r update of few tiles: its time is the epilogue of one tile; 256 x 512 in four tiles of 256 columns 12 us)
   if (!cg2 && BN == 256 && g.epi != EPI_STORE && g.tri == TRI_FULL && ((g.M + BM - 1) / BM) * ((g.N + 255) / 256) * nbat * 2 <= sm_count) BN = 128;
@@ -2029,10 +2027,7 @@ int umma_try_launch(const GemmArgs& g_in, int precision, int sm_count, float* pa
   }
   int splits = 1;
   if (g.epi == EPI_STORE && !g.klimit && part != nullptr && tiles < workers_max) {
-    i64 want = workers_max / tiles;
-    const i64 kmax = p.nkb / 4;                       // at least four K blocks per split
-    if (want > kmax) want = kmax;
-    if (want > 32) want = 32;
+    i64 want = umma_split_count(tiles, workers_max, p.nkb);
     while (want > 1 && want * g.M * g.N > part_floats) --want;
     if (want > 1) splits = (int)want;
   }
@@ -2147,7 +2142,10 @@ int umma_try_launch(const GemmArgs& g_in, int precision, int sm_count, float* pa
     }
   }
   if (cudaGetLastError() != cudaSuccess) return DION_ERR_CUDA;
-  if (g.splits_out != nullptr) { *g.splits_out = splits; return 1; }      // (the caller sums the partial products itself)
+  if (g.splits_out != nullptr) {      // (the caller sums that many partial products itself)
+    if (splits <= *g.splits_out) { *g.splits_out = splits; return 1; }
+    *g.splits_out = 1;
+  }
   if (splits > 1) {
     const i64 total = (g.M * g.N + 3) / 4;
     int blocks = (int)((total + 255) / 256);
