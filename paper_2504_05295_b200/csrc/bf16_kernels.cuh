@@ -416,8 +416,9 @@ __device__ __forceinline__ void range_of_blocks(const float* __restrict__ part, 
 // The ranges of arrays from a table (blockIdx.y; 16-byte aligned rows), of rows0 or, from the second on, rows1 rows: gridDim.x
 // blocks' partial results `stride` floats apart.
 __global__ void __launch_bounds__(256) k_range_partial(const ChainPtrs srcs, i64 ld, i64 rows0, i64 rows1, i64 cols, float* __restrict__ part,
-                                                       i64 stride, const int* __restrict__ skip_flag, i64 skip_stride) {
+                                                       i64 stride, const int* __restrict__ skip_flag, i64 skip_stride, int* __restrict__ slots) {
   pdl_enter();
+  if (blockIdx.y == 0) clear_slot(slots);      // (of one matrix)
   if (skip_flag != nullptr && skip_flag[(i64)blockIdx.y * skip_stride] != 0) return;
   Range g;
   range_scan(g, reinterpret_cast<const float*>(srcs.p[blockIdx.y]), ld, blockIdx.y == 0 ? rows0 : rows1, cols, true,
@@ -481,9 +482,10 @@ __device__ __forceinline__ void form_sum_range(Range& g, const float* __restrict
 template <bool VEC>
 __global__ void __launch_bounds__(256, 3) k_form_sum_amax(const ChainPtrs Ms, i64 ldm, const ChainPtrs Gs, i64 ldg, int g_mode, i64 rows, i64 cols,
                                                        const ChainPtrs Qs, i64 ldq, i64 qrows, i64 qcols, int qvec, float* __restrict__ out,
-                                                       float* __restrict__ part, i64 wstride, int* __restrict__ slots) {
+                                                       float* __restrict__ part, i64 wstride, int* __restrict__ slots, int* __restrict__ flag) {
   pdl_enter();
   clear_slot(slots);
+  if (flag != nullptr && blockIdx.x == 0 && threadIdx.x == 0) *flag = 0;      // (the caller's, of one matrix)
   const i64 b = blockIdx.y;
   part += b * wstride;
   Range g, gq;

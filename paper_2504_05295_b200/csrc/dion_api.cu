@@ -781,7 +781,7 @@ int potrf_blocked(StepCtx& s, i64 r, int mode, const std::function<int(i64, i64)
           cst = c->side;
         }
         dim3 grid((unsigned)grid_for(c, rem * sz, s.nb), (unsigned)s.nb);
-        launch_pdl(k_copy_block, grid, dim3(256), 0, cst, ptmp, r, panel, r, rem, sz, skip, s.wstride, (const int*)nullptr, (int*)nullptr);
+        launch_pdl(k_copy_block, grid, dim3(256), 0, cst, ptmp, r, panel, r, rem, sz, skip, s.wstride, (const int*)nullptr, (int*)nullptr, (int*)nullptr);
         DION_CHECK_LAUNCH(c);
       }
       const float* lp = side_copy ? ptmp : panel;
@@ -884,7 +884,7 @@ int cholqr_round(StepCtx& s, i64 pin_off, i64 pout_off, i64 rows, i64 r, int mod
     float* range = s.ws + s.L.part;      // (read before the product writes its partial sums there)
     ChainPtrs t;
     for (int b = 0; b < s.nb; ++b) t.p[b] = s.W(b, pin_off);
-    launch_pdl(k_range_partial, dim3((unsigned)parts, (unsigned)s.nb), dim3(256), 0, s.st, t, r, rows, rows, r, range, s.wstride, sk, (i64)OS_SLOT_INTS);
+    launch_pdl(k_range_partial, dim3((unsigned)parts, (unsigned)s.nb), dim3(256), 0, s.st, t, r, rows, rows, r, range, s.wstride, sk, (i64)OS_SLOT_INTS, (int*)nullptr);
     DION_CHECK_LAUNCH(c);
     launch_pdl(k_split_f16_scaled, dim3((unsigned)grid_for(c, rows * r / 8, s.nb), (unsigned)s.nb), dim3(256), 0, s.st,
                (const float*)(s.ws + pin_off), r, rows, r, (const float*)range, (int)parts, hi, lo, s.ws + s.L.gmax + AMAX_PARTS,
@@ -1180,7 +1180,7 @@ int rcqr(StepCtx& s, i64 rows, i64 r) {
     g.C = stack; g.ldc = r; g.epi = EPI_STORE; g.precise = 1;
     DION_TRY(launch_gemm(s, g, b));
     dim3 grid((unsigned)grid_for(c, rows * r), 1);
-    launch_pdl(k_copy_block, grid, dim3(256), 0, s.st, (const float*)s.W(b, s.L.P0), r, stack + k * r, r, rows, r, nullptr, 0, (const int*)nullptr, (int*)nullptr);
+    launch_pdl(k_copy_block, grid, dim3(256), 0, s.st, (const float*)s.W(b, s.L.P0), r, stack + k * r, r, rows, r, nullptr, 0, (const int*)nullptr, (int*)nullptr, (int*)nullptr);
     DION_CHECK_LAUNCH(c);
   }
   s.wt_off = s.L.SkW;
@@ -1493,7 +1493,7 @@ int validate(const dion_matrix* a, bool shard = false) {
   return DION_OK;
 }
 
-int begin_step(dion_ctx* c, const dion_matrix* a, int nb, cudaStream_t st, StepCtx* s, int fixed_slot = -1, bool clear = true) {
+int begin_step(dion_ctx* c, const dion_matrix* a, int nb, cudaStream_t st, StepCtx* s, int fixed_slot = -1) {
   s->c = c;
   s->st = st;
   s->L = make_layout(c, a->m, a->n, a->r);
@@ -1510,8 +1510,14 @@ int begin_step(dion_ctx* c, const dion_matrix* a, int nb, cudaStream_t st, StepC
   s->flag = s->os + OS_FAIL;
   s->tensor = (c->cfg.engine != DION_ENGINE_SIMT);
   s->in_orth = false;
-  if (clear && cudaMemsetAsync(s->os, 0, sizeof(int) * OS_SLOT_INTS * nb, st) != cudaSuccess) return DION_ERR_CUDA;
   return DION_OK;
+}
+
+// The state slots of a chain start at zero: cleared by the first kernel of a step where it can (a memset is a launch of its own and
+// lets nothing start beside it: 3 us; the step of one data-parallel rank, 4096 x 2048, r = 256: 296 -> 285 us), else here; flag (optional): the caller's flag too.
+int clear_slots(const StepCtx& s, int* flag = nullptr) {
+  if (cudaMemsetAsync(s.os, 0, sizeof(int) * OS_SLOT_INTS * s.nb, s.st) != cudaSuccess) return DION_ERR_CUDA;
+  return flag == nullptr || cudaMemsetAsync(flag, 0, sizeof(int), s.st) == cudaSuccess ? DION_OK : DION_ERR_CUDA;
 }
 
 // R = (M + G)^T U on bf16 pairs (transposed form: (M + G) U): where M + G is kept in scratch (sum_in_scratch) the
@@ -1536,8 +1542,8 @@ bool step_on_half_pairs(const StepCtx& s, i64 m, i64 n, i64 r, i64 short_dim) {
 
 // M + G and the half pairs of it and of Q (in S16) for every matrix of the chain: in one pair of launches when they share
 // leading dimensions and alignment.  ranges: matrices of wide range are flagged and get what the other formats need instead
-// (Q dense in P1, a bf16 pair of the sum).
-int half_sum_chain(StepCtx& s, const dion_matrix* const* list, i64 qrow, bool clear, bool ranges) {
+// (Q dense in P1, a bf16 pair of the sum).  clear: the state slots are cleared here; flag (one matrix): the caller's flag too.
+int half_sum_chain(StepCtx& s, const dion_matrix* const* list, i64 qrow, bool clear, bool ranges, int* flag = nullptr) {
   dion_ctx* c = s.c;
   const dion_matrix* a0 = list[0];
   const i64 m = a0->m, n = a0->n, r = a0->r;
@@ -1560,8 +1566,8 @@ int half_sum_chain(StepCtx& s, const dion_matrix* const* list, i64 qrow, bool cl
     const dim3 fg((unsigned)grid_for(c, 32 * pieces, per), (unsigned)per), sg((unsigned)grid_for(c, (m * n + qrow * r) / 8, per), (unsigned)per);
     float* part = s.W(b, s.L.part);      // (the ranges are read before the products write their partial sums there)
     const int qv = qvec_ok(a) ? 1 : 0;
-    if (vec_ok(a)) launch_pdl(k_form_sum_amax<true>, fg, dim3(256), 0, s.st, Ms, a->ldm, Gs, a->ldg, g_mode, m, n, Qs, a->ldq, qrow, r, qv, s.W(b, s.L.B32), part, s.wstride, clear ? s.OS(b) : (int*)nullptr);
-    else launch_pdl(k_form_sum_amax<false>, fg, dim3(256), 0, s.st, Ms, a->ldm, Gs, a->ldg, g_mode, m, n, Qs, a->ldq, qrow, r, qv, s.W(b, s.L.B32), part, s.wstride, clear ? s.OS(b) : (int*)nullptr);
+    if (vec_ok(a)) launch_pdl(k_form_sum_amax<true>, fg, dim3(256), 0, s.st, Ms, a->ldm, Gs, a->ldg, g_mode, m, n, Qs, a->ldq, qrow, r, qv, s.W(b, s.L.B32), part, s.wstride, clear ? s.OS(b) : (int*)nullptr, flag);
+    else launch_pdl(k_form_sum_amax<false>, fg, dim3(256), 0, s.st, Ms, a->ldm, Gs, a->ldg, g_mode, m, n, Qs, a->ldq, qrow, r, qv, s.W(b, s.L.B32), part, s.wstride, clear ? s.OS(b) : (int*)nullptr, flag);
     DION_CHECK_LAUNCH(c);
     launch_pdl(k_split_sum, sg, dim3(256), 0, s.st, (const float*)s.W(b, s.L.B32), m * n, Qs, a->ldq, qrow, r, qv, (const float*)part, (int)fg.x,
                reinterpret_cast<__half*>(s.W(b, s.L.Bp)), reinterpret_cast<__half*>(s.W(b, s.L.S16)), s.W(b, s.L.P1), s.W(b, s.L.lz),
@@ -1777,7 +1783,7 @@ int step_batch(dion_ctx* c, const dion_matrix* const* list, int nb, float lr, cu
                const float* x_scale = nullptr, int fixed_slot = -1) {
   StepCtx s;
   const dion_matrix* a0 = list[0];
-  DION_TRY(begin_step(c, a0, nb, st, &s, fixed_slot, false));      // (the state slots: by the kernel that forms M + G)
+  DION_TRY(begin_step(c, a0, nb, st, &s, fixed_slot));
   const i64 m = a0->m, n = a0->n, r = a0->r;
   s.list = list;
   if (c->cfg.orth == DION_ORTH_RCQR) {
@@ -1836,7 +1842,7 @@ int step_batch(dion_ctx* c, const dion_matrix* const* list, int nb, float lr, cu
   i64 lds[MAX_CHAIN];
   if (hstep) DION_TRY(half_sum_chain(s, list, qrow, true, true));
   else if (b32) DION_TRY(form_sum_chain(s, list, bpair, true));
-  else if (!d16 && cudaMemsetAsync(s.os, 0, sizeof(int) * OS_SLOT_INTS * nb, st) != cudaSuccess) return DION_ERR_CUDA;
+  else if (!d16) DION_TRY(clear_slots(s));
   const bool phalf = b32 && s.L.Bh > 0;
   bool p_half_ready = false;
   if (phalf) {      // the scaled half pairs of M + G and of Q, for the whole chain
@@ -2275,7 +2281,7 @@ int lazy_pairs(StepCtx& s, const dion_matrix* a, float lr, int refresh) {
     float* pm = s.ws + s.L.part;      // (read before the next product writes its partial sums there)
     ChainPtrs t;
     t.p[0] = src;
-    launch_pdl(k_range_partial, dim3((unsigned)nparts), dim3(256), 0, st, t, ld, rows, rows, cols, pm, (i64)0, (const int*)nullptr, (i64)0);
+    launch_pdl(k_range_partial, dim3((unsigned)nparts), dim3(256), 0, st, t, ld, rows, rows, cols, pm, (i64)0, (const int*)nullptr, (i64)0, (int*)nullptr);
     DION_CHECK_LAUNCH(c);
     launch_pdl(k_split_f16_scaled, dim3((unsigned)grid_for(c, rows * cols / 8)), dim3(256), 0, st, src, ld, rows, cols, (const float*)pm, (int)nparts,
                halves(off), halves(off) + rows * cols, sc + slot, (i64)0, (const int*)nullptr, (i64)0, ldexpf(1.f, HS_U_BITS),
@@ -2305,7 +2311,7 @@ int lazy_pairs(StepCtx& s, const dion_matrix* a, float lr, int refresh) {
     g.M = M_; g.N = N_; g.K = K_; g.C = C; g.ldc = ldc; g.epi = epi;
     return g;
   };
-  DION_TRY(half_sum_chain(s, &a, n, false, true));      // M + G, its pair and Q's
+  DION_TRY(half_sum_chain(s, &a, n, true, true));      // M + G, its pair and Q's
   if (refresh) {
     PhaseScope ps_orth(c, st, DION_PHASE_ORTH);
     // T = (M + G) Q  (m x r), Z = (M + G)^T T (n x r), Q <- Orthonormalize(Z)
@@ -2357,6 +2363,7 @@ int lazy_one(dion_ctx* c, const dion_matrix* a, float lr, int refresh, cudaStrea
   StepCtx s;
   DION_TRY(begin_step(c, a, 1, st, &s));
   if (lazy_on_pairs(s, a)) return lazy_pairs(s, a, lr, refresh);
+  DION_TRY(clear_slots(s));
   const i64 m = a->m, n = a->n, r = a->r;
   const int gmode = (a->g_dtype == DION_BF16) ? ADD_BF16 : ADD_F32;
   float* P0 = s.ws + s.L.P0;
@@ -2649,9 +2656,9 @@ GemmArgs dp_b_product(const dion_matrix* a, bool transposed_b, const float* rhs,
 }
 
 // The pieces of a step on half pairs (step_on_half_pairs) as calls of their own.  P = (M + G) Q:
-int half_project(StepCtx& s, const dion_matrix* a, float* P) {
+int half_project(StepCtx& s, const dion_matrix* a, float* P, int* flag) {
   const i64 m = a->m, n = a->n, r = a->r;
-  DION_TRY(half_sum_chain(s, &a, n, false, true));
+  DION_TRY(half_sum_chain(s, &a, n, true, true, flag));
   const __half* bh = reinterpret_cast<const __half*>(s.ws + s.L.Bp);
   const __half* qh = reinterpret_cast<const __half*>(s.ws + s.L.S16);
   GemmArgs p = gemm_args();
@@ -2689,7 +2696,7 @@ int half_finish(StepCtx& s, const dion_matrix* a, const float* U, const float* W
   const i64 pieces = (((m > n) ? m : n) + RANGE_ROWS - 1) / RANGE_ROWS * ((r + 127) / 128);
   x.nrange = grid_for(c, 32 * pieces, 2);
   float* range = s.ws + s.L.part;
-  launch_pdl(k_range_partial, dim3((unsigned)x.nrange, 2), dim3(256), 0, s.st, t, r, n, m, r, range, (i64)2 * x.nrange, (const int*)nullptr, (i64)0);
+  launch_pdl(k_range_partial, dim3((unsigned)x.nrange, 2), dim3(256), 0, s.st, t, r, n, m, r, range, (i64)2 * x.nrange, (const int*)nullptr, (i64)0, s.os);
   DION_CHECK_LAUNCH(c);
   const i64 u_one = s.L.P0 + ((m > n) ? m : n) * r / 2;      // (behind Q's half array)
   x.kind = CN_HALF; x.qh = s.ws + s.L.P0; x.qscale = half_scale(n); x.hi = s.ws + s.L.S16; x.os = s.os; x.range = range;
@@ -2711,8 +2718,8 @@ int dion_dp_project(dion_ctx* ctx, const dion_matrix* a, float* P, int* dp_flag,
   StepCtx s;
   cudaStream_t st = (cudaStream_t)cuda_stream;
   DION_TRY(begin_step(ctx, a, 1, st, &s));
-  if (cudaMemsetAsync(dp_flag, 0, sizeof(int), st) != cudaSuccess) return DION_ERR_CUDA;
-  if (step_on_half_pairs(s, a->m, a->n, a->r, (a->m < a->n) ? a->m : a->n)) return half_project(s, a, P);
+  if (step_on_half_pairs(s, a->m, a->n, a->r, (a->m < a->n) ? a->m : a->n)) return half_project(s, a, P, dp_flag);
+  DION_TRY(clear_slots(s, dp_flag));
   GemmArgs p = dp_b_product(a, false, (const float*)a->Q, P);
   p.b_sk = a->ldq;
   p.precise = (resolve_orth(ctx, a->r, (a->m < a->n) ? a->m : a->n) == DION_ORTH_SHIFTED3) ? 1 : 0;
@@ -2728,14 +2735,14 @@ int dion_dp_factor(dion_ctx* ctx, const dion_matrix* a, float* PU, float* W, int
   const i64 m = a->m, n = a->n, r = a->r;
   dim3 grid((unsigned)grid_for(ctx, (m * r + 3) / 4), 1);
   const i64 pin_off = panel_offset(s, r, (m < n) ? m : n);
-  launch_pdl(k_copy_block, grid, dim3(256), 0, st, PU, r, s.ws + pin_off, r, m, r, nullptr, 0, (const int*)nullptr, (int*)nullptr);
+  launch_pdl(k_copy_block, grid, dim3(256), 0, st, PU, r, s.ws + pin_off, r, m, r, nullptr, 0, (const int*)nullptr, (int*)nullptr, s.os);
   DION_CHECK_LAUNCH(ctx);
   i64 U_off = 0;
   s.in_orth = true;
   const int rc = orthonormalize(s, m, r, (m < n) ? m : n, pin_off, &U_off);
   s.in_orth = false;
   DION_TRY(rc);
-  launch_pdl(k_copy_block, grid, dim3(256), 0, st, s.ws + U_off, r, PU, r, m, r, nullptr, 0, (const int*)s.flag, dp_flag);      // (a breakdown cancels dion_dp_finish)
+  launch_pdl(k_copy_block, grid, dim3(256), 0, st, s.ws + U_off, r, PU, r, m, r, nullptr, 0, (const int*)s.flag, dp_flag, (int*)nullptr);      // (a breakdown cancels dion_dp_finish)
   DION_CHECK_LAUNCH(ctx);
   if (step_on_half_pairs(s, m, n, r, (m < n) ? m : n)) return half_factor(s, a, PU, W, nullptr);
   if (r_on_pairs(s, m, n, r)) {       // as dion_step: W on the bf16 pairs of M + G and U
@@ -2756,6 +2763,7 @@ int dion_dp_finish(dion_ctx* ctx, const dion_matrix* a, const float* U, const fl
   if (step_on_half_pairs(s, m, n, r, (m < n) ? m : n)) {
     DION_TRY(half_finish(s, a, U, W, nullptr, alpha, dp_flag));
   } else {
+    DION_TRY(clear_slots(s));
     // M <- (M + G) - (1 - mu) U W^T, with this rank's M and G (as in dion_step)
     DION_TRY(ef_update(s, 0, a, U, r, W, r, s.ws + s.L.P1, s.ws + s.L.S16, nullptr, dp_flag));
     DION_TRY(colnorm(s, 0, W, n, r, (float*)a->Q, a->ldq, a->colnorm_out, dp_flag));
@@ -2785,8 +2793,8 @@ int dion_shard_project(dion_ctx* ctx, const dion_matrix* a, int64_t n_total, flo
   StepCtx s;
   cudaStream_t st = (cudaStream_t)cuda_stream;
   DION_TRY(begin_step(ctx, a, 1, st, &s));
-  if (cudaMemsetAsync(flag, 0, sizeof(int), st) != cudaSuccess) return DION_ERR_CUDA;
-  if (step_on_half_pairs(s, a->m, a->n, a->r, (a->m < n_total) ? a->m : n_total)) return half_project(s, a, P);
+  if (step_on_half_pairs(s, a->m, a->n, a->r, (a->m < n_total) ? a->m : n_total)) return half_project(s, a, P, flag);
+  DION_TRY(clear_slots(s, flag));
   GemmArgs p = dp_b_product(a, false, (const float*)a->Q, P);
   p.b_sk = a->ldq;
   p.precise = (resolve_orth(ctx, a->r, (a->m < n_total) ? a->m : n_total) == DION_ORTH_SHIFTED3) ? 1 : 0;
@@ -2809,14 +2817,14 @@ int dion_orthonormalize(dion_ctx* ctx, int64_t m, int64_t r, int64_t n_total, fl
   const i64 sd = (m < n_total) ? m : n_total;
   const i64 pin_off = panel_offset(s, r, sd);
   dim3 grid((unsigned)grid_for(ctx, (m * r + 3) / 4), 1);
-  launch_pdl(k_copy_block, grid, dim3(256), 0, st, (const float*)PU, r, s.ws + pin_off, r, m, r, nullptr, 0, (const int*)nullptr, (int*)nullptr);
+  launch_pdl(k_copy_block, grid, dim3(256), 0, st, (const float*)PU, r, s.ws + pin_off, r, m, r, nullptr, 0, (const int*)nullptr, (int*)nullptr, s.os);
   DION_CHECK_LAUNCH(ctx);
   i64 U_off = 0;
   s.in_orth = true;
   const int rc = orthonormalize(s, m, r, sd, pin_off, &U_off);
   s.in_orth = false;
   DION_TRY(rc);
-  launch_pdl(k_copy_block, grid, dim3(256), 0, st, (const float*)(s.ws + U_off), r, PU, r, m, r, nullptr, 0, (const int*)s.flag, flag);
+  launch_pdl(k_copy_block, grid, dim3(256), 0, st, (const float*)(s.ws + U_off), r, PU, r, m, r, nullptr, 0, (const int*)s.flag, flag, (int*)nullptr);
   DION_CHECK_LAUNCH(ctx);
   return DION_OK;
 }
@@ -2828,6 +2836,7 @@ int dion_shard_factor(dion_ctx* ctx, const dion_matrix* a, int64_t n_total, cons
   StepCtx s;
   cudaStream_t st = (cudaStream_t)cuda_stream;
   DION_TRY(begin_step(ctx, a, 1, st, &s));
+  DION_TRY(clear_slots(s));
   if (step_on_half_pairs(s, a->m, a->n, a->r, (a->m < n_total) ? a->m : n_total)) {
     DION_TRY(half_factor(s, a, U, W, flag));
   } else if (r_on_pairs(s, a->m, a->n, a->r)) {       // as dion_step: W on the bf16 pairs of M + G and U
@@ -2867,6 +2876,7 @@ int dion_shard_finish(dion_ctx* ctx, const dion_matrix* a, int64_t n_total, cons
   if (step_on_half_pairs(s, m, n, r, (m < n_total) ? m : n_total)) {
     DION_TRY(half_finish(s, a, U, W, colsumsq, alpha, flag));
   } else {
+    DION_TRY(clear_slots(s));
     // M <- (M + G) - (1 - mu) U W^T on the shard's columns; Q <- W / (sqrt(colsumsq) + eps) with the all-reduced squared norms
     DION_TRY(ef_update(s, 0, a, U, r, W, r, s.ws + s.L.P1, s.ws + s.L.S16, nullptr, flag));
     DION_TRY(colnorm(s, 0, W, n, r, (float*)a->Q, a->ldq, a->colnorm_out, flag, ColnormPairs(), colsumsq));

@@ -1089,8 +1089,9 @@ __device__ __forceinline__ void copy_rows(const float* __restrict__ src, i64 lds
 // breakdown carried from one call of a multi-call step to the next).
 __global__ void k_copy_block(const float* __restrict__ src, i64 lds, float* __restrict__ dst, i64 ldd,
                              i64 rows, i64 cols, const int* __restrict__ skip_flag, i64 wstride,
-                             const int* __restrict__ latch_from, int* __restrict__ latch_to) {
+                             const int* __restrict__ latch_from, int* __restrict__ latch_to, int* __restrict__ slots) {
   pdl_enter();
+  clear_slot(slots);
   if (latch_to != nullptr && blockIdx.x == 0 && threadIdx.x == 0 && *latch_from != 0) *latch_to = 1;
   if (skip_flag != nullptr && skip_flag[(i64)blockIdx.y * OS_SLOT_INTS] != 0) return;
   copy_rows(src + (i64)blockIdx.y * wstride, lds, dst + (i64)blockIdx.y * wstride, ldd, rows, cols);     // batched over blockIdx.y
