@@ -962,6 +962,14 @@ __global__ void __launch_bounds__(256) k_cgs_fallback(const float* __restrict__ 
   const i64 rpc = (rows + G - 1) / G;
   const i64 i0 = min(rows, (i64)c * rpc), i1 = min(rows, i0 + rpc);
   const int nmy = (int)(i1 - i0);
+  {      // nearly always there is nothing to do: all flags at once (one after another 48 matrices were 14 us of a step; twelve blocks of hidden size 768 in one call: 1606 -> 1588 us)
+    bool busy = false;
+    for (int b = tid; b < nb; b += 256) {
+      const int* os = os_base + (i64)b * OS_SLOT_INTS;
+      busy = busy || os[OS_FAIL] != 0 || (second != nullptr && os[OS_DONE] == 0);
+    }
+    if (!__syncthreads_or(busy)) return;
+  }
   for (int b = 0; b < nb; ++b) {
     int* os = os_base + (i64)b * OS_SLOT_INTS;
     if (os[OS_FAIL] == 0) {                         // written by an earlier launch: every CTA reads the same value
