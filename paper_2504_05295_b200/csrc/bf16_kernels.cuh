@@ -178,10 +178,10 @@ __global__ void __launch_bounds__(256) k_to_bf16(const float* __restrict__ src, 
 
 // hi = bf16(src), lo = bf16(src - hi): src ~ hi + lo to 16 significant bits.  rows x cols (cols a multiple of 8,
 // src rows 16-byte aligned), hi and lo dense.  skip_flag (optional): nothing is written when *skip_flag != 0.
-// copy (optional): src also as a dense fp32 array
+// copy (optional): src also as a dense fp32 array; one (optional): half(one_scale src), dense (k_round_f16's values)
 __device__ __forceinline__ void split_bf16_body(const float* __restrict__ src, i64 lds, i64 rows, i64 cols,
                                                 __nv_bfloat16* __restrict__ hi, __nv_bfloat16* __restrict__ lo,
-                                                float* __restrict__ copy = nullptr) {
+                                                float* __restrict__ copy, __half* __restrict__ one, float one_scale) {
   const i64 per_row = cols / 8;
   const i64 total = rows * per_row;
   for (i64 e = (i64)blockIdx.x * blockDim.x + threadIdx.x; e < total; e += (i64)gridDim.x * blockDim.x) {
@@ -204,26 +204,32 @@ __device__ __forceinline__ void split_bf16_body(const float* __restrict__ src, i
       *reinterpret_cast<float4*>(copy + i * cols + c) = a;
       *(reinterpret_cast<float4*>(copy + i * cols + c) + 1) = b;
     }
+    if (one != nullptr) {
+      __half t[8];
+#pragma unroll
+      for (int q = 0; q < 8; ++q) t[q] = __float2half_rn(one_scale * v[q]);
+      *reinterpret_cast<uint4*>(one + i * cols + c) = *reinterpret_cast<const uint4*>(t);
+    }
   }
 }
 __global__ void __launch_bounds__(256) k_split_bf16(const float* __restrict__ src, i64 lds, i64 rows, i64 cols,
                                                     __nv_bfloat16* __restrict__ hi, __nv_bfloat16* __restrict__ lo,
-                                                    const int* __restrict__ skip_flag) {
+                                                    const int* __restrict__ skip_flag, __half* __restrict__ one, float one_scale) {
   pdl_enter();
   if (skip_flag != nullptr && *skip_flag != 0) return;
-  split_bf16_body(src, lds, rows, cols, hi, lo);
+  split_bf16_body(src, lds, rows, cols, hi, lo, nullptr, one, one_scale);
 }
 // One launch over the matrices of a chain (blockIdx.y): sources from a pointer table, outputs `ostride` floats
 // apart in the scratch slices, skip flags `skip_stride` ints apart.
 __global__ void __launch_bounds__(256) k_split_bf16_chain(const ChainPtrs srcs, i64 lds, i64 rows, i64 cols,
                                                           __nv_bfloat16* __restrict__ hi, __nv_bfloat16* __restrict__ lo,
                                                           i64 ostride, const int* __restrict__ skip_flag, i64 skip_stride,
-                                                          float* __restrict__ copy) {
+                                                          float* __restrict__ copy, __half* __restrict__ one, float one_scale) {
   pdl_enter();
   const i64 b = blockIdx.y;
   if (skip_flag != nullptr && skip_flag[b * skip_stride] != 0) return;
   split_bf16_body(reinterpret_cast<const float*>(srcs.p[b]), lds, rows, cols, hi + 2 * b * ostride, lo + 2 * b * ostride,
-                  copy != nullptr ? copy + b * ostride : nullptr);
+                  copy != nullptr ? copy + b * ostride : nullptr, one != nullptr ? one + 2 * b * ostride : nullptr, one_scale);
 }
 
 // Dense fp32 copies of a chain's matrices (blockIdx.y; sources from a pointer table, 16-byte aligned rows, cols a multiple

@@ -1376,8 +1376,9 @@ int colnorm_chain(StepCtx& s, const dion_matrix* const* list, i64 rows, i64 r, i
 // hi / lo bf16 pair of src[b] (rows x cols, leading dimension ld[b]) into the scratch slices at out_off.
 // skip0: the flag of matrix 0 (a state slot apart per matrix), or nullptr.
 // copy_off >= 0 (chain launch only): a dense fp32 copy of the sources in the scratch slices too; *copied says whether it was made.
+// one_off >= 0: half(one_scale src) too.
 int split_chain(StepCtx& s, const float* const* src, const i64* ld, i64 rows, i64 cols, i64 out_off, const int* skip0,
-                i64 copy_off = -1, bool* copied = nullptr) {
+                i64 copy_off = -1, bool* copied = nullptr, i64 one_off = -1, float one_scale = 0.f) {
   dion_ctx* c = s.c;
   bool one = s.nb > 1 && s.nb <= GEMM_TAB_MAX && c->chain_batch;
   for (int b = 1; b < s.nb && one; ++b) one = ld[b] == ld[0];
@@ -1387,7 +1388,8 @@ int split_chain(StepCtx& s, const float* const* src, const i64* ld, i64 rows, i6
     for (int b = 0; b < s.nb; ++b) t.p[b] = src[b];
     __nv_bfloat16* hi = reinterpret_cast<__nv_bfloat16*>(s.ws + out_off);
     launch_pdl(k_split_bf16_chain, dim3(gx, (unsigned)s.nb), dim3(256), 0, s.st, t, ld[0], rows, cols, hi, hi + rows * cols, s.wstride, skip0,
-               (i64)OS_SLOT_INTS, copy_off >= 0 ? s.ws + copy_off : (float*)nullptr);
+               (i64)OS_SLOT_INTS, copy_off >= 0 ? s.ws + copy_off : (float*)nullptr,
+               one_off >= 0 ? reinterpret_cast<__half*>(s.ws + one_off) : (__half*)nullptr, one_scale);
     DION_CHECK_LAUNCH(c);
     if (copied != nullptr) *copied = copy_off >= 0;
     return DION_OK;
@@ -1396,7 +1398,8 @@ int split_chain(StepCtx& s, const float* const* src, const i64* ld, i64 rows, i6
   for (int b = 0; b < s.nb; ++b) {
     __nv_bfloat16* hi = reinterpret_cast<__nv_bfloat16*>(s.W(b, out_off));
     launch_pdl(k_split_bf16, dim3(gx), dim3(256), 0, s.st, src[b], ld[b], rows, cols, hi, hi + rows * cols,
-               skip0 != nullptr ? skip0 + (i64)b * OS_SLOT_INTS : (const int*)nullptr);
+               skip0 != nullptr ? skip0 + (i64)b * OS_SLOT_INTS : (const int*)nullptr,
+               one_off >= 0 ? reinterpret_cast<__half*>(s.W(b, one_off)) : (__half*)nullptr, one_scale);
     DION_CHECK_LAUNCH(c);
   }
   return DION_OK;
@@ -1646,7 +1649,7 @@ int r_pairs(StepCtx& s, int b, const dion_matrix* a, bool tr, const float* U, fl
   __nv_bfloat16* uh = reinterpret_cast<__nv_bfloat16*>(upair);
   __nv_bfloat16* ul = uh + prow * r;
   if (!split_done) {      // (the step splits U for the whole chain beforehand)
-    launch_pdl(k_split_bf16, dim3((unsigned)grid_for(c, prow * r / 8)), dim3(256), 0, s.st, U, r, prow, r, uh, ul, skip);
+    launch_pdl(k_split_bf16, dim3((unsigned)grid_for(c, prow * r / 8)), dim3(256), 0, s.st, U, r, prow, r, uh, ul, skip, (__half*)nullptr, 0.f);
     DION_CHECK_LAUNCH(c);
   }
   __nv_bfloat16* bh = reinterpret_cast<__nv_bfloat16*>(s.W(b, s.L.Bp));
@@ -1709,11 +1712,11 @@ int ef_update(StepCtx& s, int b, const dion_matrix* a, const float* F1, i64 ld1,
     __nv_bfloat16* h2 = reinterpret_cast<__nv_bfloat16*>(p2);
     __nv_bfloat16* l2 = h2 + n * r;
     if (!ready1) {
-      launch_pdl(k_split_bf16, dim3((unsigned)grid_for(c, m * r / 8)), dim3(256), 0, s.st, F1, ld1, m, r, h1, l1, skip);
+      launch_pdl(k_split_bf16, dim3((unsigned)grid_for(c, m * r / 8)), dim3(256), 0, s.st, F1, ld1, m, r, h1, l1, skip, (__half*)nullptr, 0.f);
       DION_CHECK_LAUNCH(c);
     }
     if (!ready2) {
-      launch_pdl(k_split_bf16, dim3((unsigned)grid_for(c, n * r / 8)), dim3(256), 0, s.st, F2, ld2, n, r, h2, l2, skip);
+      launch_pdl(k_split_bf16, dim3((unsigned)grid_for(c, n * r / 8)), dim3(256), 0, s.st, F2, ld2, n, r, h2, l2, skip, (__half*)nullptr, 0.f);
       DION_CHECK_LAUNCH(c);
     }
     e.ab16 = 1;
@@ -1919,7 +1922,7 @@ int step_batch(dion_ctx* c, const dion_matrix* const* list, int nb, float lr, cu
       __nv_bfloat16* ql = qh + qrow * r;
       if (!q_split) {
         launch_pdl(k_split_bf16, dim3((unsigned)grid_for(c, qrow * r / 8)), dim3(256), 0, st, (const float*)a->Q, a->ldq, qrow, r, qh, ql,
-                   (const int*)nullptr);
+                   (const int*)nullptr, (__half*)nullptr, 0.f);
         DION_CHECK_LAUNCH(c);
       }
       __nv_bfloat16* bh = reinterpret_cast<__nv_bfloat16*>(s.W(b, s.L.Bp));
@@ -1968,8 +1971,10 @@ int step_batch(dion_ctx* c, const dion_matrix* const* list, int nb, float lr, cu
 
   // U = Orthonormalize(P)
   i64 U_off = 0;
-  // (steps on half pairs: U as a half array for the weight update, behind Q's in the panel's save buffer, free by then)
+  // (U as a half array for the weight update, made beside U's pair: behind Q's in the panel's save buffer, free by then;
+  // a rounding of its own read U again: 4096 x 4096, r = 1024, 619 -> 616 us)
   const i64 u_one = s.L.Psave + ((m > n) ? m : n) * r / 2;
+  bool u_one_made = hstep;
   {
   PhaseScope ps(c, st, DION_PHASE_ORTH);
   const std::function<int()> redo = [&]() -> int {
@@ -2004,7 +2009,14 @@ int step_batch(dion_ctx* c, const dion_matrix* const* list, int nb, float lr, cu
     i64 lds[MAX_CHAIN];
     for (int b = 0; b < nb; ++b) { srcs[b] = s.W(b, U_off); lds[b] = r; }
     if (hstep) DION_TRY(split_half_chain(s, srcs, r, prow, r, other_off, HS_U_BITS, s.os + OS_FAIL, u_one));
-    else DION_TRY(split_chain(s, srcs, lds, prow, r, other_off, s.os + OS_FAIL));
+    else {
+      u_one_made = s.L.Psave > 0 && x_half(a0);
+      for (int b = 0; b < nb; ++b) {
+        const float *Uf = srcs[b], *Qf = (const float*)list[b]->Q;
+        u_one_made = u_one_made && (tr ? x_single_pass(s, list[b], Qf, list[b]->ldq, Uf, r) : x_single_pass(s, list[b], Uf, r, Qf, list[b]->ldq));
+      }
+      DION_TRY(split_chain(s, srcs, lds, prow, r, other_off, s.os + OS_FAIL, -1, nullptr, u_one_made ? u_one : -1, half_scale(prow)));
+    }
   }
   for (int b = 0; b < nb; ++b) {
     const dion_matrix* a = list[b];
@@ -2128,7 +2140,7 @@ int step_batch(dion_ctx* c, const dion_matrix* const* list, int nb, float lr, cu
     if (all_one) {
       for (int b = 0; b < nb; ++b) { srcs[b] = s.W(b, U_off); lds[b] = r; }
       const bool half = x_half(a0);
-      if (hstep && half) u_half = ldexpf(1.f, HS_U_BITS);      // (made beside U's pair)
+      if (u_one_made && half) u_half = hstep ? ldexpf(1.f, HS_U_BITS) : half_scale(prow);      // (made beside U's pair)
       else DION_TRY(round_chain(s, srcs, lds, prow, r, other_off, s.os + OS_FAIL, half ? half_scale(prow) : 0.f));
       if (cn_kind == 0) {
         for (int b = 0; b < nb; ++b) { srcs[b] = (const float*)list[b]->Q; lds[b] = list[b]->ldq; }
