@@ -420,6 +420,22 @@ int launch_gemm_simt(dion_ctx* c, GemmArgs g, cudaStream_t st, float* part, i64 
   return DION_OK;
 }
 
+// Two updates of C of one shape (no split, no batch) in one launch: each as launch_gemm_simt computes it.
+int launch_gemm_simt_two(dion_ctx* c, const GemmArgs& a, const GemmArgs& b, cudaStream_t st) {
+  const i64 t128 = ((a.M + 127) / 128) * ((a.N + 127) / 128);
+  const bool thin = a.N <= SIMT_THIN_N, use128 = !thin && t128 >= c->sm_count && a.K >= SIMT_WIDE_MIN_K;
+  const i64 bm = (use128 || thin) ? 128 : 64, bn = use128 ? 128 : thin ? 32 : 64;
+  const i64 gm = (a.M + bm - 1) / bm, gn = (a.N + bn - 1) / bn;
+  if (gm > 65535) return DION_ERR_UNSUPPORTED;
+  const dim3 grid((unsigned)gn, (unsigned)gm, 2);
+  const GemmSecond second = {b};
+  if (use128) launch_pdl(k_gemm_simt<128, 128, 8, 8, 8, 1, GemmSecond>, grid, dim3(256), 0, st, a, second, 1);
+  else if (thin) launch_pdl(k_gemm_simt<128, 32, 16, 4, 4, 2, GemmSecond>, grid, dim3(256), 0, st, a, second, 1);
+  else launch_pdl(k_gemm_simt<64, 64, 16, 4, 4, 2, GemmSecond>, grid, dim3(256), 0, st, a, second, 1);
+  DION_CHECK_LAUNCH(c);
+  return DION_OK;
+}
+
 cudaEvent_t prof_event(dion_ctx* c) {
   if (c->prof_used == c->prof_pool.size()) {
     cudaEvent_t e = nullptr;
@@ -2069,6 +2085,13 @@ int step_batch(dion_ctx* c, const dion_matrix* const* list, int nb, float lr, cu
   DION_TRY(colnorm_chain(s, list, qrow, r, cn_kind, cn_kind == CN_ONE ? s.L.Q16 : s.L.Psave, half_scale(qrow), cn_kind == CN_ONE ? s.L.R16 : s.L.S16));
   }
 
+  // On the FMA engine the two rank-r updates, which share nothing that either writes, are one launch (small or ragged matrices:
+  // each is a few tens of blocks; 1001 x 333, r = 83: 8 + 11 us one after the other; the step 129.7 -> 119.1 us).
+  auto on_simt = [&](const GemmArgs& g) {
+    return c->cfg.engine != DION_ENGINE_TENSOR && !g.ab16 && !g.tf32x1 && !(s.tensor && umma_shape_ok(g, c->cfg.precision));
+  };
+  bool two = false;
+  GemmArgs ef_args;
   // Under graph capture (small matrices: a few CTAs each) the two rank-r updates, which share nothing that either writes, are two
   // branches of the graph -- where the update of X has nothing left to prepare (its rounded factors would go where the error
   // feedback's lie).  256 x 512, r = 64, replayed: 77.8 -> 72.4 us.
@@ -2129,7 +2152,9 @@ int step_batch(dion_ctx* c, const dion_matrix* const* list, int nb, float lr, cu
     else DION_TRY(ef_update(s, b, a, Uf, r, Rf, r, other, sbuf, sum32, s.OS(b) + OS_FAIL, bpair || ef_split, ef_split, &group[b]));
     if (hstep && group[b].ab16) { group[b].f16 = 1; group[b].wide_flag = s.OS(b) + OS_WIDE; group[b].alpha_dev = s.W(b, s.L.lz) + HS_EF; }
   }
-  DION_TRY(launch_gemm_group(s, group));
+  two = nb == 1 && !c->prof_on && on_simt(group[0]);
+  if (two) ef_args = group[0];
+  else DION_TRY(launch_gemm_group(s, group));
   }
 
   // X <- X - lr sqrt(m/n) U Q^T   (transposed form: Q U^T)
@@ -2183,7 +2208,11 @@ int step_batch(dion_ctx* c, const dion_matrix* const* list, int nb, float lr, cu
     if (tr) DION_TRY(x_update(s, b, a, Qf, a->ldq, Uf, r, rbuf, other, x_alpha, s.OS(b) + OS_FAIL, x_scale, &group[b], x_rounded, 0.f, u_half));
     else DION_TRY(x_update(s, b, a, Uf, r, Qf, a->ldq, other, rbuf, x_alpha, s.OS(b) + OS_FAIL, x_scale, &group[b], x_rounded, u_half, 0.f));
   }
-  DION_TRY(launch_gemm_group(s, group));
+  if (two && on_simt(group[0])) DION_TRY(launch_gemm_simt_two(c, ef_args, group[0], s.st));
+  else {
+    if (two) DION_TRY(launch_gemm(s, ef_args, 0));
+    DION_TRY(launch_gemm_group(s, group));
+  }
   s.st = st;
   if (fork) DION_TRY(order(c->side, st));
   }

@@ -15,10 +15,16 @@ namespace dion {
 // their sums as k_splitk_reduce would.
 struct GemmTabs { const void *A[GEMM_TAB_MAX], *A2[GEMM_TAB_MAX], *B[GEMM_TAB_MAX], *C[GEMM_TAB_MAX], *C2[GEMM_TAB_MAX]; };
 struct NoTabs {};
+// Two products of the same shape that write different arrays: blockIdx.z tells them apart (no splits, no batch).
+struct GemmSecond { GemmArgs g; };
 
 template <int BM, int BN, int BK, int TM, int TN, int MINB, typename TABS>
-__global__ void __launch_bounds__(256, MINB) k_gemm_simt(const __grid_constant__ GemmArgs g, const __grid_constant__ TABS tabs, int inner) {
+__global__ void __launch_bounds__(256, MINB) k_gemm_simt(const __grid_constant__ GemmArgs first, const __grid_constant__ TABS tabs, int inner) {
   pdl_enter();
+  constexpr bool TWO = std::is_same<TABS, GemmSecond>::value;
+  const GemmArgs* args = &first;
+  if constexpr (TWO) { if (blockIdx.z != 0) args = &tabs.g; }
+  const GemmArgs& g = *args;
   static_assert((BM / TM) * (BN / TN) == 256, "256 threads per tile");
   static_assert(TM % 4 == 0 && TN % 4 == 0, "micro tile in groups of 4");
   // blockIdx.z = inner batch index + batch * outer batch index (or the K split)
@@ -26,8 +32,8 @@ __global__ void __launch_bounds__(256, MINB) k_gemm_simt(const __grid_constant__
   int split = 0;
   constexpr bool TAB = std::is_same<TABS, GemmTabs>::value;
   if (TAB) { outer = blockIdx.z / g.splits; split = blockIdx.z % g.splits; }      // (splits: those of the grid)
-  else if (g.splits > 1) split = blockIdx.z;
-  else { batch = blockIdx.z % g.batch; outer = blockIdx.z / g.batch; }
+  else if (!TWO && g.splits > 1) split = blockIdx.z;
+  else if (!TWO) { batch = blockIdx.z % g.batch; outer = blockIdx.z / g.batch; }
   if (g.skip_flag != nullptr && g.skip_flag[outer * g.skip_stride] != 0) return;
 
   constexpr int LDA_S = BM + 4, LDB_S = BN + 4;
@@ -229,8 +235,8 @@ __global__ void __launch_bounds__(256, MINB) k_gemm_simt(const __grid_constant__
 #pragma unroll
         for (int q = 0; q < BATCH; ++q) {
           if (q * RSTEP >= left) break;
-          const float v = scale * T[tr + (q0 + q) * RSTEP][tc];
-          C[(r0 + q * RSTEP) * ldc + gj] = epi == EPI_STORE ? v : (with_c ? c[q] + t[q] : t[q]) - v;
+          const float v = T[tr + (q0 + q) * RSTEP][tc];      // (an explicit FMA: the same bits from every instance of this kernel)
+          C[(r0 + q * RSTEP) * ldc + gj] = epi == EPI_STORE ? scale * v : fmaf(-scale, v, with_c ? c[q] + t[q] : t[q]);
         }
       }
     }
