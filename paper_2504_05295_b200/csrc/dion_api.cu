@@ -3081,7 +3081,8 @@ bool touch_kernel(K kernel) {
 bool preload_kernels() {
   bool ok = true;
   ok = ok && touch_kernel(k_gemm_simt<128, 128, 8, 8, 8, 1, NoTabs>) && touch_kernel(k_gemm_simt<64, 64, 16, 4, 4, 2, NoTabs>) &&
-       touch_kernel(k_gemm_simt<128, 32, 16, 4, 4, 2, NoTabs>);
+       touch_kernel(k_gemm_simt<128, 32, 16, 4, 4, 2, NoTabs>) && touch_kernel(k_gemm_simt<128, 128, 8, 8, 8, 1, GemmSecond>) &&
+       touch_kernel(k_gemm_simt<64, 64, 16, 4, 4, 2, GemmSecond>) && touch_kernel(k_gemm_simt<128, 32, 16, 4, 4, 2, GemmSecond>);
   ok = ok && touch_kernel(k_splitk_reduce) && touch_kernel(k_round_begin) && touch_kernel(k_chol_flow<true>);
   ok = ok && touch_kernel(k_chol_flow<false>) && touch_kernel(k_round_end) && touch_kernel(k_tiny_cholqr2);
   ok = ok && touch_kernel(k_probe_fused) && touch_kernel(k_probe_y) && touch_kernel(k_probe_y4) && touch_kernel(k_probe_w) && touch_kernel(k_probe_w4) && touch_kernel(k_probe_decide) && touch_kernel(k_reset_rounds);

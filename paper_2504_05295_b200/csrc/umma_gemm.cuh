@@ -580,11 +580,15 @@ struct Cfg {
                                         : (((BF16 && !X2) || ONE) ? 1 : 2) * (A_BYTES + B_BYTES);
   // D16: the producer warps have no conversion work and serve as epilogue warps too
   // (with operand pairs the stages leave room for 8 warps' epilogue tiles only)
-  static constexpr int EPI_WARPS = (((D16 && !X2) || ONE) && !TE) ? NUM_EPI_WARPS + NUM_PROD_WARPS : NUM_EPI_WARPS;
+  // LEAN (ONE with 16-bit arrays): plain stores of single 16-bit arrays.  Such a product reads its operands once, mostly from DRAM,
+  // and has one MMA per K step to hide that: the room of eight warps' epilogue tiles goes to operand stages (four -> six).
+  // 16-bit momentum and gradient, 8192 x 8192, r = 512: the step 688 -> 669 us.
+  static constexpr bool LEAN = D16 && ONE;
+  static constexpr int EPI_WARPS = (((D16 && !X2) || ONE) && !TE && !LEAN) ? NUM_EPI_WARPS + NUM_PROD_WARPS : NUM_EPI_WARPS;
   // Operand pairs: nothing to convert and no room for more epilogue tiles, so the kernel runs without the producer
   // warps (10 warps in all); the registers they would hold go to the epilogue warps' loads in flight (DEEP).
-  static constexpr bool DEEP = X2;
-  static constexpr int MMA_WARP = (X2 || TE) ? NUM_EPI_WARPS : NUM_EPI_WARPS + NUM_PROD_WARPS;   // the warp that issues the MMAs
+  static constexpr bool DEEP = X2 || LEAN;
+  static constexpr int MMA_WARP = (X2 || TE || LEAN) ? NUM_EPI_WARPS : NUM_EPI_WARPS + NUM_PROD_WARPS;   // the warp that issues the MMAs
   static constexpr int THREADS = (MMA_WARP + (TMA ? 2 : 1)) * 32;                         // ... then the TMA warp
   // CE (coalesced epilogue): an epilogue warp owns 32 rows x EPI_W columns of the tile and passes them
   // through a private shared-memory tile in passes of EPI_RPP rows (EPI_RPP * EPI_W = 1024 elements),
@@ -636,7 +640,8 @@ k_gemm_umma(const __grid_constant__ PT p) {
   static_assert(!(BF16 && SPLIT) || X2, "split accumulators belong to the 3xTF32 mode and to operand pairs");
   static_assert(!D16 || (BF16 && TMA), "bf16 operands in memory are loaded by TMA");
   static_assert(!CE || (TMA && (D16 || !BF16)), "the coalesced epilogue serves the bf16-array and the fp32 TMA variants");
-  static_assert(!ONE || (TMA && CE && !BF16 && !SPLIT && !A_MN && !B_MN), "single pass: k-contiguous fp32 operands by TMA");
+  static_assert(!ONE || D16 || (TMA && CE && !BF16 && !SPLIT && !A_MN && !B_MN), "single pass: k-contiguous fp32 operands by TMA");
+  static_assert(!ONE || !D16 || (CE && CG2 && !X2 && !SPLIT && !TE), "lean: single 16-bit arrays on CTA pairs");
   using C = Cfg<BN, BF16, SPLIT, TMA, D16, CE, ONE, CG2, X2, TE>;
   constexpr bool NOCONV = D16 || ONE;    // the operand tiles are what TMA writes: nothing to convert
   constexpr bool PAIRLOAD = CG2 && NOCONV;   // both CTAs' loads complete on the leader's barrier
@@ -846,8 +851,8 @@ k_gemm_umma(const __grid_constant__ PT p) {
       const i64 n0 = (i64)it.ni * BN;
       // (a device scalar: the learning rate under graph replay, or a matrix's own scale)
       const float alpha = g.alpha * (g.alpha_dev != nullptr ? __ldg(g.alpha_dev + (i64)it.b * g.alpha_dev_stride) : 1.f);
-      if constexpr (X2 && !SPLIT && CE) {
-        // Plain stores of operand pairs: the chunks of a tile are summed in registers (these variants run without the
+      if constexpr ((X2 || C::LEAN) && !SPLIT && CE) {
+        // Plain stores of operand pairs (and of the lean variant): the chunks of a tile are summed in registers (these variants run without the
         // producer warps, so a lane has room for its row of W columns) and the tile is written once.
         if (g.epi == EPI_STORE) {
           constexpr int W = C::EPI_W, RPP = C::EPI_RPP, LPR = W / 4, RPI = 32 / LPR, TS = W + 4;
@@ -1349,7 +1354,7 @@ k_gemm_umma(const __grid_constant__ PT p) {
             if (++stage == STAGES) { stage = 0; phase ^= 1u; }
             continue;
           }
-          if (ONE) {   // raw fp32 tiles, [rows][32 k] boxes
+          if (ONE && !D16) {   // raw fp32 tiles, [rows][32 k] boxes
             expect((uint32_t)(C::A_BYTES + C::B_BYTES));
             ld3(sa, &p.tmA, k0, row0a, it.b);
             ld3(sb, &p.tmB, k0, row0b, it.b);
@@ -1615,6 +1620,20 @@ inline cudaError_t launch_d16_pair_one(const Params& p, int grid, cudaStream_t s
   attr[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr; cfg.numAttrs = 2;
   return cudaLaunchKernelEx(&cfg, k_gemm_umma<256, A_MN, B_MN, true, false, true, true, true, false, true, false>, p);
+}
+// ... lean (plain stores, B row-index contiguous: P and R)
+template <bool A_MN>
+inline cudaError_t launch_lean_pair(const Params& p, int grid, cudaStream_t st) {
+  using CF = Cfg<256, true, false, true, true, true, true, true, false>;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)grid); cfg.blockDim = dim3(CF::THREADS); cfg.dynamicSmemBytes = CF::SMEM_BYTES; cfg.stream = st;
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = 2; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
+  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[1].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr; cfg.numAttrs = 2;
+  return cudaLaunchKernelEx(&cfg, k_gemm_umma<256, A_MN, true, true, false, true, true, true, true, true, false>, p);
 }
 inline cudaError_t launch_d16_pair(const Params& p, bool a_mn, bool b_mn, int grid, cudaStream_t st) {
   if (!a_mn && !b_mn) return launch_d16_pair_one<false, false>(p, grid, st);
@@ -1884,6 +1903,8 @@ int umma_configure() {
   if (e == cudaSuccess) e = set_d16_pair_attr<false, true>();
   if (e == cudaSuccess) e = set_d16_pair_attr<true, true>();
   if (e == cudaSuccess) e = set_d16_pair_attr<true, false>();
+  if (e == cudaSuccess) e = set_smem_attr<256, false, true, true, false, true, true, true, true, true, false>();
+  if (e == cudaSuccess) e = set_smem_attr<256, true, true, true, false, true, true, true, true, true, false>();
   if (e == cudaSuccess) {      // (no attribute to set, but asking loads it: this unit's copy is the one the products launch)
     cudaFuncAttributes fa;
     e = cudaFuncGetAttributes(&fa, k_splitk_reduce);
@@ -2096,6 +2117,9 @@ int umma_try_launch(const GemmArgs& g_in, int precision, int sm_count, float* pa
     }
   } else if (cg2 && x2) {
     if (launch_x2_pair(p, a_mn, b_mn, grid, st) != cudaSuccess) { cudaGetLastError(); return DION_ERR_CUDA; }
+  } else if (cg2 && d16 && b_mn && g.epi == EPI_STORE) {
+    const cudaError_t e = a_mn ? launch_lean_pair<true>(p, grid, st) : launch_lean_pair<false>(p, grid, st);
+    if (e != cudaSuccess) { cudaGetLastError(); return DION_ERR_CUDA; }
   } else if (cg2 && d16) {
     if (launch_d16_pair(p, a_mn, b_mn, grid, st) != cudaSuccess) { cudaGetLastError(); return DION_ERR_CUDA; }
   } else if (cg2) {
