@@ -627,7 +627,8 @@ int launch_gemm_group(StepCtx& s, const std::vector<GemmArgs>& v) {
 int configure_kernels() {
   if (umma_configure() != DION_OK) return DION_ERR_CUDA;
   if (cudaFuncSetAttribute(k_probe_y4, cudaFuncAttributeMaxDynamicSharedMemorySize, PY_SMEM) != cudaSuccess ||
-      cudaFuncSetAttribute(k_probe_fused, cudaFuncAttributeMaxDynamicSharedMemorySize, PF_SMEM_MAX) != cudaSuccess ||
+      cudaFuncSetAttribute(k_probe_fused<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, PF_SMEM_MAX) != cudaSuccess ||
+      cudaFuncSetAttribute(k_probe_fused<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, PF_SMEM_MAX) != cudaSuccess ||
       cudaFuncSetAttribute(k_chol_flow<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, FLOW_SMEM) != cudaSuccess ||
       cudaFuncSetAttribute(k_chol_flow<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, FLOW_SMEM) != cudaSuccess ||
       cudaFuncSetAttribute(k_tiny_cholqr2, cudaFuncAttributeMaxDynamicSharedMemorySize, tiny_cholqr2_smem(TINY_MAX_ROWS)) != cudaSuccess) {
@@ -823,11 +824,14 @@ int probe(StepCtx& s, i64 off, i64 rows, i64 r, int phase) {
   probe_chunks(s.L, rows, &chunks, &per);
   const int* keep = (phase == PROBE_AFTER_REDO) ? (const int*)(s.os + OS_DONE) : nullptr;
   const float* U = s.ws + off;
-  if (r % 4 == 0 && r <= PF_MAX_R) {
+  if (r <= PF_MAX_R) {
     int ct_log = 3;                         // threads by columns: 8 .. 256
     while (4 << ct_log < r) ++ct_log;
     const size_t smem = (size_t)(((r + 127) / 128 * 128) * NPROBE + PF_RED + 32 * NPROBE) * sizeof(float);
-    launch_pdl(k_probe_fused, dim3((unsigned)chunks, (unsigned)s.nb), dim3(256), smem, s.st, U, r, rows, r, per, s.ws + s.L.probe_part, s.wstride, keep, ct_log);
+    auto go = [&](auto kernel) {
+      launch_pdl(kernel, dim3((unsigned)chunks, (unsigned)s.nb), dim3(256), smem, s.st, U, r, rows, r, per, s.ws + s.L.probe_part, s.wstride, keep, ct_log);
+    };
+    if (r % 4 == 0) go(k_probe_fused<true>); else go(k_probe_fused<false>);
   } else {
     if (r % 4 == 0) {
       i64 blocks = (rows + 31) / 32;          // a block of 8 warps takes 32 rows at a time
@@ -3085,7 +3089,7 @@ bool preload_kernels() {
        touch_kernel(k_gemm_simt<64, 64, 16, 4, 4, 2, GemmSecond>) && touch_kernel(k_gemm_simt<128, 32, 16, 4, 4, 2, GemmSecond>);
   ok = ok && touch_kernel(k_splitk_reduce) && touch_kernel(k_round_begin) && touch_kernel(k_chol_flow<true>);
   ok = ok && touch_kernel(k_chol_flow<false>) && touch_kernel(k_round_end) && touch_kernel(k_tiny_cholqr2);
-  ok = ok && touch_kernel(k_probe_fused) && touch_kernel(k_probe_y) && touch_kernel(k_probe_y4) && touch_kernel(k_probe_w) && touch_kernel(k_probe_w4) && touch_kernel(k_probe_decide) && touch_kernel(k_reset_rounds);
+  ok = ok && touch_kernel(k_probe_fused<true>) && touch_kernel(k_probe_fused<false>) && touch_kernel(k_probe_y) && touch_kernel(k_probe_y4) && touch_kernel(k_probe_w) && touch_kernel(k_probe_w4) && touch_kernel(k_probe_decide) && touch_kernel(k_reset_rounds);
   ok = ok && touch_kernel(k_orth_finish) && touch_kernel(k_cgs_fallback) && touch_kernel(k_copy_block);
   ok = ok && touch_kernel(k_colsumsq_partial<true>) && touch_kernel(k_colsumsq_partial<false>) &&
        touch_kernel(k_colnorm_apply<true, false>) && touch_kernel(k_colnorm_apply<false, false>) && touch_kernel(k_copy_panel);

@@ -675,13 +675,15 @@ __global__ void __launch_bounds__(128) k_probe_w4(const float* __restrict__ U, i
   }
 }
 
-// Both passes in one launch for r a multiple of 4 up to PF_MAX_R: a block takes 32 rows at a time (they stay in L1 between the
+// Both passes in one launch for r up to PF_MAX_R: a block takes 32 rows at a time (they stay in L1 between the
 // passes), its warps four rows each for Y = U z, then (1 << ct_log) threads by four columns and the rest by row groups for
 // U^T Y.  Two launches read the panel twice from L2 and met in memory: 2048 x 128 14.5 us, 4096 x 1024 23 us (now 5 and 15 us).
+// VEC: r a multiple of 4 (rows on 16-byte boundaries); other r read entry by entry (1001 x 83: the step 119.8 -> 113.8 us).
 // grid = (chunks, matrices); part[chunk][j][p] as in k_probe_w.
 constexpr i64 PF_MAX_R = 1024;      // 256 threads by four columns
 constexpr int PF_RED = 256 * 4 * NPROBE;      // floats: row groups x columns x probes
 constexpr int PF_SMEM_MAX = ((int)PF_MAX_R * NPROBE + PF_RED + 32 * NPROBE) * 4;
+template <bool VEC>
 __global__ void __launch_bounds__(256) k_probe_fused(const float* __restrict__ U, i64 ld, i64 rows, i64 r, i64 rows_per_chunk,
                                                      float* __restrict__ part, i64 wstride, const int* __restrict__ keep, int ct_log) {
   extern __shared__ __align__(16) float pf_smem[];
@@ -692,11 +694,15 @@ __global__ void __launch_bounds__(256) k_probe_fused(const float* __restrict__ U
   float* red = ys + 32 * NPROBE;                   // [row group][column][probe]
   float* sign = red + PF_RED;                      // (layout of k_probe_y4)
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nr = (int)r;
-  for (int e = threadIdx.x; e < nr * NPROBE; e += 256) {
+  for (int e = threadIdx.x; e < (nr + 3) / 4 * 4 * NPROBE; e += 256) {
     const int col = e / NPROBE, pr = e % NPROBE;
     sign[((((col >> 7) * 4 + (col & 3)) * 2 + (pr >> 2)) * 32 + ((col & 127) >> 2)) * 4 + (pr & 3)] = probe_sign(col, pr);
   }
   __syncthreads();
+  auto row4 = [&](const float* p, int j) -> float4 {      // columns j .. j + 3 of a row
+    if (VEC) return *reinterpret_cast<const float4*>(p);
+    return make_float4(p[0], j + 1 < nr ? p[1] : 0.f, j + 2 < nr ? p[2] : 0.f, j + 3 < nr ? p[3] : 0.f);
+  };
   const int groups = 256 >> ct_log, per = 32 / groups;      // row groups, rows of each (groups <= 32)
   const int j0 = 4 * ((int)threadIdx.x & ((1 << ct_log) - 1)), grp = (int)threadIdx.x >> ct_log;
   float w[4][NPROBE];
@@ -716,7 +722,7 @@ __global__ void __launch_bounds__(256) k_probe_fused(const float* __restrict__ U
       float4 v[4];
 #pragma unroll
       for (int q = 0; q < 4; ++q)
-        v[q] = (i0 + q < b1) ? *reinterpret_cast<const float4*>(U + (i0 + q) * ld + j) : make_float4(0.f, 0.f, 0.f, 0.f);
+        v[q] = (i0 + q < b1) ? row4(U + (i0 + q) * ld + j, j) : make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
       for (int cc = 0; cc < 4; ++cc) {
         const float4* su = reinterpret_cast<const float4*>(sign) + (((j >> 7) * 4 + cc) * 2) * 32 + lane;
@@ -753,7 +759,7 @@ __global__ void __launch_bounds__(256) k_probe_fused(const float* __restrict__ U
       for (int q = 0; q < per; ++q) {
         const int i = grp * per + q;
         if (ib + i >= b1) break;
-        const float4 u4 = *reinterpret_cast<const float4*>(U + (ib + i) * ld + j0);
+        const float4 u4 = row4(U + (ib + i) * ld + j0, j0);
         const float4 y0 = *reinterpret_cast<const float4*>(ys + i * NPROBE), y1 = *reinterpret_cast<const float4*>(ys + i * NPROBE + 4);
 #pragma unroll
         for (int c = 0; c < 4; ++c) {
@@ -769,6 +775,7 @@ __global__ void __launch_bounds__(256) k_probe_fused(const float* __restrict__ U
     float4* out = reinterpret_cast<float4*>(groups > 1 ? red + ((grp << ct_log) * 4 + j0) * NPROBE : part + ((i64)blockIdx.x * r + j0) * NPROBE);
 #pragma unroll
     for (int c = 0; c < 4; ++c) {
+      if (!VEC && groups == 1 && j0 + c >= nr) break;
       out[2 * c] = make_float4(w[c][0], w[c][1], w[c][2], w[c][3]);
       out[2 * c + 1] = make_float4(w[c][4], w[c][5], w[c][6], w[c][7]);
     }
