@@ -5,16 +5,17 @@
 #include <stddef.h>
 
 #include "dion_common.cuh"
+#include "umma_ptx.cuh"
 
 namespace dion {
 
 // ---------------------------------------------------------------------------------------------------------------
-// fp32 products on the warp-level tensor path: x = h + m + l with h, m, l bf16 (8 + 8 + 8 significant bits, every
-// remainder rounded to nearest), six of the nine cross products (those dropped are below 2^-26 of the product).  The
-// h h terms go to one accumulator, the rest to a second one that is added at the end: one truncating add per K step
-// on the main sum.  As accurate as a chain of fp32 FMAs, at 1.3 times their rate -- and, what counts here, an
-// operand fragment of a 16 x 8 tile is a few words per lane: a shared-memory load returns at most 128 bytes a cycle
-// to the registers of an SM, broadcast or not, which held a 64^3 product with 4 x 4 outputs per thread at 3900 cycles.
+// fp32 products of bf16 ones: x = h + m + l with h, m, l bf16 (8 + 8 + 8 significant bits, every remainder rounded to nearest), six
+// of the nine cross products (those dropped are below 2^-26 of the product).  The h h terms go to one accumulator, the rest to
+// others that are added at the end: one truncating add per K step on the main sum.  As accurate as a chain of fp32 FMAs.  Inside a
+// diagonal block they are on the warp-level path (mma.sync: an operand fragment of a 16 x 8 tile is a few words per lane, and a
+// shared-memory load returns at most 128 bytes a cycle to the registers of an SM, broadcast or not, which held a 64^3 product
+// with 4 x 4 outputs per thread at 3900 cycles); products of whole tiles are further below.
 // ---------------------------------------------------------------------------------------------------------------
 struct Bf3 { uint32_t h, m, l; };      // a pair of neighbouring k (the even one in the low half)
 
@@ -59,86 +60,110 @@ constexpr int CB = 64;      // tile
 constexpr int CLD = 72;     // row stride of a tile in shared memory (= 8 mod 32: the fragment loads are free of bank conflicts)
 typedef float (*ctile_t)[CLD];
 
-// A 64 x 64 tile over eight warps: warp w holds rows 16 (w / 2) .. + 15 and the 8-column groups 2 j + (w & 1), j = 0 .. 3;
-// lane (g, t) = (lane / 4, lane % 4) holds of group j: v[j][0], v[j][1] at row g, columns 2 t, 2 t + 1, v[j][2], v[j][3] at row g + 8.
-struct TileLane {
-  int row, col;      // of v[0][0]
-  __device__ __forceinline__ TileLane(int tid) : row(16 * (tid >> 6) + ((tid & 31) >> 2)), col(8 * ((tid >> 5) & 1) + 2 * (tid & 3)) {}
-  __device__ __forceinline__ int r(int e) const { return row + ((e & 2) ? 8 : 0); }
-  __device__ __forceinline__ int c(int j, int e) const { return col + 16 * j + (e & 1); }
+// ---------------------------------------------------------------------------------------------------------------
+// Products on the tensor cores: C = A B^T of tiles whose rows are contiguous along k, 64 of them, each as three bf16 planes (h, m, l)
+// of 128 bytes a row (128-byte swizzle), with the six cross products above.  A has 128 rows, the lanes of TMEM; where a tile has
+// 64, the MMA also reads the 64 rows behind a plane, whatever lies there, and nothing reads the lanes they go to.
+// (mma.sync took 3900 cycles for such a product on eight warps, bound by splitting an operand's fragments in every warp that
+// reads them; here an operand is split once and the MMAs, 768 cycles of operand reads, run beside the next operands' split.)
+// ---------------------------------------------------------------------------------------------------------------
+constexpr uint32_t PLANE = 64 * 128, PLANES = 3 * PLANE;      // bytes
+__device__ __forceinline__ uint32_t plane_at(int row, int col) {      // byte offset of an entry (its 8-column unit swizzled)
+  return (uint32_t)(row * 128 + ((((col >> 3) ^ row) & 7) << 4) + (col & 7) * 2);
+}
+__device__ __forceinline__ void planes_put4(uint32_t base, int row, int col, float4 x, uint32_t plane = PLANE) {      // col a multiple of 4
+  const Bf3 p = split3(x.x, x.y), q = split3(x.z, x.w);
+  const uint32_t a = base + plane_at(row, col);
+  asm volatile("st.shared.v2.b32 [%0], {%1, %2};" ::"r"(a), "r"(p.h), "r"(q.h) : "memory");
+  asm volatile("st.shared.v2.b32 [%0], {%1, %2};" ::"r"(a + plane), "r"(p.m), "r"(q.m) : "memory");
+  asm volatile("st.shared.v2.b32 [%0], {%1, %2};" ::"r"(a + 2 * plane), "r"(p.l), "r"(q.l) : "memory");
+}
+// (The pieces below that are called from several places are functions of their own: what a launch costs on a small matrix is to a
+// good part the fetching of its code.)
+// One thread: the product of the planes at a and b into the TMEM columns d .. d + 191.  The planes of b lie behind one another, so
+// that one MMA takes an operand of 64, 128 or 192 rows of them: what bounds these small MMAs is reading their operands from shared
+// memory (A's 128 rows 32 cycles, 64 rows of B 16), and A's planes are read once each.  Three accumulators: h h; h m + m h;
+// h l + m m + l h.
+static __device__ __noinline__ void planes_mma(uint32_t d, uint32_t a, uint32_t b, uint32_t plane_a) {
+#pragma unroll
+  for (uint32_t k = 0; k < 128; k += 32) {      // bytes of 16 columns
+    const uint64_t bd = umma::make_desc<true>(b + k, false, 0);
+    const uint32_t more = k != 0 ? 1u : 0u;
+    umma::umma<true>(d, umma::make_desc<true>(a + k, false, 0), bd, umma::make_idesc(true, false, false, 192), more);
+    umma::umma<true>(d + 64, umma::make_desc<true>(a + plane_a + k, false, 0), bd, umma::make_idesc(true, false, false, 128), 1u);
+    umma::umma<true>(d + 128, umma::make_desc<true>(a + 2 * plane_a + k, false, 0), bd, umma::make_idesc(true, false, false, 64), 1u);
+  }
+}
+// 16 columns of the three accumulators of this lane's row, the small ones added first
+__device__ __forceinline__ void planes_take16(uint32_t d, float (&v)[16]) {
+  uint32_t r[48];
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
+      "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%48];\n\t"
+      "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
+      "{%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%49];\n\t"
+      "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
+      "{%32, %33, %34, %35, %36, %37, %38, %39, %40, %41, %42, %43, %44, %45, %46, %47}, [%50];\n\t"
+      "tcgen05.wait::ld.sync.aligned;"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
+        "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]),
+        "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]),
+        "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31]),
+        "=r"(r[32]), "=r"(r[33]), "=r"(r[34]), "=r"(r[35]), "=r"(r[36]), "=r"(r[37]), "=r"(r[38]), "=r"(r[39]),
+        "=r"(r[40]), "=r"(r[41]), "=r"(r[42]), "=r"(r[43]), "=r"(r[44]), "=r"(r[45]), "=r"(r[46]), "=r"(r[47])
+      : "r"(d), "r"(d + 64), "r"(d + 128)
+      : "memory");
+#pragma unroll
+  for (int e = 0; e < 16; ++e) v[e] = (__uint_as_float(r[32 + e]) + __uint_as_float(r[16 + e])) + __uint_as_float(r[e]);
+}
+// The entries of a product that a thread reads: a row of TMEM is a lane, and a warp
+// reaches the 32 lanes of its rank mod 4.  Of eight warps, w and w + 4 hold rows 32 w .. 32 w + 31, the first four columns 0 .. 31.
+struct RowLane {
+  int row, col;
+  uint32_t tm;      // TMEM offset of its columns
+  bool owner;       // of a tile of 64 rows
+  __device__ __forceinline__ RowLane(int tid)
+      : row(32 * ((tid >> 5) & 3) + (tid & 31)), col(32 * ((tid >> 7) & 1)), tm(((uint32_t)(32 * ((tid >> 5) & 3)) << 16) + (uint32_t)col),
+        owner((tid >> 5 & 2) == 0) {}
 };
-
-// v = A B^T of 64 x 64 tiles in shared memory (k contiguous in both).  TRI: B is lower triangular (its zeros above the
-// diagonal are stored): column c needs k <= c only.  LOWER: only the groups that reach the diagonal or lie below it.
-enum : int { MM_FULL = 0, MM_TRI = 1, MM_LOWER = 2 };
-__device__ __forceinline__ void tile_nt(ctile_t A, ctile_t B, int mode, int tid, float (&v)[4][4]) {
-  const int warp = tid >> 5, lane = tid & 31, g = lane >> 2, t = lane & 3, rt = warp >> 1, par = warp & 1;
-  float s[4][4];
+// ... of the diagonal block: Lb = s2 (C - the product), identity beyond n rows (whole warps; d == ~0: no product)
+static __device__ __noinline__ void planes_diag(uint32_t d, const float* C, float* Lb, float s2, int row, int col, int n) {
+#pragma unroll 1
+  for (int h = 0; h < 2; ++h, C += 16, Lb += 16, col += 16) {
+    float v[16];
+    if (d != ~0u) planes_take16(d + 16 * h, v);
+    else {
 #pragma unroll
-  for (int j = 0; j < 4; ++j)
-#pragma unroll
-    for (int e = 0; e < 4; ++e) v[j][e] = s[j][e] = 0.f;
-  const float* pa = &A[16 * rt + g][2 * t];
-  const float* pb = &B[8 * par + g][2 * t];
-#pragma unroll 2      // (short on purpose: code that runs once costs more to fetch than to execute)
-  for (int kk = 0; kk < CB; kk += 16) {
-    float2 fa[4], fb[4][2];
-    fa[0] = *reinterpret_cast<const float2*>(pa); fa[1] = *reinterpret_cast<const float2*>(pa + 8 * CLD);
-    fa[2] = *reinterpret_cast<const float2*>(pa + 8); fa[3] = *reinterpret_cast<const float2*>(pa + 8 * CLD + 8);
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const float* q = pb + 16 * j * CLD;
-      fb[j][0] = *reinterpret_cast<const float2*>(q);
-      fb[j][1] = *reinterpret_cast<const float2*>(q + 8);
+      for (int e = 0; e < 16; ++e) v[e] = 0.f;
     }
-    const Bf3 a0 = split3(fa[0]), a1 = split3(fa[1]), a2 = split3(fa[2]), a3 = split3(fa[3]);
-    // (two column groups at a time, term by term: it is tens of cycles to the next mma on the same accumulator)
 #pragma unroll
-    for (int j0 = 0; j0 < 4; j0 += 2) {
-      // (one group decides for both: the other one's operands are zero, or its entries unused)
-      if (mode == MM_TRI && kk > 8 * (2 * (j0 + 1) + par) + 7) continue;      // (uniform)
-      if (mode == MM_LOWER && 2 * j0 + par > 2 * rt + 1) continue;
-      Bf3 b[2][2];
+    for (int q = 0; q < 4; ++q) {
+      const float4 c = *reinterpret_cast<const float4*>(C + 4 * q);
+      float o[4] = {c.x, c.y, c.z, c.w};
 #pragma unroll
-      for (int i = 0; i < 2; ++i) { b[i][0] = split3(fb[j0 + i][0]); b[i][1] = split3(fb[j0 + i][1]); }
-#pragma unroll
-      for (int i = 0; i < 2; ++i) mma_k16(s[j0 + i], a0.l, a1.l, a2.l, a3.l, b[i][0].h, b[i][1].h);
-#pragma unroll
-      for (int i = 0; i < 2; ++i) mma_k16(v[j0 + i], a0.h, a1.h, a2.h, a3.h, b[i][0].h, b[i][1].h);
-#pragma unroll
-      for (int i = 0; i < 2; ++i) mma_k16(s[j0 + i], a0.h, a1.h, a2.h, a3.h, b[i][0].l, b[i][1].l);
-#pragma unroll
-      for (int i = 0; i < 2; ++i) mma_k16(s[j0 + i], a0.m, a1.m, a2.m, a3.m, b[i][0].m, b[i][1].m);
-#pragma unroll
-      for (int i = 0; i < 2; ++i) mma_k16(s[j0 + i], a0.m, a1.m, a2.m, a3.m, b[i][0].h, b[i][1].h);
-#pragma unroll
-      for (int i = 0; i < 2; ++i) mma_k16(s[j0 + i], a0.h, a1.h, a2.h, a3.h, b[i][0].m, b[i][1].m);
+      for (int e = 0; e < 4; ++e) o[e] = (row >= n && row == col + 4 * q + e) ? 1.f : (o[e] - v[4 * q + e]) * s2;
+      *reinterpret_cast<float4*>(Lb + 4 * q) = make_float4(o[0], o[1], o[2], o[3]);
     }
-    pa += 16;
-    pb += 16;
-  }
-#pragma unroll
-  for (int j = 0; j < 4; ++j)
-#pragma unroll
-    for (int e = 0; e < 4; ++e) v[j][e] += s[j][e];
-}
-// tile in shared memory from the lanes' entries
-__device__ __forceinline__ void tile_put(ctile_t T, const TileLane& l, const float (&v)[4][4]) {
-#pragma unroll
-  for (int j = 0; j < 4; ++j) {
-    *reinterpret_cast<float2*>(&T[l.row][l.col + 16 * j]) = make_float2(v[j][0], v[j][1]);
-    *reinterpret_cast<float2*>(&T[l.row + 8][l.col + 16 * j]) = make_float2(v[j][2], v[j][3]);
   }
 }
-
-__device__ __forceinline__ void tile_get(ctile_t T, const TileLane& l, float (&v)[4][4]) {
+// 32 entries of a product into a row of a tile, or off it (whole warps)
+template <bool OFF>
+static __device__ __noinline__ void planes_take(uint32_t d, float* p) {
+#pragma unroll 1
+  for (int h = 0; h < 2; ++h, d += 16, p += 16) {
+    float v[16];
+    planes_take16(d, v);
 #pragma unroll
-  for (int j = 0; j < 4; ++j) {
-    const float2 a = *reinterpret_cast<const float2*>(&T[l.row][l.col + 16 * j]), b = *reinterpret_cast<const float2*>(&T[l.row + 8][l.col + 16 * j]);
-    v[j][0] = a.x; v[j][1] = a.y; v[j][2] = b.x; v[j][3] = b.y;
+    for (int q = 0; q < 4; ++q) {
+      float4 o = make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
+      if (OFF) {
+        const float4 c = *reinterpret_cast<const float4*>(p + 4 * q);
+        o = make_float4(c.x - o.x, c.y - o.y, c.z - o.z, c.w - o.w);
+      }
+      *reinterpret_cast<float4*>(p + 4 * q) = o;
+    }
   }
 }
-
 // ---------------------------------------------------------------------------------------------------------------
 // Cholesky factor and inverse of one 64 x 64 block by 256 threads, both in shared memory.
 //
@@ -161,6 +186,8 @@ __device__ __forceinline__ void tile_get(ctile_t T, const TileLane& l, float (&v
 // threads), 2 and 3 (192).
 // Pivot rules: see k_chol_flow.
 // ---------------------------------------------------------------------------------------------------------------
+template <int ID, int N>
+__device__ __forceinline__ void bar_arrive() { asm volatile("bar.arrive %0, %1;" ::"n"(ID), "n"(N) : "memory"); }      // (without waiting)
 template <int ID, int N>
 __device__ __forceinline__ void bar_named() { asm volatile("bar.sync %0, %1;" ::"n"(ID), "n"(N) : "memory"); }
 
@@ -445,28 +472,33 @@ __device__ __forceinline__ void potrf64(ctile_t L, ctile_t X, const Potrf64Set& 
 // A diagonal entry of A that is not finite means a NaN or Inf in M, G or Q: os[OS_FAIL] and DION_STATUS_NONFINITE.
 //
 // The right-looking form took one launch per 64 columns, ~21 us each, whatever the trailing work (r = 1024: 19 launches, 440 us
-// with the solve's products; now 160 us and one product).  Bound by the chain of diagonal blocks, ~8.5 us each: under ncu at
-// r = 1024 160 us at 1.85 GHz, 9 % of the SMs' issue slots, 0.4 % of DRAM, 18.5 of a warp's 25 cycles per instruction at barriers
-// (the runner's service warps, and helpers without a task).  Here the chain
+// with the solve's products).  With many tiles the launch is bound by the helpers' products: on mma.sync they took 3900 cycles
+// each (a 2048^2 panel of full rank, three rounds: 1402 us; on tcgen05, 128 rows to a task, 1101).  With few it is bound by the chain of
+// diagonal blocks, 8.3 to 9.8 us each (r = 1024: 157 us), of which potrf64 4.3 (its barriers, 64 dependent columns), the two products
+// and the passing of their operands 3.3.  Here the chain
 // D_k -> L_{k+1,k} -> A_{k+1,k+1} -> D_{k+1} stays inside ONE CTA (the "runner" of its matrix: two 64^3 products
 // and potrf64 per step), and every other tile is a task of a helper CTA, left-looking:
 //   L(i,k)    = (A_ik - sum_{j<k} L_ij L_kj^T) D_k^T                       i >= k + 3  (the runner makes i = k + 1)
 //   DIAG(k)   = A_kk - sum_{j<k-1} L_kj L_kj^T     for the runner's step k (it adds the last term); also makes L_{k,k-2}
 //   SUB(k)    = A_{k,k-1} - sum_{j<k-1} L_kj L_{k-1,j}^T     for the runner's step k; makes L_{k,k-2} for itself: fetched from
 //               DIAG it would come one trip through memory later on the chain's second loop, D_{k-2} -> L_{k,k-2} -> step k
-//   PANEL(I,k)= (P_Ik - sum_{j<k} U_Ij L_kj^T) D_k^T       64 panel rows (inverse: P = I, the sum starts at j = I)
-// A tile's terms are added as soon as their factors exist (double-buffered cp.async), in the order of j whoever runs
+//   PANEL(I,k)= (P_Ik - sum_{j<k} U_Ij L_kj^T) D_k^T       (inverse: P = I, the sum starts at j = I)
+// L and PANEL take 128 rows at a time: an MMA reads 128 rows of A anyway, row kt of L and D are read and split once for them, and
+// what bounds a term is shared memory (768 cycles of operand reads by its MMAs; their split and the sums hide behind).  They fetch
+// their operands into registers a term ahead; the preparations, which have three operands, by cp.async.
+// A tile's terms are added as soon as their factors exist, in the order of j whoever runs
 // the task: the result does not depend on the schedule.  Progress is published as one counter per row of L and U
 // (tiles of a row are finished in the order of k) and one for D; a consumer's thread 0 polls with acquire loads.
 // Helper tasks are handed out in the order of steps (the panel's a few steps behind the factor's), so a task only
 // ever waits for tasks handed out before it and for the runners, which are resident: the launch is cooperative.  Only the
-// preparations are handed out `ahead` steps early; they hold no more than half of the helpers.  Every wait has a cycle limit (then DION_STATUS_TIMEOUT and os[OS_FAIL], and every CTA leaves).
+// preparations are handed out `ahead` steps early; they hold no more than half of the helpers.  Every wait, those for the MMAs too,
+// has a cycle limit (then DION_STATUS_TIMEOUT and os[OS_FAIL], and every CTA leaves with its TMEM given back).
 // The last CTA to leave clears the counters for the next launch and evaluates the round (adaptive rounds).
 // ---------------------------------------------------------------------------------------------------------------
-enum : int { FLOW_TICKET = 0, FLOW_LEFT = 1, FLOW_ABORT = 2, FLOW_SM_BITS = 8, FLOW_SM_WORDS = 8, FLOW_HEAD_INTS = 32 };   // head of the control block
+enum : int { FLOW_TICKET = 0, FLOW_LEFT = 1, FLOW_ABORT = 2, FLOW_HEAD_INTS = 32 };   // head of the control block
 constexpr int FLOW_CTL_INTS = 64 * 1024;      // ints of a context's control block (zero between launches)
 constexpr int FLOW_COMPUTE = 256;            // threads that compute ...
-constexpr int FLOW_SERVICE = 128;            // ... and the service warps of a runner (four: nothing else fits beside eight anyway)
+constexpr int FLOW_SERVICE = 128;            // ... and the service warps of a runner
 constexpr int FLOW_THREADS = FLOW_COMPUTE + FLOW_SERVICE;
 constexpr int FLOW_IZ = 4;                    // the inverse's rows are stored (as zeros below the diagonal) up to a multiple of this many tiles
 // rows of tiles of column k of the inverse that are written (whole: of a square whose largest entry is looked for afterwards)
@@ -498,8 +530,8 @@ struct FlowArgs {
   int* status_always;
   int* ctl; int ctl_stride; // control block; ints per matrix after its head
   i64 wstride; int nb;
+  int prows;                // tiles of rows that a task of the panel takes, 1 or 2
   int ahead;                // steps by which the preparations are handed out early (they take on every term since the first column)
-  int exclusive;            // a runner has its SM to itself: the helper beside it leaves
   int near;                 // a matrix whose OS_GOOD is 2 is left alone too (k_near_identity has formed its factor)
   int round_end;            // evaluate the adaptive round
   float good_rel, done_rel;
@@ -537,11 +569,6 @@ __device__ __forceinline__ void flow_publish(int* p, int v) {     // the CTA's w
   asm volatile("fence.acq_rel.gpu;" ::: "memory");
   asm volatile("st.relaxed.gpu.global.s32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
 }
-__device__ __forceinline__ unsigned flow_smid() {
-  unsigned r;
-  asm volatile("mov.u32 %0, %%smid;" : "=r"(r));
-  return min(r, (unsigned)(32 * FLOW_SM_WORDS - 1));
-}
 // thread 0: waits until *p >= want; returns the value seen, or -1 when the wait ran out (or another CTA's did)
 __device__ __forceinline__ int flow_wait(const int* p, int want, const FlowArgs& f) {
   int v = flow_ld(p);
@@ -562,31 +589,97 @@ __device__ __forceinline__ int flow_wait(const int* p, int want, const FlowArgs&
   }
 }
 
-// rows x cols (<= 64 x 64) of src into a tile, zeros elsewhere.  VEC: 16-byte aligned rows, cols a multiple of 4:
-// asynchronous (cp.async, the caller waits); else plain loads.  Reads go to L2: other CTAs have written the data.
-template <bool VEC, int NT = FLOW_COMPUTE>
-__device__ __forceinline__ void flow_load(ctile_t T, const float* __restrict__ src, i64 ld, int rows, int cols, int tid) {
-  if (VEC) {
-#pragma unroll 4
-    for (int e = tid; e < CB * CB / 4; e += NT) {
-      const int i = e >> 4, c = (e & 15) * 4;
-      const bool ok = i < rows && c < cols;
-      const uint32_t dst = (uint32_t)__cvta_generic_to_shared(&T[i][c]);
-      const float* g = ok ? src + (i64)i * ld + c : src;
-      asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(g), "r"(ok ? 16 : 0) : "memory");
-    }
-  } else {
-#pragma unroll 8
-    for (int e = tid; e < CB * CB; e += NT) {
-      const int i = e >> 6, c = e & 63;
-      T[i][c] = (i < rows && c < cols) ? __ldcg(src + (i64)i * ld + c) : 0.f;
+// Tiles are handled by 256 threads, four float4 each: row tid / 16 + 16 q, columns 4 (tid % 16) ...  VEC: 16-byte aligned rows,
+// a multiple of four columns.  Reads go to L2: other CTAs have written the data.
+__device__ __forceinline__ void flow_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+__device__ __forceinline__ void flow_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+template <bool VEC>
+__device__ __forceinline__ float4 flow_ld4(const float* p, int left) {      // left: columns there are
+  if (VEC) return left > 0 ? __ldcg(reinterpret_cast<const float4*>(p)) : make_float4(0.f, 0.f, 0.f, 0.f);
+  return make_float4(left > 0 ? __ldcg(p) : 0.f, left > 1 ? __ldcg(p + 1) : 0.f, left > 2 ? __ldcg(p + 2) : 0.f, left > 3 ? __ldcg(p + 3) : 0.f);
+}
+// scale * the sum of n arrays `stride` apart, rows x cols of it, into a tile (zeros elsewhere).  Four arrays' loads in flight: one after
+// another, 16 partial sums of the first three tiles were 19 us of latency; one array by itself without the other three's predicates.
+template <bool VEC>
+static __device__ __noinline__ void flow_tile_in(ctile_t T, const float* __restrict__ src, i64 stride, int n, float scale, i64 ld, int rows, int cols, int tid) {
+  const int i = tid >> 4, c = (tid & 15) * 4;
+  const float* p = src + (i64)i * ld + c;
+  float4 v[4];
+#pragma unroll
+  for (int q = 0; q < 4; ++q) v[q] = flow_ld4<VEC>(p + (i64)(16 * q) * ld, i + 16 * q < rows ? cols - c : 0);
+#pragma unroll 1
+  for (int k = 1; k < n; k += 3) {
+    float4 w[3][4];
+#pragma unroll
+    for (int u = 0; u < 3; ++u)
+#pragma unroll
+      for (int q = 0; q < 4; ++q) w[u][q] = flow_ld4<VEC>(p + (k + u) * stride + (i64)(16 * q) * ld, (k + u < n && i + 16 * q < rows) ? cols - c : 0);
+#pragma unroll
+    for (int u = 0; u < 3; ++u)
+#pragma unroll
+      for (int q = 0; q < 4; ++q) { v[q].x += w[u][q].x; v[q].y += w[u][q].y; v[q].z += w[u][q].z; v[q].w += w[u][q].w; }
+  }
+#pragma unroll
+  for (int q = 0; q < 4; ++q) st4(&T[i + 16 * q][c], make_float4(scale * v[q].x, scale * v[q].y, scale * v[q].z, scale * v[q].w));
+}
+// A tile on its way to shared memory: 16-byte units `step` bytes apart per q from `at` on, where the thread that asked finds them
+// again itself.  (VEC: cp.async, the caller commits and waits.)
+template <bool VEC>
+static __device__ __noinline__ void flow_bring(unsigned char* at, int step, const float* __restrict__ src, i64 ld, int rows, int cols, int tid) {
+  const int i = tid >> 4, c = (tid & 15) * 4;
+  const float* p = src + (i64)i * ld + c;
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    const int left = i + 16 * q < rows ? cols - c : 0;
+    const float* g = p + (i64)(16 * q) * ld;
+    if (VEC) {
+      const uint32_t dst = umma::smem_u32(at) + (uint32_t)(q * step);
+      asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(left > 0 ? g : src), "r"(left > 0 ? 16 : 0) : "memory");
+    } else {
+      *reinterpret_cast<float4*>(at + q * step) = flow_ld4<false>(g, left);
     }
   }
 }
-__device__ __forceinline__ void flow_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-__device__ __forceinline__ void flow_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+// ... and from there into planes
+static __device__ __noinline__ void flow_split(uint32_t planes, const unsigned char* at, int step, int tid) {
+#pragma unroll
+  for (int q = 0; q < 4; ++q) planes_put4(planes, (tid >> 4) + 16 * q, (tid & 15) * 4, *reinterpret_cast<const float4*>(at + q * step));
+}
+constexpr int FLOW_TILE_STEP = 16 * CLD * (int)sizeof(float), FLOW_RAW_STEP = 4096;
+__device__ __forceinline__ unsigned char* tile_at4(ctile_t T, int tid) { return reinterpret_cast<unsigned char*>(&T[tid >> 4][(tid & 15) * 4]); }
+// rows x cols of a tile to global memory
+template <bool VEC>
+static __device__ __noinline__ void flow_store(ctile_t T, float* __restrict__ dst, i64 ld, int rows, int cols, int tid) {
+  const int i = tid >> 4, c = (tid & 15) * 4;
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    if (i + 16 * q >= rows || c >= cols) continue;
+    const float4 v = ld4(&T[i + 16 * q][c]);
+    float* p = dst + (i64)(i + 16 * q) * ld + c;
+    if (VEC) {
+      st4(p, v);
+    } else {
+      p[0] = v.x;
+      if (c + 1 < cols) p[1] = v.y;
+      if (c + 2 < cols) p[2] = v.z;
+      if (c + 3 < cols) p[3] = v.w;
+    }
+  }
+}
 
-constexpr int FLOW_SMEM = 6 * CB * CLD * (int)sizeof(float);
+// Shared memory, from a 1024-byte boundary: two stages of operand planes (128 and 64 rows, or, of a preparation, three tiles in the
+// first one and tiles on their way in the second's place) and 128 rows of results; a runner has the planes of its three operands and its
+// tiles there.
+constexpr int FLOW_TILE = CB * CLD * (int)sizeof(float);
+constexpr uint32_t FLOW_STAGE = 3 * PLANES;
+constexpr uint32_t FLOW_COMING = FLOW_STAGE;
+constexpr uint32_t FLOW_RAW = CB * CB * sizeof(float);
+constexpr uint32_t FLOW_RESULTS = 2 * FLOW_STAGE;
+static_assert(FLOW_COMING + 4 * FLOW_RAW <= FLOW_RESULTS && FLOW_STAGE + 4 * FLOW_TILE <= FLOW_RESULTS, "tiles lie behind the first planes");
+constexpr int FLOW_SMEM = 1024 + (int)FLOW_RESULTS + 2 * FLOW_TILE;
+constexpr int FLOW_ROWS = 2;                  // tiles of rows that a task of the factor takes, and most of a task of the panel
+constexpr int FLOW_TMEM = 512;                // columns: two buffers of a product, or one of a preparation's two
+constexpr int FLOW_MMA_THREAD = 64;           // issues the MMAs (its warp holds no rows)
 
 template <bool VEC>
 __global__ void __launch_bounds__(FLOW_THREADS, 1) k_chol_flow(const __grid_constant__ FlowArgs f) {
@@ -596,18 +689,20 @@ __global__ void __launch_bounds__(FLOW_THREADS, 1) k_chol_flow(const __grid_cons
     return (f.skips && os[OS_DONE] != 0) || (f.near && os[OS_GOOD] == 2);
   };
   if ((f.skips || f.near) && __syncthreads_and((int)threadIdx.x >= f.nb || skipped((int)threadIdx.x))) return;      // (nb <= 64)
-  extern __shared__ __align__(16) float flow_smem[];
-  ctile_t SA[2] = {reinterpret_cast<ctile_t>(flow_smem), reinterpret_cast<ctile_t>(flow_smem + 2 * CB * CLD)};
-  ctile_t SB[2] = {reinterpret_cast<ctile_t>(flow_smem + CB * CLD), reinterpret_cast<ctile_t>(flow_smem + 3 * CB * CLD)};
-  ctile_t SC[2] = {reinterpret_cast<ctile_t>(flow_smem + 4 * CB * CLD), reinterpret_cast<ctile_t>(flow_smem + 5 * CB * CLD)};
+  extern __shared__ unsigned char flow_smem[];
+  const uint32_t smem0 = (umma::smem_u32(flow_smem) + 1023u) & ~1023u;
+  unsigned char* const smem_al = flow_smem + (smem0 - umma::smem_u32(flow_smem));
+  auto tile_in = [&](uint32_t off) { return reinterpret_cast<ctile_t>(smem_al + off); };
+  const ctile_t V = tile_in(FLOW_RESULTS), Wt = tile_in(FLOW_RESULTS + FLOW_TILE);
+  __shared__ uint64_t s_bar[2];      // the products of a TMEM buffer are done
+  __shared__ uint32_t s_tmem;
   __shared__ Potrf64Set s_set[2];
   __shared__ Potrf64Aux aux;
-  __shared__ float s_diag[2][CB];
   __shared__ int s_ready[2];
-  __shared__ int s_ok, s_prep;
+  __shared__ int s_ok, s_prep, s_first, s_inv;
   __shared__ FlowTask s_task;
   const int tid = threadIdx.x;
-  const TileLane tl(tid);      // this thread's 16 entries of a tile
+  const RowLane rl(tid);
   const int T = (int)((f.sz + CB - 1) / CB);
   const bool solve = f.Pin != nullptr;
   const int NR = solve ? (int)((f.rows + CB - 1) / CB) : 0;      // row blocks of the panel
@@ -620,85 +715,12 @@ __global__ void __launch_bounds__(FLOW_THREADS, 1) k_chol_flow(const __grid_cons
   auto doneD = [&](int b) { return ctl_of(b) + 2 * T; };
   auto xmaxbits = [&](int b) { return ctl_of(b) + 2 * T + 1; };
   auto rowU = [&](int b, int I) { return ctl_of(b) + 2 * T + 2 + I; };
-  // entries of the square of matrix b's Gram matrix as the product left it: this thread's 16 of tile (i, k) (zeros
-  // beyond the square) ...
-  auto raw_tile = [&](int b, int i, int k, float (&v)[4][4]) {
-    const int nr = cols_of(i) - tl.row, nc = cols_of(k) - tl.col;
-    const i64 e = (f.o + (i64)i * CB + tl.row) * ld + f.o + (i64)k * CB + tl.col;
-    const float* p = (f.part == nullptr ? f.A : f.part) + (i64)b * f.wstride + e;
-    const int n = f.part == nullptr ? 1 : f.nsplit;
-#pragma unroll
-    for (int j = 0; j < 4; ++j)
-#pragma unroll
-      for (int x = 0; x < 4; ++x) v[j][x] = 0.f;
-    // (four partial sums' loads in flight: one after another, 16 partial sums of the first three tiles were 19 us of latency)
-#pragma unroll 1
-    for (int q = 0; q < n; q += 4, p += 4 * ld * ld) {
-      float w[4][4][4];
-#pragma unroll
-      for (int u = 0; u < 4; ++u)
-#pragma unroll
-        for (int j = 0; j < 4; ++j)
-#pragma unroll
-          for (int h = 0; h < 2; ++h) {
-            const int dr = 8 * h, dc = 16 * j;
-            const float* e = p + u * ld * ld + dr * ld + dc;
-            if (VEC) {      // (cols is even; whole sectors: with single words the CTA moved twice the bytes)
-              const float2 t = (q + u < n && dr < nr && dc < nc) ? __ldcg(reinterpret_cast<const float2*>(e)) : make_float2(0.f, 0.f);
-              w[u][j][2 * h] = t.x; w[u][j][2 * h + 1] = t.y;
-            } else {
-              w[u][j][2 * h] = (q + u < n && dr < nr && dc < nc) ? __ldcg(e) : 0.f;
-              w[u][j][2 * h + 1] = (q + u < n && dr < nr && dc + 1 < nc) ? __ldcg(e + 1) : 0.f;
-            }
-          }
-#pragma unroll
-      for (int u = 0; u < 4; ++u)
-#pragma unroll
-        for (int j = 0; j < 4; ++j)
-#pragma unroll
-          for (int x = 0; x < 4; ++x) v[j][x] += w[u][j][x];
-    }
-    if (f.part != nullptr && f.alpha_dev != nullptr) {
-      const float al = f.alpha_dev[(i64)b * f.alpha_stride];
-#pragma unroll
-      for (int j = 0; j < 4; ++j)
-#pragma unroll
-        for (int x = 0; x < 4; ++x) v[j][x] *= al;
-    }
-  };
-  // ... and of a rows x cols block at p (leading dimension ld), from L2: other CTAs have written it
-  auto get_tile = [&](const float* p, int rows, int cols, float (&v)[4][4]) {
-    p += (i64)tl.row * ld + tl.col;
-    const int nr = rows - tl.row, nc = cols - tl.col;
-#pragma unroll
-    for (int j = 0; j < 4; ++j)
-#pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        const int dr = 8 * h, dc = 16 * j;
-        if (VEC) {
-          const float2 t = (dr < nr && dc < nc) ? __ldcg(reinterpret_cast<const float2*>(p + dr * ld + dc)) : make_float2(0.f, 0.f);
-          v[j][2 * h] = t.x; v[j][2 * h + 1] = t.y;
-        } else {
-          v[j][2 * h] = (dr < nr && dc < nc) ? __ldcg(p + dr * ld + dc) : 0.f;
-          v[j][2 * h + 1] = (dr < nr && dc + 1 < nc) ? __ldcg(p + dr * ld + dc + 1) : 0.f;
-        }
-      }
-  };
-  auto store_tile = [&](float* p, int rows, int cols, const float (&v)[4][4]) {
-    p += (i64)tl.row * ld + tl.col;
-    const int nr = rows - tl.row, nc = cols - tl.col;
-#pragma unroll
-    for (int j = 0; j < 4; ++j)
-#pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        const int dr = 8 * h, dc = 16 * j;
-        if (VEC) {      // (cols is even)
-          if (dr < nr && dc < nc) *reinterpret_cast<float2*>(p + dr * ld + dc) = make_float2(v[j][2 * h], v[j][2 * h + 1]);
-        } else {
-          if (dr < nr && dc < nc) p[dr * ld + dc] = v[j][2 * h];
-          if (dr < nr && dc + 1 < nc) p[dr * ld + dc + 1] = v[j][2 * h + 1];
-        }
-      }
+  // tile (i, k) of the square of matrix b's Gram matrix as the product left it
+  auto raw_tile = [&](ctile_t W, int b, int i, int k, int t) {
+    const bool parts = f.part != nullptr;
+    const float* p = (parts ? f.part : f.A) + (i64)b * f.wstride + (f.o + (i64)i * CB) * ld + f.o + (i64)k * CB;
+    const float scale = (parts && f.alpha_dev != nullptr) ? f.alpha_dev[(i64)b * f.alpha_stride] : 1.f;
+    flow_tile_in<VEC>(W, p, ld * ld, parts ? f.nsplit : 1, scale, ld, cols_of(i), cols_of(k), t);
   };
   auto wait_all = [&](const int* p, int want) -> bool {      // every thread: thread 0 waits, all learn the outcome
     if (tid == 0) s_ok = flow_wait(p, want, f);
@@ -707,9 +729,39 @@ __global__ void __launch_bounds__(FLOW_THREADS, 1) k_chol_flow(const __grid_cons
     bar_named<1, FLOW_COMPUTE>();
     return ok;
   };
-  if (tid == 0) s_ok = 0;
+  if (tid == 0) {
+    s_ok = s_inv = 0;
+    umma::mbar_init(umma::smem_u32(&s_bar[0]), 1);
+    umma::mbar_init(umma::smem_u32(&s_bar[1]), 1);
+    umma::fence_barrier_init();
+  }
+  if (tid >= FLOW_COMPUTE && tid < FLOW_COMPUTE + 32) {      // (one service warp; nothing that holds TMEM fits beside this CTA)
+    umma::tmem_alloc(umma::smem_u32(&s_tmem), FLOW_TMEM);
+    umma::tmem_relinquish();
+  }
+  umma::tc_fence_before();
   __syncthreads();
-
+  umma::tc_fence_after();
+  const uint32_t tmem0 = *reinterpret_cast<volatile uint32_t*>(&s_tmem);
+  unsigned phase = 0;      // parities of s_bar, per buffer
+  auto tmem_of = [&](int buf) { return tmem0 + (uint32_t)buf * 256u; };
+  auto commit = [&](int buf) { umma::umma_commit(umma::smem_u32(&s_bar[buf])); };
+  // Every compute thread: the products of `buf` are done (false: the wait ran out; the launch is given up).
+  auto mma_wait = [&](int buf) -> bool {
+    const uint32_t bar = umma::smem_u32(&s_bar[buf]), par = (phase >> buf) & 1u;
+    phase ^= 1u << buf;
+    bool ok = umma::mbar_try_wait(bar, par);
+    if (!ok) {
+      const long long t0 = clock64();
+      while (!(ok = umma::mbar_try_wait(bar, par)) && clock64() - t0 <= f.limit) {}
+      if (!ok) {
+        atomicExch(f.ctl + FLOW_ABORT, 1);
+        atomicOr(f.status_always, DION_STATUS_TIMEOUT);
+      }
+    }
+    umma::tc_fence_after();
+    return ok;
+  };
   bool alive = true;
   if ((int)blockIdx.x < f.nb) {
     // ------------------------------------------------------------------------------------------ runner of matrix b
@@ -723,8 +775,10 @@ __global__ void __launch_bounds__(FLOW_THREADS, 1) k_chol_flow(const __grid_cons
       float* gdiag = f.gdiag + (i64)b * f.wstride;
       float* Dinv = f.Dinv + (i64)b * f.wstride;
       float* DinvP = f.DinvP + (i64)b * f.wstride;
-      ctile_t TS[2] = {SA[0], SA[1]};                     // A'_{k,k-1}, then L_{k,k-1}; by parity of k
-      ctile_t Lb = SB[0], X = SB[1], C = SC[0];              // the diagonal block; D; A'_kk
+      const uint32_t PA = smem0, PX = PA + PLANES, PL = PX + PLANES;      // planes of A'_{k,k-1}, D_{k-1}, L_{k,k-1}
+      const ctile_t Lb = tile_in(FLOW_STAGE), X = tile_in(FLOW_STAGE + FLOW_TILE),       // the diagonal block; D
+                    TS = tile_in(FLOW_STAGE + 2 * FLOW_TILE);                            // L_{k,k-1}
+      auto C = [&](int k) { return (k & 1) != 0 ? V : tile_in(FLOW_STAGE + 3 * FLOW_TILE); };      // A'_kk
       auto tile_at = [&](int i, int k) { return G + (f.o + (i64)i * CB) * ld + f.o + (i64)k * CB; };
       const int lane = tid & 31;
       // reference values of block k's pivots: diag(A) as the product left it
@@ -743,91 +797,122 @@ __global__ void __launch_bounds__(FLOW_THREADS, 1) k_chol_flow(const __grid_cons
         const int sid = tid - FLOW_COMPUTE, swarp = sid >> 5;
         if (sid == 0) {
           if (f.o == 0) { os[OS_FLOORED] = 0; os[OS_MINREL] = 0x7f800000; }      // (+inf)
-          if (f.exclusive) {
-            const unsigned sm = flow_smid();
-            atomicOr(f.ctl + FLOW_SM_BITS + (sm >> 5), 1 << (sm & 31));
-          }
         }
-        bar_named<5, FLOW_THREADS>();      // the first blocks' diagonals are in s_diag
-        if (swarp == 0) setup(0, s_diag[0][lane], s_diag[0][lane + 32]);
-        if (swarp == 1 && T > 1) setup(1, s_diag[1][lane], s_diag[1][lane + 32]);
+        auto two = [&](auto go) {      // the work of 256 threads
+#pragma unroll 1
+          for (int h = 0; h < 2; ++h) go(sid + h * FLOW_SERVICE);
+        };
+        if (f.part != nullptr && T > 1) two([&](int t) { raw_tile(Wt, b, 1, 0, t); });      // (many loads: beside those of the first block)
+        bar_named<5, FLOW_THREADS>();      // the first block is in C
+        if (swarp == 0)
+          setup(0, f.gdiag_given ? diag_of(0, lane) : C(0)[lane][lane], f.gdiag_given ? diag_of(0, lane + 32) : C(0)[lane + 32][lane + 32]);
+        int given = 0;      // (thread 0) inverses that are published
+        auto publish_d = [&](int n) {
+          if (n > given) { flow_publish(doneD(b), n); given = n; }
+        };
+        // Waits for a preparation (bit 0: SUB, bit 1: DIAG); an inverse that is finished meanwhile is published at once, not behind
+        // the next step's beginning, which may be waiting for the same helpers.
+        auto wait_prep = [&](int k, int bit) -> bool {
+          if (sid == 0) {
+            const long long t0 = clock64();
+            s_prep = 0;
+            for (unsigned polls = 1; (flow_ld(prep(b, k)) & bit) == 0; ++polls) {
+              const int n = *reinterpret_cast<volatile int*>(&s_inv);
+              if (n > given) { __threadfence_block(); publish_d(n); }
+              if ((polls & 15u) != 0) continue;
+              if (flow_ld(f.ctl + FLOW_ABORT) != 0) { s_prep = -1; break; }
+              if (clock64() - t0 > f.limit) {
+                atomicExch(f.ctl + FLOW_ABORT, 1);
+                atomicOr(f.status_always, DION_STATUS_TIMEOUT);
+                s_prep = -1;
+                break;
+              }
+            }
+            if (s_prep < 0) s_ok = -1;      // (every barrier up to the next step's is still met)
+          }
+          bar_named<8, FLOW_SERVICE>();
+          return s_prep >= 0;
+        };
         for (int k = 0; k <= T; ++k) {
-          bar_named<6, FLOW_THREADS>();      // step k may start: its operands are there; D_{k-1} is stored
+          bar_named<6, FLOW_THREADS>();      // step k may start: A'_{k,k-1} is there; D_{k-1} is stored
           if (s_ok < 0) break;
-          if (k > 0 && sid == 0) flow_publish(doneD(b), k);
+          if (sid == 0) publish_d(k);
           if (k == T) break;
           if (k > 0) {
-            bar_named<7, FLOW_THREADS>();      // L_{k,k-1} is stored
-            if (sid == FLOW_SERVICE - 1) flow_publish(rowL(b, k), k);      // (row k of L is complete)
-          }
-          if (k + 1 < T && k + 1 >= 2) {
-            if (sid == 0) s_prep = flow_wait(prep(b, k + 1), 2, f);
-            bar_named<8, FLOW_SERVICE>();
-            if (s_prep < 0) {
-              if (sid == 0) s_ok = -1;
-            } else {
-              const int nk = cols_of(k + 1);
-              flow_load<VEC, FLOW_SERVICE>(TS[(k + 1) & 1], tile_at(k + 1, k), ld, nk, CB, sid);
-              flow_load<VEC, FLOW_SERVICE>(C, tile_at(k + 1, k + 1), ld, nk, nk, sid);
+            if (k >= 2 && wait_prep(k, 2)) {      // A'_kk and its pivots' reference values
+              const int nk = cols_of(k);
+              two([&](int t) { flow_bring<VEC>(tile_at4(C(k), t), FLOW_TILE_STEP, tile_at(k, k), ld, nk, nk, t); });
               flow_commit();
-              if (swarp == 0) setup(k + 1, diag_of(k + 1, lane), diag_of(k + 1, lane + 32));
+              if (swarp == 0) setup(k, diag_of(k, lane), diag_of(k, lane + 32));
               flow_wait_all();
             }
+            bar_arrive<9, FLOW_THREADS>();
+            bar_named<7, FLOW_THREADS>();      // L_{k,k-1} is in TS
+            two([&](int t) { flow_store<VEC>(TS, tile_at(k, k - 1), ld, cols_of(k), CB, t); });
+            bar_named<8, FLOW_SERVICE>();
+            if (sid == FLOW_SERVICE - 1) flow_publish(rowL(b, k), k);      // (row k of L is complete)
+          }
+          if (k + 1 < T) {      // the next step's operand (the products that read A' are over)
+            if (k == 0) {
+              const ctile_t Cn = C(1);
+              two([&](int t) {
+                if (f.part == nullptr) raw_tile(Wt, b, 1, 0, t);
+                raw_tile(Cn, b, 1, 1, t);
+              });
+              bar_named<8, FLOW_SERVICE>();
+              if (swarp == 0)
+                setup(1, f.gdiag_given ? diag_of(1, lane) : Cn[lane][lane], f.gdiag_given ? diag_of(1, lane + 32) : Cn[lane + 32][lane + 32]);
+            } else {
+              if (!wait_prep(k + 1, 1)) continue;
+              two([&](int t) { flow_bring<VEC>(tile_at4(Wt, t), FLOW_TILE_STEP, tile_at(k + 1, k), ld, cols_of(k + 1), CB, t); });
+              flow_commit();
+              flow_wait_all();
+            }
+            two([&](int t) { flow_split(PA, tile_at4(Wt, t), FLOW_TILE_STEP, t); });
+            umma::fence_proxy_async();
           }
         }
       } else {
         // ---------------------------------------------------------------- compute threads
-        float c[4][4];
-        {
-          float v1[4][4], c1[4][4];
-          raw_tile(b, 0, 0, c);
-          if (T > 1) { raw_tile(b, 1, 0, v1); raw_tile(b, 1, 1, c1); }
-#pragma unroll
-          for (int j = 0; j < 4; ++j)
-#pragma unroll
-            for (int x = 0; x < 4; ++x)
-              if (tl.r(x) == tl.c(j, x)) {
-                s_diag[0][tl.r(x)] = f.gdiag_given ? diag_of(0, tl.r(x)) : c[j][x];
-                if (T > 1) s_diag[1][tl.r(x)] = f.gdiag_given ? diag_of(1, tl.r(x)) : c1[j][x];
-              }
-          if (T > 1) { tile_put(TS[1], tl, v1); tile_put(C, tl, c1); }
-        }
+        raw_tile(C(0), b, 0, 0, tid);
         bar_named<5, FLOW_THREADS>();
         for (int k = 0; k <= T; ++k) {
           bar_named<6, FLOW_THREADS>();
           if (s_ok < 0) { alive = false; break; }
           if (k == T) break;
           const int nk = cols_of(k);
+          const Potrf64Set& set = s_set[k & 1];
           if (k > 0) {
             // L_{k,k-1} = A' D_{k-1}^T (the deflated rows of D zeroed), then the last term of the diagonal block
-            tile_get(C, tl, c);
+            bool ok = true;
+            flow_split(PX, tile_at4(X, tid), FLOW_TILE_STEP, tid);
 #pragma unroll 1
-            for (int h = 0; h < 2; ++h) {      // (one copy of the product's code)
-              float v[4][4];
-              tile_nt(TS[k & 1], h == 0 ? X : TS[k & 1], h == 0 ? MM_TRI : MM_LOWER, tid, v);
+            for (int h = 0; h < 2; ++h) {
+              umma::fence_proxy_async();
+              umma::tc_fence_before();
+              bar_named<1, FLOW_COMPUTE>();
+              if (tid == FLOW_MMA_THREAD) {
+                umma::tc_fence_after();
+                planes_mma(tmem_of(h), h == 0 ? PA : PL, h == 0 ? PX : PL, PLANE);
+                commit(h);
+              }
+              ok = mma_wait(h) && ok;
               if (h == 0) {
+                if (rl.owner) planes_take<false>(tmem_of(0) + rl.tm, &TS[rl.row][rl.col]);
+                bar_arrive<7, FLOW_THREADS>();      // (the service warps store it)
                 bar_named<1, FLOW_COMPUTE>();
-                tile_put(TS[k & 1], tl, v);
-                store_tile(tile_at(k, k - 1), nk, CB, v);
-                bar_named<7, FLOW_THREADS>();
-              } else {
-#pragma unroll
-                for (int j = 0; j < 4; ++j)
-#pragma unroll
-                  for (int x = 0; x < 4; ++x) c[j][x] -= v[j][x];
+                flow_split(PL, tile_at4(TS, tid), FLOW_TILE_STEP, tid);
               }
             }
+            if (!ok) s_ok = -1;      // (seen behind the next step's barrier)
+            bar_named<9, FLOW_THREADS>();      // A'_kk is there
           }
-          const Potrf64Set& set = s_set[k & 1];
-          const float s2 = set.s2;
-#pragma unroll
-          for (int j = 0; j < 4; ++j)
-#pragma unroll
-            for (int x = 0; x < 4; ++x) c[j][x] = (tl.r(x) == tl.c(j, x) && tl.r(x) >= nk) ? 1.f : c[j][x] * s2;      // (identity padding)
-          tile_put(Lb, tl, c);
+          if (rl.owner) planes_diag(k > 0 ? tmem_of(1) + rl.tm : ~0u, &C(k)[rl.row][rl.col], &Lb[rl.row][rl.col], set.s2, rl.row, rl.col, nk);
+          umma::tc_fence_before();
           bar_named<1, FLOW_COMPUTE>();
           const i64 d = (i64)(f.o / CB + k) * (CB * CB);
           potrf64(Lb, X, set, aux, f.floor_rel, os, f.status, tid, Dinv + d, DinvP + d);
+          if (tid == 0) { __threadfence_block(); *reinterpret_cast<volatile int*>(&s_inv) = k + 1; }
         }
       }
     }
@@ -842,11 +927,11 @@ __global__ void __launch_bounds__(FLOW_THREADS, 1) k_chol_flow(const __grid_cons
   // tasks of list step s: the preparations for the runner's steps up to s + 2 + ahead, the factor's tiles of step s, the
   // panel's of step s - LAG
   auto step_tasks = [&](int s, int& nS, int& nL, int& nP) {
-    nL = max(T - 3 - s, 0);
+    nL = (max(T - 3 - s, 0) + FLOW_ROWS - 1) / FLOW_ROWS;
     nS = (s == 0) ? 2 * min(max(T - 2, 0), f.ahead + 1) : 2 * min(max(T - 2 - s - f.ahead, 0), 1);
     nP = 0;
     const int k = s - FLOW_LAG;
-    if (k >= 0 && k < T) nP = solve ? NR : flow_inverse_rows(T, k, f.sz < f.r);
+    if (k >= 0 && k < T) nP = ((solve ? NR : flow_inverse_rows(T, k, f.sz < f.r)) + f.prows - 1) / f.prows;
   };
   auto fetch_task = [&](int ticket) -> FlowTask {
     FlowTask t;
@@ -862,10 +947,10 @@ __global__ void __launch_bounds__(FLOW_THREADS, 1) k_chol_flow(const __grid_cons
           t.type = (e & 1) ? FT_DIAG : FT_SUB;
           t.i = t.k = (step == 0) ? 2 + (e >> 1) : step + 2 + f.ahead;
         } else if ((e -= nS) < nL) {
-          t.type = FT_L; t.i = step + 3 + e; t.k = step;
+          t.type = FT_L; t.i = step + 3 + FLOW_ROWS * e; t.k = step;
         } else {
           t.type = FT_PANEL; t.k = step - FLOW_LAG;
-          t.i = e - nL;
+          t.i = f.prows * (e - nL);
         }
         return t;
       }
@@ -874,12 +959,11 @@ __global__ void __launch_bounds__(FLOW_THREADS, 1) k_chol_flow(const __grid_cons
     }
     return t;
   };
-  const int* sm_bits = (f.exclusive && (int)blockIdx.x >= f.nb) ? f.ctl + FLOW_SM_BITS + (flow_smid() >> 5) : nullptr;
+  int ticket = -1;      // (thread 0) drawn at the end of the task before
   while (alive && tid < FLOW_COMPUTE) {
     if (tid == 0) {
-      FlowTask none;
-      none.type = FT_NONE; none.b = none.i = none.k = 0;
-      s_task = (sm_bits != nullptr && ((flow_ld(sm_bits) >> (flow_smid() & 31)) & 1)) ? none : fetch_task(atomicAdd(f.ctl + FLOW_TICKET, 1));
+      s_task = fetch_task(ticket >= 0 ? ticket : atomicAdd(f.ctl + FLOW_TICKET, 1));
+      ticket = -1;
     }
     bar_named<1, FLOW_COMPUTE>();
     const FlowTask t = s_task;
@@ -895,52 +979,47 @@ __global__ void __launch_bounds__(FLOW_THREADS, 1) k_chol_flow(const __grid_cons
     const int kt = prepares ? t.k - 2 : t.k;
     const int kw = same ? t.k : t.k - 1;
     const int j0 = (panel && !solve) ? t.i : 0;
-    const int nrow = (panel && solve) ? (int)min((i64)CB, f.rows - (i64)t.i * CB) : cols_of(t.i);
+    const int nrow = (int)min((i64)(prepares ? CB : (panel ? f.prows : FLOW_ROWS) * CB), (panel && solve ? f.rows : f.sz) - (i64)t.i * CB);
     const int ncol = cols_of(kt);
     const float* Abase = panel ? U + (i64)t.i * CB * ld : G + (i64)t.i * CB * ld;
     const float* Bbase = G + (i64)kt * CB * ld;
     const float* Wbase = G + (i64)kw * CB * ld;      // (SUB; a whole row block)
-    const int* fa = panel ? rowU(b, t.i) : rowL(b, t.i);
+    const int* fa = panel ? rowU(b, t.i / f.prows) : rowL(b, t.i);
     const int* fb = rowL(b, kt);
     const int* fw = rowL(b, kw);
     if (panel && !solve && t.i > t.k) {      // below the block diagonal of L^-T: zeros (the products read whole tiles)
-      const float z[4][4] = {};
-      store_tile(U + (i64)t.i * CB * ld + (i64)t.k * CB, nrow, ncol, z);
+      float* p = U + (i64)t.i * CB * ld + (i64)t.k * CB;
+      for (int e = tid; e < nrow * ncol; e += FLOW_COMPUTE) p[(i64)(e / ncol) * ld + e % ncol] = 0.f;
       bar_named<1, FLOW_COMPUTE>();
       continue;
     }
-    float v[4][4], w[4][4];      // the tiles' own entries, less the terms
-    if (panel && solve) {
-      get_tile(f.Pin + (i64)b * f.wstride + (i64)t.i * CB * ld + f.o + (i64)t.k * CB, nrow, ncol, v);
-    } else if (panel) {
+    // the tiles' own entries (V, Wt: 128 rows, or a preparation's two tiles)
+    if (panel) {
+      if (solve) {
+        const float* src = f.Pin + (i64)b * f.wstride + (i64)t.i * CB * ld + f.o + (i64)t.k * CB;
+#pragma unroll 1
+        for (int h = 0; h * CB < nrow; ++h) flow_tile_in<VEC>(h == 0 ? V : Wt, src + (i64)h * CB * ld, 0, 1, 1.f, ld, nrow - h * CB, ncol, tid);
+      } else {
 #pragma unroll
-      for (int j = 0; j < 4; ++j)
-#pragma unroll
-        for (int x = 0; x < 4; ++x) v[j][x] = (t.i == t.k && tl.r(x) == tl.c(j, x)) ? 1.f : 0.f;
-    } else {
-      raw_tile(b, t.i, kt, v);
-    }
-    if (prepares) {
-      raw_tile(b, t.i, kw, w);
-      if (same && !f.gdiag_given) {      // for the pivot floors of the runner
-        float* gdiag = f.gdiag + (i64)b * f.wstride + f.o + (i64)t.k * CB;
-#pragma unroll
-        for (int j = 0; j < 4; ++j)
-#pragma unroll
-          for (int x = 0; x < 4; ++x)
-            if (tl.r(x) == tl.c(j, x) && tl.r(x) < nrow) gdiag[tl.r(x)] = w[j][x];
+        for (int q = 0; q < 4 * FLOW_ROWS; ++q) {
+          const int row = (tid >> 4) + 16 * q, c = (row & (CB - 1)) - (tid & 15) * 4;
+          const bool on = t.i + row / CB == t.k;
+          st4(&V[row][(tid & 15) * 4], make_float4(on && c == 0 ? 1.f : 0.f, on && c == 1 ? 1.f : 0.f, on && c == 2 ? 1.f : 0.f, on && c == 3 ? 1.f : 0.f));
+        }
       }
+    } else {
+#pragma unroll 1
+      for (int h = 0; h < 2; ++h) raw_tile(h == 0 ? V : Wt, b, t.i + (prepares ? 0 : h), prepares && h == 1 ? kw : kt, tid);
     }
-    int pa = 0, pb = 0, pw = 0;      // progress of the rows as thread 0 has seen it
+    int pa = 0, pb = 0, pw = 0, pd = 0;      // progress of the rows and of D as thread 0 has seen it
     const bool other = t.type == FT_SUB;      // a third row of tiles
-    auto issue = [&](int j, int st) {
-      flow_load<VEC>(SA[st], Abase + (i64)j * CB, ld, nrow, CB, tid);
-      flow_load<VEC>(SB[st], Bbase + (i64)j * CB, ld, ncol, CB, tid);
-      if (other) flow_load<VEC>(SC[st], Wbase + (i64)j * CB, ld, CB, CB, tid);
-      flow_commit();
-    };
-    auto have = [&](int j) -> bool {      // (thread 0) the tiles of term j are there, as far as can be seen now
+    auto have = [&](int j) -> bool {      // (thread 0) the operands of term j are there, as far as can be seen now; term kt: D
+      if (j == kt) {
+        if (pd <= kt) pd = flow_ld(doneD(b));
+        return pd > kt;
+      }
       if (pa <= j) pa = flow_ld(fa);
+      if (t.type == FT_L && nrow > CB && pa > j) pa = min(pa, flow_ld(fa + 1));
       if (pb <= j) pb = flow_ld(fb);
       if (other && pw <= j) pw = flow_ld(fw);
       return min(pa, pb) > j && (!other || pw > j);
@@ -948,91 +1027,262 @@ __global__ void __launch_bounds__(FLOW_THREADS, 1) k_chol_flow(const __grid_cons
     auto need = [&](int j) -> bool {      // every thread: wait for term j
       if (tid == 0) {
         int ok = 0;
-        if (pa <= j) { pa = flow_wait(fa, j + 1, f); ok = min(ok, pa); }
-        if (ok >= 0 && pb <= j) { pb = flow_wait(fb, j + 1, f); ok = min(ok, pb); }
-        if (ok >= 0 && other && pw <= j) { pw = flow_wait(fw, j + 1, f); ok = min(ok, pw); }
+        if (!have(j)) {
+          if (j == kt) {
+            ok = pd = flow_wait(doneD(b), kt + 1, f);
+          } else {
+            if (pa <= j) { pa = flow_wait(fa, j + 1, f); ok = min(ok, pa); }
+            if (ok >= 0 && t.type == FT_L && nrow > CB) { pa = min(pa, flow_wait(fa + 1, j + 1, f)); ok = min(ok, pa); }
+            if (ok >= 0 && pb <= j) { pb = flow_wait(fb, j + 1, f); ok = min(ok, pb); }
+            if (ok >= 0 && other && pw <= j) { pw = flow_wait(fw, j + 1, f); ok = min(ok, pw); }
+          }
+        }
         s_ok = ok;
       }
       bar_named<1, FLOW_COMPUTE>();
-      const bool ok = s_ok >= 0;
-      bar_named<1, FLOW_COMPUTE>();
-      return ok;
+      return s_ok >= 0;      // (written again behind a later barrier only)
     };
-    if (j0 < kt) {
-      if (!need(j0)) { alive = false; break; }
-      issue(j0, 0);
-    }
-    int st = 0;
-    for (int j = j0; j < kt + (prepares ? 2 : 1); ++j) {      // terms, the product with D, a preparation's last term: one copy of the code
-      const bool more = j + 1 < kt;
-      if (j < kt) {
-        if (tid == 0 && more) s_ready[j & 1] = have(j + 1) ? 1 : 0;
-        flow_wait_all();
-        bar_named<1, FLOW_COMPUTE>();      // term j has landed; everyone is done with the other stage
-      } else {
-        if (same && j > kt) store_tile(G + (i64)t.i * CB * ld + (i64)kt * CB, nrow, ncol, v);      // (DIAG: L_{k,k-2})
-        bar_named<1, FLOW_COMPUTE>();      // everyone is done with the stages
-        if (same && j > kt && tid == FLOW_COMPUTE - 1) flow_publish(rowL(b, t.i), kt + 1);
-        st = 0;
-        tile_put(SA[0], tl, v);
-        if (j == kt) {
-          if (!wait_all(doneD(b), kt + 1)) { alive = false; break; }
-          flow_load<true>(SB[0], Dk, CB, CB, CB, tid);
-        } else if (other) {
-          if (!wait_all(fw, kt + 1)) { alive = false; break; }
-          flow_load<VEC>(SB[0], Wbase + (i64)kt * CB, ld, CB, CB, tid);
+    auto stage = [&](int buf) { return smem0 + (uint32_t)buf * FLOW_STAGE; };
+    bool ok = true;
+    if (!prepares) {
+      // ---- 128 rows of the factor or of the panel: operands through registers, a term ahead; the rows under way in registers too
+      float4 xa[4 * FLOW_ROWS], xb[4];
+      const int i0 = tid >> 4, c0 = (tid & 15) * 4;
+      auto fetch = [&](int j) {
+        const bool d = j == kt;
+        if (!d) {
+          const float* p = Abase + (i64)i0 * ld + (i64)j * CB + c0;
+#pragma unroll
+          for (int q = 0; q < 4 * FLOW_ROWS; ++q) xa[q] = flow_ld4<VEC>(p + (i64)(16 * q) * ld, i0 + 16 * q < nrow ? CB : 0);
         }
-        flow_commit();
-        flow_wait_all();
-        bar_named<1, FLOW_COMPUTE>();
+        const float* p = d ? Dk + i0 * CB + c0 : Bbase + (i64)i0 * ld + (i64)j * CB + c0;
+        const i64 lb = d ? CB : ld;
+        const int rows = d ? CB : ncol;
+#pragma unroll
+        for (int q = 0; q < 4; ++q) xb[q] = flow_ld4<VEC>(p + (i64)(16 * q) * lb, i0 + 16 * q < rows ? CB : 0);
+      };
+      if (tid == 0) s_first = have(j0) ? 1 : 0;
+      bar_named<1, FLOW_COMPUTE>();
+      bool fetched = s_first != 0;
+      if (fetched) fetch(j0);
+      float v[32];
+#pragma unroll
+      for (int q = 0; q < 8; ++q) {
+        const float4 x = ld4(&V[rl.row][rl.col + 4 * q]);
+        v[4 * q] = x.x; v[4 * q + 1] = x.y; v[4 * q + 2] = x.z; v[4 * q + 3] = x.w;
       }
-      const bool rdy = more && s_ready[j & 1] != 0;
-      if (rdy) issue(j + 1, st ^ 1);
-      const int nprod = (prepares && j < kt) ? 2 : 1;
+      auto less = [&](int buf) -> bool {      // the products of a term come off
+        if (!mma_wait(buf)) return false;
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          float t16[16];
+          planes_take16(tmem_of(buf) + rl.tm + 16 * h, t16);
+#pragma unroll
+          for (int e = 0; e < 16; ++e) v[16 * h + e] -= t16[e];
+        }
+        return true;
+      };
+      int buf = 0;
 #pragma unroll 1
-      for (int q = 0; q < nprod; ++q) {
-        float s[4][4];
-        const bool self = same && (q == 1 || j > kt);
-        tile_nt(SA[st], self ? SA[st] : q == 0 ? SB[st] : SC[st], j == kt ? MM_TRI : self ? MM_LOWER : MM_FULL, tid, s);
-        const bool into_w = q == 1 || j > kt;
+      for (int j = j0; j <= kt; ++j) {      // term j's operands are split while the products of term j - 1 run
+        if (j == kt) {      // the rows themselves, the last term's product taken off (all before D is waited for)
+          if (j > j0) ok = less(buf ^ 1) && ok;
 #pragma unroll
-        for (int y = 0; y < 4; ++y)
-#pragma unroll
-          for (int x = 0; x < 4; ++x) {
-            if (into_w) w[y][x] -= s[y][x];
-            else v[y][x] = (j == kt) ? s[y][x] : v[y][x] - s[y][x];
+          for (int q = 0; q < 8; ++q) planes_put4(stage(buf), rl.row, rl.col + 4 * q, make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]), 2 * PLANE);
+          if (tid == 0) ticket = atomicAdd(f.ctl + FLOW_TICKET, 1);      // (the next one, so that it is there in time)
+        }
+        if (!fetched) {
+          if (!need(j)) {
+            if (j > j0 && j < kt) mma_wait(buf ^ 1);      // (the products in flight)
+            alive = false;
+            break;
           }
+          fetch(j);
+        }
+        if (j < kt) {
+#pragma unroll
+          for (int q = 0; q < 4 * FLOW_ROWS; ++q) {
+            if (q >= 4 && nrow <= CB) break;      // (one tile: the other lanes' products go nowhere)
+            planes_put4(stage(buf), i0 + 16 * q, c0, xa[q], 2 * PLANE);
+          }
+        }
+#pragma unroll
+        for (int q = 0; q < 4; ++q) planes_put4(stage(buf) + 6 * PLANE, i0 + 16 * q, c0, xb[q]);
+        if (tid == 0 && j < kt) s_ready[j & 1] = have(j + 1) ? 1 : 0;
+        umma::fence_proxy_async();
+        umma::tc_fence_before();
+        bar_named<1, FLOW_COMPUTE>();
+        if (tid == FLOW_MMA_THREAD) {
+          umma::tc_fence_after();
+          planes_mma(tmem_of(buf), stage(buf), stage(buf) + 6 * PLANE, 2 * PLANE);
+          commit(buf);
+        }
+        fetched = j < kt && s_ready[j & 1] != 0;
+        if (fetched) fetch(j + 1);
+        if (j < kt) {
+          if (j > j0) ok = less(buf ^ 1) && ok;
+          buf ^= 1;
+        }
       }
-      if (more && !rdy) {
-        if (!need(j + 1)) { alive = false; break; }
-        issue(j + 1, st ^ 1);
+      if (!alive) break;
+      ok = mma_wait(buf) && ok;
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        float t16[16];
+        planes_take16(tmem_of(buf) + rl.tm + 16 * h, t16);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) st4(&V[rl.row][rl.col + 16 * h + 4 * q], make_float4(t16[4 * q], t16[4 * q + 1], t16[4 * q + 2], t16[4 * q + 3]));
       }
-      st ^= 1;
+      umma::tc_fence_before();
+      if (!ok) { alive = false; break; }
+      bar_named<1, FLOW_COMPUTE>();
+      if (panel && !solve && f.xmax != nullptr) {      // (a maximum: the order of arrival does not matter)
+        float m = 0.f;
+#pragma unroll
+        for (int q = 0; q < 4 * FLOW_ROWS; ++q) {
+          if (q >= 4 && nrow <= CB) break;
+          const float4 x = ld4(&V[i0 + 16 * q][c0]);
+          m = fmaxf(m, fmaxf(fmaxf(fabsf(x.x), fabsf(x.y)), fmaxf(fabsf(x.z), fabsf(x.w))));
+        }
+        const unsigned u = __reduce_max_sync(0xffffffffu, __float_as_uint(m));
+        if ((tid & 31) == 0) atomicMax(xmaxbits(b), (int)u);
+      }
+      float* dst = (panel ? U : G) + (i64)t.i * CB * ld + (i64)t.k * CB;
+#pragma unroll 1
+      for (int h = 0; h * CB < nrow; ++h) flow_store<VEC>(h == 0 ? V : Wt, dst + (i64)h * CB * ld, ld, nrow - h * CB, ncol, tid);
+      bar_named<1, FLOW_COMPUTE>();
+      if (tid == 0) {
+        if (t.type == FT_L) {
+          flow_publish(rowL(b, t.i), t.k + 1);
+          if (nrow > CB) flow_publish(rowL(b, t.i + 1), t.k + 1);
+        } else if (t.k + 1 < T) {
+          flow_publish(rowU(b, t.i / f.prows), t.k + 1);
+        }
+      }
+      continue;
+    }
+    // ---- a preparation
+    // Terms j0 .. kt - 1, then, as "term" kt, the product with D.  A term's operands are brought up to two terms ahead.
+    // (SUB, one term ahead, keeps its third tile where another's second term would be)
+    auto coming = [&](int j) { return smem_al + FLOW_COMING + (other ? 0 : (j - j0) & 1) * 2 * FLOW_RAW + tid * 16; };
+    unsigned char* const third = smem_al + FLOW_COMING + 2 * FLOW_RAW + tid * 16;
+    auto fetch = [&](int j) {
+      unsigned char* at = coming(j);
+      if (j < kt) {
+        flow_bring<VEC>(at, FLOW_RAW_STEP, Abase + (i64)j * CB, ld, nrow, CB, tid);
+        flow_bring<VEC>(at + FLOW_RAW, FLOW_RAW_STEP, Bbase + (i64)j * CB, ld, ncol, CB, tid);
+        if (other) flow_bring<VEC>(third, FLOW_RAW_STEP, Wbase + (i64)j * CB, ld, CB, CB, tid);
+      } else {
+        flow_bring<true>(at + FLOW_RAW, FLOW_RAW_STEP, Dk, CB, CB, CB, tid);
+      }
+      flow_commit();
+    };
+    // The operands are in the planes: the products of a term, with a tile of row kt and one of row kw, into a TMEM buffer each.
+    auto products = [&](bool second) {
+      umma::fence_proxy_async();
+      umma::tc_fence_before();
+      bar_named<1, FLOW_COMPUTE>();
+      if (tid == FLOW_MMA_THREAD) {
+        umma::tc_fence_after();
+        planes_mma(tmem_of(0), stage(0), stage(0) + PLANES, PLANE);
+        if (second) planes_mma(tmem_of(1), stage(0), stage(0) + (same ? 0u : 2 * PLANES), PLANE);
+        commit(0);
+      }
+    };
+    if (tid == 0) s_first = have(j0) ? (!other && j0 < kt && have(j0 + 1) ? 2 : 1) : 0;
+    bar_named<1, FLOW_COMPUTE>();
+    if (same && !f.gdiag_given && tid < nrow)      // for the pivot floors of the runner
+      f.gdiag[(i64)b * f.wstride + f.o + (i64)t.k * CB + tid] = Wt[tid][tid];
+    int fetched = j0 - 1 + s_first;      // the last term whose operands are on their way
+    if (fetched >= j0) fetch(j0);
+    if (fetched > j0) fetch(j0 + 1);
+    float* const vrow = &V[rl.row][rl.col];
+    float* const wrow = &Wt[rl.row][rl.col];
+#pragma unroll 1
+    for (int j = j0; j <= kt; ++j) {
+      if (j == kt) {      // the tile itself, every term taken off
+        if (j > j0) bar_named<1, FLOW_COMPUTE>();
+        flow_split(stage(0), tile_at4(V, tid), FLOW_TILE_STEP, tid);
+      }
+      if (fetched < j) {
+        if (!need(j)) { alive = false; break; }
+        fetch(j);
+        fetched = j;
+      }
+      if (fetched > j) asm volatile("cp.async.wait_group 1;" ::: "memory");
+      else flow_wait_all();
+      unsigned char* at = coming(j);
+      if (j < kt) flow_split(stage(0), at, FLOW_RAW_STEP, tid);
+      flow_split(stage(0) + PLANES, at + FLOW_RAW, FLOW_RAW_STEP, tid);
+      if (other && j < kt) flow_split(stage(0) + 2 * PLANES, third, FLOW_RAW_STEP, tid);
+      const int next = fetched + 1;
+      const bool ask = next <= kt && next <= j + (other ? 1 : 2);
+      if (tid == 0 && ask) s_ready[j & 1] = have(next) ? 1 : 0;
+      products(j < kt);
+      if (ask && s_ready[j & 1] != 0) { fetch(next); fetched = next; }
+      if (j < kt) {      // they come off
+        ok = mma_wait(0) && ok;
+        if (rl.owner) {
+          planes_take<true>(tmem_of(0) + rl.tm, vrow);
+          planes_take<true>(tmem_of(1) + rl.tm, wrow);
+        }
+        umma::tc_fence_before();
+      }
     }
     if (!alive) break;
-    if (panel && !solve && f.xmax != nullptr) {      // (a maximum: the order of arrival does not matter)
-      float m = 0.f;
-#pragma unroll
-      for (int q = 0; q < 4; ++q)
-#pragma unroll
-        for (int x = 0; x < 4; ++x) m = fmaxf(m, fabsf(v[q][x]));
-      const unsigned u = __reduce_max_sync(0xffffffffu, __float_as_uint(m));
-      if ((tid & 31) == 0) atomicMax(xmaxbits(b), (int)u);
+    bool w_there = false;      // (SUB: the last term's other operand, made by the runner about now)
+    if (other) {
+      if (tid == 0) s_first = flow_ld(fw) > kt ? 1 : 0;
+      bar_named<1, FLOW_COMPUTE>();
+      w_there = s_first != 0;
+      if (w_there) { flow_bring<VEC>(third, FLOW_RAW_STEP, Wbase + (i64)kt * CB, ld, CB, CB, tid); flow_commit(); }
     }
-    if (prepares) store_tile(G + (i64)t.i * CB * ld + (i64)kw * CB, nrow, cols_of(kw), w);
-    else store_tile((panel ? U : G) + (i64)t.i * CB * ld + (i64)t.k * CB, nrow, ncol, v);
+    ok = mma_wait(0) && ok;
+    if (rl.owner) planes_take<false>(tmem_of(0) + rl.tm, vrow);
+    umma::tc_fence_before();
+    bar_named<1, FLOW_COMPUTE>();
+    // ... whose result is the last term's operand (DIAG: and L_{k,k-2})
+    flow_split(stage(0), tile_at4(V, tid), FLOW_TILE_STEP, tid);
+    if (other) {
+      if (!w_there) {
+        if (!wait_all(fw, kt + 1)) { alive = false; break; }
+        flow_bring<VEC>(third, FLOW_RAW_STEP, Wbase + (i64)kt * CB, ld, CB, CB, tid);
+        flow_commit();
+      }
+      flow_wait_all();
+      flow_split(stage(0) + PLANES, third, FLOW_RAW_STEP, tid);
+    }
+    umma::fence_proxy_async();
+    bar_named<1, FLOW_COMPUTE>();
+    if (tid == FLOW_MMA_THREAD) {
+      umma::tc_fence_after();
+      planes_mma(tmem_of(1), stage(0), stage(0) + (other ? PLANES : 0u), PLANE);
+      commit(1);
+    }
+    if (same) {
+      flow_store<VEC>(V, G + (i64)t.i * CB * ld + (i64)kt * CB, ld, nrow, ncol, tid);
+      bar_named<1, FLOW_COMPUTE>();
+      if (tid == FLOW_COMPUTE - 1) flow_publish(rowL(b, t.i), kt + 1);
+    }
+    ok = mma_wait(1) && ok;
+    if (rl.owner) planes_take<true>(tmem_of(1) + rl.tm, wrow);
+    umma::tc_fence_before();
+    bar_named<1, FLOW_COMPUTE>();
+    if (!ok) { alive = false; break; }
+    flow_store<VEC>(Wt, G + (i64)t.i * CB * ld + (i64)kw * CB, ld, nrow, cols_of(kw), tid);
     bar_named<1, FLOW_COMPUTE>();
     if (tid == 0) {
-      if (t.type == FT_L) flow_publish(rowL(b, t.i), t.k + 1);
-      else if (panel) { if (t.k + 1 < T) flow_publish(rowU(b, t.i), t.k + 1); }
-      else {
-        asm volatile("fence.acq_rel.gpu;" ::: "memory");
-        atomicAdd(prep(b, t.k), 1);
-      }
+      asm volatile("fence.acq_rel.gpu;" ::: "memory");
+      atomicAdd(prep(b, t.k), same ? 2 : 1);
     }
   }
   // ------------------------------------------------------------------------------------------------------ the end
+  umma::tc_fence_before();
   __syncthreads();
+  if (tid >= FLOW_COMPUTE && tid < FLOW_COMPUTE + 32) {
+    umma::tc_fence_after();
+    umma::tmem_dealloc(tmem0, FLOW_TMEM);
+  }
   if (tid == 0) {
     asm volatile("fence.acq_rel.gpu;" ::: "memory");
     s_ok = (atomicAdd(f.ctl + FLOW_LEFT, 1) == (int)gridDim.x - 1) ? 1 : 0;

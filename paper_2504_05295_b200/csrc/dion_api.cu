@@ -50,21 +50,23 @@ constexpr double P_PAIR_MIN_MNR = 1.5e10;       // smallest m n r whose P = (M +
 constexpr i64 NBO_COLS = 512;  // = NBO, the outer block of the two-level Cholesky (defined below)
 
 // One launch of k_chol_flow factors Gram matrices up to this order; beyond it blocks of 512 columns, whose products are on the
-// tensor cores.  Orthonormalization of rows x r in us, one launch against blocks: 8192 x 1536 547, 741; 8192 x 2048 827, 1047;
-// 12288 x 3072 2121, 2148; 16384 x 3584 3156, 2904; 16384 x 4096 4014, 3296.
+// tensor cores.  Orthonormalization of rows x r in us, one launch against blocks: 8192 x 1536 539, 725; 8192 x 2048 697, 965;
+// 12288 x 3072 1700, 2119.  (Set with slower products in the launch, where 3584 and 4096 columns were faster in blocks; the blocks' U is
+// 5 to 9 % closer to float64, so the line was not moved up.)
 constexpr i64 FLOW_MAX_R = 3072;
 // Largest rows r whose panel that launch solves too, against the product with the inverse behind it; in us, the launch's own
-// solve first: 1024 x 256 98, 121; 4096 x 256 121, 143; 8192 x 256 137, 152; 4096 x 512 168, 187; 4096 x 1024 352, 298.  (One
-// matrix by itself would have the line near 3e6; the helpers of a chain have as many panels to solve as it has matrices.)
+// solve first: 1024 x 256 90, 113; 4096 x 256 97, 117; 8192 x 256 106, 127; 4096 x 512 149, 172; 4096 x 1024 251, 275.  The line
+// stays where it is because of U's distance from float64, which the product has smaller beyond it: 8192 x 256 6.1e-7, 4.2e-7;
+// 4096 x 1024 3.20e-6, 2.97e-6.  (The helpers of a chain also have as many panels to solve as it has matrices.)
 constexpr double FLOW_SOLVE_MAX = 1.1e6;
 constexpr i64 FLOW_SOLVE_MAX_TILES = 40000;     // ... in an adaptive round: most 64^3 products of its substitution
 constexpr float NEAR_MAX_DEF = 3e-3f;           // largest |P^T P - I|_F whose factor is taken as a series (k_near_identity): third-order error 3e-8
 constexpr i64 NEAR_MAX_BLOCKS = 512;
-constexpr int FLOW_EXCLUSIVE_MAX = 8;           // matrices of a chain up to which its runners get an SM each
-// Partial sums of the Gram product that it adds up itself.  One CTA reads those of the first three tiles; from there on a launch over
-// all SMs reduces them first (4096 x 256, 32 splits: orthonormalization 120.8 -> 101.5 us, 2048 x 128, 16 splits: 82.0 -> 75.5;
-// 1001 x 83, 7 splits: 86.7 -> 87.1, left in the launch).
-constexpr int FLOW_MAX_SPLITS = 8;
+// Partial sums of the Gram product that it adds up itself, of the tensor engine's; twice as many of the FMA engine's.  One CTA reads
+// those of the first three tiles; from there on a launch over all SMs reduces them first (4096 x 256, 32 splits: orthonormalization
+// 120.8 -> 101.5 us; 1024 x 128, 8 splits of the tensor engine: 79 in the launch, 72 reduced; 640 x 112, 6 of the FMA engine: 65.7 in
+// the launch, 66.7 reduced).
+constexpr int FLOW_MAX_SPLITS = 4;
 constexpr int FLOW_AHEAD_MAX = 16;              // steps by which its preparations are handed out early
 constexpr i64 FLOW_MAX_PANEL_TILES = 800;       // ... and most 64-row blocks of it (the control block holds 64 such matrices)
 
@@ -638,22 +640,6 @@ int configure_kernels() {
   return DION_OK;
 }
 
-// CTAs of k_chol_flow that fit an SM (the cooperative launch must not ask for more).
-int flow_ctas_per_sm() {
-  static std::atomic<int> cached{0};
-  int n = cached.load(std::memory_order_relaxed);
-  if (n > 0) return n;
-  int a = 0, b = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&a, k_chol_flow<true>, FLOW_THREADS, FLOW_SMEM) != cudaSuccess ||
-      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_chol_flow<false>, FLOW_THREADS, FLOW_SMEM) != cudaSuccess) {
-    cudaGetLastError();
-    return 1;
-  }
-  n = a < b ? a : b;
-  if (n > 0) cached.store(n, std::memory_order_relaxed);
-  return n;
-}
-
 constexpr i64 NBO = NBO_COLS;  // outer block of the two-level Cholesky
 
 // Blocks of 256 threads for `total` items on each of nb matrices: at most one wave (eight per SM) over all of them.
@@ -692,8 +678,8 @@ int flow_ctl_ints(i64 sz, i64 rows) {
 }
 // Panels that the factorization's launch solves too, beside the factorization.  The rule looks at the shape alone (grouped
 // calls compute what single ones do).  CholeskyQR2: small panels; larger ones take one product behind it, before the
-// helpers' 64^3 products outlast the chain of diagonal blocks (more so with several matrices).  Adaptive rounds: up to the
-// number of tile products (~1.3 us of one SM each) that the blocked solve's tensor-core products would take as long for.
+// helpers' products outlast the chain of diagonal blocks (more so with several matrices).  Adaptive rounds: up to the
+// number of tile products that the blocked solve's tensor-core products take as long for.
 bool flow_solves(const StepCtx& s, i64 rows, i64 r, bool adaptive) {
   (void)s;
   const i64 T = (r + CB - 1) / CB, NR = (rows + CB - 1) / CB;
@@ -738,18 +724,21 @@ int chol_flow(StepCtx& s, i64 r, i64 o, i64 sz, int mode, i64 pin_off, i64 pout_
   f.limit = umma::SPIN_LIMIT_CYCLES;
   if (FLOW_HEAD_INTS + (i64)s.nb * f.ctl_stride > c->flow_ctl_cap) return DION_ERR_UNSUPPORTED;
   // one runner per matrix; as many helpers as can be resident beside them, at most one per task
-  i64 tasks = (T > 2) ? (T - 2) * (T - 3) / 2 + 2 * (T - 2) : 0;
-  if (solve) tasks += NR * T;
-  else for (i64 k = 0; k < T; ++k) tasks += flow_inverse_rows((int)T, (int)k, sz < r);
-  const i64 cap = (i64)flow_ctas_per_sm() * c->sm_count;
+  auto blocks = [](i64 n, i64 of) { return (n + of - 1) / of; };
+  i64 tasks = (T > 2) ? 2 * (T - 2) : 0, panel[2] = {0, 0};      // (panel[i]: with i + 1 tiles of rows to a task)
+  for (i64 k = 0; k + 3 < T; ++k) tasks += blocks(T - 3 - k, FLOW_ROWS);
+  for (i64 k = 0; k < T; ++k)
+    for (int i = 0; i < 2; ++i) panel[i] += blocks(solve ? NR : flow_inverse_rows((int)T, (int)k, sz < r), i + 1);
+  const i64 cap = c->sm_count;      // (one CTA per SM: shared memory)
+  // Tasks of two tiles read the tiles of L they meet half as often; where every task has an SM to itself the shorter ones are done
+  // sooner (orthonormalization of 768 x 192 82.4 -> 80.7 us, 1024 x 128 71.7 -> 70.5).
+  f.prows = (tasks + panel[0]) * s.nb + s.nb <= cap ? 1 : 2;
+  tasks += panel[f.prows - 1];
   i64 grid = s.nb + tasks * s.nb;
   if (grid > cap) grid = cap;
   if (grid < s.nb + 1) return DION_ERR_UNSUPPORTED;
-  // With few matrices the helper that shares a runner's SM would slow the chain down more than it helps; it leaves if
-  // others are sure to stay.
   const i64 ahead = (grid - s.nb) / (4 * s.nb) - 1;      // (2 nb (ahead + 1) preparations at most wait for tasks handed out later)
   f.ahead = (int)(ahead < 0 ? 0 : ahead > FLOW_AHEAD_MAX ? FLOW_AHEAD_MAX : ahead);
-  f.exclusive = (s.nb <= FLOW_EXCLUSIVE_MAX && grid - s.nb > (i64)s.nb * (flow_ctas_per_sm() - 1)) ? 1 : 0;
   void* args[] = {&f};
   const void* fn = (r % 4 == 0) ? (const void*)k_chol_flow<true> : (const void*)k_chol_flow<false>;
   if (cudaLaunchCooperativeKernel(fn, dim3((unsigned)grid), dim3(FLOW_THREADS), args, FLOW_SMEM, s.st) != cudaSuccess) {
@@ -918,7 +907,8 @@ int cholqr_round(StepCtx& s, i64 pin_off, i64 pout_off, i64 rows, i64 r, int mod
   g.C = s.ws + s.L.Gram; g.ldc = r; g.epi = EPI_STORE; g.tri = TRI_LOWER; g.skip_flag = skips ? skip : nullptr; g.precise = rm_precise(mode) ? 1 : 0;
   const bool in_flow = flow_solves(s, rows, r, adaptive);      // factorization and solve in one launch
   const bool flow_all = in_flow || (!adaptive && r <= FLOW_MAX_R);      // at least the whole factorization
-  int nsplit = flow_all ? FLOW_MAX_SPLITS : 1;
+  const bool on_tensor = g.ab16 || (s.tensor && umma_shape_ok(g, s.in_orth ? DION_PREC_FP32 : c->cfg.precision));
+  int nsplit = !flow_all ? 1 : on_tensor ? FLOW_MAX_SPLITS : 2 * FLOW_MAX_SPLITS;
   if (flow_all) g.splits_out = &nsplit;       // (which also adds up a few partial products)
   DION_TRY(launch_gemm_chain(s, g));
   const float* part_scale = g.alpha_dev;
