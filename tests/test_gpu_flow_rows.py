@@ -8,8 +8,6 @@ torch = pytest.importorskip("torch")
 from paper_2504_05295_b200 import binding  # noqa: E402
 from test_gpu_orth_sizes import test_against_float64 as check  # noqa: E402
 
-check.__test__ = False      # (collected in its own file)
-
 # rows, r: the panel solved in the launch (1 to 5 row blocks, 2 to 5 column blocks), then the inverse (rows r > 1.1e6)
 PANELS = [(128, 65), (129, 65), (192, 128), (193, 128), (256, 132), (260, 132), (1027, 250), (900, 257), (4100, 320), (5000, 321),
           (8200, 192), (8192, 196)]
