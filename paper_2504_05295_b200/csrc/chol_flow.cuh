@@ -191,6 +191,16 @@ __device__ __forceinline__ void bar_arrive() { asm volatile("bar.arrive %0, %1;"
 template <int ID, int N>
 __device__ __forceinline__ void bar_named() { asm volatile("bar.sync %0, %1;" ::"n"(ID), "n"(N) : "memory"); }
 
+// ... and whether v holds in any of the threads
+template <int ID, int N>
+__device__ __forceinline__ bool bar_any(bool v) {
+  int any;
+  asm volatile(
+      "{\n\t.reg .pred p, q;\n\tsetp.ne.s32 p, %1, 0;\n\tbar.red.or.pred q, %2, %3, p;\n\tselp.s32 %0, 1, 0, q;\n\t}"
+      : "=r"(any) : "r"((int)v), "n"(ID), "n"(N) : "memory");
+  return any != 0;
+}
+
 __device__ __forceinline__ float4 ld4(const float* p) { return *reinterpret_cast<const float4*>(p); }
 __device__ __forceinline__ void st4(float* p, float4 v) { *reinterpret_cast<float4*>(p) = v; }
 __device__ __forceinline__ void ld8(float (&v)[8], const float* p) {
@@ -492,7 +502,9 @@ __device__ __forceinline__ void potrf64(ctile_t L, ctile_t X, const Potrf64Set& 
 // Helper tasks are handed out in the order of steps (the panel's a few steps behind the factor's), so a task only
 // ever waits for tasks handed out before it and for the runners, which are resident: the launch is cooperative.  Only the
 // preparations are handed out `ahead` steps early; they hold no more than half of the helpers.  Every wait, those for the MMAs too,
-// has a cycle limit (then DION_STATUS_TIMEOUT and os[OS_FAIL], and every CTA leaves with its TMEM given back).
+// has a cycle limit (then DION_STATUS_TIMEOUT and os[OS_FAIL], and every CTA leaves with its TMEM given back).  Waits on other CTAs are
+// one thread's; those for the MMAs are every thread's own and may end differently, so a CTA goes on to a task's end and leaves behind
+// a barrier that tells all threads whether one of them has lost a wait.
 // The last CTA to leave clears the counters for the next launch and evaluates the round (adaptive rounds).
 // ---------------------------------------------------------------------------------------------------------------
 enum : int { FLOW_TICKET = 0, FLOW_LEFT = 1, FLOW_ABORT = 2, FLOW_HEAD_INTS = 32 };   // head of the control block
@@ -537,6 +549,7 @@ struct FlowArgs {
   float good_rel, done_rel;
   int* rounds_total;
   long long limit;
+  int lose_cta, lose;       // test hook: the first `lose` threads of that CTA (< 0: of every helper) say that they lost a wait
 };
 
 // End of an adaptive round (one thread).  `minrel`, the smallest pivot relative to its column's squared norm, estimates
@@ -679,7 +692,7 @@ static_assert(FLOW_COMING + 4 * FLOW_RAW <= FLOW_RESULTS && FLOW_STAGE + 4 * FLO
 constexpr int FLOW_SMEM = 1024 + (int)FLOW_RESULTS + 2 * FLOW_TILE;
 constexpr int FLOW_ROWS = 2;                  // tiles of rows that a task of the factor takes, and most of a task of the panel
 constexpr int FLOW_TMEM = 512;                // columns: two buffers of a product, or one of a preparation's two
-constexpr int FLOW_MMA_THREAD = 64;           // issues the MMAs (its warp holds no rows)
+constexpr int FLOW_MMA_THREAD = 64;           // issues the MMAs (of a warp that holds no rows of a 64-row tile)
 
 template <bool VEC>
 __global__ void __launch_bounds__(FLOW_THREADS, 1) k_chol_flow(const __grid_constant__ FlowArgs f) {
@@ -746,22 +759,20 @@ __global__ void __launch_bounds__(FLOW_THREADS, 1) k_chol_flow(const __grid_cons
   unsigned phase = 0;      // parities of s_bar, per buffer
   auto tmem_of = [&](int buf) { return tmem0 + (uint32_t)buf * 256u; };
   auto commit = [&](int buf) { umma::umma_commit(umma::smem_u32(&s_bar[buf])); };
-  // Every compute thread: the products of `buf` are done (false: the wait ran out; the launch is given up).
-  auto mma_wait = [&](int buf) -> bool {
+  // Every compute thread: the products of `buf` are done, or this thread has lost a wait.
+  bool lost = false;
+  auto mma_wait = [&](int buf) {
     const uint32_t bar = umma::smem_u32(&s_bar[buf]), par = (phase >> buf) & 1u;
     phase ^= 1u << buf;
-    bool ok = umma::mbar_try_wait(bar, par);
-    if (!ok) {
+    if (!umma::mbar_try_wait(bar, par)) {
       const long long t0 = clock64();
-      while (!(ok = umma::mbar_try_wait(bar, par)) && clock64() - t0 <= f.limit) {}
-      if (!ok) {
-        atomicExch(f.ctl + FLOW_ABORT, 1);
-        atomicOr(f.status_always, DION_STATUS_TIMEOUT);
-      }
+      while (!umma::mbar_try_wait(bar, par))
+        if (lost || clock64() - t0 > f.limit) { lost = true; break; }      // (waited for that long once only)
     }
+    __syncwarp();      // (the loads from TMEM that follow are a warp's)
     umma::tc_fence_after();
-    return ok;
   };
+  auto loses = [&]() -> bool { return lost || (tid < f.lose && (f.lose_cta < 0 ? (int)blockIdx.x >= f.nb : (int)blockIdx.x == f.lose_cta)); };
   bool alive = true;
   if ((int)blockIdx.x < f.nb) {
     // ------------------------------------------------------------------------------------------ runner of matrix b
@@ -884,7 +895,6 @@ __global__ void __launch_bounds__(FLOW_THREADS, 1) k_chol_flow(const __grid_cons
           const Potrf64Set& set = s_set[k & 1];
           if (k > 0) {
             // L_{k,k-1} = A' D_{k-1}^T (the deflated rows of D zeroed), then the last term of the diagonal block
-            bool ok = true;
             flow_split(PX, tile_at4(X, tid), FLOW_TILE_STEP, tid);
 #pragma unroll 1
             for (int h = 0; h < 2; ++h) {
@@ -896,7 +906,7 @@ __global__ void __launch_bounds__(FLOW_THREADS, 1) k_chol_flow(const __grid_cons
                 planes_mma(tmem_of(h), h == 0 ? PA : PL, h == 0 ? PX : PL, PLANE);
                 commit(h);
               }
-              ok = mma_wait(h) && ok;
+              mma_wait(h);
               if (h == 0) {
                 if (rl.owner) planes_take<false>(tmem_of(0) + rl.tm, &TS[rl.row][rl.col]);
                 bar_arrive<7, FLOW_THREADS>();      // (the service warps store it)
@@ -904,7 +914,7 @@ __global__ void __launch_bounds__(FLOW_THREADS, 1) k_chol_flow(const __grid_cons
                 flow_split(PL, tile_at4(TS, tid), FLOW_TILE_STEP, tid);
               }
             }
-            if (!ok) s_ok = -1;      // (seen behind the next step's barrier)
+            if (lost) s_ok = -1;      // (seen behind the next step's barrier)
             bar_named<9, FLOW_THREADS>();      // A'_kk is there
           }
           if (rl.owner) planes_diag(k > 0 ? tmem_of(1) + rl.tm : ~0u, &C(k)[rl.row][rl.col], &Lb[rl.row][rl.col], set.s2, rl.row, rl.col, nk);
@@ -1043,7 +1053,6 @@ __global__ void __launch_bounds__(FLOW_THREADS, 1) k_chol_flow(const __grid_cons
       return s_ok >= 0;      // (written again behind a later barrier only)
     };
     auto stage = [&](int buf) { return smem0 + (uint32_t)buf * FLOW_STAGE; };
-    bool ok = true;
     if (!prepares) {
       // ---- 128 rows of the factor or of the panel: operands through registers, a term ahead; the rows under way in registers too
       float4 xa[4 * FLOW_ROWS], xb[4];
@@ -1071,8 +1080,8 @@ __global__ void __launch_bounds__(FLOW_THREADS, 1) k_chol_flow(const __grid_cons
         const float4 x = ld4(&V[rl.row][rl.col + 4 * q]);
         v[4 * q] = x.x; v[4 * q + 1] = x.y; v[4 * q + 2] = x.z; v[4 * q + 3] = x.w;
       }
-      auto less = [&](int buf) -> bool {      // the products of a term come off
-        if (!mma_wait(buf)) return false;
+      auto less = [&](int buf) {      // the products of a term come off
+        mma_wait(buf);
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
           float t16[16];
@@ -1080,13 +1089,12 @@ __global__ void __launch_bounds__(FLOW_THREADS, 1) k_chol_flow(const __grid_cons
 #pragma unroll
           for (int e = 0; e < 16; ++e) v[16 * h + e] -= t16[e];
         }
-        return true;
       };
       int buf = 0;
 #pragma unroll 1
       for (int j = j0; j <= kt; ++j) {      // term j's operands are split while the products of term j - 1 run
         if (j == kt) {      // the rows themselves, the last term's product taken off (all before D is waited for)
-          if (j > j0) ok = less(buf ^ 1) && ok;
+          if (j > j0) less(buf ^ 1);
 #pragma unroll
           for (int q = 0; q < 8; ++q) planes_put4(stage(buf), rl.row, rl.col + 4 * q, make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]), 2 * PLANE);
           if (tid == 0) ticket = atomicAdd(f.ctl + FLOW_TICKET, 1);      // (the next one, so that it is there in time)
@@ -1120,12 +1128,12 @@ __global__ void __launch_bounds__(FLOW_THREADS, 1) k_chol_flow(const __grid_cons
         fetched = j < kt && s_ready[j & 1] != 0;
         if (fetched) fetch(j + 1);
         if (j < kt) {
-          if (j > j0) ok = less(buf ^ 1) && ok;
+          if (j > j0) less(buf ^ 1);
           buf ^= 1;
         }
       }
       if (!alive) break;
-      ok = mma_wait(buf) && ok;
+      mma_wait(buf);
 #pragma unroll
       for (int h = 0; h < 2; ++h) {
         float t16[16];
@@ -1134,8 +1142,7 @@ __global__ void __launch_bounds__(FLOW_THREADS, 1) k_chol_flow(const __grid_cons
         for (int q = 0; q < 4; ++q) st4(&V[rl.row][rl.col + 16 * h + 4 * q], make_float4(t16[4 * q], t16[4 * q + 1], t16[4 * q + 2], t16[4 * q + 3]));
       }
       umma::tc_fence_before();
-      if (!ok) { alive = false; break; }
-      bar_named<1, FLOW_COMPUTE>();
+      if (bar_any<1, FLOW_COMPUTE>(loses())) { alive = false; break; }
       if (panel && !solve && f.xmax != nullptr) {      // (a maximum: the order of arrival does not matter)
         float m = 0.f;
 #pragma unroll
@@ -1221,7 +1228,7 @@ __global__ void __launch_bounds__(FLOW_THREADS, 1) k_chol_flow(const __grid_cons
       products(j < kt);
       if (ask && s_ready[j & 1] != 0) { fetch(next); fetched = next; }
       if (j < kt) {      // they come off
-        ok = mma_wait(0) && ok;
+        mma_wait(0);
         if (rl.owner) {
           planes_take<true>(tmem_of(0) + rl.tm, vrow);
           planes_take<true>(tmem_of(1) + rl.tm, wrow);
@@ -1237,7 +1244,7 @@ __global__ void __launch_bounds__(FLOW_THREADS, 1) k_chol_flow(const __grid_cons
       w_there = s_first != 0;
       if (w_there) { flow_bring<VEC>(third, FLOW_RAW_STEP, Wbase + (i64)kt * CB, ld, CB, CB, tid); flow_commit(); }
     }
-    ok = mma_wait(0) && ok;
+    mma_wait(0);
     if (rl.owner) planes_take<false>(tmem_of(0) + rl.tm, vrow);
     umma::tc_fence_before();
     bar_named<1, FLOW_COMPUTE>();
@@ -1264,17 +1271,20 @@ __global__ void __launch_bounds__(FLOW_THREADS, 1) k_chol_flow(const __grid_cons
       bar_named<1, FLOW_COMPUTE>();
       if (tid == FLOW_COMPUTE - 1) flow_publish(rowL(b, t.i), kt + 1);
     }
-    ok = mma_wait(1) && ok;
+    mma_wait(1);
     if (rl.owner) planes_take<true>(tmem_of(1) + rl.tm, wrow);
     umma::tc_fence_before();
-    bar_named<1, FLOW_COMPUTE>();
-    if (!ok) { alive = false; break; }
+    if (bar_any<1, FLOW_COMPUTE>(loses())) { alive = false; break; }
     flow_store<VEC>(Wt, G + (i64)t.i * CB * ld + (i64)kw * CB, ld, nrow, cols_of(kw), tid);
     bar_named<1, FLOW_COMPUTE>();
     if (tid == 0) {
       asm volatile("fence.acq_rel.gpu;" ::: "memory");
       atomicAdd(prep(b, t.k), same ? 2 : 1);
     }
+  }
+  if (!alive && loses()) {
+    atomicExch(f.ctl + FLOW_ABORT, 1);
+    atomicOr(f.status_always, DION_STATUS_TIMEOUT);
   }
   // ------------------------------------------------------------------------------------------------------ the end
   umma::tc_fence_before();

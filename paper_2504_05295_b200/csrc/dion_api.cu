@@ -133,6 +133,7 @@ struct dion_ctx {
   };
   std::vector<GraphEntry> graphs;
   bool graphs_on = false;
+  int flow_lose_cta = 0, flow_lose = 0;      // test hook: see FlowArgs
   bool chain_batch = true;          // tensor-engine products of a grouped chain in one launch over its matrices
   cudaStream_t cap = nullptr;       // the stream the chains are captured on (never the caller's: it may be the legacy stream)
   float* graph_scalars = nullptr;   // MAX_GRAPHS device floats
@@ -722,6 +723,7 @@ int chol_flow(StepCtx& s, i64 r, i64 o, i64 sz, int mode, i64 pin_off, i64 pout_
   f.round_end = (round_end && adaptive) ? 1 : 0;
   f.good_rel = GOOD_REL; f.done_rel = DONE_REL; f.rounds_total = c->dev_ints + 2;
   f.limit = umma::SPIN_LIMIT_CYCLES;
+  f.lose_cta = c->flow_lose_cta; f.lose = c->flow_lose;
   if (FLOW_HEAD_INTS + (i64)s.nb * f.ctl_stride > c->flow_ctl_cap) return DION_ERR_UNSUPPORTED;
   // one runner per matrix; as many helpers as can be resident beside them, at most one per task
   auto blocks = [](i64 n, i64 of) { return (n + of - 1) / of; };
@@ -3188,6 +3190,14 @@ extern "C" int dion_debug_chunks(int64_t m, int64_t n, int64_t r, int64_t rows, 
   probe_chunks(L, rows, &chunks, &per);
   out[2] = chunks * per >= rows ? chunks : -1;
   out[3] = (L.probe_sums - L.probe_part) / (r * NPROBE);
+  return DION_OK;
+}
+
+extern "C" int dion_debug_flow_lose(dion_ctx* ctx, int cta, int threads) {
+  if (ctx == nullptr) return DION_ERR_INVALID;
+  ctx->flow_lose_cta = cta;
+  ctx->flow_lose = threads;
+  graphs_clear(ctx);
   return DION_OK;
 }
 

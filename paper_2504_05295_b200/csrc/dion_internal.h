@@ -52,6 +52,11 @@ int dion_debug_chunks(int64_t m, int64_t n, int64_t r, int64_t rows, int sm_coun
  * over all matrices of the chain (the results must not depend on it). */
 int dion_debug_chain_batch(struct dion_ctx* ctx, int on);
 
+/* In the Cholesky launches from now on, the first `threads` threads of block `cta` (-1: of every block but the first, the runner) report
+ * that a wait for tensor-core products ran out for them (the waits themselves are not cut short).  The block must leave as a whole, the
+ * launch end with DION_STATUS_TIMEOUT.  threads = 0: none. */
+int dion_debug_flow_lose(struct dion_ctx* ctx, int cta, int threads);
+
 #ifdef __cplusplus
 }
 #endif
