@@ -839,14 +839,14 @@ __global__ void __launch_bounds__(FLOW_THREADS, 1) k_chol_flow(const __grid_cons
                 break;
               }
             }
-            if (s_prep < 0) s_ok = -1;      // (every barrier up to the next step's is still met)
           }
           bar_named<8, FLOW_SERVICE>();
+          lost = lost || s_prep < 0;      // (every barrier up to the next step's is still met)
           return s_prep >= 0;
         };
         for (int k = 0; k <= T; ++k) {
-          bar_named<6, FLOW_THREADS>();      // step k may start: A'_{k,k-1} is there; D_{k-1} is stored
-          if (s_ok < 0) break;
+          // step k may start: A'_{k,k-1} is there, D_{k-1} is stored; and whether it does is the same to every thread
+          if (bar_any<6, FLOW_THREADS>(loses())) { alive = false; break; }
           if (sid == 0) publish_d(k);
           if (k == T) break;
           if (k > 0) {
@@ -888,8 +888,7 @@ __global__ void __launch_bounds__(FLOW_THREADS, 1) k_chol_flow(const __grid_cons
         raw_tile(C(0), b, 0, 0, tid);
         bar_named<5, FLOW_THREADS>();
         for (int k = 0; k <= T; ++k) {
-          bar_named<6, FLOW_THREADS>();
-          if (s_ok < 0) { alive = false; break; }
+          if (bar_any<6, FLOW_THREADS>(loses())) { alive = false; break; }
           if (k == T) break;
           const int nk = cols_of(k);
           const Potrf64Set& set = s_set[k & 1];
@@ -914,7 +913,6 @@ __global__ void __launch_bounds__(FLOW_THREADS, 1) k_chol_flow(const __grid_cons
                 flow_split(PL, tile_at4(TS, tid), FLOW_TILE_STEP, tid);
               }
             }
-            if (lost) s_ok = -1;      // (seen behind the next step's barrier)
             bar_named<9, FLOW_THREADS>();      // A'_kk is there
           }
           if (rl.owner) planes_diag(k > 0 ? tmem_of(1) + rl.tm : ~0u, &C(k)[rl.row][rl.col], &Lb[rl.row][rl.col], set.s2, rl.row, rl.col, nk);
@@ -926,8 +924,6 @@ __global__ void __launch_bounds__(FLOW_THREADS, 1) k_chol_flow(const __grid_cons
         }
       }
     }
-    __syncthreads();
-    alive = s_ok >= 0;
     __syncthreads();
   }
   // -------------------------------------------------------------------------------------------------- helper tasks

@@ -46,3 +46,10 @@ def _check(rows, r, short, cta, threads):
 @pytest.mark.parametrize("threads", [1, 40, 65, 200, 256])
 def test_helpers_leave_as_a_whole(rows, r, short, threads):
     _check(rows, r, short, -1, threads)
+
+
+@pytest.mark.parametrize("rows,r,short", PANELS + [(640, 112, 448)])
+@pytest.mark.parametrize("threads", [1, 65, 256, 257, 300])
+def test_runner_leaves_as_a_whole(rows, r, short, threads):
+    # (threads 256 on: its service warps too)
+    _check(rows, r, short, 0, threads)
