@@ -65,8 +65,10 @@ constexpr i64 NEAR_MAX_BLOCKS = 512;
 // Partial sums of the Gram product that it adds up itself, of the tensor engine's; twice as many of the FMA engine's.  One CTA reads
 // those of the first three tiles; from there on a launch over all SMs reduces them first (4096 x 256, 32 splits: orthonormalization
 // 120.8 -> 101.5 us; 1024 x 128, 8 splits of the tensor engine: 79 in the launch, 72 reduced; 640 x 112, 6 of the FMA engine: 65.7 in
-// the launch, 66.7 reduced).
+// the launch, 66.7 reduced; 1500 x 100, 9 of it: 80 and 77).  Of a Gram matrix of one tile up to sixteen: nothing else waits for that
+// CTA's loads (2048 x 16, 11 splits: 55.9 in the launch, 59.0 reduced; 3136 x 48, 14: 68.5 and 70.0; 9888 x 22, 24: 96.0 and 92.4).
 constexpr int FLOW_MAX_SPLITS = 4;
+constexpr int FLOW_MAX_SPLITS_ONE = 16;
 constexpr int FLOW_AHEAD_MAX = 16;              // steps by which its preparations are handed out early
 constexpr i64 FLOW_MAX_PANEL_TILES = 800;       // ... and most 64-row blocks of it (the control block holds 64 such matrices)
 
@@ -910,7 +912,7 @@ int cholqr_round(StepCtx& s, i64 pin_off, i64 pout_off, i64 rows, i64 r, int mod
   const bool in_flow = flow_solves(s, rows, r, adaptive);      // factorization and solve in one launch
   const bool flow_all = in_flow || (!adaptive && r <= FLOW_MAX_R);      // at least the whole factorization
   const bool on_tensor = g.ab16 || (s.tensor && umma_shape_ok(g, s.in_orth ? DION_PREC_FP32 : c->cfg.precision));
-  int nsplit = !flow_all ? 1 : on_tensor ? FLOW_MAX_SPLITS : 2 * FLOW_MAX_SPLITS;
+  int nsplit = !flow_all ? 1 : r <= CB ? FLOW_MAX_SPLITS_ONE : on_tensor ? FLOW_MAX_SPLITS : 2 * FLOW_MAX_SPLITS;
   if (flow_all) g.splits_out = &nsplit;       // (which also adds up a few partial products)
   DION_TRY(launch_gemm_chain(s, g));
   const float* part_scale = g.alpha_dev;

@@ -53,3 +53,22 @@ def test_probe_of_ranks_that_are_no_multiple_of_four(rows, r):
             torch.cuda.synchronize()
             assert rounds[0] <= opt.orth_rounds() <= rounds[1], spread
         assert opt.get_status() == (0, 0)
+
+
+@pytest.mark.parametrize("r", [4, 22, 64])
+def test_partial_sums_of_one_block_take_no_launch_of_their_own(r):
+    # rows as the inner dimension: the Gram product is cut in 8, 11 and 16 parts
+    launches = []
+    with binding.Dion(orth=binding.ORTH_CHOLQR2) as opt:
+        flag = torch.zeros(1, dtype=torch.int32, device="cuda")
+        for rows in (1024, 2048, 4096):
+            g = torch.Generator(device="cuda"); g.manual_seed(rows + r)
+            P = torch.randn(rows, r, generator=g, device="cuda")
+            l0 = opt.launch_count()
+            opt.orthonormalize(rows, r, rows, P, flag)
+            torch.cuda.synchronize()
+            launches.append(opt.launch_count() - l0)
+            E = P.double().t() @ P.double() - torch.eye(r, device="cuda", dtype=torch.float64)
+            assert E.norm().item() <= 2 * 3e-5 * r ** 0.5      # (as in test_gpu_orth_sizes.py)
+        assert opt.get_status() == (0, 0)
+    assert len(set(launches)) == 1, launches
