@@ -1966,6 +1966,9 @@ int umma_try_launch(const GemmArgs& g_in, int precision, int sm_count, float* pa
     p.kc = p.kb_per_split;
     p.kb_per_split = p.nkb;
     splits = 1;
+  } else {      // chains of equal length (19 K blocks in 10 + 9 instead of 16 + 3: what the adds truncate grows with a chain's length)
+    const int chains = (p.kb_per_split + p.kc - 1) / p.kc;
+    p.kc = (p.kb_per_split + chains - 1) / chains;
   }
   // 128 < N < 256 in 256-column tiles where those fill the chip: the products of operand pairs are bound by the tiles they read
   // from L2, and a row block of A is then read once instead of twice (48 of 768 x 192 x 768: 57 -> 50 us).  The splits above are

@@ -220,6 +220,18 @@ def test_bf16_arrays_epilogues_and_lower_triangle(lib):
     assert run(lib, 2, 1, 2048, 128, 2048, False, True, ab16=True) < 1e-5      # split-K
 
 
+@pytest.mark.parametrize("M,N,chain,parts,kw", [(2048, 2560, 1024, 1, {}), (2048, 2560, 1024, 1, {"variant": 4}),
+                                                (1024, 1280, 1024, 3, {}), (2048, 2560, 2048, 1, {"ab16": True})])
+def test_accumulation_chains_of_a_tile_are_of_equal_length(lib, M, N, chain, parts, kw):
+    # The tensor cores truncate each sum, so the distance from float64 grows in proportion to the length of a chain.  One K block
+    # more than a full chain makes two chains of half the length (17 + 16 or 33 / 2 blocks: 0.52 of the distance), not a full
+    # one and a rest (32 + 1: 0.97).
+    block = 64 if kw.get("ab16") else 32
+    full = run(lib, 2, 1 if kw.get("ab16") else 0, M, N, parts * chain, False, True, seed=1, **kw)
+    more = run(lib, 2, 1 if kw.get("ab16") else 0, M, N, parts * (chain + block), False, True, seed=1, **kw)
+    assert more < 0.75 * full, (more, full)
+
+
 @pytest.mark.parametrize("a_mn,b_mn", LAYOUTS)
 def test_split_accumulators_reach_fma_accuracy(lib, a_mn, b_mn):
     for (M, N, K) in [(512, 512, 1024), (640, 388, 2052), (256, 128, 4096)]:
