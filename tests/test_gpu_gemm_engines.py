@@ -213,6 +213,37 @@ def test_bf16_arrays_on_cta_pairs(lib, a_mn, b_mn):
         assert torch.equal(got[0], got[1]), (M, N, K, epi)
 
 
+@pytest.mark.parametrize("a_mn,b_mn", LAYOUTS)
+def test_bf16_arrays_of_several_chunks_on_cta_pairs(lib, a_mn, b_mn):
+    # plain stores over more than one accumulation chunk (2048 k): with B row-contiguous the pairs sum a tile's chunks in registers,
+    # the single-CTA tiles in memory: same bits.  Ragged rows and columns; K not split, or split in as many parts on either side (six:
+    # 12 tiles for 74 pairs, 24 for 148 CTAs; 1032 rows would have four and five, and other sums).
+    for (M, N, K) in [(8200, 520, 4160), (1016, 520, 16448)]:
+        got = []
+        err = run(lib, 2, 1, M, N, K, a_mn, b_mn, ab16=True, seed=M + K, out=got)
+        assert err < 1e-5, (M, N, K, err)
+        err1 = run(lib, 2, 1, M, N, K, a_mn, b_mn, ab16=True, seed=M + K, variant=4, out=got)
+        assert err1 < 1e-5, (M, N, K, err1)
+        assert torch.equal(got[0], got[1]), (M, N, K)
+
+
+@pytest.mark.parametrize("m,n,r,count", [(1024, 768, 256, 3), (776, 4608, 264, 4), (4608, 1032, 512, 2)])
+def test_bf16_operands_of_a_chain_equal_single_steps(m, n, r, count):
+    # ranks and heights that take CTA pairs for P and R
+    g = torch.Generator(device="cuda"); g.manual_seed(m + r)
+    rn = lambda *s: torch.randn(*s, generator=g, device="cuda")
+    mats = [(rn(m, n), rn(m, n), rn(m, n).to(torch.bfloat16), torch.nn.functional.normalize(rn(n, r), dim=0)) for _ in range(count)]
+    single = [tuple(t.clone() for t in a) for a in mats]
+    with binding.Dion(precision=binding.PREC_BF16_OPERANDS) as opt:
+        for X, M, G, Q in single:
+            opt.step(X, M, G, Q, 0.01)
+        opt.step_grouped(mats, 0.01)
+        assert opt.get_status() == (0, 0)
+    for k, (a, b) in enumerate(zip(single, mats)):
+        for name, u, v in zip("XMGQ", a, b):
+            assert torch.equal(u, v), f"matrix {k}: {name}"
+
+
 def test_bf16_arrays_epilogues_and_lower_triangle(lib):
     assert run(lib, 2, 1, 1024, 768, 256, False, False, ab16=True, epi=2, alpha=0.05) < 1e-5
     assert run(lib, 2, 1, 1024, 768, 256, False, False, ab16=True, epi=1, alpha=0.01) < 1e-5
