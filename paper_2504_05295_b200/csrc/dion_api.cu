@@ -50,14 +50,15 @@ constexpr double P_PAIR_MIN_MNR = 1.5e10;       // smallest m n r whose P = (M +
 constexpr i64 NBO_COLS = 512;  // = NBO, the outer block of the two-level Cholesky (defined below)
 
 // One launch of k_chol_flow factors Gram matrices up to this order; beyond it blocks of 512 columns, whose products are on the
-// tensor cores.  Orthonormalization of rows x r in us, one launch against blocks: 8192 x 1536 539, 725; 8192 x 2048 697, 965;
-// 12288 x 3072 1700, 2119.  (Set with slower products in the launch, where 3584 and 4096 columns were faster in blocks; the blocks' U is
-// 5 to 9 % closer to float64, so the line was not moved up.)
+// tensor cores.  Orthonormalization of rows x r in us, one launch against blocks, and U's distance from float64: 8192 x 2048 686, 958
+// (2.93, 2.72e-6); 12288 x 3072 1672, 2100 (2.93, 2.66e-6); 16384 x 3584 2380, 2838 (2.80, 2.57e-6); 16384 x 4096 2842, 3211 (2.95,
+// 2.65e-6).  The launch is faster beyond the line too; the line stays for U's distance, which the blocks have 8 to 10 % smaller.
 constexpr i64 FLOW_MAX_R = 3072;
 // Largest rows r whose panel that launch solves too, against the product with the inverse behind it; in us, the launch's own
-// solve first: 1024 x 256 90, 113; 4096 x 256 97, 117; 8192 x 256 106, 127; 4096 x 512 149, 172; 4096 x 1024 251, 275.  The line
-// stays where it is because of U's distance from float64, which the product has smaller beyond it: 8192 x 256 6.1e-7, 4.2e-7;
-// 4096 x 1024 3.20e-6, 2.97e-6.  (The helpers of a chain also have as many panels to solve as it has matrices.)
+// solve first, and U's distance from float64: 2048 x 128 71.7, 81.3 (3.3, 2.5e-7); 1024 x 256 90, 114 (3.9, 5.8e-7); 1536 x 384 113, 139
+// (3.7, 8.2e-7); 4096 x 256 98, 117 (3.3, 3.6e-7); beyond the line 8192 x 256 106, 128 (6.1, 4.2e-7); 4096 x 512 147, 170 (9.5, 8.4e-7);
+// 4096 x 1024 244, 272 (3.20, 2.97e-6).  The launch is faster on both sides; the line lies where the smaller distance goes from the
+// launch (but for 2048 x 128) to the product.  (The helpers of a chain also have as many panels to solve as it has matrices.)
 constexpr double FLOW_SOLVE_MAX = 1.1e6;
 constexpr i64 FLOW_SOLVE_MAX_TILES = 40000;     // ... in an adaptive round: most 64^3 products of its substitution
 constexpr float NEAR_MAX_DEF = 3e-3f;           // largest |P^T P - I|_F whose factor is taken as a series (k_near_identity): third-order error 3e-8
@@ -220,8 +221,8 @@ Layout make_layout(const dion_ctx* c, i64 m, i64 n, i64 r) {
   // split-K partials: the largest plain-store product of a step is max(m,n) x r
   i64 pf = 4 * (i64)c->sm_count * 64 * 64;
   // ... and enough for as many splits as give every SM work: 148 tiles of 64 x 64 held two splits of a 4096 x 256 product, which
-  // left more than half of the chip idle (from 4096^2: 50 us with two, 37 with four).  The fixed scratch keeps its size: what fits it is
-  // what fitted before.
+  // left more than half of the chip idle (from 4096^2: 50 us with two, 37 with four).  (By the shape's usual tiles; where a launch's
+  // own would want more, it takes as many as fit.)  The fixed scratch keeps its size: what fits it is what fitted before.
   if (c->form_sum) {
     const i64 need[4] = {umma_split_floats(m, r, n, false, c->sm_count), umma_split_floats(n, r, m, false, c->sm_count),
                          umma_split_floats(r, r, big, true, c->sm_count), pf};

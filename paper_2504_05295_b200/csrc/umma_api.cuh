@@ -41,7 +41,9 @@ inline i64 umma_split_count(i64 tiles, i64 workers, i64 nkb) {
 }
 constexpr i64 UMMA_PAIR_MIN_ROWS = 512;   // smallest output height given to CTA pairs
 constexpr i64 UMMA_PAIR_MIN_TRI = 2048;   // smallest lower-triangular output given to CTA pairs
-// Floats of partial sums that the splits of an M x N product take (an upper bound over the operand types).
+// Floats of partial sums that the splits of an M x N product take in the tiles that its shape usually gets and whole K blocks of 32.  Not
+// a bound: a product that its operands keep from CTA pairs (a bf16 addend, no tensor maps) has other tiles and may want more
+// splits (600 x 256: 29 against 24), K blocks that are not whole one more; the launch takes as many as the scratch holds.
 inline i64 umma_split_floats(i64 M, i64 N, i64 K, bool tri, int sm_count) {
   if (M < 128 || N < 64) return 0;
   const bool pairs = N >= 256 && M >= UMMA_PAIR_MIN_ROWS && (!tri || N >= UMMA_PAIR_MIN_TRI);

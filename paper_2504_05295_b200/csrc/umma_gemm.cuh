@@ -1538,6 +1538,7 @@ inline cudaError_t launch_lean_pair(const Params& p, int grid, cudaStream_t st) 
   cfg.attrs = attr; cfg.numAttrs = 2;
   return cudaLaunchKernelEx(&cfg, k_gemm_umma<256, A_MN, true, true, false, true, true, true, true, true, false>, p);
 }
+// (B row-index contiguous: updates of C in that layout, which the isolated tests of the engine ask for; the steps' have it k-contiguous)
 inline cudaError_t launch_d16_pair(const Params& p, bool a_mn, bool b_mn, int grid, cudaStream_t st) {
   if (!a_mn && !b_mn) return launch_d16_pair_one<false, false>(p, grid, st);
   if (!a_mn && b_mn) return launch_d16_pair_one<false, true>(p, grid, st);
