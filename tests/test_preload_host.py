@@ -37,6 +37,16 @@ def test_first_call_loads_what_the_step_launches():
     assert set(ELSEWHERE) <= launched
 
 
+def test_first_call_loads_every_instance_of_a_template():
+    # (also those that a helper launches for its caller: go(...))
+    api = source("dion_api.cu")
+    named = lambda text, call: {re.sub(r"\s", "", k) for k in re.findall(call + r"\((k_\w+(?:<[^>]*>)?)", text)}
+    launched = named(api, r"(?:launch_pdl|\bgo)")
+    assert {"k_probe_fused<true>", "k_probe_fused<false>", "k_gemm_simt<64,64,16,4,4,2,GemmSecond>"} <= launched
+    missing = launched - named(body(api, "bool preload_kernels()"), "touch_kernel")
+    assert {k for k in missing if k.split("<")[0] not in ELSEWHERE and "GemmTabs" not in k} == set()      # (GemmTabs: chains)
+
+
 def test_the_tensor_engine_loads_its_own_reduction():
     # a static kernel of a header is one kernel per translation unit
     umma = source("umma_gemm.cuh")
